@@ -325,10 +325,10 @@ void colour_config(ovl_ctx *c, int *cluster, int *slots) {
 }
 
 // Dynamic shared memory a solver CTA may use with 1 or 2 resident CTAs per SM
-// (the solver's static shared memory -- row-bucket offsets, reductions -- is
-// under 1 KB)
+// (the solver's static shared memory -- row-bucket offsets, reductions -- takes
+// up to 2.2 KB, the system 1 KB per CTA)
 int solve_smem_budget(ovl_ctx *c, int ctas_per_sm) {
-    return ctas_per_sm == 1 ? c->smem_optin - 2 * 1024 : (c->smem_per_sm / 2) - 3 * 1024;
+    return ctas_per_sm == 1 ? c->smem_optin - 2560 : (c->smem_per_sm / 2) - 3584;
 }
 
 // Shared-memory body slots per CTA (24 B each, the layout without masses: the
@@ -348,23 +348,30 @@ bool solve_masses_fit(ovl_ctx *c, int slots, int ctas_per_sm) {
 // Per-worker CTA counts for the default launch: every worker starts at the
 // fewest CTAs (1, 2, 3, 4, 6 or 8) whose shares of its bodies fit one CTA's
 // shared memory; while all CTAs still fit the SMs, the worker with the most
-// rows per CTA moves to the next count.  Workers with the same count form one launch, and
+// rows per CTA moves to the next count while kGrow allows.  Workers with the same count form one launch, and
 // the launches run side by side on the context's streams.  Every launch
 // shape gives the same bits (no implicit FMA contraction in the solver),
 // so the plan changes only the time.  Returns false when some worker does
 // not fit even 8 CTAs (the uniform launch then takes it to global memory).
-struct SolveClass { int C, first, count, slots; };
+struct SolveClass { int C, first, count, slots, rows; };
 
-// the growth stops at this many CTAs per worker (more only where a
-// worker's bodies need them), and leaves this many SMs unclaimed: clusters
-// must fit inside one GPC, so a launch that claims every SM can leave a
-// cluster waiting for a second wave
-#ifndef OVL_SOLVE_MAX_GROW
-#define OVL_SOLVE_MAX_GROW 4
-#endif
-#ifndef OVL_SOLVE_SM_SLACK
-#define OVL_SOLVE_SM_SLACK 8
-#endif
+// The growth leaves this many SMs unclaimed: clusters must fit inside one GPC,
+// so a launch that claims every SM can leave a cluster waiting for a second
+// wave.
+constexpr int kSolveSmSlack = 8;
+// A worker grows past one CTA above the first number of constraints, and
+// further, up to four, while its CTAs hold more than the second each (rows with a box end take
+// longer, so a context with boxes grows sooner).  A
+// colour step of one CTA costs about 900 cycles plus 3 per row; a cluster
+// adds its barrier (560 cycles against 95) and the traffic between its CTAs
+// (6 B per cycle), which fewer rows have to pay for.  Measured solves: 2
+// workers of 392 constraints 0.14 ms with one CTA each, 0.26 with four; 8 of
+// 906 (a chain) 0.19 and 0.31; 12 of 8600 0.63 with one and 0.50 with three or
+// four; 16 of 40,000 1.29 with four, 1.65 with eight (of which 15 clusters fit
+// at once); boxes: 16 of 4200 2.57 with one and 2.94 with four, 16 of 6100
+// 3.7 with one or two and 3.24 with four.
+constexpr double kGrow[2][2] = {{5000, 3000}, {3000, 1000}};   // [boxes][first, next]
+constexpr int kMaxGrow = 4;
 
 // CTA shapes of the per-class launches: threads, rows per thread, CTAs per SM
 struct SolveShape { int threads, unroll, per_sm; };
@@ -381,7 +388,7 @@ int default_solve_shape(const ovl_ctx *c) { return c->n_parts <= c->num_sms ? 0 
 // CTA count of every worker (shared by the colouring and the solve): the
 // fewest of kClusterSizes whose shares of its bodies fit `cap` slots; then,
 // while the total stays within `budget`, the worker with the most rows per
-// CTA moves to the next size (at most OVL_SOLVE_MAX_GROW).  Empty if some
+// CTA moves to the next size if it is worth one.  Empty if some
 // worker needs more than 8.  (Sizes 5 and 7 were tried: the workers of the
 // large pile need 1-4 CTAs each, so they changed no plan.)
 std::vector<int> plan_worker_counts(ovl_ctx *c, int cap, long long budget) {
@@ -408,7 +415,11 @@ std::vector<int> plan_worker_counts(ovl_ctx *c, int cap, long long budget) {
             std::pop_heap(heap.begin(), heap.end(), less);
             const int p = heap.back();
             const int up = next(C[p]);
-            if (!up || up > OVL_SOLVE_MAX_GROW || total + (up - C[p]) > budget) break;
+            if (load(p) < kGrow[c->has_boxes][C[p] > 1]) {
+                heap.pop_back();
+                continue;
+            }
+            if (!up || up > kMaxGrow || total + (up - C[p]) > budget) break;
             total += up - C[p];
             C[p] = up;
             std::push_heap(heap.begin(), heap.end(), less);
@@ -432,10 +443,13 @@ void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveC
     classes.clear();
     for (int i = 0; i < P; ++i) {
         const int p = order[i], nb = pb[p + 1] - pb[p];
-        if (classes.empty() || classes.back().C != C[p]) classes.push_back({C[p], i, 0, 1});
+        if (classes.empty() || classes.back().C != C[p]) classes.push_back({C[p], i, 0, 1, 0});
         SolveClass &k = classes.back();
         k.count++;
         k.slots = std::max(k.slots, (nb + C[p] - 1) / C[p]);
+        // a CTA's rows: the worker's even share, plus a quarter for uneven owners
+        const int np = pp[p + 1] - pp[p];
+        k.rows = std::max(k.rows, C[p] == 1 ? np : (int)(1.25 * np / C[p]) + 64);
     }
     std::vector<uint32_t> o(order.begin(), order.end());
     upload(buf, o.data(), o.size(), c->stream);
@@ -473,7 +487,7 @@ long long fewest_ctas(ovl_ctx *c, int cap) {
 // masses.  (Measured on the large pile: planning 32 B per body past one wave
 // made the solve up to 40 % slower than the 24 B plan.)
 bool plan_solve_classes(ovl_ctx *c, const SolveShape &shape, std::vector<SolveClass> &classes) {
-    const long long budget = (long long)shape.per_sm * c->num_sms - OVL_SOLVE_SM_SLACK;
+    const long long budget = (long long)shape.per_sm * c->num_sms - kSolveSmSlack;
     const long long slots = (long long)shape.per_sm * c->num_sms;
     const int cap_plain = solve_slot_capacity(c, shape.per_sm);
     int cap = cap_plain;
@@ -532,8 +546,9 @@ void launch_solve_classes(ovl_ctx *c, const SolveArgs &a, const SolveShape &shap
         b.n_parts = classes[k].count;
         b.order = c->class_order.p + classes[k].first;
         b.smem_slots = classes[k].slots;
-        launch_solve(b, shape.threads, classes[k].C, shape.unroll,
-                     solve_masses_fit(c, classes[k].slots, shape.per_sm), sk);
+        b.smem_rows = classes[k].rows;
+        launch_solve(b, shape.threads, classes[k].C, shape.unroll, solve_masses_fit(c, classes[k].slots, shape.per_sm),
+                     solve_smem_budget(c, shape.per_sm), sk);
     }, class_launch_order(c, classes));
 }
 
@@ -563,7 +578,7 @@ void phase_colour(ovl_ctx *c) {
     const bool fixed = c->P.pgs_cluster > 0 || c->P.smem_slot_limit > 0;
     std::vector<SolveClass> classes;
     if (!fixed && P > 0 &&
-        plan_worker_classes(c, colour_smem_capacity(c), (long long)c->num_sms - OVL_SOLVE_SM_SLACK,
+        plan_worker_classes(c, colour_smem_capacity(c), (long long)c->num_sms - kSolveSmSlack,
                             classes, c->colour_order)) {
         run_on_streams(c, classes.size(), [&](size_t k, cudaStream_t sk) {
             ColourArgs b = a;
@@ -713,11 +728,15 @@ void apply_solve_order(ovl_ctx *c, const SolvePlan &pl) {
         std::fill(M.begin(), M.end(), solve_masses_fit(c, pl.slots, solve_ctas_per_sm(pl.unroll)) ? 1 : 0);
     }
     upload(c->solve_M, M.data(), (size_t)P, c->stream);
+    // the bank order is for k_solve_m's rows
+    if (c->has_boxes) std::fill(M.begin(), M.end(), 0);
+    upload(c->solve_banked, M.data(), (size_t)P, c->stream);
     c->col_off2.ensure((size_t)P * OWNER_NB + 1);
     c->pair_of_row2.ensure((size_t)c->npairs + 1);
     c->row_owner.ensure((size_t)c->npairs + 1);
-    launch_row_owner(P, c->part_bstart.p, c->part_ncol.p, c->solve_C.p, c->col_off.p, c->pair_of_row.p,
-                     c->p_slot.p, c->row_owner.p, c->pair_of_row2.p, c->col_off2.p, c->stream);
+    c->row_by_owner.ensure((size_t)c->npairs + 1);
+    launch_row_owner(P, c->part_bstart.p, c->part_ncol.p, c->solve_C.p, c->col_off.p, c->pair_of_row.p, c->p_slot.p,
+                     c->solve_banked.p, c->row_owner.p, c->row_by_owner.p, c->pair_of_row2.p, c->col_off2.p, c->stream);
 }
 
 void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int iters) {
@@ -744,7 +763,8 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
     }
     a.smem_slots = pl.slots;
     const bool masses = solve_masses_fit(c, pl.slots, solve_ctas_per_sm(pl.unroll));
-    launch_solve(a, pl.threads, pl.cluster, pl.unroll, masses, c->stream);
+    a.smem_rows = *std::max_element(c->h_pp.begin(), c->h_pp.end());
+    launch_solve(a, pl.threads, pl.cluster, pl.unroll, masses, solve_smem_budget(c, solve_ctas_per_sm(pl.unroll)), c->stream);
     c->last_ctas = (long long)pl.cluster * P;
     c->last_ctas_masses = masses ? c->last_ctas : 0;
     c->last_cluster = pl.cluster;
@@ -1090,8 +1110,8 @@ void release_all(ovl_ctx *c) {
     c->ball_root.release(); c->ball_size.release(); c->ball_start.release(); c->ball_vtx.release();
     c->ball_list.release();
     c->worker_order.release(); c->wk.release(); c->wk2.release(); c->wv2.release();
-    c->class_order.release(); c->colour_order.release(); c->solve_C.release(); c->solve_M.release(); c->col_off2.release();
-    c->row_owner.release();
+    c->class_order.release(); c->colour_order.release(); c->solve_C.release(); c->solve_M.release(); c->solve_banked.release(); c->col_off2.release();
+    c->row_owner.release(); c->row_by_owner.release();
     c->pair_of_row2.release(); c->lb_loads.release();
     c->half.release(); c->iib.release(); c->c_p.release(); c->row_full.release(); c->rfull.release();
 }

@@ -103,9 +103,12 @@ __device__ __forceinline__ int body_slot(const MemberArgs &a, int x, int w) {
     return a.entry_slot[e];
 }
 
-// One block per (worker, colour); warp w takes the w-th contiguous chunk of
-// the colour's rows.  A row's owner is the CTA that holds its first dynamic
-// body.  The warps count their rows per (owner rank, kind); a colour step
+// The rows of every colour in the order the solve takes them.  A block takes a
+// worker's colours in turn; warp w takes the w-th contiguous chunk of a
+// colour's (or a bucket's) rows.
+//
+// Owners (C > 1): a row's owner is the CTA that holds its first dynamic body.
+// The warps count their rows per (owner rank, kind); a colour step
 // lasts as long as its fullest CTA, so a CTA with more rows of a kind than
 // the even share (total / C) passes half of the excess on: it keeps its own
 // rows up to its new share, in order, and the rows beyond it go, in order, to
@@ -115,34 +118,40 @@ __device__ __forceinline__ int body_slot(const MemberArgs &a, int x, int w) {
 // balance gained.)  Buckets
 // are laid out rank by rank (contacts, then joints).  Rows of one colour are
 // independent, so any assignment gives the same result.
+//
+// Order inside a bucket's contacts: rows with a body in another CTA's shared
+// memory first (their latency then runs beside the local rows), then the
+// local rows so that eight consecutive ones name bodies in eight different
+// 16-byte bank groups, on both sides: rows with the same d = (slot_b - slot_a)
+// mod 8 together, and inside a d the slots a mod 8 in turn.  Row order was
+// canonical before, and eight random slots meet 2.6 deep in the fullest bank
+// group: shared memory's data path was 58 % busy at 114 wavefronts per 32
+// rows, of which 41 are needed; now 59 (a solve of 12 one-CTA workers 0.82 ->
+// 0.59 ms, the large pile's 1.24 -> 0.94 ms with the local and remote paths
+// apart).  Only for launches with the masses in shared memory: at 24 B per
+// slot the large pile's late solve (3.9 ms) gained nothing from it, and the
+// order takes 0.14 ms there.
 constexpr int OWNER_THREADS = 256, OWNER_WARPS = OWNER_THREADS / 32;
+constexpr int OWNER_GRID_Y = 16;   // blocks per worker, colours round robin
+constexpr int BANK_KEYS = 65;      // remote rows, then (d, slot_a mod 8)
 
-__global__ void __launch_bounds__(OWNER_THREADS)
-k_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solve_C,
-            const int *off_in, const int *pair_of_row, const int2 *p_slot, uint8_t *owner_of_row,
-            int *pair_of_row_out, int *off_out) {
+struct OwnerShared {
+    int cnt[OWNER_WARPS][2 * OWNER_RANKS];   // a warp's rows per (owner, kind), then its first index in the group
+    int total[2 * OWNER_RANKS], share[2 * OWNER_RANKS], start[2 * OWNER_RANKS], exc0[2 * OWNER_RANKS],
+        def0[2 * OWNER_RANKS];
+    int bcnt[OWNER_WARPS][BANK_KEYS];        // the same per bank key
+    int btot[BANK_KEYS], dbase[8];
+};
+
+// rows [s0, s2) of one colour (joints from s1) to their owners' buckets:
+// src -> dst, the buckets' offsets to o2
+__device__ void colour_owners(OwnerShared &sh, int C, int per, int s0, int s1, int s2, const int *src, const int2 *p_slot,
+                              uint8_t *key_of_row, int *dst, int *o2) {
     constexpr int NK = 2 * OWNER_RANKS;
-    __shared__ int cnt[OWNER_WARPS][NK];    // a warp's rows per (owner, kind), then its first index in the group
-    __shared__ int total[NK], share[NK], start[NK], exc0[NK], def0[NK];
-    const int p = blockIdx.x, c = blockIdx.y;
-    if (p >= P) return;
-    const int ncol = part_ncol[p];
-    const int *off = off_in + (size_t)p * (2 * OVL_MAX_COLOURS + 1);
-    int *o2 = off_out + (size_t)p * OWNER_NB;
-    const int end = off[2 * ncol];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (c >= ncol) {
-        if (tid < NK) o2[c * NK + tid] = end;
-        if (c == OVL_MAX_COLOURS - 1 && tid == 0) o2[OWNER_NB - 1] = end;
-        return;
-    }
-    const int nb = part_bstart[p + 1] - part_bstart[p];
-    const int C = max(1, min(solve_C[p], OWNER_RANKS));
-    const int per = max(1, (nb + C - 1) / C);
-    const int s0 = off[2 * c], s1 = off[2 * c + 1], s2 = off[2 * c + 2];
     const int chunk = (s2 - s0 + OWNER_WARPS - 1) / OWNER_WARPS;
     const int w0 = min(s2, s0 + warp * chunk), w1 = min(s2, w0 + chunk);
-    if (lane < NK) cnt[warp][lane] = 0;
+    if (lane < NK) sh.cnt[warp][lane] = 0;
     __syncwarp();
     const unsigned full = 0xffffffffu;
     const unsigned lt = (1u << lane) - 1u;
@@ -151,13 +160,13 @@ k_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solv
         const int r = b + lane;
         int key = -1;
         if (r < w1) {
-            const int2 sl = p_slot[pair_of_row[r]];
+            const int2 sl = p_slot[src[r]];
             const int sa = sl.x >= 0 ? sl.x : max(sl.y, 0);
             key = 2 * min(sa / per, C - 1) + (r >= s1 ? 1 : 0);
-            owner_of_row[r] = (uint8_t)key;
+            key_of_row[r] = (uint8_t)key;
         }
         const unsigned peers = __match_any_sync(full, key);
-        if (key >= 0 && (peers & lt) == 0) cnt[warp][key] += __popc(peers);
+        if (key >= 0 && (peers & lt) == 0) sh.cnt[warp][key] += __popc(peers);
         __syncwarp();
     }
     __syncthreads();
@@ -165,70 +174,180 @@ k_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solv
         for (int k = 0; k < NK; ++k) {
             int t = 0;
             for (int w = 0; w < OWNER_WARPS; ++w) {   // counts -> each warp's first index in its group
-                const int x = cnt[w][k];
-                cnt[w][k] = t;
+                const int x = sh.cnt[w][k];
+                sh.cnt[w][k] = t;
                 t += x;
             }
-            total[k] = t;
+            sh.total[k] = t;
         }
         for (int kind = 0; kind < 2; ++kind) {
             int all = 0;
-            for (int r = 0; r < OWNER_RANKS; ++r) all += total[2 * r + kind];
+            for (int r = 0; r < OWNER_RANKS; ++r) all += sh.total[2 * r + kind];
             // a CTA above the even share passes on half of its excess; the
             // CTAs below it take those rows in rank order
             int moved = 0;
             for (int r = 0; r < OWNER_RANKS; ++r) {
                 const int k = 2 * r + kind;
                 const int even = r < C ? all / C + (r < all % C ? 1 : 0) : 0;
-                share[k] = total[k] > even ? total[k] - (total[k] - even) / 2 : even;
-                moved += total[k] - min(total[k], share[k]);
+                sh.share[k] = sh.total[k] > even ? sh.total[k] - (sh.total[k] - even) / 2 : even;
+                moved += sh.total[k] - min(sh.total[k], sh.share[k]);
             }
             int e = 0, d = 0;
             for (int r = 0; r < OWNER_RANKS; ++r) {
                 const int k = 2 * r + kind;
-                if (share[k] > total[k]) {
-                    const int take = min(share[k] - total[k], moved);
-                    share[k] = total[k] + take;
+                if (sh.share[k] > sh.total[k]) {
+                    const int take = min(sh.share[k] - sh.total[k], moved);
+                    sh.share[k] = sh.total[k] + take;
                     moved -= take;
                 }
-                exc0[k] = e;
-                def0[k] = d;
-                e += max(0, total[k] - share[k]);
-                d += max(0, share[k] - total[k]);
+                sh.exc0[k] = e;
+                sh.def0[k] = d;
+                e += max(0, sh.total[k] - sh.share[k]);
+                d += max(0, sh.share[k] - sh.total[k]);
             }
         }
         int pos = s0;
         for (int k = 0; k < NK; ++k) {
-            start[k] = pos;
-            o2[c * NK + k] = pos;
-            pos += share[k];
+            sh.start[k] = pos;
+            o2[k] = pos;
+            pos += sh.share[k];
         }
-        if (c == OVL_MAX_COLOURS - 1) o2[OWNER_NB - 1] = end;
     }
     __syncthreads();
     for (int b = w0; b < w1; b += 32) {
         const int r = b + lane;
-        const int key = r < w1 ? (int)owner_of_row[r] : -1;
+        const int key = r < w1 ? (int)key_of_row[r] : -1;
         const unsigned peers = __match_any_sync(full, key);
         if (key >= 0) {
-            const int idx = cnt[warp][key] + __popc(peers & lt);   // index in its (owner, kind) group
-            int dst;
-            if (idx < share[key]) {
-                dst = start[key] + idx;
+            const int idx = sh.cnt[warp][key] + __popc(peers & lt);   // index in its (owner, kind) group
+            int to;
+            if (idx < sh.share[key]) {
+                to = sh.start[key] + idx;
             } else {
                 // the e-th row beyond its owner's share (over owners in rank
                 // order) fills the e-th free place of the same kind
                 const int kind = key & 1;
-                const int e = exc0[key] + (idx - share[key]);
+                const int e = sh.exc0[key] + (idx - sh.share[key]);
                 int k = kind;
-                while (k + 2 < NK && def0[k + 2] <= e) k += 2;
-                dst = start[k] + total[k] + (e - def0[k]);
+                while (k + 2 < NK && sh.def0[k + 2] <= e) k += 2;
+                to = sh.start[k] + sh.total[k] + (e - sh.def0[k]);
             }
-            pair_of_row_out[dst] = pair_of_row[r];
+            dst[to] = src[r];
         }
         __syncwarp();
-        if (key >= 0 && (peers & lt) == 0) cnt[warp][key] += __popc(peers);
+        if (key >= 0 && (peers & lt) == 0) sh.cnt[warp][key] += __popc(peers);
         __syncwarp();
+    }
+    __syncthreads();
+}
+
+// the contacts [r0, r1) of CTA k's bucket in bank order: src -> dst
+__device__ void bucket_banks(OwnerShared &sh, int k, int per, int r0, int r1, const int *src, const int2 *p_slot,
+                             uint8_t *key_of_row, int *dst) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int chunk = (r1 - r0 + OWNER_WARPS - 1) / OWNER_WARPS;
+    const int w0 = min(r1, r0 + warp * chunk), w1 = min(r1, w0 + chunk);
+    for (int i = lane; i < BANK_KEYS; i += 32) sh.bcnt[warp][i] = 0;
+    __syncwarp();
+    const unsigned full = 0xffffffffu;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int b = w0; b < w1; b += 32) {
+        const int r = b + lane;
+        int key = -1;
+        if (r < w1) {
+            const int2 sl = p_slot[src[r]];
+            // indexes in the CTA's range; a static end reads the zero slot `per`
+            const int x = sl.x >= 0 ? sl.x - k * per : per, y = sl.y >= 0 ? sl.y - k * per : per;
+            const bool remote = x < 0 || x > per || y < 0 || y > per || (sl.x >= 0 && x == per) || (sl.y >= 0 && y == per);
+            key = remote ? 0 : 1 + 8 * ((y - x) & 7) + (x & 7);
+            key_of_row[r] = (uint8_t)key;
+        }
+        const unsigned peers = __match_any_sync(full, key);
+        if (key >= 0 && (peers & lt) == 0) sh.bcnt[warp][key] += __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    if (tid < BANK_KEYS) {
+        int t = 0;
+        for (int w = 0; w < OWNER_WARPS; ++w) {
+            const int x = sh.bcnt[w][tid];
+            sh.bcnt[w][tid] = t;
+            t += x;
+        }
+        sh.btot[tid] = t;
+    }
+    __syncthreads();
+    if (tid < 8) {
+        int t = r0 + sh.btot[0];
+        for (int i = 1; i <= 8 * tid; ++i) t += sh.btot[i];
+        sh.dbase[tid] = t;
+    }
+    __syncthreads();
+    for (int b = w0; b < w1; b += 32) {
+        const int r = b + lane;
+        const int key = r < w1 ? (int)key_of_row[r] : -1;
+        const unsigned peers = __match_any_sync(full, key);
+        if (key >= 0) {
+            const int i = sh.bcnt[warp][key] + __popc(peers & lt);   // index among the key's rows
+            int to = r0 + i;
+            if (key > 0) {
+                // the i-th row of slot_a mod 8 = g comes in round i of its d, after the smaller g of that round
+                const int d = (key - 1) >> 3, g = (key - 1) & 7;
+                to = sh.dbase[d];
+#pragma unroll
+                for (int h = 0; h < 8; ++h) {
+                    const int n = sh.btot[1 + 8 * d + h];
+                    to += min(n, i) + (h < g && n > i ? 1 : 0);
+                }
+            }
+            dst[to] = src[r];
+        }
+        __syncwarp();
+        if (key >= 0 && (peers & lt) == 0) sh.bcnt[warp][key] += __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(OWNER_THREADS)
+k_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solve_C, const int *off_in,
+            const int *pair_of_row, const int2 *p_slot, const int *banked, uint8_t *key_of_row, int *by_owner,
+            int *pair_of_row_out, int *off_out) {
+    __shared__ OwnerShared sh;
+    const int p = blockIdx.x;
+    const int ncol = part_ncol[p];
+    const int *off = off_in + (size_t)p * (2 * OVL_MAX_COLOURS + 1);
+    int *o2 = off_out + (size_t)p * OWNER_NB;
+    const int nb = part_bstart[p + 1] - part_bstart[p];
+    const int C = max(1, min(solve_C[p], OWNER_RANKS));
+    const int per = max(1, (nb + C - 1) / C);
+    if (blockIdx.y == 0 && threadIdx.x == 0) {
+        o2[OWNER_NB - 1] = off[2 * ncol];
+        if (ncol == 0) o2[0] = off[0];
+    }
+    for (int c = blockIdx.y; c < ncol; c += gridDim.y) {
+        const int s0 = off[2 * c], s1 = off[2 * c + 1], s2 = off[2 * c + 2];
+        int *oc = o2 + c * 2 * OWNER_RANKS;
+        const int *src = pair_of_row;
+        if (C == 1) {
+            if (threadIdx.x < 2 * OWNER_RANKS) oc[threadIdx.x] = threadIdx.x == 0 ? s0 : (threadIdx.x == 1 ? s1 : s2);
+        } else {
+            colour_owners(sh, C, per, s0, s1, s2, pair_of_row, p_slot, key_of_row, banked[p] ? by_owner : pair_of_row_out, oc);
+            src = by_owner;
+        }
+        if (c + 1 == ncol && threadIdx.x == 0) oc[2 * OWNER_RANKS] = s2;
+        if (!banked[p]) {
+            if (C == 1)
+                for (int r = s0 + threadIdx.x; r < s2; r += OWNER_THREADS) pair_of_row_out[r] = src[r];
+            continue;
+        }
+        for (int k = 0; k < C; ++k) {
+            const int b0 = C == 1 ? s0 : sh.start[2 * k], b1 = C == 1 ? s1 : sh.start[2 * k + 1];
+            const int b2 = C == 1 || 2 * k + 2 == 2 * OWNER_RANKS ? s2 : sh.start[2 * k + 2];
+            bucket_banks(sh, k, per, b0, b1, src, p_slot, key_of_row, pair_of_row_out);
+            for (int r = b1 + threadIdx.x; r < b2; r += OWNER_THREADS) pair_of_row_out[r] = src[r];
+        }
+        __syncthreads();
     }
 }
 
@@ -878,13 +997,12 @@ void launch_pair_setup(const MemberArgs &a, const WarmArgs &w, int np, cudaStrea
     CK(cudaGetLastError());
 }
 
-void launch_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solve_C,
-                      const int *off_in, const int *pair_of_row, const int2 *p_slot,
-                      uint8_t *owner_of_row, int *pair_of_row_out, int *off_out, cudaStream_t s) {
+void launch_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solve_C, const int *off_in,
+                      const int *pair_of_row, const int2 *p_slot, const int *banked, uint8_t *key_of_row,
+                      int *by_owner, int *pair_of_row_out, int *off_out, cudaStream_t s) {
     if (P <= 0) return;
-    k_row_owner<<<dim3(P, OVL_MAX_COLOURS), OWNER_THREADS, 0, s>>>(P, part_bstart, part_ncol, solve_C, off_in,
-                                                                   pair_of_row, p_slot, owner_of_row,
-                                                                   pair_of_row_out, off_out);
+    k_row_owner<<<dim3(P, OWNER_GRID_Y), OWNER_THREADS, 0, s>>>(P, part_bstart, part_ncol, solve_C, off_in, pair_of_row,
+                                                                p_slot, banked, key_of_row, by_owner, pair_of_row_out, off_out);
     note_launch();
     CK(cudaGetLastError());
 }

@@ -15,10 +15,11 @@
 // colours -- the same result as sweeping the constraints one by one in colour
 // order.  Inside a colour every CTA takes the rows whose first dynamic body
 // it holds (the rows are grouped that way beforehand), so most body accesses
-// stay in the CTA's own shared memory.  In full-size CTAs (one per SM) with
-// the masses in shared memory, a thread loads its next rows' records and
-// impulses into registers ahead of use: the next pass's during the current
-// one, the next colour's between the two halves of the colour barrier.
+// stay in the CTA's own shared memory.  A thread loads its next rows' records
+// into registers ahead of use, across the colour barrier too.  With the
+// masses in shared memory (k_solve_m) the impulses stay there as well when
+// they fit; otherwise (k_solve) a full-size CTA loads them ahead with the
+// records.
 //
 // Row model (sphere contact, normal n from a to b, lever arms r_a n and
 // -r_b n, tangents t1 and t2 = n x t1):
@@ -43,6 +44,8 @@
 // layouts compute the same bits; t1 = normalise(e_k - (n . e_k) n) (k the
 // axis of the smallest |n_k|) is formed here.
 #include <cooperative_groups.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "geom.cuh"
@@ -97,7 +100,6 @@ struct LocalSlots {
     static constexpr bool kMasses = false;
     float4 *A;   // (vx, vy, vz, wx)
     float2 *B;   // (wy, wz)
-    __device__ __forceinline__ uint32_t code_of(int s) const { return (uint32_t)s; }
     __device__ __forceinline__ void load(uint32_t c, Body &b) const {
         const uint32_t i = code_index(c);
         const float4 x = A[i];
@@ -112,14 +114,15 @@ struct LocalSlots {
     }
 };
 
-// (v, 1/m) and (w, 1/I) of slot i at S[2i], S[2i + 1]
+// (v, 1/m) of slot i at V[i], (w, 1/I) at W[i].  Two arrays: eight lanes read
+// eight 16-byte words at a time, and a 32-byte stride would leave them only
+// four of the eight bank groups.
 struct LocalSlotsM {
     static constexpr bool kMasses = true;
-    float4 *S;
-    __device__ __forceinline__ uint32_t code_of(int s) const { return (uint32_t)s; }
+    float4 *V, *W;
     __device__ __forceinline__ void load(uint32_t c, Body &b) const {
         const uint32_t i = code_index(c);
-        const float4 x = S[2 * i], y = S[2 * i + 1];
+        const float4 x = V[i], y = W[i];
         b.v = make_float3(x.x, x.y, x.z);
         b.w = make_float3(y.x, y.y, y.z);
         b.im = x.w;
@@ -127,8 +130,8 @@ struct LocalSlotsM {
     }
     __device__ __forceinline__ void store(uint32_t c, const Body &b) const {
         const uint32_t i = code_index(c);
-        S[2 * i] = make_float4(b.v.x, b.v.y, b.v.z, b.im);
-        S[2 * i + 1] = make_float4(b.w.x, b.w.y, b.w.z, b.ii);
+        V[i] = make_float4(b.v.x, b.v.y, b.v.z, b.im);
+        W[i] = make_float4(b.w.x, b.w.y, b.w.z, b.ii);
     }
 };
 
@@ -148,7 +151,6 @@ struct ClusterSlots {
     static constexpr bool kMasses = false;
     uint32_t A, B;   // shared-window offsets of this CTA's arrays (same in every CTA)
     uint32_t per;    // slots per CTA
-    __device__ __forceinline__ uint32_t code_of(int s) const { return ((uint32_t)s / per) << 24 | (uint32_t)s % per; }
     __device__ __forceinline__ void load(uint32_t c, Body &b) const {
         const uint32_t r = code_rank(c), i = code_index(c);
         const uint32_t a = mapa(A + 16u * i, r), d = mapa(B + 8u * i, r);
@@ -169,31 +171,30 @@ struct ClusterSlots {
     }
 };
 
-// the same with the masses: one 32 B slot, one mapa per access
+// LocalSlotsM over the C CTAs of a cluster, every access through distributed
+// shared memory
 template <int C>
 struct ClusterSlotsM {
     static constexpr bool kMasses = true;
-    uint32_t S;      // shared-window offset of this CTA's slots (same in every CTA)
-    uint32_t per;    // slots per CTA
-    __device__ __forceinline__ uint32_t code_of(int s) const { return ((uint32_t)s / per) << 24 | (uint32_t)s % per; }
+    uint32_t V, W;   // shared-window offsets of this CTA's arrays (same in every CTA)
     __device__ __forceinline__ void load(uint32_t c, Body &b) const {
-        const uint32_t a = mapa(S + 32u * code_index(c), code_rank(c));
+        const uint32_t r = code_rank(c), i = 16u * code_index(c);
         float4 x, y;
         asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
-                     : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(a));
+                     : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(mapa(V + i, r)));
         asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
-                     : "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w) : "r"(a + 16u));
+                     : "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w) : "r"(mapa(W + i, r)));
         b.v = make_float3(x.x, x.y, x.z);
         b.w = make_float3(y.x, y.y, y.z);
         b.im = x.w;
         b.ii = y.w;
     }
     __device__ __forceinline__ void store(uint32_t c, const Body &b) const {
-        const uint32_t a = mapa(S + 32u * code_index(c), code_rank(c));
+        const uint32_t r = code_rank(c), i = 16u * code_index(c);
         asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};"
-                     :: "r"(a), "f"(b.v.x), "f"(b.v.y), "f"(b.v.z), "f"(b.im));
+                     :: "r"(mapa(V + i, r)), "f"(b.v.x), "f"(b.v.y), "f"(b.v.z), "f"(b.im));
         asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};"
-                     :: "r"(a + 16u), "f"(b.w.x), "f"(b.w.y), "f"(b.w.z), "f"(b.ii));
+                     :: "r"(mapa(W + i, r)), "f"(b.w.x), "f"(b.w.y), "f"(b.w.z), "f"(b.ii));
     }
 };
 
@@ -205,7 +206,6 @@ struct GlobalSlots {
     float4 *A;
     float2 *B;
     uint32_t per;    // slots per CTA of the worker's launch (the codes' ranges)
-    __device__ __forceinline__ uint32_t code_of(int s) const { return ((uint32_t)s / per) << 24 | (uint32_t)s % per; }
     __device__ __forceinline__ void load(uint32_t c, Body &b) const {
         const uint32_t i = code_index(c);
         if (i >= per) { b.v = make_float3(0.f, 0.f, 0.f); b.w = b.v; return; }
@@ -600,13 +600,32 @@ __device__ float rows_residual_sq(const SolveArgs &a, const S &st, const Buckets
     return sq;
 }
 
+// integrates one body, x += h v; q <- normalise(q + h/2 (0, w) (x) q), and
+// writes the worker's copy (entry e of body b)
+__device__ __forceinline__ void integrate_copy(const SolveArgs &a, int e, int b, float h, float3 v, float3 w) {
+    const float4 x = a.st[4 * b], q = a.st[4 * b + 1], v0 = a.st[4 * b + 2], w0 = a.st[4 * b + 3];
+    const float4 xn = make_float4(x.x + h * v.x, x.y + h * v.y, x.z + h * v.z, x.w);
+    // (0, w) (x) q = (-w.qv, qw w + w x qv)
+    const float dqw = -(w.x * q.y + w.y * q.z + w.z * q.w);
+    const float dqx = q.x * w.x + (w.y * q.w - w.z * q.z);
+    const float dqy = q.x * w.y + (w.z * q.y - w.x * q.w);
+    const float dqz = q.x * w.z + (w.x * q.z - w.y * q.y);
+    const float hh = 0.5f * h;
+    const float4 qn = make_float4(q.x + hh * dqw, q.y + hh * dqx, q.z + hh * dqy, q.w + hh * dqz);
+    const float L = sqrtf(qn.x * qn.x + qn.y * qn.y + qn.z * qn.z + qn.w * qn.w);
+    a.copies[4 * (size_t)e] = xn;
+    a.copies[4 * (size_t)e + 1] = make_float4(qn.x / L, qn.y / L, qn.z / L, qn.w / L);
+    a.copies[4 * (size_t)e + 2] = make_float4(v.x, v.y, v.z, v0.w);
+    a.copies[4 * (size_t)e + 3] = make_float4(w.x, w.y, w.z, w0.w);
+}
+
 // One worker solved by a group of C CTAs.  CTA `rank` holds the body slots
 // [rank per, min(nb, (rank + 1) per)) and, in every colour, takes the rows of
 // its owner bucket, thread tid the rows tid, tid + T, ..., U of them at a
 // time.  With C = 1 (one CTA, or the global-memory path) the CTA holds every
-// slot and takes every bucket.
+// slot and takes every bucket.  cper: slots per CTA in the rows' slot codes.
 template <int C, int U, bool P, bool X, class S>
-__device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, int per, const Buckets &bk,
+__device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, int per, int cper, const Buckets &bk,
                              int row0, int row1) {
     __shared__ float red[32];
     __shared__ float part_sum;
@@ -617,6 +636,8 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
     const int scene = a.part_scene[p];
     const float h = a.dt_override > 0.f ? a.dt_override : a.scene_dt[scene];
     const float mu = a.scene_mu[scene];
+    // the code of worker slot s
+    auto slot_code = [&](int s) { return (uint32_t)(s / cper) << 24 | (uint32_t)(s % cper); };
     // velocities after the external force (h f), from the blended state; each
     // CTA loads the slots it holds
     for (int s = s_lo + tid; s < s_hi; s += T) {
@@ -627,7 +648,7 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
         x.w = make_float3(w.x, w.y, w.z);
         x.im = v.w;
         x.ii = w.w;
-        st.store(st.code_of(s), x);
+        st.store(slot_code(s), x);
     }
     // this CTA's zero slot (static ends of its rows)
     if (tid == 0) {
@@ -779,32 +800,272 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
     if (rank == 0 && tid == 0) a.part_iters[p] = it_done;
     // impulses back in canonical pair order (next step's warm start)
     for (int r = row0 + g; r < row1; r += G) a.lam_out[a.rpair[r]] = a.rlam[r];
-    // integrate: x += h v; q <- normalise(q + h/2 (0, w) (x) q); write this
-    // worker's copy of each body the CTA holds
+    // integrate and write this worker's copy of each body the CTA holds
     for (int s = s_lo + tid; s < s_hi; s += T) {
         int e = a.part_list[b0 + s];
         int b = a.entry_body[e];
-        float4 x = a.st[4 * b], q = a.st[4 * b + 1], v0 = a.st[4 * b + 2], w0 = a.st[4 * b + 3];
         Body y;
-        st.load(st.code_of(s), y);
-        float3 v = y.v, w = y.w;
-        float4 xn = make_float4(x.x + h * v.x, x.y + h * v.y, x.z + h * v.z, x.w);
-        // (0, w) (x) q = (-w.qv, qw w + w x qv)
-        float dqw = -(w.x * q.y + w.y * q.z + w.z * q.w);
-        float dqx = q.x * w.x + (w.y * q.w - w.z * q.z);
-        float dqy = q.x * w.y + (w.z * q.y - w.x * q.w);
-        float dqz = q.x * w.z + (w.x * q.z - w.y * q.y);
-        float hh = 0.5f * h;
-        float4 qn = make_float4(q.x + hh * dqw, q.y + hh * dqx, q.z + hh * dqy, q.w + hh * dqz);
-        float L = sqrtf(qn.x * qn.x + qn.y * qn.y + qn.z * qn.z + qn.w * qn.w);
-        qn = make_float4(qn.x / L, qn.y / L, qn.z / L, qn.w / L);
-        a.copies[4 * (size_t)e] = xn;
-        a.copies[4 * (size_t)e + 1] = qn;
-        a.copies[4 * (size_t)e + 2] = make_float4(v.x, v.y, v.z, v0.w);
-        a.copies[4 * (size_t)e + 3] = make_float4(w.x, w.y, w.z, w0.w);
+        st.load(slot_code(s), y);
+        integrate_copy(a, e, b, h, y.v, y.w);
     }
     // no CTA may leave while another can still reach its shared memory
     if (C > 1) group_sync<C>();
+}
+
+// ---- sphere and joint rows, masses in shared memory -------------------------
+// The impulses of a CTA's rows: in shared memory (three words per row, an odd
+// stride, so consecutive rows meet no bank conflict; k_n formed from the
+// masses as the row build forms it), or, when they do not fit beside the
+// bodies, in the global records.  (A store to global memory before a cluster
+// barrier costs its release fence the write's way to L2: 1790 cycles per
+// barrier with 512 threads against 575.)
+struct LamShared {
+    float *l;
+    __device__ __forceinline__ float4 load(int i, int, const Body &A, const Body &B) const {
+        const float *q = l + 3 * i;
+        return make_float4(q[0], q[1], q[2], __frcp_rn(A.im + B.im));
+    }
+    __device__ __forceinline__ void store(int i, int, float4 v) const {
+        float *q = l + 3 * i;
+        q[0] = v.x;
+        q[1] = v.y;
+        q[2] = v.z;
+    }
+};
+struct LamGlobal {
+    float4 *l;
+    __device__ __forceinline__ float4 load(int, int r, const Body &, const Body &) const { return l[r]; }
+    __device__ __forceinline__ void store(int, int r, float4 v) const { l[r] = v; }
+};
+
+// a row's two records, read once per sweep and never written during the solve
+struct RowHead {
+    float4 x, y;
+};
+__device__ __forceinline__ void fetch_head(const SolveArgs &a, int r, int end, RowHead &q) {
+    if (r < end) {
+        q.x = __ldg(a.r0 + r);
+        q.y = __ldg(a.r1 + r);
+    }
+}
+
+// The body slots of a group as 16-bit codes name them (rank << 13 | i).
+// LOCAL: every code names this CTA's own slots, plain shared memory.
+// (Measured on this GPU, dependent 16-byte loads by 512 threads: 65 cycles
+// plain, 102 through shared::cluster to the own CTA, 1390 to another -- 6 B
+// per cycle -- so the rows of a bucket come remote ones first, then local
+// ones, and few warps hold both.)
+template <bool LOCAL>
+struct CodeSlots {
+    LocalSlotsM own;
+    __device__ __forceinline__ void load(uint32_t c, Body &b) const {
+        const uint32_t i = c & 0x1fffu;
+        float4 x, y;
+        if (LOCAL) {
+            x = own.V[i];
+            y = own.W[i];
+        } else {
+            const uint32_t v = mapa((uint32_t)__cvta_generic_to_shared(own.V + i), c >> 13),
+                           w = mapa((uint32_t)__cvta_generic_to_shared(own.W + i), c >> 13);
+            asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
+                         : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(v) : "memory");
+            asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
+                         : "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w) : "r"(w) : "memory");
+        }
+        b.v = make_float3(x.x, x.y, x.z);
+        b.w = make_float3(y.x, y.y, y.z);
+        b.im = x.w;
+        b.ii = y.w;
+    }
+    __device__ __forceinline__ void store(uint32_t c, const Body &b) const {
+        const uint32_t i = c & 0x1fffu;
+        if (LOCAL) {
+            own.V[i] = make_float4(b.v.x, b.v.y, b.v.z, b.im);
+            own.W[i] = make_float4(b.w.x, b.w.y, b.w.z, b.ii);
+        } else {
+            const uint32_t v = mapa((uint32_t)__cvta_generic_to_shared(own.V + i), c >> 13),
+                           w = mapa((uint32_t)__cvta_generic_to_shared(own.W + i), c >> 13);
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};"
+                         :: "r"(v), "f"(b.v.x), "f"(b.v.y), "f"(b.v.z), "f"(b.im) : "memory");
+            asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};"
+                         :: "r"(w), "f"(b.w.x), "f"(b.w.y), "f"(b.w.z), "f"(b.ii) : "memory");
+        }
+    }
+};
+
+// One row: loads, f, stores if f says so.  i: the row's place in the CTA's
+// impulses.  The group's CTAs take a warp's rows as local ones when all of
+// them are.
+template <int C, class LM, class F>
+__device__ __forceinline__ void visit_row(const SolveArgs &a, const LocalSlotsM &own, uint32_t rank, const LM &lam, int i,
+                                          int r, bool joint, const RowHead &q, F &&f) {
+    Row w;
+    w.x = q.x;
+    w.y = q.y;
+    w.joint = joint;
+    uint32_t c = __float_as_uint(q.y.w);
+    if (joint) {
+        // a joint's codes are the 24-bit ones of r2
+        w.z = a.r2[r];
+        const uint32_t ca = __float_as_uint(w.z.z), cb = __float_as_uint(w.z.w);
+        c = (code_rank(ca) << 13 | code_index(ca)) | (code_rank(cb) << 13 | code_index(cb)) << 16;
+    }
+    auto body = [&](const auto &st) {
+        Body A, B;
+        st.load(c & 0xffffu, A);
+        st.load(c >> 16, B);
+        float4 l = lam.load(i, r, A, B);
+        if (!f(A, B, w, l)) return;
+        st.store(c & 0xffffu, A);
+        st.store(c >> 16, B);
+        lam.store(i, r, l);
+    };
+    bool out = false;
+    if constexpr (C > 1) out = __any_sync(__activemask(), (c >> 13 & 7u) != rank || c >> 29 != rank);
+    if (out) body(CodeSlots<C == 1>{own});
+    else body(CodeSlots<true>{own});
+}
+
+// Warm start, sweeps, residual of one CTA's rows; tab[c] = (first row, first
+// joint, end, rows of earlier colours) of colour c.  A thread's first row of
+// the next colour is loaded before the current colour is solved, its further
+// rows of a colour one ahead.
+template <int C, class LM>
+__device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM &lam, const int4 *tab, int ncol, float mu,
+                           int p, int rank, int nrows, float *red, float *part_sum) {
+    const int tid = threadIdx.x, T = blockDim.x;
+    RowHead nx;
+    if (ncol > 0) fetch_head(a, tab[0].x + tid, tab[0].z, nx);
+    auto colour = [&](int c, auto &&f) {
+        const int4 o = tab[c], on = tab[c + 1 < ncol ? c + 1 : 0];
+        RowHead cur = nx;
+        fetch_head(a, on.x + tid, on.z, nx);
+        for (int r = o.x + tid; r < o.z; r += T) {
+            RowHead ahead;
+            fetch_head(a, r + T, o.z, ahead);
+            visit_row<C>(a, own, (uint32_t)rank, lam, r - o.x + o.w, r, r >= o.y, cur, f);
+            cur = ahead;
+        }
+        group_sync<C>();
+    };
+    auto warm = [&](Body &A, Body &B, const Row &w, float4 &l) {
+        if (l.x == 0.f && l.y == 0.f && l.z == 0.f) return false;
+        if (w.joint) {
+            joint_impulse(A, B, f3(w.x), f3(w.y), 0, l.x);
+            joint_impulse(A, B, f3(w.x), f3(w.y), 1, l.y);
+            joint_impulse(A, B, f3(w.x), f3(w.y), 2, l.z);
+        } else {
+            const float3 t1 = contact_t1(w), n = f3(w.x);
+            contact_impulse(A, B, n, t1, cross3(n, t1), w.y.x, w.y.y, l.x, l.y, l.z);
+        }
+        return true;
+    };
+    auto solve = [&](Body &A, Body &B, const Row &w, float4 &l) {
+        solve_row<LocalSlotsM>(A, B, w, mu, l);
+        return true;
+    };
+    auto residual = [&]() {
+        float sq = 0.f;
+        for (int c = 0; c < ncol; ++c) {
+            const int4 o = tab[c];
+            for (int r = o.x + tid; r < o.z; r += T) {
+                RowHead q;
+                fetch_head(a, r, o.z, q);
+                visit_row<C>(a, own, (uint32_t)rank, lam, r - o.x + o.w, r, r >= o.y, q, [&](Body &A, Body &B, const Row &w, float4 &l) {
+                    sq += w.joint ? joint_residual_sq(A, B, w.x, w.y, w.z)
+                                  : contact_residual_sq(A, B, w.x, w.y, contact_t1(w), l.w, w.x.w, mu, l);
+                    return false;
+                });
+            }
+        }
+        return group_sum<C>(sq, red, part_sum);
+    };
+    for (int c = 0; c < ncol; ++c) colour(c, warm);
+    int it = 0;
+    while (it < a.iters) {
+        for (int c = 0; c < ncol; ++c) colour(c, solve);
+        ++it;
+        if (a.res_tol > 0.f && a.res_check_every > 0 && it % a.res_check_every == 0 && it < a.iters) {
+            const float tot = residual();
+            if (nrows == 0 || sqrtf(tot / nrows) <= a.res_tol) break;   // the same total in every CTA
+        }
+    }
+    if (a.flags & OVL_FLAG_RESIDUAL) {
+        const float tot = residual();
+        if (rank == 0 && tid == 0) a.part_res_sq[p] = (double)tot;
+    }
+    if (rank == 0 && tid == 0) a.part_iters[p] = it;
+}
+
+// A launch whose slots hold the masses (no boxes): CTA `rank` of worker p's
+// group holds the slots [rank per, (rank + 1) per), their zero slot and, when
+// they fit, the impulses of its rows.  Latency-bound: a colour step of few
+// rows takes about 900 cycles, of which 95 are the CTA barrier (560 a
+// cluster's), the rest one row's chain; 512 threads (measured on the large
+// pile: 256 1.14 ms, 384 1.00, 512 0.94, 768 0.92 but slower on small piles).
+template <int C>
+__global__ void __launch_bounds__(SOLVE_THREADS, 1) k_solve_m(SolveArgs a) {
+    extern __shared__ float4 sm[];
+    __shared__ int4 tab[OVL_MAX_COLOURS];
+    __shared__ float red[32];
+    __shared__ float part_sum;
+    const int tid = threadIdx.x, T = blockDim.x;
+    const int rank = C == 1 ? 0 : (int)cg::this_cluster().block_rank();
+    const int p = a.order ? (int)a.order[blockIdx.x / C] : (int)(blockIdx.x / C);
+    const int b0 = a.part_bstart[p], nb = a.part_bstart[p + 1] - b0;
+    const int per = (nb + C - 1) / C;
+    const int *goff = a.col_off + (size_t)p * OWNER_NB;
+    const int ncol = a.part_ncol[p];
+    const int row0 = goff[0], row1 = goff[OWNER_NB - 1];
+    for (int c = tid; c < ncol; c += T) {
+        const int *o = goff + (c * OWNER_RANKS + rank) * 2;
+        tab[c] = make_int4(o[0], o[1], o[2], 0);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        int t = 0;
+        for (int c = 0; c < ncol; ++c) {
+            tab[c].w = t;
+            t += tab[c].z - tab[c].x;
+        }
+        red[0] = __int_as_float(t);
+    }
+    __syncthreads();
+    const int mine = __float_as_int(red[0]);   // this CTA's rows
+    const int scene = a.part_scene[p];
+    const float h = a.dt_override > 0.f ? a.dt_override : a.scene_dt[scene];
+    const float mu = a.scene_mu[scene];
+    const int s_lo = rank * per, s_hi = min(nb, (rank + 1) * per);
+    float4 *const V = sm, *const W = sm + per + 1;   // (v, 1/m), (w, 1/I) of the CTA's slots and its zero slot
+    float *const L = reinterpret_cast<float *>(sm + 2 * (per + 1));
+    const bool fits = 32ll * (per + 1) + 12ll * mine <= a.smem_bytes;
+    // velocities after the external force (h f), from the blended state; the
+    // zero slot (static ends); the impulses
+    for (int s = s_lo + tid; s < s_hi; s += T) {
+        const int b = a.entry_body[a.part_list[b0 + s]];
+        const float4 v = a.st[4 * b + 2], w = a.st[4 * b + 3];
+        V[s - s_lo] = make_float4(v.x + h * a.gravity.x, v.y + h * a.gravity.y, v.z + h * a.gravity.z, v.w);
+        W[s - s_lo] = w;
+    }
+    if (tid == 0) V[per] = W[per] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const LamShared ls{L};
+    if (fits)
+        for (int c = 0; c < ncol; ++c)
+            for (int r = tab[c].x + tid; r < tab[c].z; r += T) ls.store(r - tab[c].x + tab[c].w, r, a.rlam[r]);
+    group_sync<C>();
+    const LocalSlotsM own{V, W};
+    if (fits) sweep_rows<C>(a, own, ls, tab, ncol, mu, p, rank, 3 * (row1 - row0), red, &part_sum);
+    else sweep_rows<C>(a, own, LamGlobal{a.rlam}, tab, ncol, mu, p, rank, 3 * (row1 - row0), red, &part_sum);
+    // impulses back in canonical pair order (next step's warm start)
+    for (int c = 0; c < ncol; ++c)
+        for (int r = tab[c].x + tid; r < tab[c].z; r += T) {
+            const int i = r - tab[c].x + tab[c].w;
+            a.lam_out[a.rpair[r]] = fits ? make_float4(L[3 * i], L[3 * i + 1], L[3 * i + 2], 0.f) : a.rlam[r];
+        }
+    for (int s = s_lo + tid; s < s_hi; s += T) {
+        const int e = a.part_list[b0 + s], b = a.entry_body[e];
+        integrate_copy(a, e, b, h, f3(V[s - s_lo]), f3(W[s - s_lo]));
+    }
 }
 
 // C CTAs per worker; a worker's slots are spread over their shared memory when
@@ -832,29 +1093,25 @@ __global__ void __launch_bounds__(SOLVE_THREADS, U == 1 ? 2 : 1) k_solve(SolveAr
         // per + 1 slots: the CTA's range and its zero slot
         float4 *A = sm;
         if (M) {
-            if (C == 1) {
-                LocalSlotsM st{A};
-                solve_worker<C, U, P, X>(a, st, p, rank, per, Buckets{boff, 3, 1}, row0, row1);
-            } else {
-                ClusterSlotsM<C> st{(uint32_t)__cvta_generic_to_shared(A), (uint32_t)per};
-                solve_worker<C, U, P, X>(a, st, p, rank, per, Buckets{boff, 3, 1}, row0, row1);
-            }
+            const LocalSlotsM own{A, A + per + 1};
+            if constexpr (C == 1) solve_worker<C, U, P, X>(a, own, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
+            else solve_worker<C, U, P, X>(a, ClusterSlotsM<C>{(uint32_t)__cvta_generic_to_shared(own.V), (uint32_t)__cvta_generic_to_shared(own.W)}, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
         } else {
             float2 *B = reinterpret_cast<float2 *>(sm + per + 1);
             if (C == 1) {
                 LocalSlots st{A, B};
-                solve_worker<C, U, P, X>(a, st, p, rank, per, Buckets{boff, 3, 1}, row0, row1);
+                solve_worker<C, U, P, X>(a, st, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
             } else {
                 ClusterSlots<C> st{(uint32_t)__cvta_generic_to_shared(A), (uint32_t)__cvta_generic_to_shared(B),
                                    (uint32_t)per};
-                solve_worker<C, U, P, X>(a, st, p, rank, per, Buckets{boff, 3, 1}, row0, row1);
+                solve_worker<C, U, P, X>(a, st, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
             }
         }
     } else if (rank == 0) {
         // one CTA takes the whole worker: every owner bucket of every colour
         GlobalSlots st{a.scratch + (size_t)b0, reinterpret_cast<float2 *>(a.scratch + (size_t)a.n_entries) + b0,
                        (uint32_t)per};
-        solve_worker<1, U, false, X>(a, st, p, 0, nb, Buckets{goff, 2 * OWNER_RANKS, OWNER_RANKS}, row0, row1);
+        solve_worker<1, U, false, X>(a, st, p, 0, nb, per, Buckets{goff, 2 * OWNER_RANKS, OWNER_RANKS}, row0, row1);
     }
 }
 
@@ -897,8 +1154,41 @@ static void launch_solve_u(const SolveArgs &a, int threads, int cluster, cudaStr
     }
 }
 
-void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool masses, cudaStream_t s) {
+template <int C>
+static void launch_solve_m(const SolveArgs &a, int threads, int budget, cudaStream_t s) {
+    SolveArgs b = a;
+    b.smem_bytes = std::min(budget, solve_smem_bytes(a.smem_slots, true) + 12 * a.smem_rows);
+    CK(cudaFuncSetAttribute(k_solve_m<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a.n_parts * C);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = b.smem_bytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CK(cudaLaunchKernelEx(&cfg, k_solve_m<C>, b));
+    note_launch();
+}
+
+void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool masses, int budget, cudaStream_t s) {
     if (!a.n_parts) return;
+    if (masses && !a.row_full) {
+        switch (cluster) {
+            case 8: launch_solve_m<8>(a, threads, budget, s); break;
+            case 6: launch_solve_m<6>(a, threads, budget, s); break;
+            case 4: launch_solve_m<4>(a, threads, budget, s); break;
+            case 3: launch_solve_m<3>(a, threads, budget, s); break;
+            case 2: launch_solve_m<2>(a, threads, budget, s); break;
+            default: launch_solve_m<1>(a, threads, budget, s); break;
+        }
+        CK(cudaGetLastError());
+        return;
+    }
     if (threads > SOLVE_THREADS) threads = SOLVE_THREADS;
     if (a.row_full) {
         // a context with boxes: the kernels that hold the full rows (two rows
@@ -907,17 +1197,10 @@ void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool
         else launch_solve_u<2, false, false, true>(a, threads, cluster, s);
     } else if (unroll == 2) {
         // a full-size CTA (one per SM) loads rows ahead
-        if (threads == SOLVE_THREADS) {
-            if (masses) launch_solve_u<2, true, true>(a, threads, cluster, s);
-            else launch_solve_u<2, false, true>(a, threads, cluster, s);
-        } else if (masses) {
-            launch_solve_u<2, true, false>(a, threads, cluster, s);
-        } else {
-            launch_solve_u<2, false, false>(a, threads, cluster, s);
-        }
+        if (threads == SOLVE_THREADS) launch_solve_u<2, false, true>(a, threads, cluster, s);
+        else launch_solve_u<2, false, false>(a, threads, cluster, s);
     } else {
-        if (masses) launch_solve_u<1, true, false>(a, threads, cluster, s);
-        else launch_solve_u<1, false, false>(a, threads, cluster, s);
+        launch_solve_u<1, false, false>(a, threads, cluster, s);
     }
     CK(cudaGetLastError());
 }

@@ -115,17 +115,22 @@ struct WarmArgs {
     float factor;
 };
 void launch_pair_setup(const MemberArgs &a, const WarmArgs &w, int np, cudaStream_t s);
-// Rows of every colour regrouped by the CTA that owns them in the solve:
-// worker p's bodies are split into solve_C[p] contiguous slot ranges of
+// Rows of every colour in the order of the solve: worker p's bodies are split
+// into solve_C[p] contiguous slot ranges of
 // ceil(nb / C) slots, one per CTA, and a row belongs to the CTA holding its
-// first dynamic body.  off_in: [P][2*OVL_MAX_COLOURS+1] (colour, kind)
+// first dynamic body (up to the balancing of the CTAs' shares); inside a CTA's bucket rows that reach another
+// CTA come first, then the local ones in an order that spreads their slots
+// over the shared-memory banks.  off_in: [P][2*OVL_MAX_COLOURS+1] (colour, kind)
 // offsets of pair_of_row; off_out: [P][OWNER_NB] offsets of (colour, owner
-// rank, kind) buckets, ranks 0..7, contacts before joints, then the end.
+// rank, kind) buckets, ranks 0..7, contacts before joints, of the worker's
+// colours (the offset after the last colour follows them), and in the last
+// place the end.  banked [P]: 0 leaves a worker's buckets in canonical order.
+// key_of_row [np], by_owner [np]: scratch.
 #define OWNER_RANKS 8
 #define OWNER_NB (OVL_MAX_COLOURS * OWNER_RANKS * 2 + 1)
-void launch_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solve_C,
-                      const int *off_in, const int *pair_of_row, const int2 *p_slot,
-                      uint8_t *owner_of_row, int *pair_of_row_out, int *off_out, cudaStream_t s);
+void launch_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solve_C, const int *off_in,
+                      const int *pair_of_row, const int2 *p_slot, const int *banked, uint8_t *key_of_row,
+                      int *by_owner, int *pair_of_row_out, int *off_out, cudaStream_t s);
 // keys[p] = 2^24 - 1 - min(pairs of worker p, 2^24 - 1), vals[p] = p: an
 // ascending stable sort of the keys lists the workers longest first
 void launch_worker_cost_keys(const int *part_pstart, int P, uint32_t *keys, uint32_t *vals,
@@ -228,6 +233,8 @@ struct SolveArgs {
     float4 *scratch;           // [ne] float4 + [ne] float2: velocities of workers too large for shared memory
     int iters;
     int smem_slots;
+    int smem_rows;             // room asked for: rows per CTA whose impulses are kept in shared memory
+    int smem_bytes;            // dynamic shared memory of the launch
     int flags;                 // OVL_FLAG_*
     float res_tol;
     int res_check_every;
@@ -239,7 +246,8 @@ struct SolveArgs {
 };
 // masses: the shared-memory slots hold the inverse masses and inertias (32 B
 // per slot; contact rows read as two records); else 24 B per slot
-void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool masses, cudaStream_t s);
+// budget: dynamic shared memory a CTA may take
+void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool masses, int budget, cudaStream_t s);
 int solve_ctas_per_sm(int unroll);
 int solve_slot_bytes(bool masses);              // bytes of one shared-memory body slot
 int solve_smem_bytes(int slots, bool masses);   // a CTA's slots plus its zero slot
