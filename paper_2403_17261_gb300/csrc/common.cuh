@@ -95,17 +95,23 @@ long long launch_count();
 // ---------------------------------------------------------------------------
 // utility kernels (k_util.cu)
 // ---------------------------------------------------------------------------
-// exclusive scan of n int32 values; out has n+1 entries (out[n] = total)
-void scan_i32(const int *in, int *out, int n, DBuf<int> &tmp, cudaStream_t s);
-// stable LSD radix sort of (key, val) pairs by the low nbits of key
-void radix_sort_u32(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt, int n,
-                    int nbits, DBuf<int> &hist, DBuf<int> &tmp, cudaStream_t s,
-                    bool *result_in_alt);
-void fill_i32(int *p, int v, size_t n, cudaStream_t s);
+// exclusive scan of n int32 values; out (not in) has n+1 entries (out[n] =
+// total); the total also goes to host_total, pinned host memory, when given.
+// tmp: scratch of scans on one stream only
+void scan_i32(const int *in, int *out, int n, DBuf<int> &tmp, cudaStream_t s, int *host_total = nullptr);
+// Stable grouping of n items by a key below 2^nbits (LSD radix sort, 8-bit
+// digits): out = the items' indexes in key order; returns the sorted keys (in
+// b, until its next use)
+struct GroupBuf {
+    DBuf<uint32_t> k0, k1, v0, v1;
+    DBuf<int> hist, offs;
+    void release() { k0.release(); k1.release(); v0.release(); v1.release(); hist.release(); offs.release(); }
+};
+const uint32_t *group_by_key(const uint32_t *key, int n, int nbits, uint32_t *out, GroupBuf &b, DBuf<int> &tmp,
+                             cudaStream_t s);
+// start[p] = host_start[p] (pinned) = first index of the n sorted keys whose key is >= p, p = 0 .. P
+void key_starts(const uint32_t *keys, int n, int P, int *start, int *host_start, cudaStream_t s);
 void fill_u8(uint8_t *p, uint8_t v, size_t n, cudaStream_t s);
-void iota_u32(uint32_t *p, int n, cudaStream_t s);
-// counts[key[i]]++ for i < n
-void histogram_i32(const int *key, int n, int *counts, int nbins, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // host-side algorithms (host_alg.cpp): Algorithms 2, 3, 6, 7

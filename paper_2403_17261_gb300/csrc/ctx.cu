@@ -96,8 +96,9 @@ void phase_contacts(ovl_ctx *c) {
     scan_i32(c->bucket_count.p, c->bucket_start.p, (int)c->tsize, c->scan_tmp, s);
     launch_bucket_fill(a, s);
     launch_find_pairs(a, s);
-    scan_i32(c->ccount.p, c->cstart.p, n, c->scan_tmp, s);
-    c->nc = read_i32(c, c->cstart.p + n);
+    scan_i32(c->ccount.p, c->cstart.p, n, c->scan_tmp, s, c->h_counts.p + COUNT_CONTACTS);
+    CK(cudaStreamSynchronize(s));
+    c->nc = c->h_counts.p[COUNT_CONTACTS];
     c->c_ab.ensure(c->nc + 1);
     c->c_n.ensure(c->nc + 1);
     c->c_t1.ensure(c->nc + 1);
@@ -119,14 +120,15 @@ void phase_graph(ovl_ctx *c) {
     CK(cudaMemsetAsync(c->cursor2.p, 0, sizeof(int) * ((size_t)n + 1), s));
     launch_edge_degree(c->c_ab.p, c->nc, c->jab.p, c->nj, c->im.p, n, c->deg.p, s);
     scan_i32(c->deg.p, c->tptr.p, n, c->scan_tmp, s);
-    int e2 = read_i32(c, c->tptr.p + n);
-    c->tcol.ensure((size_t)e2 + 1);
+    // at most two directed edges per constraint, so neither count is waited
+    // for here: the adjacency's is read after the next wait
+    const size_t most = 2 * ((size_t)c->nc + c->nj) + 1;
+    c->tcol.ensure(most);
+    c->col.ensure(most);
     launch_edge_fill(c->c_ab.p, c->nc, c->jab.p, c->nj, c->im.p, n, c->tptr.p, c->cursor2.p,
                      c->tcol.p, s);
     launch_adj_unique(c->tptr.p, n, c->tcol.p, c->ucount.p, s);
-    scan_i32(c->ucount.p, c->row_ptr.p, n, c->scan_tmp, s);
-    c->nadj = read_i32(c, c->row_ptr.p + n);
-    c->col.ensure((size_t)c->nadj + 1);
+    scan_i32(c->ucount.p, c->row_ptr.p, n, c->scan_tmp, s, c->h_counts.p + COUNT_ADJACENCY);
     launch_adj_compact(c->tptr.p, c->tcol.p, n, c->row_ptr.p, c->col.p, s);
 }
 
@@ -144,17 +146,19 @@ void phase_load_balance(ovl_ctx *c, bool act, bool deact) {
     c->lb_pairs.ensure(c->nc + 1);
     const auto t0 = std::chrono::steady_clock::now();
     launch_lb_flags(c->c_ab.p, c->nc, c->im.p, n, c->mask.p, deact ? 0 : 1, c->lb_flag.p, contact_points(c), s);
-    scan_i32(c->lb_flag.p, c->lb_pos.p, c->nc, c->scan_tmp, s);
-    // the graph and the masks go to the host while the candidate count is read
+    scan_i32(c->lb_flag.p, c->lb_pos.p, c->nc, c->scan_tmp, s, c->h_counts.p + COUNT_CANDIDATES);
+    CK(cudaStreamSynchronize(s));
+    c->nadj = c->h_counts.p[COUNT_ADJACENCY];
+    const int m = c->h_counts.p[COUNT_CANDIDATES];
+    c->lb_candidates = m;
+    if (m == 0) return;
+    // the graph and the masks go to the host
     c->h_rp.ensure((size_t)n + 1);
     c->h_col.ensure((size_t)c->nadj + 1);
     c->h_mask.ensure(n);
     CK(cudaMemcpyAsync(c->h_rp.p, c->row_ptr.p, sizeof(int) * ((size_t)n + 1), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(c->h_col.p, c->col.p, sizeof(int) * c->nadj, cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(c->h_mask.p, c->mask.p, sizeof(uint64_t) * n, cudaMemcpyDeviceToHost, s));
-    const int m = read_i32(c, c->lb_pos.p + c->nc);
-    c->lb_candidates = m;
-    if (m == 0) return;
     launch_lb_compact(c->c_ab.p, c->nc, c->lb_flag.p, c->lb_pos.p, c->lb_pairs.p, s);
     c->h_ab.ensure(m + 1);
     CK(cudaMemcpyAsync(c->h_ab.p, c->lb_pairs.p, sizeof(int2) * m, cudaMemcpyDeviceToHost, s));
@@ -187,8 +191,9 @@ void phase_load_balance(ovl_ctx *c, bool act, bool deact) {
         launch_ball_roots(c->lb_pairs.p, m, c->mask.p, c->ball_root.p, c->ball_list.p, nroot, s);
         launch_balls(false, max_roots, c->ball_list.p, nroot, c->row_ptr.p, c->col.p, c->sob.p, c->scene_gamma.p,
                      c->ball_size.p, nullptr, nullptr, s);
-        scan_i32(c->ball_size.p, c->ball_start.p, n, c->scan_tmp, s);
-        const int total = read_i32(c, c->ball_start.p + n);
+        scan_i32(c->ball_size.p, c->ball_start.p, n, c->scan_tmp, s, c->h_counts.p + COUNT_BALLS);
+        CK(cudaStreamSynchronize(s));
+        const int total = c->h_counts.p[COUNT_BALLS];
         c->ball_vtx.ensure((size_t)total + 1);
         launch_balls(true, max_roots, c->ball_list.p, nroot, c->row_ptr.p, c->col.p, c->sob.p, c->scene_gamma.p,
                      c->ball_size.p, c->ball_start.p, c->ball_vtx.p, s);
@@ -226,81 +231,69 @@ MemberArgs member_args(ovl_ctx *c) {
     return a;
 }
 
-// stable grouping of items by a small key (< n_parts): out = item indices
-void group_by(ovl_ctx *c, const int *key, int m, DBuf<int> &out) {
+void phase_membership(ovl_ctx *c) {
     cudaStream_t s = c->stream;
-    c->sk.ensure(m + 1); c->sv.ensure(m + 1); c->sk2.ensure(m + 1); c->sv2.ensure(m + 1);
-    out.ensure(m + 1);
-    if (m == 0) return;
-    CK(cudaMemcpyAsync(c->sk.p, key, sizeof(int) * m, cudaMemcpyDeviceToDevice, s));
-    iota_u32(c->sv.p, m, s);
-    bool alt = false;
-    radix_sort_u32(c->sk.p, c->sv.p, c->sk2.p, c->sv2.p, m, bits_for(c->n_parts), c->sort_hist,
-                   c->sort_tmp, s, &alt);
-    CK(cudaMemcpyAsync(out.p, alt ? c->sv2.p : c->sv.p, sizeof(int) * m, cudaMemcpyDeviceToDevice, s));
-}
-
-void phase_membership(ovl_ctx *c, float dt_override) {
-    (void)dt_override;
-    cudaStream_t s = c->stream;
-    const int n = c->n, P = c->n_parts;
+    const int n = c->n, P = c->n_parts, bits = bits_for(P);
     c->entry_count.ensure((size_t)n + 1);
     c->entry_ptr.ensure((size_t)n + 1);
+    c->h_starts.ensure(2 * (size_t)P + 2);
+    int *const h_bstart = c->h_starts.p, *const h_pstart = h_bstart + P + 1;
     MemberArgs a = member_args(c);
     launch_entry_count(a, s);
-    scan_i32(c->entry_count.p, c->entry_ptr.p, n, c->scan_tmp, s);
-    c->ne = read_i32(c, c->entry_ptr.p + n);
+    scan_i32(c->entry_count.p, c->entry_ptr.p, n, c->scan_tmp, s, c->h_counts.p + COUNT_ENTRIES);
+    CK(cudaStreamSynchronize(s));
+    c->nadj = c->h_counts.p[COUNT_ADJACENCY];
+    c->ne = c->h_counts.p[COUNT_ENTRIES];
     const int ne = c->ne;
     c->entry_body.ensure(ne + 1); c->entry_part.ensure(ne + 1); c->entry_slot.ensure(ne + 1);
-    c->part_count.ensure((size_t)P + 1); c->part_bstart.ensure((size_t)P + 1);
+    c->part_list.ensure(ne + 1); c->part_bstart.ensure((size_t)P + 1);
     a = member_args(c);
     launch_entry_fill(a, s);
-    group_by(c, c->entry_part.p, ne, c->part_list);
-    CK(cudaMemsetAsync(c->part_count.p, 0, sizeof(int) * ((size_t)P + 1), s));
-    histogram_i32(c->entry_part.p, ne, c->part_count.p, P, s);
-    scan_i32(c->part_count.p, c->part_bstart.p, P, c->scan_tmp, s);
-    a = member_args(c);
+    const uint32_t *keys = group_by_key(reinterpret_cast<const uint32_t *>(c->entry_part.p), ne, bits,
+                                        reinterpret_cast<uint32_t *>(c->part_list.p), c->group, c->scan_tmp, s);
+    key_starts(keys, ne, P, c->part_bstart.p, h_bstart, s);
     launch_entry_slot(a, ne, s);
     // (worker, constraint) pairs
     const int K = c->nc + c->nj;
     c->cons_count.ensure((size_t)K + 1); c->cons_start.ensure((size_t)K + 1);
     a = member_args(c);
     launch_cons_count(a, s);
-    scan_i32(c->cons_count.p, c->cons_start.p, K, c->scan_tmp, s);
-    c->npairs = read_i32(c, c->cons_start.p + K);
+    scan_i32(c->cons_count.p, c->cons_start.p, K, c->scan_tmp, s, c->h_counts.p + COUNT_PAIRS);
+    CK(cudaStreamSynchronize(s));
+    c->npairs = c->h_counts.p[COUNT_PAIRS];
     const int npr = c->npairs;
     c->pair_cons.ensure(npr + 1); c->pair_part.ensure(npr + 1); c->ps_cons.ensure(npr + 1);
-    c->ps_part.ensure(npr + 1); c->part_pcount.ensure((size_t)P + 1); c->part_pstart.ensure((size_t)P + 1);
+    c->ps_part.ensure(npr + 1); c->part_pstart.ensure((size_t)P + 1);
     c->p_key.ensure(npr + 1); c->p_slot.ensure(npr + 1); c->p_lam0.ensure(npr + 1);
     a = member_args(c);
     launch_pair_fill(a, s);
     DBuf<int> &order = c->pair_of_row;   // temporary use before colouring
     order.ensure(npr + 1);
-    group_by(c, c->pair_part.p, npr, order);
-    launch_pair_gather(a, reinterpret_cast<const uint32_t *>(order.p), npr, s);
-    CK(cudaMemsetAsync(c->part_pcount.p, 0, sizeof(int) * ((size_t)P + 1), s));
-    histogram_i32(c->pair_part.p, npr, c->part_pcount.p, P, s);
-    scan_i32(c->part_pcount.p, c->part_pstart.p, P, c->scan_tmp, s);
+    keys = group_by_key(reinterpret_cast<const uint32_t *>(c->pair_part.p), npr, bits,
+                        reinterpret_cast<uint32_t *>(order.p), c->group, c->scan_tmp, s);
+    key_starts(keys, npr, P, c->part_pstart.p, h_pstart, s);
     WarmArgs w{};
     w.ws_pstart = c->ws_pstart.p; w.ws_key = c->ws_key.p; w.ws_lam = c->ws_lam.p;
     w.factor = c->P.warmstart;
-    launch_pair_setup(a, w, npr, s);
-    // launch order of the per-worker kernels: most constraints first, so
-    // the longest workers start in the first wave
-    c->worker_order.ensure((size_t)P + 1);
-    c->wk.ensure((size_t)P + 1); c->wk2.ensure((size_t)P + 1); c->wv2.ensure((size_t)P + 1);
-    launch_worker_cost_keys(c->part_pstart.p, P, c->wk.p, c->worker_order.p, s);
-    bool alt = false;
-    radix_sort_u32(c->wk.p, c->worker_order.p, c->wk2.p, c->wv2.p, P, 24, c->sort_hist, c->sort_tmp, s, &alt);
-    if (alt) std::swap(c->worker_order, c->wv2);
+    launch_pair_setup(a, w, reinterpret_cast<const uint32_t *>(order.p), npr, s);
     // per-worker bodies and constraints on the host, for the launch plans
-    c->h_pb.resize((size_t)P + 1);
-    c->h_pp.resize((size_t)P + 1);
-    download(c->h_pb.data(), c->part_bstart.p, (size_t)P + 1, s);
-    download(c->h_pp.data(), c->part_pstart.p, (size_t)P + 1, s);
     CK(cudaStreamSynchronize(s));
+    c->h_pb.assign(h_bstart, h_bstart + P + 1);
+    c->h_pp.assign(h_pstart, h_pstart + P + 1);
     c->nb_max = 0;
     for (int p = 0; p < P; ++p) c->nb_max = std::max(c->nb_max, c->h_pb[p + 1] - c->h_pb[p]);
+}
+
+// The workers of a uniform launch, most constraints first, so the longest
+// start in the first wave
+const uint32_t *uniform_order(ovl_ctx *c) {
+    std::vector<uint32_t> o(c->n_parts);
+    std::iota(o.begin(), o.end(), 0u);
+    std::stable_sort(o.begin(), o.end(), [&](uint32_t x, uint32_t y) {
+        return c->h_pp[x + 1] - c->h_pp[x] > c->h_pp[y + 1] - c->h_pp[y];
+    });
+    upload(c->worker_order, o.data(), o.size(), c->stream);
+    return c->worker_order.p;
 }
 
 int colour_smem_capacity(ovl_ctx *c) {
@@ -566,7 +559,6 @@ void phase_colour(ovl_ctx *c) {
     c->wprio2.ensure(npr + 1);
     ColourArgs a{};
     a.n_parts = P; a.part_bstart = c->part_bstart.p; a.part_pstart = c->part_pstart.p;
-    a.order = c->worker_order.p;
     a.part_list = c->part_list.p; a.entry_body = c->entry_body.p;
     a.p_key = c->p_key.p; a.p_slot = c->p_slot.p; a.p_colour = c->p_colour.p;
     a.part_ncol = c->part_ncol.p; a.col_off = c->col_off.p; a.pair_of_row = c->pair_of_row.p;
@@ -592,6 +584,7 @@ void phase_colour(ovl_ctx *c) {
     int cluster = 1, slots = 0;
     colour_config(c, &cluster, &slots);
     a.smem_slots = slots;
+    a.order = uniform_order(c);
     launch_colour(a, cluster, c->stream);
 }
 
@@ -663,7 +656,6 @@ int solve_threads(ovl_ctx *c) {
 SolveArgs solve_args(ovl_ctx *c, float dt_override, int iters) {
     SolveArgs a{};
     a.n_parts = c->n_parts; a.part_bstart = c->part_bstart.p; a.part_list = c->part_list.p;
-    a.order = c->worker_order.p;
     a.entry_body = c->entry_body.p; a.part_ncol = c->part_ncol.p; a.col_off = c->col_off2.p;
     a.part_scene = c->part_scene.p; a.scene_dt = c->scene_dt.p; a.dt_override = dt_override;
     a.gravity = make_float3(c->P.gravity[0], c->P.gravity[1], c->P.gravity[2]);
@@ -762,6 +754,7 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
         return;
     }
     a.smem_slots = pl.slots;
+    a.order = uniform_order(c);
     const bool masses = solve_masses_fit(c, pl.slots, solve_ctas_per_sm(pl.unroll));
     a.smem_rows = *std::max_element(c->h_pp.begin(), c->h_pp.end());
     launch_solve(a, pl.threads, pl.cluster, pl.unroll, masses, solve_smem_budget(c, solve_ctas_per_sm(pl.unroll)), c->stream);
@@ -934,7 +927,7 @@ ovl_status run_step(ovl_ctx *c, float dt, int iters) {
     mark(c, 2);
     phase_load_balance(c, c->P.lb_activate != 0, deact);
     mark(c, 3);
-    phase_membership(c, dt);
+    phase_membership(c);
     phase_warmstart(c, dt);
     // The geodesic weights need only the membership and the graph.  When the
     // workers do not outnumber the SMs (the solve is one wave), they run on
@@ -1059,6 +1052,7 @@ ovl_status ovl_create(ovl_ctx **out, const ovl_params *p, void *cuda_stream) {
         for (auto &e : c->join) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         c->lb_threads = (int)std::max(1u, std::min(16u, std::thread::hardware_concurrency()));
         c->status.ensure(4);
+        c->h_counts.ensure(COUNT_N);
         CK(cudaMemsetAsync(c->status.p, 0, 4 * sizeof(int), c->stream));
         return OVL_OK;
     });
@@ -1095,21 +1089,19 @@ void release_all(ovl_ctx *c) {
     c->deg.release(); c->tptr.release(); c->cursor2.release(); c->tcol.release(); c->ucount.release();
     c->row_ptr.release(); c->col.release(); c->entry_count.release(); c->entry_ptr.release();
     c->entry_body.release(); c->entry_part.release(); c->entry_slot.release(); c->part_list.release();
-    c->part_count.release(); c->part_bstart.release(); c->sk.release(); c->sv.release();
-    c->sk2.release(); c->sv2.release(); c->cons_count.release(); c->cons_start.release();
+    c->part_bstart.release(); c->group.release(); c->cons_count.release(); c->cons_start.release();
     c->pair_cons.release(); c->pair_part.release(); c->ps_cons.release(); c->ps_part.release();
-    c->part_pcount.release(); c->part_pstart.release(); c->p_colour.release(); c->part_ncol.release(); c->part_rounds.release();
+    c->part_pstart.release(); c->p_colour.release(); c->part_ncol.release(); c->part_rounds.release();
     c->col_off.release(); c->pair_of_row.release(); c->p_key.release(); c->p_slot.release();
     c->p_lam0.release(); c->colour_scratch.release(); c->worklist.release(); c->worklist2.release(); c->wprio.release(); c->wprio2.release(); c->r0.release(); c->r1.release();
     c->r2.release(); c->rlam.release(); c->lam_out.release(); c->r3.release(); c->rpair.release(); c->ws_pstart.release();
     c->ws_key.release(); c->ws_lam.release(); c->copies.release(); c->solve_scratch.release();
     c->part_iters.release(); c->part_res_sq.release(); c->visited.release(); c->queue.release();
     c->qctl.release(); c->D.release(); c->weight.release(); c->stage13.release(); c->scan_tmp.release();
-    c->sort_hist.release(); c->sort_tmp.release();
     c->lb_flag.release(); c->lb_pos.release(); c->lb_pairs.release();
     c->ball_root.release(); c->ball_size.release(); c->ball_start.release(); c->ball_vtx.release();
     c->ball_list.release();
-    c->worker_order.release(); c->wk.release(); c->wk2.release(); c->wv2.release();
+    c->worker_order.release();
     c->class_order.release(); c->colour_order.release(); c->solve_C.release(); c->solve_M.release(); c->solve_banked.release(); c->col_off2.release();
     c->row_owner.release(); c->row_by_owner.release();
     c->pair_of_row2.release(); c->lb_loads.release();
@@ -1149,7 +1141,7 @@ ovl_status ovl_destroy(ovl_ctx *c) {
     release_mlp(c);
     c->h_loads.release();
     c->h_ball_start.release(); c->h_ball_vtx.release();
-    c->h_i32.release(); c->h_ab.release(); c->h_rp.release(); c->h_col.release(); c->h_mask.release();
+    c->h_i32.release(); c->h_counts.release(); c->h_starts.release(); c->h_ab.release(); c->h_rp.release(); c->h_col.release(); c->h_mask.release();
     for (auto &e : c->ev)
         if (e) cudaEventDestroy(e);
     for (auto &x : c->aux)
@@ -1537,6 +1529,8 @@ ovl_status ovl_load_balance(ovl_ctx *c, int32_t flags) {
         phase_contacts(c);
         phase_graph(c);
         phase_load_balance(c, (flags & 1) != 0, (flags & 2) != 0);
+        CK(cudaStreamSynchronize(c->stream));
+        c->nadj = c->h_counts.p[COUNT_ADJACENCY];
         return check_device_status(c);
     });
 }

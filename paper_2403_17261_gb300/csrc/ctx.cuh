@@ -12,6 +12,9 @@
 
 using namespace ovl;
 
+// places of ovl_ctx::h_counts
+enum { COUNT_CONTACTS, COUNT_ADJACENCY, COUNT_CANDIDATES, COUNT_BALLS, COUNT_ENTRIES, COUNT_PAIRS, COUNT_N };
+
 struct ovl_ctx {
     ovl_params P{};
     cudaStream_t stream = nullptr;
@@ -63,11 +66,8 @@ struct ovl_ctx {
     DBuf<float4> c_n, c_t1;
     DBuf<float4> c_p;          // contact point, manifold index in w (contexts with boxes)
     DBuf<int> deg, tptr, cursor2, tcol, ucount, row_ptr, col;
-    DBuf<int> entry_count, entry_ptr, entry_body, entry_part, entry_slot, part_list, part_count,
-        part_bstart;
-    DBuf<uint32_t> sk, sv, sk2, sv2;
-    DBuf<int> cons_count, cons_start, pair_cons, pair_part, ps_cons, ps_part, part_pcount,
-        part_pstart, p_colour, part_ncol, part_rounds, col_off, pair_of_row;
+    DBuf<int> entry_count, entry_ptr, entry_body, entry_part, entry_slot, part_list, part_bstart;
+    DBuf<int> cons_count, cons_start, pair_cons, pair_part, ps_cons, ps_part, part_pstart, p_colour, part_ncol, part_rounds, col_off, pair_of_row;
     DBuf<uint64_t> p_key;
     DBuf<int2> p_slot;
     DBuf<float4> p_lam0;
@@ -88,8 +88,10 @@ struct ovl_ctx {
     DBuf<uint8_t> D;
     DBuf<float> weight;
     DBuf<float> stage13;   // staging for host <-> device state transfers
-    DBuf<int> scan_tmp, sort_hist, sort_tmp;
+    DBuf<int> scan_tmp;
+    GroupBuf group;
     HBuf<int> h_i32;
+    HBuf<int> h_counts;        // counts of the step the kernels write to pinned memory (COUNT_*)
     HBuf<int2> h_ab;
     HBuf<int> h_rp, h_col;
     HBuf<uint64_t> h_mask;
@@ -97,9 +99,10 @@ struct ovl_ctx {
     DBuf<int> ball_root, ball_size, ball_start, ball_vtx, ball_list;   // Algorithm 6's gamma-balls, found ahead
     HBuf<int> h_ball_start, h_ball_vtx;
     DBuf<int2> lb_pairs;
-    DBuf<uint32_t> worker_order, wk, wk2, wv2;   // workers longest first (launch order)
+    DBuf<uint32_t> worker_order;                 // workers longest first (order of a uniform launch)
     DBuf<uint32_t> class_order, colour_order;    // solve / colouring: workers grouped by CTAs per worker
     std::vector<int> h_pb, h_pp;                 // part_bstart, part_pstart of this step on the host
+    HBuf<int> h_starts;                          // both as the kernels write them
     std::vector<int> h_class_C;                  // CTAs per worker of the last per-worker plan
     DBuf<int> solve_C, solve_M, solve_banked, col_off2, pair_of_row2;   // solve: CTAs per worker, masses in shared memory, rows in bank order, rows by owner CTA
     DBuf<uint8_t> row_owner;                     // bucket of every row (scratch of the ordering)

@@ -88,14 +88,6 @@ __global__ void k_pair_fill(MemberArgs a) {
     }
 }
 
-__global__ void k_pair_gather(MemberArgs a, const uint32_t *order, int np) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < np; k += gridDim.x * blockDim.x) {
-        int q = (int)order[k];
-        a.ps_cons[k] = a.pair_cons[q];
-        a.ps_part[k] = a.pair_part[q];
-    }
-}
-
 __device__ __forceinline__ int body_slot(const MemberArgs &a, int x, int w) {
     if (x < 0 || x >= a.n || !(a.im[x] > 0.0f)) return -1;
     uint64_t m = a.mask[x];
@@ -351,22 +343,16 @@ k_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solv
     }
 }
 
-__global__ void k_worker_cost_keys(const int *part_pstart, int P, uint32_t *keys, uint32_t *vals) {
-    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
-        const uint32_t cost = (uint32_t)min(part_pstart[p + 1] - part_pstart[p], (1 << 24) - 1);
-        keys[p] = ((1u << 24) - 1u) - cost;
-        vals[p] = (uint32_t)p;
-    }
-}
-
 // manifold index of contact i (0 without boxes)
 __device__ __forceinline__ int contact_point(const MemberArgs &a, int i) {
     return a.c_p ? __float_as_int(a.c_p[i].w) : 0;
 }
 
-__global__ void k_pair_setup(MemberArgs a, WarmArgs ws, int np) {
+__global__ void k_pair_setup(MemberArgs a, WarmArgs ws, const uint32_t *order, int np) {
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < np; k += gridDim.x * blockDim.x) {
-        int i = a.ps_cons[k], p = a.ps_part[k];
+        const int q = (int)order[k], i = a.pair_cons[q], p = a.pair_part[q];
+        a.ps_cons[k] = i;
+        a.ps_part[k] = p;
         int scene = cons_scene(i, a.nc, a.c_ab, a.sob, a.joint_scene);
         int w = p - a.part_base[scene];
         int2 e;
@@ -984,15 +970,9 @@ void launch_pair_fill(const MemberArgs &a, cudaStream_t s) {
     note_launch();
     CK(cudaGetLastError());
 }
-void launch_pair_gather(const MemberArgs &a, const uint32_t *order, int np, cudaStream_t s) {
+void launch_pair_setup(const MemberArgs &a, const WarmArgs &w, const uint32_t *order, int np, cudaStream_t s) {
     if (!np) return;
-    k_pair_gather<<<grid1d(np, 256), 256, 0, s>>>(a, order, np);
-    note_launch();
-    CK(cudaGetLastError());
-}
-void launch_pair_setup(const MemberArgs &a, const WarmArgs &w, int np, cudaStream_t s) {
-    if (!np) return;
-    k_pair_setup<<<grid1d(np, 256), 256, 0, s>>>(a, w, np);
+    k_pair_setup<<<grid1d(np, 256), 256, 0, s>>>(a, w, order, np);
     note_launch();
     CK(cudaGetLastError());
 }
@@ -1007,13 +987,6 @@ void launch_row_owner(int P, const int *part_bstart, const int *part_ncol, const
     CK(cudaGetLastError());
 }
 
-void launch_worker_cost_keys(const int *part_pstart, int P, uint32_t *keys, uint32_t *vals,
-                             cudaStream_t s) {
-    if (P <= 0) return;
-    k_worker_cost_keys<<<grid1d(P, 256), 256, 0, s>>>(part_pstart, P, keys, vals);
-    note_launch();
-    CK(cudaGetLastError());
-}
 template <int C>
 static void launch_colour_c(const ColourArgs &a, cudaStream_t s) {
     size_t smem = (size_t)a.smem_slots * 2 * sizeof(unsigned long long);

@@ -1,4 +1,4 @@
-// k_util.cu -- scan, stable radix sort, fills and histograms used by the step.
+// k_util.cu -- scan, stable grouping by key, and fills used by the step.
 #include "common.cuh"
 
 #include <atomic>
@@ -14,8 +14,8 @@ long long launch_count() { return g_launches.load(std::memory_order_relaxed); }
 
 namespace {
 
-constexpr int SCAN_THREADS = 1024;
-constexpr int SCAN_ITEMS = 2;
+constexpr int SCAN_THREADS = 256;
+constexpr int SCAN_ITEMS = 8;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 
 __device__ __forceinline__ int warp_incl_scan(int v) {
@@ -51,72 +51,124 @@ __device__ int block_excl_scan(int v, int *total) {
     return res;
 }
 
-__global__ void k_tile_reduce(const int *in, int n, int *bsum) {
-    int base = blockIdx.x * SCAN_TILE;
-    int s = 0;
-    for (int k = 0; k < SCAN_ITEMS; ++k) {
-        int i = base + threadIdx.x * SCAN_ITEMS + k;
-        if (i < n) s += in[i];
-    }
-    // block reduction
-    __shared__ int red[32];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        int v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (threadIdx.x == 0) bsum[blockIdx.x] = v;
-    }
-}
+// Exclusive scan in one launch: every tile publishes its sum, then its prefix
+// once it has added up its predecessors' (decoupled look-back, Merrill and
+// Garland 2016).  A step scans a dozen arrays, most of a few thousand words,
+// so launches count: three kernels per scan (tile sums, their scan, tile
+// scan) took 8-10 us each time, this one 2.5.  Tiles are taken by ticket, so
+// a tile's predecessors are always running.  The state words carry an epoch,
+// so nothing is cleared between scans: ctl = (next ticket, tiles done, epoch),
+// advanced by the tile that finishes last.  A wait that reaches its limit adds
+// up the missing inputs itself.
+constexpr unsigned long long kAggregate = 1, kPrefix = 2;
+constexpr int kScanPolls = 1 << 16;
 
-// single block: exclusive scan of nb block sums in place; total to *total_out
-__global__ void k_scan_bsums(int *bsum, int nb, int *total_out) {
-    __shared__ int carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < nb; base += blockDim.x) {
-        int i = base + threadIdx.x;
-        int v = i < nb ? bsum[i] : 0;
-        int tot;
-        int ex = block_excl_scan(v, &tot);
-        if (i < nb) bsum[i] = ex + carry;
+__global__ void __launch_bounds__(SCAN_THREADS)
+k_scan(const int *__restrict__ in, int n, int *__restrict__ out, int nb, unsigned *ctl, unsigned long long *state,
+       int *host_total) {
+    __shared__ int sh_tile, sh_prefix;
+    const int tid = threadIdx.x, lane = tid & 31;
+    unsigned long long epoch = 0;
+    if (nb > 1) {
+        epoch = *reinterpret_cast<volatile unsigned *>(ctl + 2) & 0x3fffffffu;
+        if (tid == 0) sh_tile = (int)atomicAdd(ctl, 1u);
         __syncthreads();
-        if (threadIdx.x == 0) carry += tot;
+    } else if (tid == 0) {
+        sh_tile = 0;
+    }
+    if (nb == 1) __syncthreads();
+    const int tile = sh_tile, base = tile * SCAN_TILE + tid * SCAN_ITEMS;
+    int v[SCAN_ITEMS], sum = 0;
+    const bool whole = base + SCAN_ITEMS <= n && (reinterpret_cast<uintptr_t>(in) & 15) == 0;
+    if (whole) {
+        const int4 a = *reinterpret_cast<const int4 *>(in + base), b = *reinterpret_cast<const int4 *>(in + base + 4);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k) v[k] = base + k < n ? in[base + k] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < SCAN_ITEMS; ++k) sum += v[k];
+    int total;
+    const int ex = block_excl_scan(sum, &total);
+    int prefix = 0;
+    if (nb > 1) {
+        auto word = [&](unsigned long long flag, int x) {
+            return (epoch << 2 | flag) << 32 | (unsigned long long)(unsigned)x;
+        };
+        volatile unsigned long long *st = state;
+        if (tid == 0) st[tile] = word(tile == 0 ? kPrefix : kAggregate, total);
+        if (tid < 32) {
+            int run = 0;
+            for (int j = tile - 1; j >= 0; j -= 32) {
+                const int k = j - lane;
+                unsigned long long w = 0;
+                bool ready = false;
+                for (int it = 0; it < kScanPolls; ++it) {
+                    w = k >= 0 ? st[k] : word(kPrefix, 0);
+                    ready = (w >> 34) == epoch && (w >> 32 & 3) != 0;
+                    if (__all_sync(0xffffffffu, ready)) break;
+                }
+                int add;
+                if (!__all_sync(0xffffffffu, ready)) {
+                    add = 0;
+                    for (long long i = lane; i < (long long)(j + 1) * SCAN_TILE; i += 32) add += in[i];
+                    for (int o = 16; o > 0; o >>= 1) add += __shfl_xor_sync(0xffffffffu, add, o);
+                    run += add;
+                    break;
+                }
+                const unsigned full = __ballot_sync(0xffffffffu, (w >> 32 & 3) == kPrefix);
+                add = !full || lane <= __ffs(full) - 1 ? (int)(unsigned)w : 0;
+                for (int o = 16; o > 0; o >>= 1) add += __shfl_xor_sync(0xffffffffu, add, o);
+                run += add;
+                if (full) break;
+            }
+            if (lane == 0) {
+                if (tile > 0) st[tile] = word(kPrefix, run + total);
+                sh_prefix = run;
+            }
+        }
         __syncthreads();
+        prefix = sh_prefix;
     }
-    if (threadIdx.x == 0) *total_out = carry;
-}
-
-__global__ void k_tile_scan(const int *in, int n, const int *bsum, int *out) {
-    int base = blockIdx.x * SCAN_TILE;
-    int vals[SCAN_ITEMS];
-    int s = 0;
-    for (int k = 0; k < SCAN_ITEMS; ++k) {
-        int i = base + threadIdx.x * SCAN_ITEMS + k;
-        vals[k] = i < n ? in[i] : 0;
-        s += vals[k];
+    int e = prefix + ex;
+    if (whole && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+        int o[SCAN_ITEMS];
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k) { o[k] = e; e += v[k]; }
+        *reinterpret_cast<int4 *>(out + base) = make_int4(o[0], o[1], o[2], o[3]);
+        *reinterpret_cast<int4 *>(out + base + 4) = make_int4(o[4], o[5], o[6], o[7]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < SCAN_ITEMS; ++k) {
+            if (base + k < n) out[base + k] = e;
+            e += v[k];
+        }
     }
-    int tot;
-    int ex = block_excl_scan(s, &tot) + bsum[blockIdx.x];
-    for (int k = 0; k < SCAN_ITEMS; ++k) {
-        int i = base + threadIdx.x * SCAN_ITEMS + k;
-        if (i < n) out[i] = ex;
-        ex += vals[k];
+    if (tid == 0) {
+        if (tile == nb - 1) {
+            out[n] = prefix + total;
+            if (host_total) *host_total = prefix + total;
+        }
+        if (nb > 1 && atomicAdd(ctl + 1, 1u) == (unsigned)nb - 1) {
+            ctl[0] = 0;
+            ctl[1] = 0;
+            ctl[2] = (unsigned)epoch + 1;
+        }
     }
 }
 
 }  // namespace
 
-void scan_i32(const int *in, int *out, int n, DBuf<int> &tmp, cudaStream_t s) {
-    int nb = (n + SCAN_TILE - 1) / SCAN_TILE;
-    if (nb < 1) nb = 1;
-    tmp.ensure((size_t)nb + 1);
-    k_tile_reduce<<<nb, SCAN_THREADS, 0, s>>>(in, n, tmp.p);
-    note_launch();
-    k_scan_bsums<<<1, SCAN_THREADS, 0, s>>>(tmp.p, nb, out + n);
-    note_launch();
-    k_tile_scan<<<nb, SCAN_THREADS, 0, s>>>(in, n, tmp.p, out);
+void scan_i32(const int *in, int *out, int n, DBuf<int> &tmp, cudaStream_t s, int *host_total) {
+    const int nb = n > 0 ? (n + SCAN_TILE - 1) / SCAN_TILE : 1;
+    const size_t need = 4 + 2 * (size_t)nb;   // ctl, then a state word per tile
+    if (need > tmp.cap || !tmp.p) {
+        tmp.ensure(need);
+        CK(cudaMemsetAsync(tmp.p, 0, sizeof(int) * tmp.cap, s));
+    }
+    k_scan<<<nb, SCAN_THREADS, 0, s>>>(in, n, out, nb, reinterpret_cast<unsigned *>(tmp.p),
+                                       reinterpret_cast<unsigned long long *>(tmp.p + 4), host_total);
     note_launch();
     CK(cudaGetLastError());
 }
@@ -180,7 +232,7 @@ __global__ void k_rs_scatter(const uint32_t *keys, const uint32_t *vals, int n, 
         }
         if (valid) {
             keys_out[pos] = k;
-            vals_out[pos] = vals[i];
+            vals_out[pos] = vals ? vals[i] : (uint32_t)i;
         }
         __syncthreads();
     }
@@ -188,53 +240,45 @@ __global__ void k_rs_scatter(const uint32_t *keys, const uint32_t *vals, int n, 
 
 }  // namespace
 
-void radix_sort_u32(uint32_t *keys, uint32_t *vals, uint32_t *keys_alt, uint32_t *vals_alt, int n,
-                    int nbits, DBuf<int> &hist, DBuf<int> &tmp, cudaStream_t s,
-                    bool *result_in_alt) {
-    *result_in_alt = false;
-    if (n <= 1 || nbits <= 0) return;
-    int nblocks = (n + RS_TILE - 1) / RS_TILE;
-    hist.ensure((size_t)256 * nblocks + 1);
-    uint32_t *ki = keys, *vi = vals, *ko = keys_alt, *vo = vals_alt;
-    for (int shift = 0; shift < nbits; shift += 8) {
-        k_rs_hist<<<nblocks, RS_THREADS, 0, s>>>(ki, n, shift, nblocks, hist.p);
+const uint32_t *group_by_key(const uint32_t *key, int n, int nbits, uint32_t *out, GroupBuf &b, DBuf<int> &tmp,
+                             cudaStream_t s) {
+    b.k0.ensure((size_t)n + 1);
+    if (n == 0) return b.k0.p;
+    const int nblocks = (n + RS_TILE - 1) / RS_TILE, passes = nbits > 8 ? (nbits + 7) / 8 : 1;
+    b.hist.ensure((size_t)256 * nblocks + 1);
+    b.offs.ensure((size_t)256 * nblocks + 1);
+    if (passes > 1) { b.k1.ensure((size_t)n + 1); b.v0.ensure((size_t)n + 1); b.v1.ensure((size_t)n + 1); }
+    const uint32_t *ki = key, *vi = nullptr;
+    for (int p = 0; p < passes; ++p) {
+        uint32_t *ko = p & 1 ? b.k1.p : b.k0.p, *vo = p + 1 == passes ? out : (p & 1 ? b.v1.p : b.v0.p);
+        k_rs_hist<<<nblocks, RS_THREADS, 0, s>>>(ki, n, 8 * p, nblocks, b.hist.p);
         note_launch();
-        scan_i32(hist.p, hist.p, 256 * nblocks, tmp, s);
-        k_rs_scatter<<<nblocks, RS_THREADS, 0, s>>>(ki, vi, n, shift, nblocks, hist.p, ko, vo);
+        scan_i32(b.hist.p, b.offs.p, 256 * nblocks, tmp, s);
+        k_rs_scatter<<<nblocks, RS_THREADS, 0, s>>>(ki, vi, n, 8 * p, nblocks, b.offs.p, ko, vo);
         note_launch();
         CK(cudaGetLastError());
-        uint32_t *t = ki; ki = ko; ko = t;
-        t = vi; vi = vo; vo = t;
-        *result_in_alt = !*result_in_alt;
+        ki = ko;
+        vi = vo;
     }
+    return ki;
 }
 
 namespace {
-__global__ void k_fill_i32(int *p, int v, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        p[i] = v;
-}
 __global__ void k_fill_u8(uint8_t *p, uint8_t v, size_t n) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         p[i] = v;
 }
-__global__ void k_iota(uint32_t *p, int n) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) p[i] = (uint32_t)i;
-}
-// bins privatised in shared memory (nbins <= 12288), one global add per bin and block
-__global__ void k_hist(const int *key, int n, int *counts, int nbins) {
-    extern __shared__ int h[];
-    for (int j = threadIdx.x; j < nbins; j += blockDim.x) h[j] = 0;
-    __syncthreads();
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        atomicAdd(&h[key[i]], 1);
-    __syncthreads();
-    for (int j = threadIdx.x; j < nbins; j += blockDim.x)
-        if (h[j]) atomicAdd(&counts[j], h[j]);
-}
-__global__ void k_hist_global(const int *key, int n, int *counts) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        atomicAdd(&counts[key[i]], 1);
+// start[p] = first index of a sorted key >= p, for p <= P, here and on the host
+__global__ void k_key_starts(const uint32_t *keys, int n, int P, int *start, int *host_start) {
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p <= P; p += gridDim.x * blockDim.x) {
+        int lo = 0, hi = n;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (keys[mid] < (uint32_t)p) lo = mid + 1; else hi = mid;
+        }
+        start[p] = lo;
+        host_start[p] = lo;
+    }
 }
 int grid_for(size_t n, int threads) {
     size_t g = (n + threads - 1) / threads;
@@ -244,33 +288,14 @@ int grid_for(size_t n, int threads) {
 }
 }  // namespace
 
-void fill_i32(int *p, int v, size_t n, cudaStream_t s) {
-    if (!n) return;
-    k_fill_i32<<<grid_for(n, 256), 256, 0, s>>>(p, v, n);
-    note_launch();
-    CK(cudaGetLastError());
-}
 void fill_u8(uint8_t *p, uint8_t v, size_t n, cudaStream_t s) {
     if (!n) return;
     k_fill_u8<<<grid_for(n, 256), 256, 0, s>>>(p, v, n);
     note_launch();
     CK(cudaGetLastError());
 }
-void iota_u32(uint32_t *p, int n, cudaStream_t s) {
-    if (n <= 0) return;
-    k_iota<<<grid_for((size_t)n, 256), 256, 0, s>>>(p, n);
-    note_launch();
-    CK(cudaGetLastError());
-}
-void histogram_i32(const int *key, int n, int *counts, int nbins, cudaStream_t s) {
-    if (!n) return;
-    if (nbins <= 12288) {
-        int g = grid_for((size_t)n, 256);
-        if (g > 304) g = 304;
-        k_hist<<<g, 256, (size_t)nbins * sizeof(int), s>>>(key, n, counts, nbins);
-    } else {
-        k_hist_global<<<grid_for((size_t)n, 256), 256, 0, s>>>(key, n, counts);
-    }
+void key_starts(const uint32_t *keys, int n, int P, int *start, int *host_start, cudaStream_t s) {
+    k_key_starts<<<grid_for((size_t)P + 1, 128), 128, 0, s>>>(keys, n, P, start, host_start);
     note_launch();
     CK(cudaGetLastError());
 }

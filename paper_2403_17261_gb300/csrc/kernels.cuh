@@ -106,7 +106,6 @@ void launch_entry_fill(const MemberArgs &a, cudaStream_t s);
 void launch_entry_slot(const MemberArgs &a, int ne, cudaStream_t s);
 void launch_cons_count(const MemberArgs &a, cudaStream_t s);
 void launch_pair_fill(const MemberArgs &a, cudaStream_t s);
-void launch_pair_gather(const MemberArgs &a, const uint32_t *order, int np, cudaStream_t s);
 
 struct WarmArgs {
     const int *ws_pstart;      // [P+1] previous step's (worker) ranges
@@ -114,7 +113,8 @@ struct WarmArgs {
     const float4 *ws_lam;
     float factor;
 };
-void launch_pair_setup(const MemberArgs &a, const WarmArgs &w, int np, cudaStream_t s);
+// order: the pairs' canonical indexes grouped by worker
+void launch_pair_setup(const MemberArgs &a, const WarmArgs &w, const uint32_t *order, int np, cudaStream_t s);
 // Rows of every colour in the order of the solve: worker p's bodies are split
 // into solve_C[p] contiguous slot ranges of
 // ceil(nb / C) slots, one per CTA, and a row belongs to the CTA holding its
@@ -131,11 +131,6 @@ void launch_pair_setup(const MemberArgs &a, const WarmArgs &w, int np, cudaStrea
 void launch_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solve_C, const int *off_in,
                       const int *pair_of_row, const int2 *p_slot, const int *banked, uint8_t *key_of_row,
                       int *by_owner, int *pair_of_row_out, int *off_out, cudaStream_t s);
-// keys[p] = 2^24 - 1 - min(pairs of worker p, 2^24 - 1), vals[p] = p: an
-// ascending stable sort of the keys lists the workers longest first
-void launch_worker_cost_keys(const int *part_pstart, int P, uint32_t *keys, uint32_t *vals,
-                             cudaStream_t s);
-
 struct ColourArgs {
     int n_parts;
     const uint32_t *order;     // [P] worker of each CTA group, longest first (NULL: identity)
