@@ -21,8 +21,7 @@
 #include "../../include/ovl.h"
 
 #define OVL_MAX_COLOURS 128
-#define OVL_MAX_NEIGH 32   // sphere neighbours with larger index kept in registers per body; bodies
-                           // whose neighbour capacity is larger continue in their global range
+#define OVL_MAX_NEIGH 32   // smallest neighbour capacity of a body; lists up to this are sorted in a thread's own memory
 
 // device status codes (first error wins)
 #define DEV_OK 0

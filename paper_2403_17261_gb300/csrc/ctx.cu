@@ -74,19 +74,18 @@ void phase_contacts(ovl_ctx *c) {
     c->cell.ensure(n);
     c->bucket_count.ensure((size_t)c->tsize + 1);
     c->bucket_start.ensure((size_t)c->tsize + 1);
-    c->cursor.ensure(c->tsize);
     c->items.ensure(n);
+    c->centres.ensure(n);
     c->nb_list.ensure((size_t)c->nb_total + 1);
     c->nb_count.ensure(n);
     c->ccount.ensure((size_t)n + 1);
     c->cstart.ensure((size_t)n + 1);
     CK(cudaMemsetAsync(c->bucket_count.p, 0, sizeof(int) * ((size_t)c->tsize + 1), s));
-    CK(cudaMemsetAsync(c->cursor.p, 0, sizeof(int) * c->tsize, s));
     ContactArgs a{};
     a.st = c->st.p; a.im = c->im.p; a.n = n; a.sob = c->sob.p; a.scene_flags = c->scene_flags.p;
     a.inv_cs = 1.0f / c->cs; a.tmask = c->tsize - 1;
     a.cell = c->cell.p; a.bucket_count = c->bucket_count.p; a.bucket_start = c->bucket_start.p;
-    a.cursor = c->cursor.p; a.items = c->items.p; a.planes = c->planes.p;
+    a.items = c->items.p; a.centres = c->centres.p; a.planes = c->planes.p;
     a.plane_ptr = c->plane_ptr.p; a.plane_list = c->plane_list.p; a.margin = c->P.margin;
     a.nb_list = c->nb_list.p; a.nb_off = c->nb_off.p; a.nb_count = c->nb_count.p;
     a.contact_count = c->ccount.p;
@@ -105,7 +104,7 @@ void phase_contacts(ovl_ctx *c) {
     if (c->has_boxes) c->c_p.ensure(c->nc + 1);
     a.c_ab = c->c_ab.p; a.c_n = c->c_n.p; a.c_t1 = c->c_t1.p;
     a.c_p = contact_points(c);
-    launch_write_contacts(a, s);
+    launch_write_contacts(a, c->nc, s);
 }
 
 void phase_graph(ovl_ctx *c) {
@@ -118,7 +117,7 @@ void phase_graph(ovl_ctx *c) {
     c->row_ptr.ensure((size_t)n + 1);
     CK(cudaMemsetAsync(c->deg.p, 0, sizeof(int) * ((size_t)n + 1), s));
     CK(cudaMemsetAsync(c->cursor2.p, 0, sizeof(int) * ((size_t)n + 1), s));
-    launch_edge_degree(c->c_ab.p, c->nc, c->jab.p, c->nj, c->im.p, n, c->deg.p, s);
+    launch_edge_degree(c->c_ab.p, c->nc, c->jab.p, c->nj, c->im.p, n, c->deg.p, contact_points(c), s);
     scan_i32(c->deg.p, c->tptr.p, n, c->scan_tmp, s);
     // at most two directed edges per constraint, so neither count is waited
     // for here: the adjacency's is read after the next wait
@@ -126,7 +125,7 @@ void phase_graph(ovl_ctx *c) {
     c->tcol.ensure(most);
     c->col.ensure(most);
     launch_edge_fill(c->c_ab.p, c->nc, c->jab.p, c->nj, c->im.p, n, c->tptr.p, c->cursor2.p,
-                     c->tcol.p, s);
+                     c->tcol.p, contact_points(c), s);
     launch_adj_unique(c->tptr.p, n, c->tcol.p, c->ucount.p, s);
     scan_i32(c->ucount.p, c->row_ptr.p, n, c->scan_tmp, s, c->h_counts.p + COUNT_ADJACENCY);
     launch_adj_compact(c->tptr.p, c->tcol.p, n, c->row_ptr.p, c->col.p, s);
@@ -1084,7 +1083,7 @@ void release_all(ovl_ctx *c) {
     c->joint_scene.release(); c->part_scene.release(); c->planes.release(); c->plane_ptr.release();
     c->plane_list.release(); c->jab.release(); c->janc.release(); c->vb_base.release();
     c->mask.release(); c->cell.release(); c->bucket_count.release(); c->bucket_start.release();
-    c->cursor.release(); c->items.release(); c->nb_list.release(); c->nb_count.release(); c->nb_off.release();
+    c->centres.release(); c->items.release(); c->nb_list.release(); c->nb_count.release(); c->nb_off.release();
     c->ccount.release(); c->cstart.release(); c->c_ab.release(); c->c_n.release(); c->c_t1.release();
     c->deg.release(); c->tptr.release(); c->cursor2.release(); c->tcol.release(); c->ucount.release();
     c->row_ptr.release(); c->col.release(); c->entry_count.release(); c->entry_ptr.release();

@@ -58,8 +58,8 @@ struct ovl_ctx {
 
     // step buffers
     DBuf<int> status;
-    DBuf<int4> cell;
-    DBuf<int> bucket_count, bucket_start, cursor, items, nb_list, nb_count, ccount, cstart;
+    DBuf<float4> centres;
+    DBuf<int> cell, bucket_count, bucket_start, items, nb_list, nb_count, ccount, cstart;
     DBuf<long long> nb_off;    // per-body neighbour capacity offsets (set at scene upload)
     long long nb_total = 0;
     DBuf<int2> c_ab;

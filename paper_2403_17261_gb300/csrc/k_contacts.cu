@@ -4,6 +4,11 @@
 //
 // Broadphase: spatial hash grid, one thread per body (cell size >= the
 // largest contact distance, so touching spheres sit in neighbouring cells).
+// Cells of one (x, y) column lie in consecutive buckets, and the centres are
+// stored in bucket order, so the 27 cells around a body are nine contiguous
+// runs of centres.  (With a bucket per cell anywhere in the table and the
+// centres read through it, four dependent loads per cell, the large pile's
+// search took 259 us, now 164.)
 // Narrowphase: sphere-sphere (a < b) and sphere-plane.  The contact test and
 // the choice of tangent axis decide integers, so they are evaluated in FP32
 // with explicit round-to-nearest operations in a fixed order (no fused
@@ -31,31 +36,35 @@ namespace ovl {
 
 namespace {
 
-__device__ __forceinline__ uint32_t cell_hash(int ix, int iy, int iz, int scene, uint32_t mask) {
-    uint32_t h = ((uint32_t)ix * 73856093u) ^ ((uint32_t)iy * 19349663u) ^
-                 ((uint32_t)iz * 83492791u) ^ ((uint32_t)scene * 2654435761u);
-    return h & mask;
+// bucket of cell (ix, iy, iz): the column's, plus iz
+__device__ __forceinline__ uint32_t column_hash(int ix, int iy, int scene) {
+    return ((uint32_t)ix * 73856093u) ^ ((uint32_t)iy * 19349663u) ^ ((uint32_t)scene * 2654435761u);
 }
 
-__global__ void k_cells(const float4 *__restrict__ st, int n, const int *__restrict__ sob,
-                        float inv_cs, uint32_t tmask, int4 *__restrict__ cell,
-                        int *__restrict__ bucket_count) {
+__device__ __forceinline__ int3 cell_of(float4 p, float inv_cs) {
+    return make_int3((int)floorf(p.x * inv_cs), (int)floorf(p.y * inv_cs), (int)floorf(p.z * inv_cs));
+}
+
+__global__ void k_cells(const float4 *__restrict__ st, int n, const int *__restrict__ sob, float inv_cs, uint32_t tmask,
+                        int *__restrict__ cell, int *__restrict__ bucket_count) {
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < n; b += gridDim.x * blockDim.x) {
-        float4 p = st[4 * b];
-        int ix = (int)floorf(p.x * inv_cs), iy = (int)floorf(p.y * inv_cs),
-            iz = (int)floorf(p.z * inv_cs);
-        uint32_t h = cell_hash(ix, iy, iz, sob[b], tmask);
-        cell[b] = make_int4(ix, iy, iz, (int)h);
+        const int3 c = cell_of(st[4 * b], inv_cs);
+        const uint32_t h = (column_hash(c.x, c.y, sob[b]) + (uint32_t)c.z) & tmask;
+        cell[b] = (int)h;
         atomicAdd(&bucket_count[h], 1);
     }
 }
 
-__global__ void k_bucket_fill(const int4 *__restrict__ cell, int n, const int *__restrict__ bstart,
-                              int *__restrict__ cursor, int *__restrict__ items) {
+// centres and radii in bucket order (any order inside a bucket); the counts
+// serve as cursors
+__global__ void k_bucket_fill(const float4 *__restrict__ st, const int *__restrict__ cell, int n,
+                              const int *__restrict__ bstart, int *__restrict__ bucket_count, int *__restrict__ items,
+                              float4 *__restrict__ centres) {
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < n; b += gridDim.x * blockDim.x) {
-        int h = cell[b].w;
-        int slot = atomicAdd(&cursor[h], 1);
-        items[bstart[h] + slot] = b;
+        const int h = cell[b];
+        const int k = bstart[h] + atomicSub(&bucket_count[h], 1) - 1;
+        items[k] = b;
+        centres[k] = st[4 * b];
     }
 }
 
@@ -121,183 +130,326 @@ __device__ __forceinline__ void write_box_contact(int o, int a, int b, int k, do
     c_p[o] = make_float4((float)p.x, (float)p.y, (float)p.z, __int_as_float(k));
 }
 
-// neighbours b > a of body a (sorted ascending) + its plane contacts
-// X: the context has boxes.  The box narrow phase (FP64 locals, a large
-// stack) is only in the X kernels, so sphere scenes keep a lean kernel.
-template <bool X>
-__global__ void k_find_pairs(const float4 *__restrict__ st, const float *__restrict__ im, int n,
-                             const int *__restrict__ sob, const int *__restrict__ scene_flags,
-                             const int4 *__restrict__ cell, const int *__restrict__ bstart,
-                             const int *__restrict__ items, uint32_t tmask,
-                             const float4 *__restrict__ planes, const int *__restrict__ plane_ptr,
-                             const int *__restrict__ plane_list, float margin,
-                             int *__restrict__ nb_list, const long long *__restrict__ nb_off,
-                             int *__restrict__ nb_count, int *__restrict__ contact_count,
-                             int *__restrict__ status, const float4 *__restrict__ half) {
-    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < n; a += gridDim.x * blockDim.x) {
-        const int s = sob[a];
-        const float4 pa = st[4 * a];   // .w = radius
-        const bool dyn_a = im[a] > 0.0f;
-        int cnt = 0;
-        int local[OVL_MAX_NEIGH];
-        int *const gl = nb_list + nb_off[a];
-        const int cap = (int)(nb_off[a + 1] - nb_off[a]);
-        bool spilled = false;   // the list continues in gl (more than OVL_MAX_NEIGH neighbours)
-        bool overflow = false;
-        if (scene_flags[s] & 1) {
-            const int4 ca = cell[a];
-            for (int dx = -1; dx <= 1; ++dx)
-                for (int dy = -1; dy <= 1; ++dy)
-                    for (int dz = -1; dz <= 1; ++dz) {
-                        const int cx = ca.x + dx, cy = ca.y + dy, cz = ca.z + dz;
-                        const uint32_t h = cell_hash(cx, cy, cz, s, tmask);
-                        for (int k = bstart[h]; k < bstart[h + 1]; ++k) {
-                            const int b = items[k];
-                            if (b <= a) continue;
-                            const int4 cb = cell[b];
-                            if (cb.x != cx || cb.y != cy || cb.z != cz || sob[b] != s) continue;
-                            if (!dyn_a && !(im[b] > 0.0f)) continue;
-                            if (!pair_touches(pa, st[4 * b], margin)) continue;
-                            if (!spilled && cnt == OVL_MAX_NEIGH && cap > OVL_MAX_NEIGH) {
-                                for (int j = 0; j < cnt; ++j) gl[j] = local[j];
-                                spilled = true;
-                            }
-                            if (cnt >= (spilled ? cap : OVL_MAX_NEIGH)) {
-                                overflow = true;
-                                continue;
-                            }
-                            // insertion into the sorted list
-                            int *lst = spilled ? gl : local;
-                            int j = cnt;
-                            while (j > 0 && lst[j - 1] > b) {
-                                lst[j] = lst[j - 1];
-                                --j;
-                            }
-                            lst[j] = b;
-                            ++cnt;
-                        }
-                    }
+// What the pair search reads (see ContactArgs).
+struct PairArgs {
+    const float4 *st;
+    const float *im;
+    int n;
+    const int *sob, *scene_flags;
+    float inv_cs;
+    const int *bstart, *items;
+    const float4 *centres;
+    uint32_t tmask;
+    const float4 *planes;
+    const int *plane_ptr, *plane_list;
+    float margin;
+    int *nb_list;
+    const long long *nb_off;
+    int *nb_count, *contact_count, *status;
+};
+
+// The centres that touch body a (centre pa, cell ca, scene s) in column c of
+// the nine around it: take(k) for each, k its place in bucket order.  A bucket
+// may hold other cells too; other scenes are left to the caller.
+template <class F>
+__device__ __forceinline__ void touching_in_column(const PairArgs &g, float4 pa, int3 ca, int s, int c, F &&take) {
+    const int cx = ca.x + c / 3 - 1, cy = ca.y + c % 3 - 1;
+    auto run = [&](int k0, int k1) {
+        for (int k = k0; k < k1; ++k) {
+            const float4 pb = g.centres[k];
+            if (!pair_touches(pa, pb, g.margin)) continue;
+            const int3 cb = cell_of(pb, g.inv_cs);
+            if (cb.x == cx && cb.y == cy && abs(cb.z - ca.z) <= 1) take(k);
         }
-        if (overflow) atomicCAS(status, DEV_OK, DEV_ERR_CAPACITY);
-        if (!spilled)
-            for (int j = 0; j < cnt; ++j) gl[j] = local[j];
-        nb_count[a] = cnt;
-        // contacts: one per sphere pair, 0-4 per pair with a box end
-        int nct = cnt;
-        if constexpr (X) {
-            const int *lst = spilled ? gl : local;
-            nct = 0;
-            for (int j = 0; j < cnt; ++j) {
-                const int b = lst[j];
-                if (!is_box(half, a) && !is_box(half, b)) { ++nct; continue; }
-                double3 pts[4], nrm;
-                double gaps[4];
-                nct += box_pair(st, half, nullptr, a, b, margin, pts, gaps, nrm);
-            }
-        }
-        int np_ = 0;
-        if (dyn_a) {
-            const bool box_a = X && is_box(half, a);
-            for (int k = plane_ptr[s]; k < plane_ptr[s + 1]; ++k) {
-                const float4 pl = planes[plane_list[k]];
-                if (plane_gap(pa, pl) > margin) continue;   // the (bounding) sphere test
-                if (!box_a) { ++np_; continue; }
-                if constexpr (X) {
-                    double3 pts[4], nrm;
-                    double gaps[4];
-                    np_ += box_plane_pair(st, half, a, pl, margin, pts, gaps, nrm);
-                }
-            }
-        }
-        contact_count[a] = nct + np_;
+    };
+    const uint32_t h0 = column_hash(cx, cy, s) + (uint32_t)(ca.z - 1), h = h0 & g.tmask;
+    if (h + 2u <= g.tmask) {
+        run(g.bstart[h], g.bstart[h + 3]);
+    } else {
+        // the column's buckets wrap around the table's end (with a table of
+        // fewer than three buckets they would repeat)
+        for (uint32_t d = 0; d < 3u && d <= g.tmask; ++d)
+            run(g.bstart[(h0 + d) & g.tmask], g.bstart[((h0 + d) & g.tmask) + 1]);
     }
 }
 
-template <bool X>
-__global__ void k_write_contacts(const float4 *__restrict__ st, const float *__restrict__ im, int n,
-                                 const int *__restrict__ sob, const float4 *__restrict__ planes,
-                                 const int *__restrict__ plane_ptr, const int *__restrict__ plane_list,
-                                 float margin, const int *__restrict__ nb_list,
-                                 const long long *__restrict__ nb_off,
-                                 const int *__restrict__ nb_count, const int *__restrict__ cstart,
-                                 int2 *__restrict__ c_ab, float4 *__restrict__ c_n,
-                                 float4 *__restrict__ c_t1, const float4 *__restrict__ half,
-                                 float4 *__restrict__ c_p) {
-    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < n; a += gridDim.x * blockDim.x) {
-        const float4 pa = st[4 * a];
-        int o = cstart[a];
-        const int cnt = nb_count[a];
-        for (int j = 0; j < cnt; ++j) {
-            const int b = nb_list[nb_off[a] + j];
-            const float4 pb = st[4 * b];
-            if constexpr (X) {
-                if (is_box(half, a) || is_box(half, b)) {
-                    double3 pts[4], nrm;
-                    double gaps[4];
-                    const int m = box_pair(st, half, nullptr, a, b, margin, pts, gaps, nrm);
-                    for (int k = 0; k < m; ++k)
-                        write_box_contact(o++, a, b, k, pts[k], gaps[k], nrm, c_ab, c_n, c_t1, c_p);
-                    continue;
-                }
-            }
-            float dx = __fsub_rn(pb.x, pa.x), dy = __fsub_rn(pb.y, pa.y), dz = __fsub_rn(pb.z, pa.z);
-            float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-            float L = __fsqrt_rn(d2);
-            float3 nn;
-            int k;
-            if (L == 0.0f) {
-                nn = make_float3(0.f, 0.f, 1.f);
-                k = 0;
-            } else {
-                nn = make_float3(__fdiv_rn(dx, L), __fdiv_rn(dy, L), __fdiv_rn(dz, L));
-                k = tangent_axis(nn.x, nn.y, nn.z);
-            }
-            float3 t = tangent_from(nn, k);
-            // The gap from the exact FP64 differences of the FP32 centres and an
-            // FP64 square root, rounded once: it enters the speculative target
-            // -phi / h, which multiplies an FP32 rounding of |d| (~1e-7 m)
-            // into ~1e-5 m/s of velocity.
-            const double ex = (double)pb.x - (double)pa.x, ey = (double)pb.y - (double)pa.y,
-                         ez = (double)pb.z - (double)pa.z;
-            const double L64 = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)));
-            const float phi = (float)((L64 - (double)pa.w) - (double)pb.w);
-            c_ab[o] = make_int2(a, b);
-            c_n[o] = make_float4(nn.x, nn.y, nn.z, phi);
-            c_t1[o] = make_float4(t.x, t.y, t.z, 0.f);
-            if (c_p) c_p[o] = make_float4(0.f, 0.f, 0.f, __int_as_float(0));
-            ++o;
-        }
-        if (im[a] > 0.0f) {
-            const int s = sob[a];
-            const bool box_a = X && is_box(half, a);
-            for (int k2 = plane_ptr[s]; k2 < plane_ptr[s + 1]; ++k2) {
-                const int pidx = plane_list[k2];
-                const float4 pl = planes[pidx];
-                if (plane_gap(pa, pl) > margin) continue;   // the FP32 (bounding-sphere) decision
-                if constexpr (X) {
-                    if (box_a) {
-                        double3 pts[4], nrm;
-                        double gaps[4];
-                        const int m = box_plane_pair(st, half, a, pl, margin, pts, gaps, nrm);
-                        for (int k = 0; k < m; ++k)
-                            write_box_contact(o++, a, n + pidx, k, pts[k], gaps[k], nrm, c_ab, c_n, c_t1, c_p);
+// whether the k-th centre is a neighbour b > a of body a; b
+__device__ __forceinline__ bool is_neighbour(const PairArgs &g, int a, int s, bool dyn_a, int k, int &b) {
+    b = g.items[k];
+    return b > a && g.sob[b] == s && (dyn_a || g.im[b] > 0.0f);
+}
+
+// inserts b into the sorted list of m bodies
+__device__ __forceinline__ void insert_sorted(int *lst, int m, int b) {
+    while (m > 0 && lst[m - 1] > b) {
+        lst[m] = lst[m - 1];
+        --m;
+    }
+    lst[m] = b;
+}
+
+// Neighbours b > a of body a (sorted ascending, by the (bounding) sphere
+// test) and, without boxes, its number of contacts.  One thread per body, or
+// PAIR_LANES (a column of cells each) while all their threads fit the chip at
+// once: the walk is a chain of loads and branches, which a small scene has too
+// few threads to hide and a large one does not need split.  Measured: 34 k
+// bodies of mixed radii 202 us with one thread, 72 with eight; 2.6 k boxes 61
+// and 28; 262 k bodies 164 and 259; 512 scenes of 1.45 M bodies 291 and 916.
+constexpr int PAIR_LANES = 8, PAIR_THREADS = 128, PAIR_LIST = 128;
+
+__global__ void __launch_bounds__(PAIR_THREADS) k_find_pairs(PairArgs g) {
+    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < g.n; a += gridDim.x * blockDim.x) {
+        const int s = g.sob[a];
+        const float4 pa = g.st[4 * a];   // .w = radius
+        const bool dyn_a = g.im[a] > 0.0f;
+        int cnt = 0;
+        int local[OVL_MAX_NEIGH];
+        int *const gl = g.nb_list + g.nb_off[a];
+        const int cap = (int)(g.nb_off[a + 1] - g.nb_off[a]);
+        bool spilled = false;   // the list continues in gl (more than OVL_MAX_NEIGH neighbours)
+        bool overflow = false;
+        if (g.scene_flags[s] & 1) {
+            const int3 ca = cell_of(pa, g.inv_cs);
+            // Touching centres are only noted while a column is walked (some
+            // lane of the warp finds one at almost every step); their bodies
+            // are looked up together afterwards.
+            int found[OVL_MAX_NEIGH], m = 0;
+            auto look_up = [&]() {
+                for (int i = 0; i < m; ++i) {
+                    int b;
+                    if (!is_neighbour(g, a, s, dyn_a, found[i], b)) continue;
+                    if (!spilled && cnt == OVL_MAX_NEIGH && cap > OVL_MAX_NEIGH) {
+                        for (int j = 0; j < cnt; ++j) gl[j] = local[j];
+                        spilled = true;
+                    }
+                    if (cnt >= (spilled ? cap : OVL_MAX_NEIGH)) {
+                        overflow = true;
                         continue;
                     }
+                    insert_sorted(spilled ? gl : local, cnt++, b);
                 }
-                // the gap itself from large coordinates: FP64, then rounded once
-                const float gap = (float)((double)pl.x * pa.x + (double)pl.y * pa.y +
-                                          (double)pl.z * pa.z - (double)pl.w - (double)pa.w);
-                // normal from the sphere towards the plane
-                float3 nn = make_float3(-pl.x, -pl.y, -pl.z);
-                int k = tangent_axis(nn.x, nn.y, nn.z);
-                float3 t = tangent_from(nn, k);
-                c_ab[o] = make_int2(a, n + pidx);
-                c_n[o] = make_float4(nn.x, nn.y, nn.z, gap);
-                c_t1[o] = make_float4(t.x, t.y, t.z, 0.f);
-                if (c_p) c_p[o] = make_float4(0.f, 0.f, 0.f, __int_as_float(0));
-                ++o;
-            }
+                m = 0;
+            };
+#pragma unroll 1
+            for (int c = 0; c < 9; ++c)
+                touching_in_column(g, pa, ca, s, c, [&](int k) {
+                    if (m == OVL_MAX_NEIGH) look_up();
+                    found[m++] = k;
+                });
+            look_up();
         }
+        if (overflow) atomicCAS(g.status, DEV_OK, DEV_ERR_CAPACITY);
+        if (!spilled)
+            for (int j = 0; j < cnt; ++j) gl[j] = local[j];
+        g.nb_count[a] = cnt;
+        int np_ = 0;
+        if (dyn_a)
+            for (int k = g.plane_ptr[s]; k < g.plane_ptr[s + 1]; ++k)
+                if (plane_gap(pa, g.planes[g.plane_list[k]]) <= g.margin) ++np_;   // the (bounding) sphere test
+        g.contact_count[a] = cnt + np_;
+    }
+}
+
+// PAIR_LANES threads per body: the accepted bodies go to a list in shared
+// memory in any order and are placed by rank; only a body with more than
+// PAIR_LIST of them is searched by one thread.
+__global__ void __launch_bounds__(PAIR_THREADS) k_find_pairs_lanes(PairArgs g) {
+    __shared__ int list[PAIR_THREADS / PAIR_LANES][PAIR_LIST];
+    __shared__ int len[PAIR_THREADS / PAIR_LANES];
+    const int sub = threadIdx.x & (PAIR_LANES - 1), q = threadIdx.x / PAIR_LANES;
+    const unsigned group = ((1u << PAIR_LANES) - 1u) << (threadIdx.x & 31 & ~(PAIR_LANES - 1));
+    const int stride = gridDim.x * (PAIR_THREADS / PAIR_LANES);
+    for (int a = blockIdx.x * (PAIR_THREADS / PAIR_LANES) + q; a < g.n; a += stride) {
+        const int s = g.sob[a];
+        const float4 pa = g.st[4 * a];
+        const bool dyn_a = g.im[a] > 0.0f, on = g.scene_flags[s] & 1;
+        int *const gl = g.nb_list + g.nb_off[a];
+        const int cap = (int)(g.nb_off[a + 1] - g.nb_off[a]);
+        const int3 ca = cell_of(pa, g.inv_cs);
+        if (sub == 0) len[q] = 0;
+        __syncwarp(group);
+        for (int c = sub; on && c < 9; c += PAIR_LANES)
+            touching_in_column(g, pa, ca, s, c, [&](int k) {
+                int b;
+                if (!is_neighbour(g, a, s, dyn_a, k, b)) return;
+                const int i = atomicAdd(&len[q], 1);
+                if (i < PAIR_LIST) list[q][i] = b;
+            });
+        __syncwarp(group);
+        const int found = len[q];
+        if (found <= PAIR_LIST) {
+            for (int i = sub; i < found; i += PAIR_LANES) {
+                const int x = list[q][i];
+                int rank = 0;
+                for (int j = 0; j < found; ++j) rank += list[q][j] < x ? 1 : 0;
+                if (rank < cap) gl[rank] = x;
+            }
+        } else if (sub == 0) {
+            int m = 0;
+            for (int c = 0; c < 9; ++c)
+                touching_in_column(g, pa, ca, s, c, [&](int k) {
+                    int b;
+                    if (m < cap && is_neighbour(g, a, s, dyn_a, k, b)) insert_sorted(gl, m++, b);
+                });
+        }
+        int np_ = 0;
+        if (dyn_a)
+            for (int k = g.plane_ptr[s] + sub; k < g.plane_ptr[s + 1]; k += PAIR_LANES)
+                if (plane_gap(pa, g.planes[g.plane_list[k]]) <= g.margin) ++np_;
+        for (int o = PAIR_LANES / 2; o > 0; o >>= 1) np_ += __shfl_xor_sync(group, np_, o);
+        if (sub == 0) {
+            if (found > cap) atomicCAS(g.status, DEV_OK, DEV_ERR_CAPACITY);
+            g.nb_count[a] = min(found, cap);
+            g.contact_count[a] = min(found, cap) + np_;
+        }
+        __syncwarp(group);
+    }
+}
+
+// the bodies of every contact, in canonical order (no boxes)
+__global__ void k_contact_bodies(const float4 *__restrict__ st, const float *__restrict__ im, int n,
+                                 const int *__restrict__ sob, const float4 *__restrict__ planes,
+                                 const int *__restrict__ plane_ptr, const int *__restrict__ plane_list, float margin,
+                                 const int *__restrict__ nb_list, const long long *__restrict__ nb_off,
+                                 const int *__restrict__ nb_count, const int *__restrict__ cstart,
+                                 int2 *__restrict__ c_ab) {
+    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < n; a += gridDim.x * blockDim.x) {
+        int o = cstart[a];
+        const int cnt = nb_count[a];
+        const int *lst = nb_list + nb_off[a];
+        for (int j = 0; j < cnt; ++j) c_ab[o++] = make_int2(a, lst[j]);
+        if (!(im[a] > 0.0f) || o == cstart[a + 1]) continue;
+        const float4 pa = st[4 * a];
+        const int s = sob[a];
+        for (int k = plane_ptr[s]; k < plane_ptr[s + 1]; ++k)
+            if (plane_gap(pa, planes[plane_list[k]]) <= margin) c_ab[o++] = make_int2(a, n + plane_list[k]);
+    }
+}
+
+// geometry of a sphere pair: normal, gap, tangent
+__device__ __forceinline__ void sphere_contact(float4 pa, float4 pb, float4 &cn, float4 &ct) {
+    float dx = __fsub_rn(pb.x, pa.x), dy = __fsub_rn(pb.y, pa.y), dz = __fsub_rn(pb.z, pa.z);
+    float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+    float L = __fsqrt_rn(d2);
+    float3 nn;
+    int k;
+    if (L == 0.0f) {
+        nn = make_float3(0.f, 0.f, 1.f);
+        k = 0;
+    } else {
+        nn = make_float3(__fdiv_rn(dx, L), __fdiv_rn(dy, L), __fdiv_rn(dz, L));
+        k = tangent_axis(nn.x, nn.y, nn.z);
+    }
+    float3 t = tangent_from(nn, k);
+    // The gap from the exact FP64 differences of the FP32 centres and an
+    // FP64 square root, rounded once: it enters the speculative target
+    // -phi / h, which multiplies an FP32 rounding of |d| (~1e-7 m)
+    // into ~1e-5 m/s of velocity.
+    const double ex = (double)pb.x - (double)pa.x, ey = (double)pb.y - (double)pa.y,
+                 ez = (double)pb.z - (double)pa.z;
+    const double L64 = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)));
+    const float phi = (float)((L64 - (double)pa.w) - (double)pb.w);
+    cn = make_float4(nn.x, nn.y, nn.z, phi);
+    ct = make_float4(t.x, t.y, t.z, 0.f);
+}
+
+// of a sphere and a plane
+__device__ __forceinline__ void plane_contact(float4 pa, float4 pl, float4 &cn, float4 &ct) {
+    // the gap itself from large coordinates: FP64, then rounded once
+    const float gap = (float)((double)pl.x * pa.x + (double)pl.y * pa.y +
+                              (double)pl.z * pa.z - (double)pl.w - (double)pa.w);
+    // normal from the sphere towards the plane
+    float3 nn = make_float3(-pl.x, -pl.y, -pl.z);
+    int k = tangent_axis(nn.x, nn.y, nn.z);
+    float3 t = tangent_from(nn, k);
+    cn = make_float4(nn.x, nn.y, nn.z, gap);
+    ct = make_float4(t.x, t.y, t.z, 0.f);
+}
+
+// One thread per contact: bound by the FP64 unit (about 30 operations for
+// the gap, two lanes per cycle and SM), which a thread per body left to a few
+// lanes of every warp (large pile, 752 k contacts: 82 us, now 42, and 10 for the bodies).
+__global__ void k_contact_geometry(const float4 *__restrict__ st, int n, const float4 *__restrict__ planes, int nc,
+                                   const int2 *__restrict__ c_ab, float4 *__restrict__ c_n, float4 *__restrict__ c_t1) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
+        const int2 e = c_ab[i];
+        const float4 pa = st[4 * e.x];
+        float4 cn, ct;
+        if (e.y < n) sphere_contact(pa, st[4 * e.y], cn, ct);
+        else plane_contact(pa, planes[e.y - n], cn, ct);
+        c_n[i] = cn;
+        c_t1[i] = ct;
+    }
+}
+
+// Contexts with boxes: BOX_LANES threads per body, one candidate (neighbour,
+// then plane) each, so that the FP64 narrow phase of a body's pairs runs side
+// by side.  WRITE = false: the number of contacts per body; true: the
+// contacts, from cstart[a] on, by the same functions on the same inputs.  (One
+// thread per body, pair after pair: building 1189 us for both passes, now 250.)
+constexpr int BOX_LANES = 8;
+
+template <bool WRITE>
+__global__ void __launch_bounds__(128)
+k_box_contacts(const float4 *__restrict__ st, const float *__restrict__ im, int n, const int *__restrict__ sob,
+               const float4 *__restrict__ planes, const int *__restrict__ plane_ptr,
+               const int *__restrict__ plane_list, float margin, const int *__restrict__ nb_list,
+               const long long *__restrict__ nb_off, const int *__restrict__ nb_count, int *__restrict__ contact_count,
+               const int *__restrict__ cstart, int2 *__restrict__ c_ab, float4 *__restrict__ c_n,
+               float4 *__restrict__ c_t1, const float4 *__restrict__ half, float4 *__restrict__ c_p) {
+    const int sub = threadIdx.x & (BOX_LANES - 1);
+    const unsigned group = ((1u << BOX_LANES) - 1u) << (threadIdx.x & 31 & ~(BOX_LANES - 1));
+    const int stride = gridDim.x * blockDim.x / BOX_LANES;
+    for (int a = (blockIdx.x * blockDim.x + threadIdx.x) / BOX_LANES; a < n; a += stride) {
+        const int s = sob[a], cnt = nb_count[a];
+        const int *lst = nb_list + nb_off[a];
+        const int p0 = plane_ptr[s], np_ = im[a] > 0.0f ? plane_ptr[s + 1] - p0 : 0;
+        const float4 pa = st[4 * a];
+        const bool box_a = is_box(half, a);
+        int o = WRITE ? cstart[a] : 0;
+        for (int base = 0; base < cnt + np_; base += BOX_LANES) {
+            const int j = base + sub;
+            int b = -1, m = 0;
+            bool full = false;   // a contact of the box functions
+            double3 pts[4], nrm;
+            double gaps[4];
+            float4 pl = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j < cnt) {
+                b = lst[j];
+                full = box_a || is_box(half, b);
+                m = full ? box_pair(st, half, nullptr, a, b, margin, pts, gaps, nrm) : 1;
+            } else if (j < cnt + np_) {
+                const int pidx = plane_list[p0 + j - cnt];
+                pl = planes[pidx];
+                b = n + pidx;
+                full = box_a;
+                if (plane_gap(pa, pl) <= margin)   // the FP32 (bounding-sphere) decision
+                    m = full ? box_plane_pair(st, half, a, pl, margin, pts, gaps, nrm) : 1;
+            }
+            int before = 0, all = 0;
+#pragma unroll
+            for (int k = 0; k < BOX_LANES; ++k) {
+                const int x = __shfl_sync(group, m, k, BOX_LANES);
+                before += k < sub ? x : 0;
+                all += x;
+            }
+            if (WRITE && m > 0) {
+                int q = o + before;
+                if (full) {
+                    for (int k = 0; k < m; ++k) write_box_contact(q++, a, b, k, pts[k], gaps[k], nrm, c_ab, c_n, c_t1, c_p);
+                } else {
+                    float4 cn, ct;
+                    if (b < n) sphere_contact(pa, st[4 * b], cn, ct);
+                    else plane_contact(pa, pl, cn, ct);
+                    c_ab[q] = make_int2(a, b);
+                    c_n[q] = cn;
+                    c_t1[q] = ct;
+                    c_p[q] = make_float4(0.f, 0.f, 0.f, __int_as_float(0));
+                }
+            }
+            o += all;
+        }
+        if (!WRITE && sub == 0) contact_count[a] = o;
     }
 }
 
@@ -305,11 +457,13 @@ __global__ void k_write_contacts(const float4 *__restrict__ st, const float *__r
 // G^t: undirected edges between two dynamic bodies from contacts and joints
 // ---------------------------------------------------------------------------
 __global__ void k_edge_degree(const int2 *__restrict__ c_ab, int nc, const int2 *__restrict__ jab,
-                              int nj, const float *__restrict__ im, int n, int *__restrict__ deg) {
+                              int nj, const float *__restrict__ im, int n, int *__restrict__ deg,
+                              const float4 *__restrict__ c_p) {
     int total = nc + nj;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         int2 e = i < nc ? c_ab[i] : jab[i - nc];
         if (e.x < 0 || e.y < 0 || e.x >= n || e.y >= n || e.x == e.y) continue;
+        if (c_p && i < nc && __float_as_int(c_p[i].w) != 0) continue;   // a box manifold gives its edge once
         if (!(im[e.x] > 0.0f) || !(im[e.y] > 0.0f)) continue;
         atomicAdd(&deg[e.x], 1);
         atomicAdd(&deg[e.y], 1);
@@ -319,35 +473,46 @@ __global__ void k_edge_degree(const int2 *__restrict__ c_ab, int nc, const int2 
 __global__ void k_edge_fill(const int2 *__restrict__ c_ab, int nc, const int2 *__restrict__ jab,
                             int nj, const float *__restrict__ im, int n,
                             const int *__restrict__ tptr, int *__restrict__ cursor,
-                            int *__restrict__ tcol) {
+                            int *__restrict__ tcol, const float4 *__restrict__ c_p) {
     int total = nc + nj;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         int2 e = i < nc ? c_ab[i] : jab[i - nc];
         if (e.x < 0 || e.y < 0 || e.x >= n || e.y >= n || e.x == e.y) continue;
+        if (c_p && i < nc && __float_as_int(c_p[i].w) != 0) continue;   // a box manifold gives its edge once
         if (!(im[e.x] > 0.0f) || !(im[e.y] > 0.0f)) continue;
         tcol[tptr[e.x] + atomicAdd(&cursor[e.x], 1)] = e.y;
         tcol[tptr[e.y] + atomicAdd(&cursor[e.y], 1)] = e.x;
     }
 }
 
-// sort each vertex's neighbours and drop duplicates in place
+// sort each vertex's neighbours and drop duplicates in place (lists of up to
+// OVL_MAX_NEIGH in a thread's own memory: the insertions' dependent loads then
+// hit L1, large pile 48 -> 23 us)
 __global__ void k_adj_unique(const int *__restrict__ tptr, int n, int *__restrict__ tcol,
                              int *__restrict__ ucount) {
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        int b = tptr[v], e = tptr[v + 1];
-        for (int i = b + 1; i < e; ++i) {
-            int x = tcol[i];
-            int j = i;
-            while (j > b && tcol[j - 1] > x) {
-                tcol[j] = tcol[j - 1];
-                --j;
+        const int b = tptr[v], d = tptr[v + 1] - b;
+        int own[OVL_MAX_NEIGH];
+        auto sort = [&](int *lst, auto &&at) {
+            for (int i = 0; i < d; ++i) {
+                const int x = at(i);
+                int j = i;
+                while (j > 0 && lst[j - 1] > x) {
+                    lst[j] = lst[j - 1];
+                    --j;
+                }
+                lst[j] = x;
             }
-            tcol[j] = x;
-        }
-        int m = 0;
-        for (int i = b; i < e; ++i)
-            if (i == b || tcol[i] != tcol[i - 1]) tcol[b + m++] = tcol[i];
-        ucount[v] = m;
+            int m = 0, last = -1;
+            for (int i = 0; i < d; ++i) {
+                const int x = lst[i];
+                if (x != last) tcol[b + m++] = x;
+                last = x;
+            }
+            ucount[v] = m;
+        };
+        if (d <= OVL_MAX_NEIGH) sort(own, [&](int i) { return tcol[b + i]; });
+        else sort(tcol + b, [&](int i) { return tcol[b + i]; });
     }
 }
 
@@ -489,47 +654,61 @@ int grid1d(size_t n, int threads) {
 }
 
 void launch_cells(const ContactArgs &a, cudaStream_t s) {
-    k_cells<<<grid1d(a.n, 256), 256, 0, s>>>(a.st, a.n, a.sob, a.inv_cs, a.tmask, a.cell,
-                                             a.bucket_count);
+    k_cells<<<grid1d(a.n, 256), 256, 0, s>>>(a.st, a.n, a.sob, a.inv_cs, a.tmask, a.cell, a.bucket_count);
     note_launch();
     CK(cudaGetLastError());
 }
 
 void launch_bucket_fill(const ContactArgs &a, cudaStream_t s) {
-    k_bucket_fill<<<grid1d(a.n, 256), 256, 0, s>>>(a.cell, a.n, a.bucket_start, a.cursor, a.items);
+    k_bucket_fill<<<grid1d(a.n, 256), 256, 0, s>>>(a.st, a.cell, a.n, a.bucket_start, a.bucket_count, a.items, a.centres);
     note_launch();
     CK(cudaGetLastError());
 }
 
 void launch_find_pairs(const ContactArgs &a, cudaStream_t s) {
-    auto k = a.half ? k_find_pairs<true> : k_find_pairs<false>;
-    k<<<grid1d(a.n, 128), 128, 0, s>>>(
-        a.st, a.im, a.n, a.sob, a.scene_flags, a.cell, a.bucket_start, a.items, a.tmask, a.planes,
-        a.plane_ptr, a.plane_list, a.margin, a.nb_list, a.nb_off, a.nb_count, a.contact_count, a.status, a.half);
+    const PairArgs g{a.st, a.im, a.n, a.sob, a.scene_flags, a.inv_cs, a.bucket_start, a.items, a.centres, a.tmask, a.planes,
+                     a.plane_ptr, a.plane_list, a.margin, a.nb_list, a.nb_off, a.nb_count, a.contact_count, a.status};
+    if ((long long)a.n * PAIR_LANES <= 152 * 2048)
+        k_find_pairs_lanes<<<grid1d((size_t)a.n * PAIR_LANES, PAIR_THREADS), PAIR_THREADS, 0, s>>>(g);
+    else
+        k_find_pairs<<<grid1d(a.n, PAIR_THREADS), PAIR_THREADS, 0, s>>>(g);
     note_launch();
+    if (a.half) {
+        k_box_contacts<false><<<grid1d((size_t)a.n * BOX_LANES, 128), 128, 0, s>>>(
+            a.st, a.im, a.n, a.sob, a.planes, a.plane_ptr, a.plane_list, a.margin, a.nb_list, a.nb_off, a.nb_count,
+            a.contact_count, nullptr, nullptr, nullptr, nullptr, a.half, nullptr);
+        note_launch();
+    }
     CK(cudaGetLastError());
 }
 
-void launch_write_contacts(const ContactArgs &a, cudaStream_t s) {
-    auto k = a.half ? k_write_contacts<true> : k_write_contacts<false>;
-    k<<<grid1d(a.n, 128), 128, 0, s>>>(a.st, a.im, a.n, a.sob, a.planes, a.plane_ptr,
-                                                      a.plane_list, a.margin, a.nb_list, a.nb_off,
-                                                      a.nb_count, a.contact_start, a.c_ab, a.c_n,
-                                                      a.c_t1, a.half, a.c_p);
-    note_launch();
+void launch_write_contacts(const ContactArgs &a, int nc, cudaStream_t s) {
+    if (nc == 0) return;
+    if (a.half) {
+        k_box_contacts<true><<<grid1d((size_t)a.n * BOX_LANES, 128), 128, 0, s>>>(
+            a.st, a.im, a.n, a.sob, a.planes, a.plane_ptr, a.plane_list, a.margin, a.nb_list, a.nb_off, a.nb_count,
+            nullptr, a.contact_start, a.c_ab, a.c_n, a.c_t1, a.half, a.c_p);
+        note_launch();
+    } else {
+        k_contact_bodies<<<grid1d(a.n, 128), 128, 0, s>>>(a.st, a.im, a.n, a.sob, a.planes, a.plane_ptr, a.plane_list,
+                                                          a.margin, a.nb_list, a.nb_off, a.nb_count, a.contact_start,
+                                                          a.c_ab);
+        k_contact_geometry<<<grid1d(nc, 128), 128, 0, s>>>(a.st, a.n, a.planes, nc, a.c_ab, a.c_n, a.c_t1);
+        note_launches(2);
+    }
     CK(cudaGetLastError());
 }
 
 void launch_edge_degree(const int2 *c_ab, int nc, const int2 *jab, int nj, const float *im, int n,
-                        int *deg, cudaStream_t s) {
-    k_edge_degree<<<grid1d(nc + nj, 256), 256, 0, s>>>(c_ab, nc, jab, nj, im, n, deg);
+                        int *deg, const float4 *c_p, cudaStream_t s) {
+    k_edge_degree<<<grid1d(nc + nj, 256), 256, 0, s>>>(c_ab, nc, jab, nj, im, n, deg, c_p);
     note_launch();
     CK(cudaGetLastError());
 }
 
 void launch_edge_fill(const int2 *c_ab, int nc, const int2 *jab, int nj, const float *im, int n,
-                      const int *tptr, int *cursor, int *tcol, cudaStream_t s) {
-    k_edge_fill<<<grid1d(nc + nj, 256), 256, 0, s>>>(c_ab, nc, jab, nj, im, n, tptr, cursor, tcol);
+                      const int *tptr, int *cursor, int *tcol, const float4 *c_p, cudaStream_t s) {
+    k_edge_fill<<<grid1d(nc + nj, 256), 256, 0, s>>>(c_ab, nc, jab, nj, im, n, tptr, cursor, tcol, c_p);
     note_launch();
     CK(cudaGetLastError());
 }

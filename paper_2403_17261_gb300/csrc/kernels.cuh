@@ -16,11 +16,11 @@ struct ContactArgs {
     const int *scene_flags;
     float inv_cs;
     uint32_t tmask;        // hash table size - 1
-    int4 *cell;            // per body (ix, iy, iz, hash)
-    int *bucket_count;     // [T]
+    int *cell;             // per body: its cell's bucket
+    int *bucket_count;     // [T] zeroed by the caller
     int *bucket_start;     // [T+1]
-    int *cursor;           // [T]
-    int *items;            // [n]
+    int *items;            // [n] bodies in bucket order
+    float4 *centres;       // [n] their centres and radii
     const float4 *planes;
     const int *plane_ptr;  // [n_scenes+1]
     const int *plane_list; // plane indices grouped by scene, ascending
@@ -40,11 +40,12 @@ struct ContactArgs {
 void launch_cells(const ContactArgs &a, cudaStream_t s);
 void launch_bucket_fill(const ContactArgs &a, cudaStream_t s);
 void launch_find_pairs(const ContactArgs &a, cudaStream_t s);
-void launch_write_contacts(const ContactArgs &a, cudaStream_t s);
+void launch_write_contacts(const ContactArgs &a, int nc, cudaStream_t s);
+// c_p: contact points of contexts with boxes (else NULL)
 void launch_edge_degree(const int2 *c_ab, int nc, const int2 *jab, int nj, const float *im, int n,
-                        int *deg, cudaStream_t s);
+                        int *deg, const float4 *c_p, cudaStream_t s);
 void launch_edge_fill(const int2 *c_ab, int nc, const int2 *jab, int nj, const float *im, int n,
-                      const int *tptr, int *cursor, int *tcol, cudaStream_t s);
+                      const int *tptr, int *cursor, int *tcol, const float4 *c_p, cudaStream_t s);
 void launch_adj_unique(const int *tptr, int n, int *tcol, int *ucount, cudaStream_t s);
 // loads [P] := |P_w| of every worker from the masks
 // number of contacts each body is an end of (planes and static ends included)
