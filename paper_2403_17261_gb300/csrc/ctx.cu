@@ -665,7 +665,7 @@ SolveArgs solve_args(ovl_ctx *c, float dt_override, int iters) {
     a.iters = iters; a.flags = c->P.flags;
     a.res_tol = c->P.res_tol; a.res_check_every = c->P.res_check_every;
     a.part_iters = c->part_iters.p; a.part_res_sq = c->part_res_sq.p; a.status = c->status.p;
-    if (c->has_boxes) { a.row_full = c->row_full.p; a.rfull = c->rfull.p; }
+    if (c->has_boxes) { a.row_full = c->row_full.p; a.rfull = c->rfull.p; a.np = c->npairs; }
     return a;
 }
 

@@ -784,7 +784,8 @@ __device__ float3 inv_inertia_times(const RowArgs &a, int b, float3 v) {
 // (-1: static or not in this worker), directions dir[3], targets tg[3]
 __device__ void write_full_row(const RowArgs &a, int r, int ea, int eb, float3 rA, float3 rB, const float3 *dir,
                                const float *tg) {
-    float4 *F = a.rfull + (size_t)r * FULL_ROW_WORDS;
+    const size_t np = (size_t)a.np;
+    float4 *F = a.rfull + r;
     const float imA = ea >= 0 ? a.st[4 * ea + 2].w : 0.f, imB = eb >= 0 ? a.st[4 * eb + 2].w : 0.f;
     for (int i = 0; i < 3; ++i) {
         const float3 d = dir[i];
@@ -793,13 +794,13 @@ __device__ void write_full_row(const RowArgs &a, int r, int ea, int eb, float3 r
         const float3 iA = ea >= 0 ? inv_inertia_times(a, ea, jA) : make_float3(0.f, 0.f, 0.f);
         const float3 iB = eb >= 0 ? inv_inertia_times(a, eb, jB) : make_float3(0.f, 0.f, 0.f);
         const float s = (imA + imB) + ((jA.x * iA.x + jA.y * iA.y + jA.z * iA.z) + (jB.x * iB.x + jB.y * iB.y + jB.z * iB.z));
-        F[i] = make_float4(d.x, d.y, d.z, tg[i]);
-        F[3 + i] = make_float4(jA.x, jA.y, jA.z, s > 0.f ? 1.f / s : 0.f);
-        F[6 + i] = make_float4(iA.x, iA.y, iA.z, 0.f);
-        F[9 + i] = make_float4(jB.x, jB.y, jB.z, 0.f);
-        F[12 + i] = make_float4(iB.x, iB.y, iB.z, 0.f);
+        F[i * np] = make_float4(d.x, d.y, d.z, tg[i]);
+        F[(3 + i) * np] = make_float4(jA.x, jA.y, jA.z, s > 0.f ? 1.f / s : 0.f);
+        F[(6 + i) * np] = make_float4(iA.x, iA.y, iA.z, 0.f);
+        F[(9 + i) * np] = make_float4(jB.x, jB.y, jB.z, 0.f);
+        F[(12 + i) * np] = make_float4(iB.x, iB.y, iB.z, 0.f);
     }
-    F[15] = make_float4(imA, imB, 0.f, 0.f);
+    F[15 * np] = make_float4(imA, imB, 0.f, 0.f);
 }
 
 __global__ void k_rows(RowArgs a) {
@@ -867,7 +868,7 @@ __global__ void k_rows(RowArgs a) {
                     dir[1] = make_float3(0.f, 1.f, 0.f);
                     dir[2] = make_float3(0.f, 0.f, 1.f);
                     a.r0[r] = z;
-                    a.r1[r] = z;
+                    a.r1[r] = make_float4(0.f, 0.f, 0.f, pack ? sw.packed : 0.f);   // where k_solve_m reads them
                     a.r2[r] = make_float4(0.f, 0.f, sw.a, sw.b);
                     a.r3[r] = z;
                 }

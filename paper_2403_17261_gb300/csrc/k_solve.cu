@@ -114,25 +114,12 @@ struct LocalSlots {
     }
 };
 
-// (v, 1/m) of slot i at V[i], (w, 1/I) at W[i].  Two arrays: eight lanes read
-// eight 16-byte words at a time, and a 32-byte stride would leave them only
-// four of the eight bank groups.
+// (v, 1/m) of slot i at V[i], (w, 1/I) at W[i] (k_solve_m; CodeSlots reads
+// them).  Two arrays: eight lanes read eight 16-byte words at a time, and a
+// 32-byte stride would leave them only four of the eight bank groups.
 struct LocalSlotsM {
     static constexpr bool kMasses = true;
     float4 *V, *W;
-    __device__ __forceinline__ void load(uint32_t c, Body &b) const {
-        const uint32_t i = code_index(c);
-        const float4 x = V[i], y = W[i];
-        b.v = make_float3(x.x, x.y, x.z);
-        b.w = make_float3(y.x, y.y, y.z);
-        b.im = x.w;
-        b.ii = y.w;
-    }
-    __device__ __forceinline__ void store(uint32_t c, const Body &b) const {
-        const uint32_t i = code_index(c);
-        V[i] = make_float4(b.v.x, b.v.y, b.v.z, b.im);
-        W[i] = make_float4(b.w.x, b.w.y, b.w.z, b.ii);
-    }
 };
 
 __device__ __forceinline__ uint32_t mapa(uint32_t a, uint32_t rank) {
@@ -168,33 +155,6 @@ struct ClusterSlots {
         asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};"
                      :: "r"(a), "f"(b.v.x), "f"(b.v.y), "f"(b.v.z), "f"(b.w.x));
         asm volatile("st.shared::cluster.v2.f32 [%0], {%1,%2};" :: "r"(d), "f"(b.w.y), "f"(b.w.z));
-    }
-};
-
-// LocalSlotsM over the C CTAs of a cluster, every access through distributed
-// shared memory
-template <int C>
-struct ClusterSlotsM {
-    static constexpr bool kMasses = true;
-    uint32_t V, W;   // shared-window offsets of this CTA's arrays (same in every CTA)
-    __device__ __forceinline__ void load(uint32_t c, Body &b) const {
-        const uint32_t r = code_rank(c), i = 16u * code_index(c);
-        float4 x, y;
-        asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
-                     : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(mapa(V + i, r)));
-        asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];"
-                     : "=f"(y.x), "=f"(y.y), "=f"(y.z), "=f"(y.w) : "r"(mapa(W + i, r)));
-        b.v = make_float3(x.x, x.y, x.z);
-        b.w = make_float3(y.x, y.y, y.z);
-        b.im = x.w;
-        b.ii = y.w;
-    }
-    __device__ __forceinline__ void store(uint32_t c, const Body &b) const {
-        const uint32_t r = code_rank(c), i = 16u * code_index(c);
-        asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};"
-                     :: "r"(mapa(V + i, r)), "f"(b.v.x), "f"(b.v.y), "f"(b.v.z), "f"(b.im));
-        asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};"
-                     :: "r"(mapa(W + i, r)), "f"(b.w.x), "f"(b.w.y), "f"(b.w.z), "f"(b.ii));
     }
 };
 
@@ -400,62 +360,79 @@ __device__ __forceinline__ float clampf(float x, float lo, float hi) { return fm
 template <bool X>
 __device__ __forceinline__ bool is_full(const SolveArgs &a, int r) { return X && a.row_full[r]; }
 
+// The FULL_ROW_WORDS float4 of a full row: F(j), from global memory or as
+// staged in shared memory.
+struct FullGlobal {
+    const float4 *p;
+    size_t stride;
+    __device__ __forceinline__ float4 operator()(int j) const { return __ldg(p + j * stride); }
+};
+struct FullStaged {
+    const float4 *p;
+    int stride;
+    __device__ __forceinline__ float4 operator()(int j) const { return p[j * stride]; }
+};
+__device__ __forceinline__ FullGlobal full_of(const SolveArgs &a, int r) { return {a.rfull + r, (size_t)a.np}; }
+
 // impulse dl along direction i of a full row
-__device__ __forceinline__ void full_impulse(const float4 *F, int i, float imA, float imB, Body &A, Body &B,
-                                             float dl) {
-    const float3 d = f3(F[i]);
+template <class FR>
+__device__ __forceinline__ void full_impulse(const FR &F, int i, float imA, float imB, Body &A, Body &B, float dl) {
+    const float3 d = f3(F(i));
     axpy(A.v, -imA * dl, d);
     axpy(B.v, imB * dl, d);
-    axpy(A.w, -dl, f3(F[6 + i]));
-    axpy(B.w, dl, f3(F[12 + i]));
+    axpy(A.w, -dl, f3(F(6 + i)));
+    axpy(B.w, dl, f3(F(12 + i)));
 }
 
-__device__ __forceinline__ float full_w(const float4 *F, int i, const Body &A, const Body &B) {
+template <class FR>
+__device__ __forceinline__ float full_w(const FR &F, int i, const Body &A, const Body &B) {
     const float3 dv = make_float3(B.v.x - A.v.x, B.v.y - A.v.y, B.v.z - A.v.z);
-    return dot3(f3(F[i]), dv) + (dot3(f3(F[9 + i]), B.w) - dot3(f3(F[3 + i]), A.w));
+    return dot3(f3(F(i)), dv) + (dot3(f3(F(9 + i)), B.w) - dot3(f3(F(3 + i)), A.w));
 }
 
 // the three rows of a constraint with a box end: contact (normal >= 0,
 // tangents within +-mu lambda_n) or ball joint (unbounded)
-__device__ void full_rows(const SolveArgs &a, int r, bool joint, Body &A, Body &B, float mu, float4 &lam) {
-    const float4 *F = a.rfull + (size_t)r * FULL_ROW_WORDS;
-    const float imA = F[15].x, imB = F[15].y;
+template <class FR>
+__device__ __forceinline__ void full_rows(const FR &F, bool joint, Body &A, Body &B, float mu, float4 &lam) {
+    const float4 m = F(15);
     float l[3] = {lam.x, lam.y, lam.z};
+#pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const float k = F[3 + i].w, target = F[i].w;
+        const float k = F(3 + i).w, target = F(i).w;
         float ln = fmaf(k, target - full_w(F, i, A, B), l[i]);
         if (!joint) ln = i == 0 ? fmaxf(ln, 0.f) : fminf(fmaxf(ln, -mu * l[0]), mu * l[0]);
         const float dl = ln - l[i];
         l[i] = ln;
-        full_impulse(F, i, imA, imB, A, B, dl);
+        full_impulse(F, i, m.x, m.y, A, B, dl);
     }
     lam = make_float4(l[0], l[1], l[2], lam.w);
 }
 
-__device__ void full_warm(const SolveArgs &a, int r, Body &A, Body &B, float4 lam) {
-    const float4 *F = a.rfull + (size_t)r * FULL_ROW_WORDS;
-    const float imA = F[15].x, imB = F[15].y;
-    full_impulse(F, 0, imA, imB, A, B, lam.x);
-    full_impulse(F, 1, imA, imB, A, B, lam.y);
-    full_impulse(F, 2, imA, imB, A, B, lam.z);
+template <class FR>
+__device__ __forceinline__ void full_warm(const FR &F, Body &A, Body &B, float4 lam) {
+    const float4 m = F(15);
+    full_impulse(F, 0, m.x, m.y, A, B, lam.x);
+    full_impulse(F, 1, m.x, m.y, A, B, lam.y);
+    full_impulse(F, 2, m.x, m.y, A, B, lam.z);
 }
 
 // a row of the sweep: full (box end) or plain
 template <class S, bool X>
 __device__ __forceinline__ void solve_any(const SolveArgs &a, int r, Body &A, Body &B, const Row &w, float mu,
                                           float4 &lam) {
-    if (is_full<X>(a, r)) full_rows(a, r, w.joint, A, B, mu, lam);
+    if (is_full<X>(a, r)) full_rows(full_of(a, r), w.joint, A, B, mu, lam);
     else solve_row<S>(A, B, w, mu, lam);
 }
 
-__device__ float full_residual_sq(const SolveArgs &a, int r, bool joint, const Body &A, const Body &B, float mu,
-                                  float4 lam) {
-    const float4 *F = a.rfull + (size_t)r * FULL_ROW_WORDS;
+template <class FR>
+__device__ __forceinline__ float full_residual_sq(const FR &F, bool joint, const Body &A, const Body &B, float mu,
+                                                  float4 lam) {
     const float l[3] = {lam.x, lam.y, lam.z};
     float s = 0.f;
+#pragma unroll
     for (int i = 0; i < 3; ++i) {
-        const float k = F[3 + i].w;
-        float p = l[i] + k * (F[i].w - full_w(F, i, A, B));
+        const float k = F(3 + i).w;
+        float p = l[i] + k * (F(i).w - full_w(F, i, A, B));
         if (!joint) p = i == 0 ? fmaxf(p, 0.f) : clampf(p, -mu * l[0], mu * l[0]);
         const float e = k > 0.f ? (l[i] - p) / k : 0.f;
         s += e * e;
@@ -589,7 +566,7 @@ __device__ float rows_residual_sq(const SolveArgs &a, const S &st, const Buckets
                 Body A, B;
                 load_pair(st, w, A, B);
                 if (is_full<X>(a, r)) {
-                    sq += full_residual_sq(a, r, w.joint, A, B, mu, lam);
+                    sq += full_residual_sq(full_of(a, r), w.joint, A, B, mu, lam);
                 } else if (w.joint) {
                     sq += joint_residual_sq(A, B, w.x, w.y, w.z);
                 } else {
@@ -674,7 +651,7 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
             Body A, B;
             load_pair(st, w, A, B);
             if (is_full<X>(a, r)) {
-                full_warm(a, r, A, B, lam);
+                full_warm(full_of(a, r), A, B, lam);
             } else if (!w.joint) {
                 const float3 t1 = contact_t1(w);
                 const float3 n = f3(w.x);
@@ -849,6 +826,21 @@ __device__ __forceinline__ void fetch_head(const SolveArgs &a, int r, int end, R
     }
 }
 
+// A full row's words copied to shared memory ahead of use, word j of thread
+// tid at stage[j T + tid]: read by the thread that copied them, so a
+// wait on its own copies is enough.
+__device__ __forceinline__ void stage_full(const SolveArgs &a, int r, float4 *stage) {
+    const float4 *src = a.rfull + r;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage + threadIdx.x);
+#pragma unroll
+    for (int j = 0; j < FULL_ROW_WORDS; ++j)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 16u * j * blockDim.x), "l"(src + (size_t)j * a.np) : "memory");
+}
+__device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the newest n groups of this thread's copies have landed
+template <int N>
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory"); }
+
 // The body slots of a group as 16-bit codes name them (rank << 13 | i).
 // LOCAL: every code names this CTA's own slots, plain shared memory.
 // (Measured on this GPU, dependent 16-byte loads by 512 threads: 65 cycles
@@ -895,16 +887,16 @@ struct CodeSlots {
 
 // One row: loads, f, stores if f says so.  i: the row's place in the CTA's
 // impulses.  The group's CTAs take a warp's rows as local ones when all of
-// them are.
+// them are.  full: a full row (its codes are in r1 for joints too).
 template <int C, class LM, class F>
 __device__ __forceinline__ void visit_row(const SolveArgs &a, const LocalSlotsM &own, uint32_t rank, const LM &lam, int i,
-                                          int r, bool joint, const RowHead &q, F &&f) {
+                                          int r, bool joint, bool full, const RowHead &q, F &&f) {
     Row w;
     w.x = q.x;
     w.y = q.y;
     w.joint = joint;
     uint32_t c = __float_as_uint(q.y.w);
-    if (joint) {
+    if (joint && !full) {
         // a joint's codes are the 24-bit ones of r2
         w.z = a.r2[r];
         const uint32_t ca = __float_as_uint(w.z.z), cb = __float_as_uint(w.z.w);
@@ -926,29 +918,9 @@ __device__ __forceinline__ void visit_row(const SolveArgs &a, const LocalSlotsM 
     else body(CodeSlots<true>{own});
 }
 
-// Warm start, sweeps, residual of one CTA's rows; tab[c] = (first row, first
-// joint, end, rows of earlier colours) of colour c.  A thread's first row of
-// the next colour is loaded before the current colour is solved, its further
-// rows of a colour one ahead.
-template <int C, class LM>
-__device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM &lam, const int4 *tab, int ncol, float mu,
-                           int p, int rank, int nrows, float *red, float *part_sum) {
-    const int tid = threadIdx.x, T = blockDim.x;
-    RowHead nx;
-    if (ncol > 0) fetch_head(a, tab[0].x + tid, tab[0].z, nx);
-    auto colour = [&](int c, auto &&f) {
-        const int4 o = tab[c], on = tab[c + 1 < ncol ? c + 1 : 0];
-        RowHead cur = nx;
-        fetch_head(a, on.x + tid, on.z, nx);
-        for (int r = o.x + tid; r < o.z; r += T) {
-            RowHead ahead;
-            fetch_head(a, r + T, o.z, ahead);
-            visit_row<C>(a, own, (uint32_t)rank, lam, r - o.x + o.w, r, r >= o.y, cur, f);
-            cur = ahead;
-        }
-        group_sync<C>();
-    };
-    auto warm = [&](Body &A, Body &B, const Row &w, float4 &l) {
+// what a pass does with a row: true if the bodies and impulses changed
+struct WarmRow {
+    __device__ __forceinline__ bool operator()(Body &A, Body &B, const Row &w, float4 &l) const {
         if (l.x == 0.f && l.y == 0.f && l.z == 0.f) return false;
         if (w.joint) {
             joint_impulse(A, B, f3(w.x), f3(w.y), 0, l.x);
@@ -959,10 +931,84 @@ __device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM 
             contact_impulse(A, B, n, t1, cross3(n, t1), w.y.x, w.y.y, l.x, l.y, l.z);
         }
         return true;
-    };
-    auto solve = [&](Body &A, Body &B, const Row &w, float4 &l) {
+    }
+    template <class FR>
+    __device__ __forceinline__ bool full(const FR &F, Body &A, Body &B, const Row &, float4 &l) const {
+        if (l.x == 0.f && l.y == 0.f && l.z == 0.f) return false;
+        full_warm(F, A, B, l);
+        return true;
+    }
+};
+struct SolveRow {
+    float mu;
+    __device__ __forceinline__ bool operator()(Body &A, Body &B, const Row &w, float4 &l) const {
         solve_row<LocalSlotsM>(A, B, w, mu, l);
         return true;
+    }
+    template <class FR>
+    __device__ __forceinline__ bool full(const FR &F, Body &A, Body &B, const Row &w, float4 &l) const {
+        full_rows(F, w.joint, A, B, mu, l);
+        return true;
+    }
+};
+
+// Warm start, sweeps, residual of one CTA's rows; tab[c] = (first row, first
+// joint, end, rows of earlier colours) of colour c.  A thread's first row of
+// the next colour is loaded before the current colour is solved, its further
+// rows of a colour one ahead.  X (contexts with boxes): with stage != NULL
+// the full rows among a thread's first rows of the colours are copied to
+// shared memory a colour ahead too (two stages of FULL_ROW_WORDS float4 per
+// thread), further ones of a colour come straight from global memory.
+template <int C, bool X, class LM>
+__device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM &lam, const int4 *tab, int ncol, float mu,
+                           int p, int rank, int nrows, float4 *stage, float *red, float *part_sum) {
+    const int tid = threadIdx.x, T = blockDim.x;
+    RowHead nx;
+    bool fullx = false;
+    int turn = 0;
+    auto ahead_of = [&](const int4 &o, float4 *st) {
+        fetch_head(a, o.x + tid, o.z, nx);
+        if (X) {
+            fullx = o.x + tid < o.z && __ldg(a.row_full + o.x + tid);
+            if (stage) {
+                if (fullx) stage_full(a, o.x + tid, st);
+                stage_commit();
+            }
+        }
+    };
+    if (ncol > 0) ahead_of(tab[0], stage);
+    auto colour = [&](int c, auto &&f) {
+        const int4 o = tab[c], on = tab[c + 1 < ncol ? c + 1 : 0];
+        RowHead cur = nx;
+        bool full = fullx;
+        float4 *const now = stage + (turn ? FULL_ROW_WORDS * T : 0), *const next = stage + (turn ? 0 : FULL_ROW_WORDS * T);
+        turn ^= 1;
+        ahead_of(on, next);
+        bool first = true;
+        for (int r = o.x + tid; r < o.z; r += T) {
+            RowHead ahead;
+            fetch_head(a, r + T, o.z, ahead);
+            const bool fa = X && r + T < o.z && __ldg(a.row_full + r + T);
+            const int i = r - o.x + o.w;
+            if (X && full) {
+                if (stage && first) {
+                    stage_wait<1>();
+                    visit_row<C>(a, own, (uint32_t)rank, lam, i, r, r >= o.y, true, cur, [&](Body &A, Body &B, const Row &w, float4 &l) {
+                        return f.full(FullStaged{now + tid, T}, A, B, w, l);
+                    });
+                } else {
+                    visit_row<C>(a, own, (uint32_t)rank, lam, i, r, r >= o.y, true, cur, [&](Body &A, Body &B, const Row &w, float4 &l) {
+                        return f.full(full_of(a, r), A, B, w, l);
+                    });
+                }
+            } else {
+                visit_row<C>(a, own, (uint32_t)rank, lam, i, r, r >= o.y, false, cur, f);
+            }
+            cur = ahead;
+            full = fa;
+            first = false;
+        }
+        group_sync<C>();
     };
     auto residual = [&]() {
         float sq = 0.f;
@@ -971,25 +1017,28 @@ __device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM 
             for (int r = o.x + tid; r < o.z; r += T) {
                 RowHead q;
                 fetch_head(a, r, o.z, q);
-                visit_row<C>(a, own, (uint32_t)rank, lam, r - o.x + o.w, r, r >= o.y, q, [&](Body &A, Body &B, const Row &w, float4 &l) {
-                    sq += w.joint ? joint_residual_sq(A, B, w.x, w.y, w.z)
-                                  : contact_residual_sq(A, B, w.x, w.y, contact_t1(w), l.w, w.x.w, mu, l);
+                const bool full = X && a.row_full[r];
+                visit_row<C>(a, own, (uint32_t)rank, lam, r - o.x + o.w, r, r >= o.y, full, q, [&](Body &A, Body &B, const Row &w, float4 &l) {
+                    if (full) sq += full_residual_sq(full_of(a, r), w.joint, A, B, mu, l);
+                    else if (w.joint) sq += joint_residual_sq(A, B, w.x, w.y, w.z);
+                    else sq += contact_residual_sq(A, B, w.x, w.y, contact_t1(w), l.w, w.x.w, mu, l);
                     return false;
                 });
             }
         }
         return group_sum<C>(sq, red, part_sum);
     };
-    for (int c = 0; c < ncol; ++c) colour(c, warm);
+    for (int c = 0; c < ncol; ++c) colour(c, WarmRow{});
     int it = 0;
     while (it < a.iters) {
-        for (int c = 0; c < ncol; ++c) colour(c, solve);
+        for (int c = 0; c < ncol; ++c) colour(c, SolveRow{mu});
         ++it;
         if (a.res_tol > 0.f && a.res_check_every > 0 && it % a.res_check_every == 0 && it < a.iters) {
             const float tot = residual();
             if (nrows == 0 || sqrtf(tot / nrows) <= a.res_tol) break;   // the same total in every CTA
         }
     }
+    if (X && stage) stage_wait<0>();   // the copies of a colour that is not solved again
     if (a.flags & OVL_FLAG_RESIDUAL) {
         const float tot = residual();
         if (rank == 0 && tid == 0) a.part_res_sq[p] = (double)tot;
@@ -997,14 +1046,18 @@ __device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM 
     if (rank == 0 && tid == 0) a.part_iters[p] = it;
 }
 
-// A launch whose slots hold the masses (no boxes): CTA `rank` of worker p's
+// A launch whose slots hold the masses: CTA `rank` of worker p's
 // group holds the slots [rank per, (rank + 1) per), their zero slot and, when
-// they fit, the impulses of its rows.  Latency-bound: a colour step of few
+// they fit, the impulses of its rows and (X) the two stages of full rows.  Latency-bound: a colour step of few
 // rows takes about 900 cycles, of which 95 are the CTA barrier (560 a
 // cluster's), the rest one row's chain; 512 threads (measured on the large
 // pile: 256 1.14 ms, 384 1.00, 512 0.94, 768 0.92 but slower on small piles).
-template <int C>
-__global__ void __launch_bounds__(SOLVE_THREADS, 1) k_solve_m(SolveArgs a) {
+// X: a context with boxes.  Rows read straight from global memory, flag, head
+// and words one after the other, made a colour step 1.4 us (building 2.93 ms,
+// bridge 1.13); with the impulses in shared memory and the words a colour
+// ahead @X.  256 threads: the stages take 512 B per thread.
+template <int C, bool X>
+__global__ void __launch_bounds__(X ? SOLVE_THREADS / 2 : SOLVE_THREADS, 1) k_solve_m(SolveArgs a) {
     extern __shared__ float4 sm[];
     __shared__ int4 tab[OVL_MAX_COLOURS];
     __shared__ float red[32];
@@ -1039,6 +1092,8 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) k_solve_m(SolveArgs a) {
     float4 *const V = sm, *const W = sm + per + 1;   // (v, 1/m), (w, 1/I) of the CTA's slots and its zero slot
     float *const L = reinterpret_cast<float *>(sm + 2 * (per + 1));
     const bool fits = 32ll * (per + 1) + 12ll * mine <= a.smem_bytes;
+    const long long used = fits ? (32ll * (per + 1) + 12ll * mine + 15) / 16 : 2ll * (per + 1);
+    float4 *const stage = X && 16 * (used + 2ll * FULL_ROW_WORDS * T) <= a.smem_bytes ? sm + used : nullptr;
     // velocities after the external force (h f), from the blended state; the
     // zero slot (static ends); the impulses
     for (int s = s_lo + tid; s < s_hi; s += T) {
@@ -1054,8 +1109,8 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) k_solve_m(SolveArgs a) {
             for (int r = tab[c].x + tid; r < tab[c].z; r += T) ls.store(r - tab[c].x + tab[c].w, r, a.rlam[r]);
     group_sync<C>();
     const LocalSlotsM own{V, W};
-    if (fits) sweep_rows<C>(a, own, ls, tab, ncol, mu, p, rank, 3 * (row1 - row0), red, &part_sum);
-    else sweep_rows<C>(a, own, LamGlobal{a.rlam}, tab, ncol, mu, p, rank, 3 * (row1 - row0), red, &part_sum);
+    if (fits) sweep_rows<C, X>(a, own, ls, tab, ncol, mu, p, rank, 3 * (row1 - row0), stage, red, &part_sum);
+    else sweep_rows<C, X>(a, own, LamGlobal{a.rlam}, tab, ncol, mu, p, rank, 3 * (row1 - row0), stage, red, &part_sum);
     // impulses back in canonical pair order (next step's warm start)
     for (int c = 0; c < ncol; ++c)
         for (int r = tab[c].x + tid; r < tab[c].z; r += T) {
@@ -1073,7 +1128,7 @@ __global__ void __launch_bounds__(SOLVE_THREADS, 1) k_solve_m(SolveArgs a) {
 // its body state in the global scratch area.  M: the shared-memory slots hold
 // the masses (32 B per slot; else 24 B, and rows carry the masses in r3).
 // P: rows loaded ahead (launches of SOLVE_THREADS threads, one CTA per SM).
-template <int C, int U, bool M, bool P, bool X>
+template <int C, int U, bool P, bool X>
 __global__ void __launch_bounds__(SOLVE_THREADS, U == 1 ? 2 : 1) k_solve(SolveArgs a) {
     extern __shared__ float4 sm[];
     const int rank = C == 1 ? 0 : (int)cg::this_cluster().block_rank();
@@ -1092,20 +1147,13 @@ __global__ void __launch_bounds__(SOLVE_THREADS, U == 1 ? 2 : 1) k_solve(SolveAr
     if (per <= a.smem_slots) {
         // per + 1 slots: the CTA's range and its zero slot
         float4 *A = sm;
-        if (M) {
-            const LocalSlotsM own{A, A + per + 1};
-            if constexpr (C == 1) solve_worker<C, U, P, X>(a, own, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
-            else solve_worker<C, U, P, X>(a, ClusterSlotsM<C>{(uint32_t)__cvta_generic_to_shared(own.V), (uint32_t)__cvta_generic_to_shared(own.W)}, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
+        float2 *B = reinterpret_cast<float2 *>(sm + per + 1);
+        if constexpr (C == 1) {
+            solve_worker<C, U, P, X>(a, LocalSlots{A, B}, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
         } else {
-            float2 *B = reinterpret_cast<float2 *>(sm + per + 1);
-            if (C == 1) {
-                LocalSlots st{A, B};
-                solve_worker<C, U, P, X>(a, st, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
-            } else {
-                ClusterSlots<C> st{(uint32_t)__cvta_generic_to_shared(A), (uint32_t)__cvta_generic_to_shared(B),
-                                   (uint32_t)per};
-                solve_worker<C, U, P, X>(a, st, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
-            }
+            const ClusterSlots<C> st{(uint32_t)__cvta_generic_to_shared(A), (uint32_t)__cvta_generic_to_shared(B),
+                                     (uint32_t)per};
+            solve_worker<C, U, P, X>(a, st, p, rank, per, per, Buckets{boff, 3, 1}, row0, row1);
         }
     } else if (rank == 0) {
         // one CTA takes the whole worker: every owner bucket of every colour
@@ -1122,10 +1170,10 @@ int solve_slot_bytes(bool masses) { return (int)(masses ? 2 * sizeof(float4) : s
 // a CTA's slots and its zero slot
 int solve_smem_bytes(int slots, bool masses) { return (slots + 1) * solve_slot_bytes(masses); }
 
-template <int C, int U, bool M, bool P, bool X>
+template <int C, int U, bool P, bool X>
 static void launch_solve_c(const SolveArgs &a, int threads, cudaStream_t s) {
-    int smem = solve_smem_bytes(a.smem_slots, M);
-    CK(cudaFuncSetAttribute(k_solve<C, U, M, P, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    int smem = solve_smem_bytes(a.smem_slots, false);
+    CK(cudaFuncSetAttribute(k_solve<C, U, P, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.n_parts * C);
     cfg.blockDim = dim3(threads);
@@ -1138,27 +1186,29 @@ static void launch_solve_c(const SolveArgs &a, int threads, cudaStream_t s) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    CK(cudaLaunchKernelEx(&cfg, k_solve<C, U, M, P, X>, a));
+    CK(cudaLaunchKernelEx(&cfg, k_solve<C, U, P, X>, a));
     note_launch();
 }
 
-template <int U, bool M, bool P, bool X = false>
+template <int U, bool P, bool X = false>
 static void launch_solve_u(const SolveArgs &a, int threads, int cluster, cudaStream_t s) {
     switch (cluster) {
-        case 8: launch_solve_c<8, U, M, P, X>(a, threads, s); break;
-        case 6: launch_solve_c<6, U, M, P, X>(a, threads, s); break;
-        case 4: launch_solve_c<4, U, M, P, X>(a, threads, s); break;
-        case 3: launch_solve_c<3, U, M, P, X>(a, threads, s); break;
-        case 2: launch_solve_c<2, U, M, P, X>(a, threads, s); break;
-        default: launch_solve_c<1, U, M, P, X>(a, threads, s); break;
+        case 8: launch_solve_c<8, U, P, X>(a, threads, s); break;
+        case 6: launch_solve_c<6, U, P, X>(a, threads, s); break;
+        case 4: launch_solve_c<4, U, P, X>(a, threads, s); break;
+        case 3: launch_solve_c<3, U, P, X>(a, threads, s); break;
+        case 2: launch_solve_c<2, U, P, X>(a, threads, s); break;
+        default: launch_solve_c<1, U, P, X>(a, threads, s); break;
     }
 }
 
-template <int C>
+template <int C, bool X>
 static void launch_solve_m(const SolveArgs &a, int threads, int budget, cudaStream_t s) {
     SolveArgs b = a;
-    b.smem_bytes = std::min(budget, solve_smem_bytes(a.smem_slots, true) + 12 * a.smem_rows);
-    CK(cudaFuncSetAttribute(k_solve_m<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
+    if (X) threads = std::min(threads, SOLVE_THREADS / 2);
+    b.smem_bytes = std::min(budget, solve_smem_bytes(a.smem_slots, true) + 12 * a.smem_rows + 16 +
+                                        (X ? 2 * FULL_ROW_WORDS * 16 * threads : 0));
+    CK(cudaFuncSetAttribute(k_solve_m<C, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.n_parts * C);
     cfg.blockDim = dim3(threads);
@@ -1171,36 +1221,38 @@ static void launch_solve_m(const SolveArgs &a, int threads, int budget, cudaStre
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    CK(cudaLaunchKernelEx(&cfg, k_solve_m<C>, b));
+    CK(cudaLaunchKernelEx(&cfg, k_solve_m<C, X>, b));
     note_launch();
+}
+
+template <bool X>
+static void launch_solve_masses(const SolveArgs &a, int threads, int cluster, int budget, cudaStream_t s) {
+    switch (cluster) {
+        case 8: launch_solve_m<8, X>(a, threads, budget, s); break;
+        case 6: launch_solve_m<6, X>(a, threads, budget, s); break;
+        case 4: launch_solve_m<4, X>(a, threads, budget, s); break;
+        case 3: launch_solve_m<3, X>(a, threads, budget, s); break;
+        case 2: launch_solve_m<2, X>(a, threads, budget, s); break;
+        default: launch_solve_m<1, X>(a, threads, budget, s); break;
+    }
 }
 
 void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool masses, int budget, cudaStream_t s) {
     if (!a.n_parts) return;
-    if (masses && !a.row_full) {
-        switch (cluster) {
-            case 8: launch_solve_m<8>(a, threads, budget, s); break;
-            case 6: launch_solve_m<6>(a, threads, budget, s); break;
-            case 4: launch_solve_m<4>(a, threads, budget, s); break;
-            case 3: launch_solve_m<3>(a, threads, budget, s); break;
-            case 2: launch_solve_m<2>(a, threads, budget, s); break;
-            default: launch_solve_m<1>(a, threads, budget, s); break;
-        }
-        CK(cudaGetLastError());
-        return;
-    }
     if (threads > SOLVE_THREADS) threads = SOLVE_THREADS;
-    if (a.row_full) {
+    if (masses) {
+        if (a.row_full) launch_solve_masses<true>(a, threads, cluster, budget, s);
+        else launch_solve_masses<false>(a, threads, cluster, budget, s);
+    } else if (a.row_full) {
         // a context with boxes: the kernels that hold the full rows (two rows
         // per thread, no rows loaded ahead; one CTA per SM at 512 threads)
-        if (masses) launch_solve_u<2, true, false, true>(a, threads, cluster, s);
-        else launch_solve_u<2, false, false, true>(a, threads, cluster, s);
+        launch_solve_u<2, false, true>(a, threads, cluster, s);
     } else if (unroll == 2) {
         // a full-size CTA (one per SM) loads rows ahead
-        if (threads == SOLVE_THREADS) launch_solve_u<2, false, true>(a, threads, cluster, s);
-        else launch_solve_u<2, false, false>(a, threads, cluster, s);
+        if (threads == SOLVE_THREADS) launch_solve_u<2, true>(a, threads, cluster, s);
+        else launch_solve_u<2, false>(a, threads, cluster, s);
     } else {
-        launch_solve_u<1, false, false>(a, threads, cluster, s);
+        launch_solve_u<1, false>(a, threads, cluster, s);
     }
     CK(cudaGetLastError());
 }

@@ -187,7 +187,7 @@ struct RowArgs {
     // inverse inertia diagonals; out: the full-row flag and record of every row
     const float4 *c_p, *half, *iib;
     uint8_t *row_full;
-    float4 *rfull;
+    float4 *rfull;               // [FULL_ROW_WORDS][np]
 };
 void launch_rows(const RowArgs &a, cudaStream_t s);
 
@@ -195,7 +195,8 @@ void launch_rows(const RowArgs &a, cudaStream_t s);
 // a box end) is a "full" row: its lever arms reach the contact point (or the
 // pivots) and a box's angular response is its world inverse inertia
 // R diag(1/I) R^T.  Per constraint FULL_ROW_WORDS float4, for its three
-// directions d_i (contact: n, t1, t2 = n x t1; joint: the world axes):
+// directions d_i (contact: n, t1, t2 = n x t1; joint: the world axes), word j
+// of row r at [j np + r]:
 //   [i]      (d_i, target_i)
 //   [3 + i]  (r_A x d_i, k_i)                k_i = 1 / (J_i M^-1 J_i^T)
 //   [6 + i]  (I_A^-1 (r_A x d_i), 0)
@@ -237,8 +238,9 @@ struct SolveArgs {
     int *part_iters;           // [P]
     double *part_res_sq;       // [P]
     int *status;
-    const uint8_t *row_full;   // contexts with boxes: rows read from rfull (FULL_ROW_WORDS each), else NULL
-    const float4 *rfull;
+    const uint8_t *row_full;   // contexts with boxes: rows read from rfull, else NULL
+    const float4 *rfull;       // [FULL_ROW_WORDS][np]
+    int np;
 };
 // masses: the shared-memory slots hold the inverse masses and inertias (32 B
 // per slot; contact rows read as two records); else 24 B per slot

@@ -70,3 +70,23 @@ def test_joint_rows_agree(links, n_sets):
         sim.close()
     for st in out[1:]:
         assert np.array_equal(st.view(np.uint32), out[0].view(np.uint32))
+
+
+@pytest.mark.parametrize("scene", ["building", "bridge", "wide"])
+def test_box_rows_agree(scene):
+    """full rows staged a colour ahead, straight from memory (buckets beyond a CTA's threads), in clusters, and with the
+    masses in the rows"""
+    from paper_2403_17261_gb300 import ovl
+    from paper_2403_17261_gb300 import scenes as S
+    sc = {"building": lambda: S.box_building(storeys=2, cells=3, n_sets=3, iters=10),
+          "bridge": lambda: S.plank_bridge(planks=40, n_sets=2, iters=10),
+          "wide": lambda: S.box_building(storeys=1, cells=24, n_sets=1, iters=6)}[scene]()
+    out = []
+    for par in ({}, dict(pgs_cluster=1), dict(pgs_cluster=4), dict(pgs_cluster=2, pgs_threads=32), dict(smem_slot_limit=5000)):
+        sim = ovl.Simulation(sc, par)
+        for _ in range(3):
+            sim.step()
+        out.append(sim.state())
+        sim.close()
+    for st in out[1:]:
+        assert np.array_equal(st.view(np.uint32), out[0].view(np.uint32))
