@@ -352,17 +352,17 @@ struct SolveClass { int C, first, count, slots, rows; };
 // wave.
 constexpr int kSolveSmSlack = 8;
 // A worker grows past one CTA above the first number of constraints, and
-// further, up to four, while its CTAs hold more than the second each (rows with a box end take
-// longer, so a context with boxes grows sooner).  A
+// further, up to four, while its CTAs hold more than the second each (boxes have more colours,
+// so fewer rows in each).  A
 // colour step of one CTA costs about 900 cycles plus 3 per row; a cluster
 // adds its barrier (560 cycles against 95) and the traffic between its CTAs
 // (6 B per cycle), which fewer rows have to pay for.  Measured solves: 2
 // workers of 392 constraints 0.14 ms with one CTA each, 0.26 with four; 8 of
 // 906 (a chain) 0.19 and 0.31; 12 of 8600 0.63 with one and 0.50 with three or
 // four; 16 of 40,000 1.29 with four, 1.65 with eight (of which 15 clusters fit
-// at once); boxes: 16 of 4200 2.57 with one and 2.94 with four, 16 of 6100
-// 3.7 with one or two and 3.24 with four.
-constexpr double kGrow[2][2] = {{5000, 3000}, {3000, 1000}};   // [boxes][first, next]
+// at once); boxes: 16 of 4200 1.59 with one and 2.14 with four, 16 of 6100
+// 1.96 and 2.35.
+constexpr double kGrow[2][2] = {{5000, 3000}, {9000, 2500}};   // [boxes][first, next]
 constexpr int kMaxGrow = 4;
 
 // CTA shapes of the per-class launches: threads, rows per thread, CTAs per SM
