@@ -517,15 +517,15 @@ std::vector<size_t> class_launch_order(ovl_ctx *c, const std::vector<SolveClass>
 // stream
 template <class F>
 void run_on_streams(ovl_ctx *c, size_t n, F &&launch, const std::vector<size_t> &ord = {}) {
-    if (n > sizeof(c->aux) / sizeof(c->aux[0])) throw std::logic_error("more launch classes than side streams");
     if (n == 0) return;
+    const size_t streams = std::min(n, sizeof(c->aux) / sizeof(c->aux[0]));   // further launches follow the first ones
     CK(cudaEventRecord(c->fork, c->stream));
     for (size_t j = 0; j < n; ++j) {
         const size_t k = ord.empty() ? j : ord[j];
-        CK(cudaStreamWaitEvent(c->aux[j], c->fork, 0));
-        launch(k, c->aux[j]);
+        if (j < streams) CK(cudaStreamWaitEvent(c->aux[j], c->fork, 0));
+        launch(k, c->aux[j % streams]);
     }
-    for (size_t j = 0; j < n; ++j) {
+    for (size_t j = 0; j < streams; ++j) {
         CK(cudaEventRecord(c->join[j], c->aux[j]));
         CK(cudaStreamWaitEvent(c->stream, c->join[j], 0));
     }
@@ -552,10 +552,6 @@ void phase_colour(ovl_ctx *c) {
     c->col_off.ensure((size_t)P * (2 * OVL_MAX_COLOURS + 1) + 1);
     c->pair_of_row.ensure(npr + 1);
     c->colour_scratch.ensure(3 * (size_t)c->ne + 1);
-    c->worklist.ensure(npr + 1);
-    c->worklist2.ensure(npr + 1);
-    c->wprio.ensure(npr + 1);
-    c->wprio2.ensure(npr + 1);
     ColourArgs a{};
     a.n_parts = P; a.part_bstart = c->part_bstart.p; a.part_pstart = c->part_pstart.p;
     a.part_list = c->part_list.p; a.entry_body = c->entry_body.p;
@@ -564,27 +560,86 @@ void phase_colour(ovl_ctx *c) {
     a.part_rounds = c->part_rounds.p;
     a.scratch = c->colour_scratch.p; a.hi_mask = c->colour_scratch.p + 2 * (size_t)c->ne;
     a.status = c->status.p;
+    const bool fixed = c->P.pgs_cluster > 0 || c->P.smem_slot_limit > 0;
+    // Workers one CTA's shared memory holds take the list kernel (a fixed
+    // cluster size keeps the rounds).  More threads than a worker has work for
+    // only lengthen its barriers, and a small worker's CTA leaves room for
+    // others on its SM: 256 threads up to kColourSmall constraints (512 scenes:
+    // 0.83 ms with the line at 512, 0.78 at 1024, 0.73 at 2048, 0.82 at 4096;
+    // the building's 4200 per worker: 0.25 ms with 1024 threads, 0.45 with 256).
+    constexpr int kColourSmall = 2048;
+    std::vector<uint32_t> lists[2], rest;
+    int smem[2] = {0, 0};
+    const int most = c->smem_optin - colour_list_static_smem() - 1024;
+    std::vector<uint32_t> longest(P);
+    std::iota(longest.begin(), longest.end(), 0u);
+    std::stable_sort(longest.begin(), longest.end(), [&](uint32_t x, uint32_t y) {
+        return c->h_pp[x + 1] - c->h_pp[x] > c->h_pp[y + 1] - c->h_pp[y];
+    });
+    for (uint32_t p : longest) {
+        const int nb = c->h_pb[p + 1] - c->h_pb[p], np = c->h_pp[p + 1] - c->h_pp[p];
+        const int need = colour_list_smem(nb, np, most);
+        if (fixed || need > most) {
+            rest.push_back(p);
+            continue;
+        }
+        const int k = np > kColourSmall ? 0 : 1;
+        lists[k].push_back(p);
+        smem[k] = std::max(smem[k], need);
+    }
+    if (!lists[0].empty() || !lists[1].empty()) {
+        c->list_prio.ensure(2 * (size_t)npr + 1);
+        c->list_sorted.ensure(2 * (size_t)npr + 1);
+        c->list_queue.ensure((size_t)npr + 1);
+    }
+    if (!rest.empty()) {
+        c->worklist.ensure(npr + 1);
+        c->worklist2.ensure(npr + 1);
+        c->wprio.ensure(npr + 1);
+        c->wprio2.ensure(npr + 1);
+    }
     a.worklist = c->worklist.p; a.worklist2 = c->worklist2.p;
     a.wprio = c->wprio.p; a.wprio2 = c->wprio2.p;
-    const bool fixed = c->P.pgs_cluster > 0 || c->P.smem_slot_limit > 0;
+    a.list_prio = c->list_prio.p; a.list_sorted = c->list_sorted.p; a.list_queue = c->list_queue.p;
     std::vector<SolveClass> classes;
-    if (!fixed && P > 0 &&
-        plan_worker_classes(c, colour_smem_capacity(c), (long long)c->num_sms - kSolveSmSlack,
-                            classes, c->colour_order)) {
-        run_on_streams(c, classes.size(), [&](size_t k, cudaStream_t sk) {
-            ColourArgs b = a;
-            b.n_parts = classes[k].count;
-            b.order = c->colour_order.p + classes[k].first;
-            b.smem_slots = classes[k].slots;
-            launch_colour(b, classes[k].C, sk);
-        });
+    if (!rest.empty() && (fixed || !plan_worker_classes(c, colour_smem_capacity(c), (long long)c->num_sms - kSolveSmSlack,
+                                                        classes, c->colour_order))) {
+        int cluster = 1, slots = 0;
+        colour_config(c, &cluster, &slots);
+        a.smem_slots = slots;
+        a.order = uniform_order(c);
+        launch_colour(a, cluster, c->stream);
         return;
     }
-    int cluster = 1, slots = 0;
-    colour_config(c, &cluster, &slots);
-    a.smem_slots = slots;
-    a.order = uniform_order(c);
-    launch_colour(a, cluster, c->stream);
+    // launch order: the clusters of the large workers, then the lists
+    std::vector<uint32_t> order;
+    struct Launch { int kind, first, count, C, slots; };   // kind: 0, 1 lists; 2 rounds
+    std::vector<Launch> launches;
+    if (!rest.empty()) {
+        std::stable_sort(rest.begin(), rest.end(), [&](uint32_t x, uint32_t y) { return c->h_class_C[x] > c->h_class_C[y]; });
+        for (size_t i = 0; i < rest.size(); ++i) {
+            const int C = c->h_class_C[rest[i]], nb = c->h_pb[rest[i] + 1] - c->h_pb[rest[i]];
+            if (launches.empty() || launches.back().C != C) launches.push_back({2, (int)order.size(), 0, C, 1});
+            launches.back().count++;
+            launches.back().slots = std::max(launches.back().slots, (nb + C - 1) / C);
+            order.push_back(rest[i]);
+        }
+    }
+    for (int k = 0; k < 2; ++k) {
+        if (lists[k].empty()) continue;
+        launches.push_back({k, (int)order.size(), (int)lists[k].size(), 1, 0});
+        order.insert(order.end(), lists[k].begin(), lists[k].end());
+    }
+    upload(c->colour_order, order.data(), order.size(), c->stream);
+    run_on_streams(c, launches.size(), [&](size_t k, cudaStream_t sk) {
+        const Launch &l = launches[k];
+        ColourArgs b = a;
+        b.n_parts = l.count;
+        b.order = c->colour_order.p + l.first;
+        b.smem_slots = l.kind == 2 ? l.slots : smem[l.kind];
+        if (l.kind == 2) launch_colour(b, l.C, sk);
+        else launch_colour_lists(b, l.kind == 0 ? 1024 : 256, smem[l.kind], sk);
+    });
 }
 
 void phase_rows(ovl_ctx *c, float dt_override) {
@@ -1092,7 +1147,7 @@ void release_all(ovl_ctx *c) {
     c->pair_cons.release(); c->pair_part.release(); c->ps_cons.release(); c->ps_part.release();
     c->part_pstart.release(); c->p_colour.release(); c->part_ncol.release(); c->part_rounds.release();
     c->col_off.release(); c->pair_of_row.release(); c->p_key.release(); c->p_slot.release();
-    c->p_lam0.release(); c->colour_scratch.release(); c->worklist.release(); c->worklist2.release(); c->wprio.release(); c->wprio2.release(); c->r0.release(); c->r1.release();
+    c->p_lam0.release(); c->colour_scratch.release(); c->worklist.release(); c->worklist2.release(); c->list_prio.release(); c->list_sorted.release(); c->list_queue.release(); c->wprio.release(); c->wprio2.release(); c->r0.release(); c->r1.release();
     c->r2.release(); c->rlam.release(); c->lam_out.release(); c->r3.release(); c->rpair.release(); c->ws_pstart.release();
     c->ws_key.release(); c->ws_lam.release(); c->copies.release(); c->solve_scratch.release();
     c->part_iters.release(); c->part_res_sq.release(); c->visited.release(); c->queue.release();

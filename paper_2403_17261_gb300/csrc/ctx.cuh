@@ -73,7 +73,8 @@ struct ovl_ctx {
     DBuf<float4> p_lam0;
     DBuf<unsigned long long> colour_scratch;
     DBuf<int4> worklist, worklist2;
-    DBuf<unsigned long long> wprio, wprio2;
+    DBuf<int2> list_sorted, list_queue;
+    DBuf<unsigned long long> wprio, wprio2, list_prio;
     DBuf<float4> r0, r1, r2, r3, rlam, lam_out;
     DBuf<int> rpair;
     DBuf<int> ws_pstart;

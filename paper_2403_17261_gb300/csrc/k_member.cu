@@ -726,6 +726,255 @@ __global__ void __launch_bounds__(COLOUR_THREADS) k_colour(ColourArgs a) {
 }
 
 // ---------------------------------------------------------------------------
+// The same colours for a worker that one CTA holds, by lists.  Every slot keeps
+// its constraints sorted by descending priority; a constraint is ready once it
+// heads the lists of both its slots, takes its colour, and both lists move
+// on.  The ready constraints of a round are exactly those of the rounds above,
+// but a constraint is looked at twice in all, where there every uncoloured one
+// posts its priority in every round: same-address shared-memory atomics (28
+// constraints per body in the building, 147 rounds) bounded it.  A round is
+// now a barrier and a chain of a few loads.  Measured, rounds and lists: the
+// building 0.51 and 0.25 ms, 512 scenes 1.14 and 0.73, a 30 k pile 0.20 and
+// 0.13, the large pile (in clusters before) 0.38-0.54 and 0.30.
+//
+// Global scratch of the worker: the priorities of every end in slot order,
+// and (constraint, other slot) sorted.
+// Shared memory: per slot the start of its list, its head and the colours
+// 0-63 taken; a bit per constraint, set when it heads its first list; and,
+// while they fit, two queues of ready constraints (no more than one per
+// slot), which else lie in global memory.
+// ---------------------------------------------------------------------------
+constexpr int LIST_SLOT_BYTES = 4 + 4 + 8, LIST_QUEUE_BYTES = 2 * 4;   // start, head, used; two queues
+
+struct ListShared {
+    int qlen[3];          // by round modulo 3
+    int ncol, scan[32];
+    int counts[NBUCKET + 1], base_b[NBUCKET + 1], running[NBUCKET];
+    uint8_t wcnt[32][NBUCKET];
+};
+
+__host__ __device__ inline long long list_bytes(int nb, int np) {
+    return (long long)LIST_SLOT_BYTES * nb + 8 + 4 * (long long)((np + 31) / 32);
+}
+
+// exclusive prefix over the block of one value per thread; *total gets the sum
+__device__ __forceinline__ int block_prefix(int v, int *warp_sums, int *total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int inc = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += x;
+    }
+    if (lane == 31) warp_sums[warp] = inc;
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int w = 0; w < nw; ++w) {
+        before += w < warp ? warp_sums[w] : 0;
+        all += warp_sums[w];
+    }
+    __syncthreads();
+    *total = all;
+    return before + inc - v;
+}
+
+template <int TMAX>
+__global__ void __launch_bounds__(TMAX) k_colour_lists(ColourArgs a) {
+    extern __shared__ unsigned long long dyn_smem[];
+    __shared__ ListShared sh;
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int p = (int)a.order[blockIdx.x];
+    const int b0 = a.part_bstart[p], nb = a.part_bstart[p + 1] - b0;
+    const int q0 = a.part_pstart[p], m = a.part_pstart[p + 1] - q0;
+    unsigned long long *used = dyn_smem;
+    int *start = reinterpret_cast<int *>(used + nb), *head = start + nb + 1;
+    uint32_t *first = reinterpret_cast<uint32_t *>(head + nb);   // (m + 31) / 32
+    const uint64_t *key = a.p_key + q0;
+    const int2 *slot = a.p_slot + q0;
+    unsigned long long *hi = a.hi_mask + b0;
+    unsigned long long *fill_pr = a.list_prio + 2 * (size_t)q0;
+    int2 *sorted = a.list_sorted + 2 * (size_t)q0;
+    // the queues: nb words each, or m each (never more constraints than that)
+    const bool near = list_bytes(nb, m) + LIST_QUEUE_BYTES * nb <= a.smem_slots;
+    int *const queue0 = near ? reinterpret_cast<int *>(first + (m + 31) / 32) : reinterpret_cast<int *>(a.list_queue + q0);
+    int *const queue1 = near ? queue0 + nb : queue0 + m;
+    for (int s = tid; s < nb; s += T) {
+        used[s] = 0ull;
+        head[s] = 0;
+        __stcg(hi + s, 0ull);
+    }
+    for (int w = tid; w < (m + 31) / 32; w += T) first[w] = 0u;
+    for (int j = tid; j <= NBUCKET; j += T) sh.counts[j] = 0;
+    for (int j = tid; j < NBUCKET; j += T) sh.running[j] = 0;
+    for (int j = tid; j < 32 * NBUCKET; j += T) (&sh.wcnt[0][0])[j] = 0;
+    if (tid < 3) sh.qlen[tid] = 0;
+    if (tid == 0) sh.ncol = 0;
+    __syncthreads();
+    // list lengths, starts, and the ends in any order (a constraint whose two
+    // ends share a slot enters it once)
+    for (int k = tid; k < m; k += T) {
+        const int2 sl = slot[k];
+        if (sl.x >= 0) atomicAdd(&head[sl.x], 1);
+        if (sl.y >= 0 && sl.y != sl.x) atomicAdd(&head[sl.y], 1);
+    }
+    __syncthreads();
+    int run = 0;
+    for (int base = 0; base < nb; base += T) {
+        const int s = base + tid, n = s < nb ? head[s] : 0;
+        int total;
+        const int e = block_prefix(n, sh.scan, &total);
+        if (s < nb) {
+            start[s] = run + e;
+            head[s] = run + e;
+        }
+        run += total;
+    }
+    if (tid == 0) start[nb] = run;
+    __syncthreads();
+    for (int k = tid; k < m; k += T) {
+        const int2 sl = slot[k];
+        const unsigned long long pr = mix64(key[k]);
+        auto put = [&](int s) {
+            const int o = atomicAdd(&head[s], 1);
+            fill_pr[o] = pr;
+        };
+        const bool loop = sl.x == sl.y;
+        if (sl.x >= 0) put(sl.x);
+        if (sl.y >= 0 && !loop) put(sl.y);
+    }
+    __syncthreads();
+    // every end to its place by priority: its rank among its list
+    for (int k = tid; k < m; k += T) {
+        const int2 sl = slot[k];
+        const unsigned long long pr = mix64(key[k]);
+        auto place = [&](int s, int other) {
+            const int lo = start[s], end = start[s + 1];
+            int rank = 0;
+            for (int i = lo; i < end; ++i) rank += fill_pr[i] > pr ? 1 : 0;
+            sorted[lo + rank] = make_int2(k, other);
+        };
+        const bool loop = sl.x == sl.y;
+        if (sl.x >= 0) place(sl.x, loop ? -1 : sl.y);
+        if (sl.y >= 0 && !loop) place(sl.y, sl.x);
+    }
+    __syncthreads();
+    // the constraint that now heads the list of slot s: ready if it is its
+    // only slot, or it heads its other list already; queued for the round
+    auto arrive = [&](int s, int *q, int *len) {
+        const int h = head[s];
+        if (h >= start[s + 1]) return;
+        const int2 e = sorted[h];
+        bool ready = e.y < 0;
+        if (!ready) {
+            __threadfence_block();
+            const uint32_t bit = 1u << (e.x & 31);
+            ready = atomicOr(first + (e.x >> 5), bit) & bit;
+        }
+        if (ready) q[atomicAdd(len, 1)] = e.x;
+    };
+    for (int s = tid; s < nb; s += T) head[s] = start[s];
+    __syncthreads();
+    for (int s = tid; s < nb; s += T) arrive(s, queue0, &sh.qlen[0]);
+    int rounds = 0, ncol = 0;
+    for (;; ++rounds) {
+        __syncthreads();
+        const int n = sh.qlen[rounds % 3];
+        if (n == 0 || rounds > m) break;
+        const int *cur = rounds & 1 ? queue1 : queue0;
+        int *next = rounds & 1 ? queue0 : queue1;
+        if (tid == 0) sh.qlen[(rounds + 2) % 3] = 0;   // last read two rounds ago, written in the next round
+        for (int i = tid; i < n; i += T) {
+            const int k = cur[i];
+            const int2 sl = slot[k];
+            const bool loop = sl.x == sl.y;
+            // only this constraint touches its slots in this round
+            unsigned long long u = 0ull;
+            if (sl.x >= 0) u |= used[sl.x];
+            if (sl.y >= 0) u |= used[sl.y];
+            int c;
+            if (~u) {   // colours 0-63
+                c = __ffsll((long long)~u) - 1;
+                const unsigned long long bit = 1ull << c;
+                if (sl.x >= 0) used[sl.x] |= bit;
+                if (sl.y >= 0) used[sl.y] |= bit;
+            } else {
+                unsigned long long v = 0ull;   // colours 64-127
+                if (sl.x >= 0) v |= __ldcg(hi + sl.x);
+                if (sl.y >= 0) v |= __ldcg(hi + sl.y);
+                if (~v) {
+                    c = 64 + __ffsll((long long)~v) - 1;
+                } else {
+                    c = OVL_MAX_COLOURS - 1;
+                    atomicCAS(a.status, DEV_OK, DEV_ERR_COLOURS);
+                }
+                const unsigned long long bit = 1ull << (c - 64);
+                if (sl.x >= 0) __stcg(hi + sl.x, __ldcg(hi + sl.x) | bit);
+                if (sl.y >= 0) __stcg(hi + sl.y, __ldcg(hi + sl.y) | bit);
+            }
+            a.p_colour[q0 + k] = c;
+            ncol = max(ncol, c + 1);
+            if (sl.x >= 0) {
+                ++head[sl.x];
+                arrive(sl.x, next, &sh.qlen[(rounds + 1) % 3]);
+            }
+            if (sl.y >= 0 && !loop) {
+                ++head[sl.y];
+                arrive(sl.y, next, &sh.qlen[(rounds + 1) % 3]);
+            }
+        }
+    }
+    if (tid == 0 && rounds > m) atomicCAS(a.status, DEV_OK, DEV_ERR_TIMEOUT);
+    // stable counting sort by (colour, kind): contacts before joints inside a
+    // colour, canonical order kept
+    for (int o = 16; o > 0; o >>= 1) ncol = max(ncol, __shfl_xor_sync(0xffffffffu, ncol, o));
+    if (lane == 0) atomicMax(&sh.ncol, ncol);
+    auto bucket_of = [&](int k) { return 2 * a.p_colour[q0 + k] + ((int)(key[k] >> 62) & 1); };
+    const unsigned lt = (1u << lane) - 1u;
+    for (int base = warp * 32; base < m; base += T) {
+        const int k = base + lane, bucket = k < m ? bucket_of(k) : -1;
+        const unsigned peers = __match_any_sync(0xffffffffu, bucket);
+        if (bucket >= 0 && (peers & lt) == 0) atomicAdd(&sh.counts[bucket], __popc(peers));
+    }
+    __syncthreads();
+    run = 0;
+    for (int base = 0; base <= NBUCKET; base += T) {
+        const int j = base + tid;
+        int total;
+        const int e = block_prefix(j <= NBUCKET ? sh.counts[j] : 0, sh.scan, &total);
+        if (j <= NBUCKET) {
+            sh.base_b[j] = run + e;
+            a.col_off[(size_t)p * (NBUCKET + 1) + j] = q0 + run + e;
+        }
+        run += total;
+    }
+    if (tid == 0) {
+        a.part_ncol[p] = sh.ncol;
+        // at least one round, as the rounds of the kernel above count
+        a.part_rounds[p] = max(rounds, 1);
+    }
+    __syncthreads();
+    for (int base = 0; base < m; base += T) {
+        const int k = base + tid;
+        const int bucket = k < m ? bucket_of(k) : NBUCKET;
+        const unsigned peers = __match_any_sync(0xffffffffu, bucket);
+        const int lrank = __popc(peers & lt);
+        if (k < m && lrank == 0) sh.wcnt[warp][bucket] = (uint8_t)__popc(peers);
+        __syncthreads();
+        if (k < m) {
+            int pre = 0;
+            for (int w = 0; w < warp; ++w) pre += sh.wcnt[w][bucket];
+            a.pair_of_row[q0 + sh.base_b[bucket] + sh.running[bucket] + pre + lrank] = q0 + k;
+        }
+        __syncthreads();
+        for (int j = tid; j < NBUCKET; j += T) {
+            int add = 0;
+            for (int w = 0; w < T / 32; ++w) { add += sh.wcnt[w][j]; sh.wcnt[w][j] = 0; }
+            sh.running[j] += add;
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Row records in colour order (the solver forms t1, t2, k_n, k_t and the
 // joint k's itself).  Contacts (sphere-sphere or sphere-plane):
 //   r0 = (n, slot_b)  r1 = (r_a, r_b, target_n, slot_a)  r3 = (1/m_a, 1/m_b, 1/I_a, 1/I_b)
@@ -1021,6 +1270,25 @@ int colour_static_smem() {
         bytes = mx;
     }
     return bytes;
+}
+
+int colour_list_smem(int nb, int np, int most) {
+    const long long need = list_bytes(nb, np), near = need + (long long)LIST_QUEUE_BYTES * nb;
+    return (int)std::min<long long>(near <= most ? near : need, 1ll << 30);
+}
+int colour_list_static_smem() { return (int)sizeof(ListShared); }
+
+void launch_colour_lists(const ColourArgs &a, int threads, int smem, cudaStream_t s) {
+    if (!a.n_parts) return;
+    if (threads > 256) {
+        CK(cudaFuncSetAttribute(k_colour_lists<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        k_colour_lists<1024><<<a.n_parts, threads, smem, s>>>(a);
+    } else {
+        CK(cudaFuncSetAttribute(k_colour_lists<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        k_colour_lists<256><<<a.n_parts, threads, smem, s>>>(a);
+    }
+    note_launch();
+    CK(cudaGetLastError());
 }
 
 void launch_colour(const ColourArgs &a, int cluster, cudaStream_t s) {

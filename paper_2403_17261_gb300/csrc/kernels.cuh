@@ -150,10 +150,18 @@ struct ColourArgs {
     unsigned long long *hi_mask;  // [ne] colours 64-127 taken at every worker slot
     int4 *worklist, *worklist2;                 // [np] each: uncoloured constraints per round
     unsigned long long *wprio, *wprio2;         // [np] each: their priorities
-    int smem_slots;            // slots that fit in shared memory
+    // the list kernel's (it runs beside the rounds): priorities and ends by slot [2 np], queues [np]
+    unsigned long long *list_prio;
+    int2 *list_sorted, *list_queue;
+    int smem_slots;            // slots that fit in shared memory (list kernel: bytes)
     int *status;
 };
 void launch_colour(const ColourArgs &a, int cluster, cudaStream_t s);
+// one CTA per worker of `order`, each within smem bytes of dynamic shared memory
+void launch_colour_lists(const ColourArgs &a, int threads, int smem, cudaStream_t s);
+// bytes for a worker of nb bodies and np constraints, its queues in shared memory too if that fits `most`
+int colour_list_smem(int nb, int np, int most);
+int colour_list_static_smem();
 int colour_static_smem();
 
 struct RowArgs {
