@@ -148,11 +148,12 @@ struct ovl_ctx {
     DBuf<float> log_feat, log_targ;
     long long log_cap = 0, log_n = 0;
     bool log_on = false;
-    DBuf<float> train_act, train_sample_loss, train_partials, train_loss_hist, infer_y;
+    DBuf<float> train_sample_loss, train_partials, train_loss_hist, infer_y;
     DBuf<float4> infer_feat;
     DBuf<double> loss_acc;
     DBuf<float> train_c12;            // Adam bias corrections per step of a training call
-    DBuf<long long> train_step;       // step counter of a training call (graph replay)
+    DBuf<long long> train_step;       // step counter of a training call (graph replay), scratch
+    DBuf<uint32_t> train_packed;      // BF16 operands of a training call
 };
 
 namespace ovl {

@@ -24,10 +24,11 @@
 // memory (tcgen05.ld), adds the bias, applies the ReLU and writes the next
 // layer's BF16 operand to shared memory.  Training runs on the tensor cores
 // too, with the same arithmetic (operands rounded to BF16, products exact,
-// FP32 sums): the forward and backward passes of 128 samples per CTA as five
-// products, the weight gradients of 128 samples per CTA as three products
-// with the samples as K, summed over blocks in block order (deterministic),
-// and Adam on FP32 master parameters.
+// FP32 sums): one kernel takes 128 samples per CTA through the forward and
+// backward passes (five products) and their weight gradients (three products
+// with the samples as K), the next sums the gradients over blocks in block
+// order (deterministic), runs Adam on FP32 master parameters and writes the
+// next step's BF16 operands.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -49,9 +50,6 @@ static_assert(OFF_B3 + 3 == MLP_N_PARAMS, "parameter layout");
 // FP32 biases b1 [64], b2 [64], b3 [16] (zero-padded)
 constexpr int PK_W1 = 0, PK_W2 = 512, PK_W3 = 2560, PK_B1 = 3072, PK_B2 = 3136, PK_B3 = 3200;
 static_assert(PK_B3 + 16 == MLP_PK_WORDS, "packed layout");
-// activation rows of the training pass
-constexpr int A_X = 0, A_H1 = 16, A_H2 = 80, A_DZ1 = 144, A_DZ2 = 208, A_DY = 272;
-static_assert(A_DY + 4 == MLP_ACT_STRIDE, "activation layout");
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
@@ -437,7 +435,7 @@ __device__ __forceinline__ long long sample_row(const TrainArgs &a, long long st
     return a.first + (long long)(z % (uint64_t)a.count);
 }
 
-// Forward, loss and the backward pass down to the pre-activation gradients
+// Forward, loss, backward pass and weight gradients
 // of one tile of 128 samples per CTA, on the tensor cores; thread t owns
 // sample t of the tile (TMEM lane t).  Five products, each M = 128 with BF16
 // operands in shared memory and FP32 accumulators in tensor memory:
@@ -446,19 +444,45 @@ __device__ __forceinline__ long long sample_row(const TrainArgs &a, long long st
 // with h1 = bf16(relu(D1 + b1)), h2 = bf16(relu(D2 + b2)), y = (D3 + b3) +
 // x[4..6] (the skip connection in FP32), dy = bf16(2 (y - t) / (3 B)),
 // dz2 = bf16(T2) where h2 > 0, dz1 = bf16(T1) where h1 > 0.  Every operand
-// of a product is BF16 (the products exact) and the sums FP32.  The B
-// operands are built from the FP32 parameters by every CTA.  Accumulators:
+// of a product is BF16 (the products exact) and the sums FP32.  Accumulators:
 // D1 and then T1 in TMEM columns 0-63, D2 in 64-127, D3 in 128-143, T2 in
-// 192-255.  Waits on the MMAs are bounded; one that gives up sets the device
+// 192-255.
+//
+// BACK: every weight gradient is a sum over samples of (operand
+// A) x (operand B) of the same values, i.e. a GEMM with the samples as K:
+//   dW1 = X^T dZ1 (12 x 64), dW2 = H1^T dZ2 (64 x 64), dW3 = H2^T dY (64 x 3),
+// and a bias gradient is the same sum with A = 1.  Each is one M = 128
+// product over K = 128 samples (eight K-steps): A holds the
+// transposed activations in its first rows and a row of ones after them (its
+// accumulator row is the bias gradient), B the transposed deltas; thread s
+// writes sample s's column of every operand as it forms the values.  The
+// other rows of A, and rows 3-15 of dY's operand, stay as they are: they reach
+// only accumulator rows and columns that are not read.  Accumulators in
+// columns 256-319, 320-383 and 384-399.  Slot MLP_N_PARAMS of a
+// block's partials holds its loss sum.
+//
+// Bound by latency (32 CTAs of four warps for a batch of 4096).  As two kernels
+// with the activations in global memory (4.5 MB per step, read back a scalar
+// at a time) and the operands built from FP32 parameters by every CTA, an Adam
+// step took 39.7 us; now 18.9.
+//
+// Waits on the MMAs are bounded; one that gives up sets the device
 // status, and the CTA waits once more and frees its tensor memory.
-constexpr int TRAIN_TILE = 128, TRAIN_COLS = 256;
+constexpr int TRAIN_TILE = 128;
 constexpr int TF_X = 0, TF_H1 = TF_X + 128 * 16 * 2, TF_H2 = TF_H1 + 128 * 64 * 2, TF_DY = TF_H2 + 128 * 64 * 2,
               TF_DZ2 = TF_DY + 128 * 16 * 2, TF_B1 = TF_DZ2 + 128 * 64 * 2, TF_B2 = TF_B1 + 64 * 16 * 2,
               TF_B3 = TF_B2 + 64 * 64 * 2, TF_B4 = TF_B3 + 16 * 64 * 2, TF_B5 = TF_B4 + 64 * 16 * 2,
               TF_SMEM = TF_B5 + 64 * 64 * 2;
-// two CTAs per SM at most: each holds half of the SM's 512 tensor-memory
-// columns, and a third would wait in tcgen05.alloc
+// the gradients' operands: X^T, H1^T, H2^T and dZ1^T, dZ2^T, dY^T
+constexpr int WG_A_BYTES = 128 * TRAIN_TILE * 2, WG_B_BYTES = 64 * TRAIN_TILE * 2, WG_B3_BYTES = 16 * TRAIN_TILE * 2;
+constexpr int WG_A1 = TF_SMEM, WG_A2 = WG_A1 + WG_A_BYTES, WG_A3 = WG_A2 + WG_A_BYTES, WG_B1 = WG_A3 + WG_A_BYTES,
+              WG_B2 = WG_B1 + WG_B_BYTES, WG_B3 = WG_B2 + WG_B_BYTES, WG_SMEM = WG_B3 + WG_B3_BYTES;
+// loss only: two CTAs per SM at most, each with half of the SM's 512
+// tensor-memory columns (a third would wait in tcgen05.alloc); with the
+// gradients one, with all of them
 static_assert(3 * (TF_SMEM + 2048) > 228 * 1024 && 2 * (TF_SMEM + 2048) <= 227 * 1024, "two CTAs per SM");
+static_assert(2 * WG_SMEM > 228 * 1024 && WG_SMEM + 2048 <= 227 * 1024, "one CTA per SM");
+static_assert(TF_SMEM - TF_B1 == 4 * MLP_TRAIN_PK_WORDS, "packed training operands");
 
 // one row (K columns) of a K-major BF16 operand from FP32 values
 template <int K>
@@ -472,45 +496,41 @@ __device__ __forceinline__ void put_row(uint8_t *op, int r, const float *v) {
     }
 }
 
-__global__ void __launch_bounds__(TRAIN_TILE) k_train_fwd(TrainArgs a) {
+__device__ __forceinline__ void put_bf16(uint8_t *op, int r, int k, int K, float v) {
+    *reinterpret_cast<__nv_bfloat16 *>(op + kmajor_off(r, k, K)) = __float2bfloat16_rn(v);
+}
+
+// parameter p's places in the packed training operands (B1 .. B5 as they lie
+// from TF_B1 on; biases are read as FP32)
+__device__ __forceinline__ void pack_param(uint8_t *pk, int p, float v) {
+    if (p < OFF_B1) {
+        put_bf16(pk, p % 64, p / 64, 16, v);                                             // W1^T
+    } else if (p >= OFF_W2 && p < OFF_B2) {
+        const int i = (p - OFF_W2) / 64, o = (p - OFF_W2) % 64;
+        put_bf16(pk + (TF_B2 - TF_B1), o, i, 64, v);                                     // W2^T
+        put_bf16(pk + (TF_B5 - TF_B1), i, o, 64, v);                                     // (W2^T)^T = W2
+    } else if (p >= OFF_W3 && p < OFF_B3) {
+        const int i = (p - OFF_W3) / 3, o = (p - OFF_W3) % 3;
+        put_bf16(pk + (TF_B3 - TF_B1), o, i, 64, v);                                     // W3^T
+        put_bf16(pk + (TF_B4 - TF_B1), i, o, 16, v);                                     // (W3^T)^T = W3
+    }
+}
+
+__global__ void k_train_pack(const float *th, uint32_t *pk) {
+    for (int i = threadIdx.x; i < MLP_TRAIN_PK_WORDS; i += blockDim.x) pk[i] = 0u;       // the padding
+    __syncthreads();
+    for (int p = threadIdx.x; p < MLP_N_PARAMS; p += blockDim.x) pack_param(reinterpret_cast<uint8_t *>(pk), p, th[p]);
+}
+
+template <bool BACK>
+__global__ void __launch_bounds__(TRAIN_TILE) k_train_grad(TrainArgs a) {
     extern __shared__ __align__(1024) uint8_t tsm[];
     __shared__ float sb[64 + 64 + 4];
+    __shared__ float lsum[TRAIN_TILE];
     __shared__ __align__(8) uint64_t mbar;
     __shared__ uint32_t tmem_base;
+    constexpr uint32_t kCols = BACK ? 512 : 256;
     const int tid = threadIdx.x, warp = tid >> 5;
-    // B operands from the parameters: row n, column k
-    {
-        const float *th = a.theta;
-        auto put = [&](int off, int r, int k, int K, float v) {
-            *reinterpret_cast<__nv_bfloat16 *>(tsm + off + kmajor_off(r, k, K)) = __float2bfloat16_rn(v);
-        };
-        for (int e = tid; e < 64 * 16; e += TRAIN_TILE) {
-            const int n = e / 16, k = e % 16;
-            put(TF_B1, n, k, 16, k < 12 ? th[OFF_W1 + k * 64 + n] : 0.f);        // W1^T
-            put(TF_B4, n, k, 16, k < 3 ? th[OFF_W3 + n * 3 + k] : 0.f);          // (W3^T)^T = W3
-        }
-        for (int e = tid; e < 64 * 64; e += TRAIN_TILE) {
-            const int n = e / 64, k = e % 64;
-            put(TF_B2, n, k, 64, th[OFF_W2 + k * 64 + n]);                       // W2^T
-            put(TF_B5, n, k, 64, th[OFF_W2 + n * 64 + k]);                       // (W2^T)^T = W2
-        }
-        for (int e = tid; e < 16 * 64; e += TRAIN_TILE) {
-            const int n = e / 64, k = e % 64;
-            put(TF_B3, n, k, 64, n < 3 ? th[OFF_W3 + k * 3 + n] : 0.f);          // W3^T
-        }
-        for (int e = tid; e < 64; e += TRAIN_TILE) { sb[e] = th[OFF_B1 + e]; sb[64 + e] = th[OFF_B2 + e]; }
-        if (tid < 4) sb[128 + tid] = tid < 3 ? th[OFF_B3 + tid] : 0.f;
-    }
-    const uint32_t mb = (uint32_t)__cvta_generic_to_shared(&mbar);
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(mb) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&tmem_base);
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(dst), "n"(TRAIN_COLS) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
     // this thread's sample: features (rounded to BF16 for the product, FP32
     // for the skip connection) and targets
     const long long step = a.step_dev ? *a.step_dev : a.step;
@@ -519,26 +539,50 @@ __global__ void __launch_bounds__(TRAIN_TILE) k_train_fwd(TrainArgs a) {
     float xraw[12], targ[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int k = 0; k < 12; ++k) xraw[k] = 0.f;
-    long long r = 0;
     if (valid) {
-        r = sample_row(a, step, j);
+        const long long r = sample_row(a, step, j);
         const float4 *f = reinterpret_cast<const float4 *>(a.log_feat + 12 * r);
         const float4 f0 = f[0], f1 = f[1], f2 = f[2];
         xraw[0] = f0.x; xraw[1] = f0.y; xraw[2] = f0.z; xraw[3] = f0.w; xraw[4] = f1.x; xraw[5] = f1.y;
         xraw[6] = f1.z; xraw[7] = f1.w; xraw[8] = f2.x; xraw[9] = f2.y; xraw[10] = f2.z; xraw[11] = f2.w;
         targ[0] = a.log_targ[3 * r]; targ[1] = a.log_targ[3 * r + 1]; targ[2] = a.log_targ[3 * r + 2];
     }
-    float *act = a.act + (size_t)(valid ? j : 0) * MLP_ACT_STRIDE;
-    const bool wr = valid && a.backward;
+    // B operands as the parameters' update packed them, biases in FP32
+    {
+        const uint4 *src = reinterpret_cast<const uint4 *>(a.packed);
+        uint4 *dst = reinterpret_cast<uint4 *>(tsm + TF_B1);
+#pragma unroll
+        for (int e = 0; e < MLP_TRAIN_PK_WORDS / 4 / TRAIN_TILE; ++e) dst[tid + e * TRAIN_TILE] = src[tid + e * TRAIN_TILE];
+        const float *th = a.theta;
+        if (tid < 64) { sb[tid] = th[OFF_B1 + tid]; sb[64 + tid] = th[OFF_B2 + tid]; }
+        if (tid < 4) sb[128 + tid] = tid < 3 ? th[OFF_B3 + tid] : 0.f;
+    }
+    static_assert(MLP_TRAIN_PK_WORDS % (4 * TRAIN_TILE) == 0, "whole copies");
+    const uint32_t mb = (uint32_t)__cvta_generic_to_shared(&mbar);
+    if (tid == 0) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(mb) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&tmem_base);
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" :: "r"(dst), "n"(kCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // sample tid's column of a gradient operand (zero past the batch)
+    auto column = [&](int off, int row, float v) {
+        if (BACK) put_bf16(tsm + off, row, tid, TRAIN_TILE, valid ? v : 0.f);
+    };
     {
         float x[16];
 #pragma unroll
         for (int k = 0; k < 12; ++k) x[k] = bf16r(xraw[k]);
         x[12] = x[13] = x[14] = x[15] = 0.f;
         put_row<16>(tsm + TF_X, tid, x);
-        if (wr)
 #pragma unroll
-            for (int c = 0; c < 16; c += 4) *reinterpret_cast<float4 *>(act + A_X + c) = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
+        for (int k = 0; k < 12; ++k) column(WG_A1, k, x[k]);
+        column(WG_A1, 12, 1.f);
+        column(WG_A2, 64, 1.f);
+        column(WG_A3, 64, 1.f);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_sync();
@@ -547,22 +591,28 @@ __global__ void __launch_bounds__(TRAIN_TILE) k_train_fwd(TrainArgs a) {
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(tsm);
     uint32_t phase = 0;
     bool ok = true;
-    // one product (ks K-steps of 16) into columns dcol, then the wait
-    auto mma = [&](uint32_t dcol, int aoff, int boff, int K, int N) {
-        if (tid == 0) {
-            const uint32_t sbo = (uint32_t)K * 16u;
-            for (int ks = 0; ks < K / 16; ++ks)
-                umma_f16(tmem + dcol, umma_desc(base + aoff + 256u * ks, 128, sbo),
-                         umma_desc(base + boff + 256u * ks, 128, sbo), umma_idesc(128, N), ks > 0);
-            umma_commit(mb);
-        }
+    auto wait = [&]() {
         ok = __syncthreads_and(mbar_wait(mb, phase));
         phase ^= 1;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     };
+    // one product (K / 16 K-steps) into columns dcol
+    auto issue = [&](uint32_t dcol, int aoff, int boff, int K, int N) {
+        const uint32_t sbo = (uint32_t)K * 16u;
+        for (int ks = 0; ks < K / 16; ++ks)
+            umma_f16(tmem + dcol, umma_desc(base + aoff + 256u * ks, 128, sbo),
+                     umma_desc(base + boff + 256u * ks, 128, sbo), umma_idesc(128, N), ks > 0);
+    };
+    auto mma = [&](uint32_t dcol, int aoff, int boff, int K, int N) {
+        if (tid == 0) {
+            issue(dcol, aoff, boff, K, N);
+            umma_commit(mb);
+        }
+        wait();
+    };
     uint64_t m1 = 0, m2 = 0;   // h1 > 0, h2 > 0 per hidden unit
-    // h = bf16(relu(D + b)) into the next operand (and the activation row)
-    auto hidden = [&](uint32_t dcol, const float *bias, int opoff, int aoff_act, uint64_t &mask) {
+    // h = bf16(relu(D + b)) into the next operand and the gradient's (woff)
+    auto hidden = [&](uint32_t dcol, const float *bias, int opoff, int woff, uint64_t &mask) {
 #pragma unroll
         for (int c0 = 0; c0 < 64; c0 += 16) {
             float v[16];
@@ -580,17 +630,15 @@ __global__ void __launch_bounds__(TRAIN_TILE) k_train_fwd(TrainArgs a) {
                 q.z = pack_bf16(v[c + 4], v[c + 5]); q.w = pack_bf16(v[c + 6], v[c + 7]);
                 *reinterpret_cast<uint4 *>(op + kmajor_off(tid, c0 + c, 64)) = q;
             }
-            if (wr)
 #pragma unroll
-                for (int c = 0; c < 16; c += 4)
-                    *reinterpret_cast<float4 *>(act + aoff_act + c0 + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+            for (int i = 0; i < 16; ++i) column(woff, c0 + i, v[i]);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_sync();
     };
-    // delta = bf16(T) where the unit is active, into the activation row (and
-    // an operand when opoff >= 0)
-    auto delta = [&](uint32_t dcol, uint64_t mask, int opoff, int aoff_act) {
+    // delta = bf16(T) where the unit is active, into the gradient's operand
+    // (and a product's when opoff >= 0)
+    auto delta = [&](uint32_t dcol, uint64_t mask, int opoff, int woff) {
 #pragma unroll
         for (int c0 = 0; c0 < 64; c0 += 16) {
             float v[16];
@@ -607,21 +655,20 @@ __global__ void __launch_bounds__(TRAIN_TILE) k_train_fwd(TrainArgs a) {
                     *reinterpret_cast<uint4 *>(op + kmajor_off(tid, c0 + c, 64)) = q;
                 }
             }
-            if (wr)
 #pragma unroll
-                for (int c = 0; c < 16; c += 4)
-                    *reinterpret_cast<float4 *>(act + aoff_act + c0 + c) = make_float4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+            for (int i = 0; i < 16; ++i) column(woff, c0 + i, v[i]);
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         tc_sync();
     };
+    float loss = 0.f;
     mma(0u, TF_X, TF_B1, 16, 64);
-    if (ok) { hidden(0u, sb, TF_H1, A_H1, m1); mma(64u, TF_H1, TF_B2, 64, 64); }
-    if (ok) { hidden(64u, sb + 64, TF_H2, A_H2, m2); mma(128u, TF_H2, TF_B3, 64, 16); }
+    if (ok) { hidden(0u, sb, TF_H1, WG_A2, m1); mma(64u, TF_H1, TF_B2, 64, 64); }
+    if (ok) { hidden(64u, sb + 64, TF_H2, WG_A3, m2); mma(128u, TF_H2, TF_B3, 64, 16); }
     if (ok) {
         float o[16];
         tmem_ld16(lane_base + 128u, o);
-        float dy[16], loss = 0.f;
+        float dy[16];
 #pragma unroll
         for (int k = 0; k < 16; ++k) dy[k] = 0.f;
 #pragma unroll
@@ -631,136 +678,69 @@ __global__ void __launch_bounds__(TRAIN_TILE) k_train_fwd(TrainArgs a) {
             loss += d * d;
             dy[k] = bf16r(2.f * d / (3.f * (float)a.batch));
         }
-        if (valid) a.sample_loss[j] = loss;
-        if (wr) *reinterpret_cast<float4 *>(act + A_DY) = make_float4(dy[0], dy[1], dy[2], 0.f);
-        if (a.backward) {
+        if (!BACK && valid) a.sample_loss[j] = loss;
+        if (BACK) {
             put_row<16>(tsm + TF_DY, tid, dy);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) column(WG_B3, k, dy[k]);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             tc_sync();
             mma(192u, TF_DY, TF_B4, 16, 64);
-            if (ok) { delta(192u, m2, TF_DZ2, A_DZ2); mma(0u, TF_DZ2, TF_B5, 64, 64); }
-            if (ok) delta(0u, m1, -1, A_DZ1);
+            if (ok) { delta(192u, m2, TF_DZ2, WG_B2); mma(0u, TF_DZ2, TF_B5, 64, 64); }
+            if (ok) {
+                delta(0u, m1, -1, WG_B1);
+                if (tid == 0) {
+                    issue(256u, WG_A1, WG_B1, TRAIN_TILE, 64);
+                    issue(320u, WG_A2, WG_B2, TRAIN_TILE, 64);
+                    issue(384u, WG_A3, WG_B3, TRAIN_TILE, 16);
+                    umma_commit(mb);
+                }
+                wait();
+            }
         }
+    }
+    if (BACK) {
+        float *out = a.partials + (size_t)blockIdx.x * (MLP_N_PARAMS + 1);
+        if (ok) {
+            // accumulator row tid (TMEM lane tid): weight rows, and the bias rows
+            float v[16];
+#pragma unroll 1
+            for (int c0 = 0; c0 < 64; c0 += 16) {
+                tmem_ld16(lane_base + 256u + c0, v);
+                if (tid <= 12) {
+                    float *o = tid < 12 ? out + OFF_W1 + tid * 64 + c0 : out + OFF_B1 + c0;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) o[i] = v[i];
+                }
+                tmem_ld16(lane_base + 320u + c0, v);
+                if (tid <= 64) {
+                    float *o = tid < 64 ? out + OFF_W2 + tid * 64 + c0 : out + OFF_B2 + c0;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) o[i] = v[i];
+                }
+            }
+            tmem_ld16(lane_base + 384u, v);
+            if (tid <= 64) {
+                float *o = tid < 64 ? out + OFF_W3 + tid * 3 : out + OFF_B3;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) o[k] = v[k];
+            }
+        }
+        // loss of this block's samples, summed in a fixed tree order
+        lsum[tid] = valid ? loss : 0.f;
+        __syncthreads();
+        for (int w = TRAIN_TILE / 2; w > 0; w >>= 1) {
+            if (tid < w) lsum[tid] += lsum[tid + w];
+            __syncthreads();
+        }
+        if (tid == 0) out[MLP_N_PARAMS] = lsum[0];
     }
     if (!ok) {
         if (tid == 0) atomicCAS(a.status, DEV_OK, DEV_ERR_TIMEOUT);
-        mbar_wait(mb, phase ^ 1u);   // the product that was not seen to finish, once more (bounded)
+        mbar_wait(mb, phase ^ 1u);   // the products that were not seen to finish, once more (bounded)
     }
     tc_sync();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(TRAIN_COLS) : "memory");
-}
-
-// Block-partial gradients over the WGRAD_CHUNK = 128 samples of one CTA, on
-// the tensor cores: every weight gradient is a sum over samples of (operand
-// A) x (operand B) of the activation rows (all BF16 values, so the products
-// are exact), i.e. a GEMM with the samples as K:
-//   dW1 = X^T dZ1 (12 x 64), dW2 = H1^T dZ2 (64 x 64), dW3 = H2^T dY (64 x 3),
-// and a bias gradient is the same sum with A = 1.  Each GEMM is one M = 128
-// tcgen05 product over K = 128 samples (eight K-steps): A holds the
-// transposed activations in its first rows and a row of ones after them (its
-// accumulator row is the bias gradient), B the transposed deltas; thread s
-// writes sample s's column of every operand.  Accumulators: dW1 in TMEM
-// columns 0-63, dW2 in 64-127, dW3 in 128-143.  Slot MLP_N_PARAMS of a
-// block's partials holds its loss sum.
-constexpr int WG_A_BYTES = 128 * WGRAD_CHUNK * 2, WG_B_BYTES = 64 * WGRAD_CHUNK * 2, WG_B3_BYTES = 16 * WGRAD_CHUNK * 2;
-constexpr int WG_SMEM = 3 * WG_A_BYTES + 2 * WG_B_BYTES + WG_B3_BYTES;
-
-__global__ void __launch_bounds__(WGRAD_CHUNK) k_train_wgrad(TrainArgs a) {
-    extern __shared__ __align__(1024) uint8_t wsm[];
-    uint8_t *A1 = wsm, *A2 = A1 + WG_A_BYTES, *A3 = A2 + WG_A_BYTES;
-    uint8_t *B1 = A3 + WG_A_BYTES, *B2 = B1 + WG_B_BYTES, *B3 = B2 + WG_B_BYTES;
-    __shared__ float lsum[WGRAD_CHUNK];
-    __shared__ __align__(8) uint64_t mbar;
-    __shared__ uint32_t tmem_base;
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int s0 = blockIdx.x * WGRAD_CHUNK, cnt = min(WGRAD_CHUNK, a.batch - s0);
-    for (int i = tid; i < WG_SMEM / 16; i += WGRAD_CHUNK) reinterpret_cast<uint4 *>(wsm)[i] = make_uint4(0u, 0u, 0u, 0u);
-    __syncthreads();
-    // this sample's column of every operand (zeros past the batch)
-    {
-        const bool valid = tid < cnt;
-        const float *r = a.act + (size_t)(s0 + (valid ? tid : 0)) * MLP_ACT_STRIDE;
-        auto put = [&](uint8_t *op, int row, float v) {
-            *reinterpret_cast<__nv_bfloat16 *>(op + kmajor_off(row, tid, WGRAD_CHUNK)) = __float2bfloat16_rn(valid ? v : 0.f);
-        };
-        for (int k = 0; k < 12; ++k) put(A1, k, r[A_X + k]);
-        put(A1, 12, 1.f);
-        for (int k = 0; k < 64; ++k) {
-            put(A2, k, r[A_H1 + k]);
-            put(A3, k, r[A_H2 + k]);
-            put(B1, k, r[A_DZ1 + k]);
-            put(B2, k, r[A_DZ2 + k]);
-        }
-        put(A2, 64, 1.f);
-        put(A3, 64, 1.f);
-        for (int j = 0; j < 3; ++j) put(B3, j, r[A_DY + j]);
-    }
-    const uint32_t mb = (uint32_t)__cvta_generic_to_shared(&mbar);
-    if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" :: "r"(mb) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) {
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&tmem_base);
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" :: "r"(dst) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    tc_sync();
-    const uint32_t tmem = tmem_base;
-    if (tid == 0) {
-        const uint32_t sbo = WGRAD_CHUNK * 16;
-        const uint32_t a1 = (uint32_t)__cvta_generic_to_shared(A1), a2 = (uint32_t)__cvta_generic_to_shared(A2),
-                       a3 = (uint32_t)__cvta_generic_to_shared(A3), b1 = (uint32_t)__cvta_generic_to_shared(B1),
-                       b2 = (uint32_t)__cvta_generic_to_shared(B2), b3 = (uint32_t)__cvta_generic_to_shared(B3);
-#pragma unroll 1
-        for (int ks = 0; ks < WGRAD_CHUNK / 16; ++ks) {
-            const uint32_t o = 256u * ks;
-            umma_f16(tmem, umma_desc(a1 + o, 128, sbo), umma_desc(b1 + o, 128, sbo), umma_idesc(128, 64), ks > 0);
-            umma_f16(tmem + 64u, umma_desc(a2 + o, 128, sbo), umma_desc(b2 + o, 128, sbo), umma_idesc(128, 64), ks > 0);
-            umma_f16(tmem + 128u, umma_desc(a3 + o, 128, sbo), umma_desc(b3 + o, 128, sbo), umma_idesc(128, 16), ks > 0);
-        }
-        umma_commit(mb);
-    }
-    const bool ok = __syncthreads_and(mbar_wait(mb, 0));
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    float *out = a.partials + (size_t)blockIdx.x * (MLP_N_PARAMS + 1);
-    if (ok) {
-        // accumulator row tid (TMEM lane tid): weight rows, and the bias rows
-        const uint32_t lane = tmem + ((uint32_t)(warp * 32) << 16);
-        float v[16];
-#pragma unroll 1
-        for (int c0 = 0; c0 < 64; c0 += 16) {
-            tmem_ld16(lane + c0, v);
-            for (int i = 0; i < 16; ++i) {
-                if (tid < 12) out[OFF_W1 + tid * 64 + c0 + i] = v[i];
-                else if (tid == 12) out[OFF_B1 + c0 + i] = v[i];
-            }
-            tmem_ld16(lane + 64u + c0, v);
-            for (int i = 0; i < 16; ++i) {
-                if (tid < 64) out[OFF_W2 + tid * 64 + c0 + i] = v[i];
-                else if (tid == 64) out[OFF_B2 + c0 + i] = v[i];
-            }
-        }
-        tmem_ld16(lane + 128u, v);
-        for (int j = 0; j < 3; ++j) {
-            if (tid < 64) out[OFF_W3 + tid * 3 + j] = v[j];
-            else if (tid == 64) out[OFF_B3 + j] = v[j];
-        }
-    } else {
-        if (tid == 0) atomicCAS(a.status, DEV_OK, DEV_ERR_TIMEOUT);
-        mbar_wait(mb, 0);   // the MMAs still in flight, once more (bounded)
-    }
-    // loss of this block's samples, summed in a fixed tree order
-    lsum[tid] = tid < cnt ? a.sample_loss[s0 + tid] : 0.f;
-    __syncthreads();
-    for (int w = WGRAD_CHUNK / 2; w > 0; w >>= 1) {
-        if (tid < w) lsum[tid] += lsum[tid + w];
-        __syncthreads();
-    }
-    if (tid == 0) out[MLP_N_PARAMS] = lsum[0];
-    tc_sync();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" :: "r"(tmem) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "n"(kCols) : "memory");
 }
 
 __global__ void k_train_reduce(const float *partials, int blocks, int batch, float *grad_out,
@@ -783,29 +763,37 @@ __global__ void k_train_reduce(const float *partials, int blocks, int batch, flo
     theta[p] -= lr * (mm * c1) / (sqrtf(vv * c2) + eps);
 }
 
-// the reduce of one Adam step with its step number read from device memory
+// the reduce of one Adam step with its step number read from device memory:
+// also packs the next step's operands, and the block that finishes last
+// advances the step (done: blocks finished, zero between launches)
 __global__ void k_train_reduce_dev(const float *partials, int blocks, int batch, float *loss_hist,
                                    float *theta, float *m, float *v, float lr, float beta1,
-                                   float beta2, float eps, const float *c12,
-                                   const long long *step_dev) {
+                                   float beta2, float eps, const float *c12, uint32_t *packed,
+                                   long long *step_dev, unsigned long long *done) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > MLP_N_PARAMS) return;
-    const long long t = *step_dev;
-    float g = 0.f;
-    for (int b = 0; b < blocks; ++b) g += partials[(size_t)b * (MLP_N_PARAMS + 1) + p];
-    if (p == MLP_N_PARAMS) {
-        loss_hist[t] = g / (3.f * (float)batch);
-        return;
+    const long long t = *reinterpret_cast<volatile long long *>(step_dev);
+    if (p <= MLP_N_PARAMS) {
+        float g = 0.f;
+#pragma unroll 8
+        for (int b = 0; b < blocks; ++b) g += partials[(size_t)b * (MLP_N_PARAMS + 1) + p];
+        if (p == MLP_N_PARAMS) {
+            loss_hist[t] = g / (3.f * (float)batch);
+        } else {
+            const float mm = beta1 * m[p] + (1.f - beta1) * g;
+            const float vv = beta2 * v[p] + (1.f - beta2) * g * g;
+            m[p] = mm;
+            v[p] = vv;
+            const float th = theta[p] - lr * (mm * c12[2 * t]) / (sqrtf(vv * c12[2 * t + 1]) + eps);
+            theta[p] = th;
+            pack_param(reinterpret_cast<uint8_t *>(packed), p, th);
+        }
     }
-    const float mm = beta1 * m[p] + (1.f - beta1) * g;
-    const float vv = beta2 * v[p] + (1.f - beta2) * g * g;
-    m[p] = mm;
-    v[p] = vv;
-    theta[p] -= lr * (mm * c12[2 * t]) / (sqrtf(vv * c12[2 * t + 1]) + eps);
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(done, 1ull) == gridDim.x - 1) {
+        *done = 0;
+        *step_dev = t + 1;
+    }
 }
-
-// after every block of the reduce has read it
-__global__ void k_step_advance(long long *step_dev) { *step_dev += 1; }
 
 __global__ void k_loss_sum(const float *sample_loss, int n, double *acc) {
     __shared__ double part[256];
@@ -881,8 +869,8 @@ void mlp_kernels_setup(int device) {
     g.pad = pad;
     g.per_sm = std::max(1, std::min(occ, 4));
     g.sms = sms;
-    CK(cudaFuncSetAttribute(k_train_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM));
-    CK(cudaFuncSetAttribute(k_train_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, TF_SMEM));
+    CK(cudaFuncSetAttribute(k_train_grad<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM));
+    CK(cudaFuncSetAttribute(k_train_grad<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TF_SMEM));
 }
 
 void launch_mlp_infer(const uint32_t *packed, const float4 *feat, int n, int mode, float4 *lam0,
@@ -913,16 +901,17 @@ void launch_log_append(const float4 *feat, const float4 *lam, const int *pos, in
     CK(cudaGetLastError());
 }
 
-void launch_train_fwd(const TrainArgs &a, cudaStream_t s) {
-    k_train_fwd<<<(a.batch + TRAIN_TILE - 1) / TRAIN_TILE, TRAIN_TILE, TF_SMEM, s>>>(a);
+int train_blocks(int batch) { return (batch + TRAIN_TILE - 1) / TRAIN_TILE; }
+
+void launch_train_pack(const float *theta, uint32_t *packed, cudaStream_t s) {
+    k_train_pack<<<1, 1024, 0, s>>>(theta, packed);
     note_launch();
     CK(cudaGetLastError());
 }
 
-int train_wgrad_blocks(int batch) { return (batch + WGRAD_CHUNK - 1) / WGRAD_CHUNK; }
-
-void launch_train_wgrad(const TrainArgs &a, cudaStream_t s) {
-    k_train_wgrad<<<train_wgrad_blocks(a.batch), WGRAD_CHUNK, WG_SMEM, s>>>(a);
+void launch_train_grad(const TrainArgs &a, cudaStream_t s) {
+    if (a.backward) k_train_grad<true><<<train_blocks(a.batch), TRAIN_TILE, WG_SMEM, s>>>(a);
+    else k_train_grad<false><<<train_blocks(a.batch), TRAIN_TILE, TF_SMEM, s>>>(a);
     note_launch();
     CK(cudaGetLastError());
 }
@@ -938,11 +927,10 @@ void launch_train_reduce(const float *partials, int blocks, int batch, float *gr
 
 void launch_train_reduce_dev(const float *partials, int blocks, int batch, float *loss_hist,
                              float *theta, float *m, float *v, float lr, float beta1, float beta2,
-                             float eps, const float *c12, long long *step_dev, cudaStream_t s) {
-    k_train_reduce_dev<<<(MLP_N_PARAMS + 1 + 255) / 256, 256, 0, s>>>(
-        partials, blocks, batch, loss_hist, theta, m, v, lr, beta1, beta2, eps, c12, step_dev);
-    note_launch();
-    k_step_advance<<<1, 1, 0, s>>>(step_dev);
+                             float eps, const float *c12, uint32_t *packed, long long *step_dev, cudaStream_t s) {
+    k_train_reduce_dev<<<(MLP_N_PARAMS + 1 + 63) / 64, 64, 0, s>>>(
+        partials, blocks, batch, loss_hist, theta, m, v, lr, beta1, beta2, eps, c12, packed, step_dev,
+        reinterpret_cast<unsigned long long *>(step_dev + 1));
     note_launch();
     CK(cudaGetLastError());
 }

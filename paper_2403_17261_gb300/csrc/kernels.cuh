@@ -308,7 +308,7 @@ void launch_unpack_state(const float4 *st, int n, float *out13, cudaStream_t s);
 #define MLP_DEPTH_CAP 8
 #define MLP_N_PARAMS 5187
 #define MLP_PK_WORDS 3216      // BF16 tensor-core operands + FP32 biases
-#define MLP_ACT_STRIDE 276     // x 16, h1 64, h2 64, dz1 64, dz2 64, dy 4
+#define MLP_TRAIN_PK_WORDS 5632   // the same for training: W1^T, W2^T, W3^T, W3, W2
 struct FeatArgs {
     int np, nc, n;
     const int *ps_cons, *ps_part, *part_scene;
@@ -349,27 +349,30 @@ struct TrainArgs {
     const long long *step_dev;          // if set: the step counter in device memory (graph replay)
     int backward;                       // 0: loss only
     const float *theta;                 // FP32 master parameters
-    float *act;                         // [batch][MLP_ACT_STRIDE]
+    const uint32_t *packed;             // the same as BF16 operands (launch_train_pack, then every Adam step)
     float *sample_loss;                 // [batch]
     float *partials;                    // [blocks][MLP_N_PARAMS + 1]
     int *status;                        // set to DEV_ERR_TIMEOUT if a tensor-core wait gives up
 };
-void launch_train_fwd(const TrainArgs &a, cudaStream_t s);
-int train_wgrad_blocks(int batch);
+// forward pass and loss per sample (backward = 0), or also the backward pass
+// and the blocks' partial gradients
+void launch_train_grad(const TrainArgs &a, cudaStream_t s);
+void launch_train_pack(const float *theta, uint32_t *packed, cudaStream_t s);
+int train_blocks(int batch);
 // Function attributes of the network's kernels on `device`: once per context,
 // before any of their launches (outside graph capture).
 void mlp_kernels_setup(int device);
-void launch_train_wgrad(const TrainArgs &a, cudaStream_t s);
 // sums the partials in block order; grad_out (optional) gets the gradient and
 // loss_out[0] the mean loss; with adam != 0 also updates theta, m, v
 void launch_train_reduce(const float *partials, int blocks, int batch, float *grad_out,
                          float *loss_out, int adam, float *theta, float *m, float *v, float lr,
                          float beta1, float beta2, float eps, float c1, float c2, cudaStream_t s);
 // the same with the step taken from step_dev: loss to loss_hist[step], bias
-// corrections from c12[2 step], c12[2 step + 1]; then step_dev += 1
+// corrections from c12[2 step], c12[2 step + 1]; the new parameters packed;
+// then step_dev += 1 (step_dev[1]: scratch, zero between launches)
 void launch_train_reduce_dev(const float *partials, int blocks, int batch, float *loss_hist,
                              float *theta, float *m, float *v, float lr, float beta1, float beta2,
-                             float eps, const float *c12, long long *step_dev, cudaStream_t s);
+                             float eps, const float *c12, uint32_t *packed, long long *step_dev, cudaStream_t s);
 void launch_loss_sum(const float *sample_loss, int n, double *acc, cudaStream_t s);
 
 }  // namespace ovl

@@ -19,9 +19,9 @@ bool features_needed(const ovl_ctx *c) {
 }
 
 void ensure_train_buffers(ovl_ctx *c, int batch) {
-    c->train_act.ensure((size_t)batch * MLP_ACT_STRIDE);
+    c->train_packed.ensure(MLP_TRAIN_PK_WORDS);
     c->train_sample_loss.ensure((size_t)batch);
-    c->train_partials.ensure((size_t)train_wgrad_blocks(batch) * (MLP_N_PARAMS + 1));
+    c->train_partials.ensure((size_t)train_blocks(batch) * (MLP_N_PARAMS + 1));
     c->mlp_grad.ensure(MLP_N_PARAMS);
     c->mlp_loss.ensure(1);
 }
@@ -33,7 +33,7 @@ TrainArgs train_args(ovl_ctx *c, long long first, long long count, int batch, in
     a.first = first; a.count = count; a.batch = batch; a.sampling = sampling;
     a.seed = seed; a.step = step; a.backward = backward;
     a.theta = c->mlp_theta.p;
-    a.act = c->train_act.p; a.sample_loss = c->train_sample_loss.p;
+    a.packed = c->train_packed.p; a.sample_loss = c->train_sample_loss.p;
     a.partials = c->train_partials.p;
     a.status = c->status.p;
     return a;
@@ -94,7 +94,7 @@ void release_mlp(ovl_ctx *c) {
     c->feat.release(); c->is_contact.release(); c->contact_pos.release(); c->depth.release();
     c->mlp_theta.release(); c->mlp_m.release(); c->mlp_v.release(); c->mlp_grad.release();
     c->mlp_loss.release(); c->mlp_packed.release(); c->log_feat.release(); c->log_targ.release();
-    c->train_act.release(); c->train_sample_loss.release(); c->train_partials.release();
+    c->train_packed.release(); c->train_sample_loss.release(); c->train_partials.release();
     c->train_loss_hist.release(); c->infer_y.release(); c->infer_feat.release(); c->loss_acc.release();
     c->train_c12.release(); c->train_step.release();
 }
@@ -260,17 +260,17 @@ ovl_status ovl_mlp_train(ovl_ctx *c, const ovl_train_desc *d, float *loss_per_st
             c12[2 * t + 1] = (float)(1.0 / (1.0 - std::pow((double)b2, k)));
         }
         upload(c->train_c12, c12.data(), c12.size(), c->stream);
-        c->train_step.ensure(1);
-        CK(cudaMemsetAsync(c->train_step.p, 0, sizeof(long long), c->stream));
-        const int blocks = train_wgrad_blocks(d->batch);
+        c->train_step.ensure(2);
+        CK(cudaMemsetAsync(c->train_step.p, 0, 2 * sizeof(long long), c->stream));
+        launch_train_pack(c->mlp_theta.p, c->train_packed.p, c->stream);
+        const int blocks = train_blocks(d->batch);
         TrainArgs a = train_args(c, d->first, d->count, d->batch, d->sampling, d->seed, 0, 1);
         a.step_dev = c->train_step.p;
         auto one_step = [&](cudaStream_t st) {
-            launch_train_fwd(a, st);
-            launch_train_wgrad(a, st);
+            launch_train_grad(a, st);
             launch_train_reduce_dev(c->train_partials.p, blocks, d->batch, c->train_loss_hist.p,
                                     c->mlp_theta.p, c->mlp_m.p, c->mlp_v.p, lr, b1, b2, eps,
-                                    c->train_c12.p, c->train_step.p, st);
+                                    c->train_c12.p, c->train_packed.p, c->train_step.p, st);
         };
         constexpr int kGraphSteps = 50;
         int done = 0;
@@ -314,9 +314,9 @@ ovl_status ovl_mlp_grad(ovl_ctx *c, int64_t first, int64_t count, float *grad, d
         const int batch = (int)count;
         ensure_train_buffers(c, batch);
         TrainArgs a = train_args(c, first, count, batch, 0, 0, 0, 1);
-        launch_train_fwd(a, c->stream);
-        launch_train_wgrad(a, c->stream);
-        launch_train_reduce(c->train_partials.p, train_wgrad_blocks(batch), batch, c->mlp_grad.p,
+        launch_train_pack(c->mlp_theta.p, c->train_packed.p, c->stream);
+        launch_train_grad(a, c->stream);
+        launch_train_reduce(c->train_partials.p, train_blocks(batch), batch, c->mlp_grad.p,
                             c->mlp_loss.p, 0, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f,
                             c->stream);
         float l = 0.f;
@@ -336,10 +336,11 @@ ovl_status ovl_mlp_loss(ovl_ctx *c, int64_t first, int64_t count, double *loss) 
         ensure_train_buffers(c, kLossChunk);
         c->loss_acc.ensure(1);
         CK(cudaMemsetAsync(c->loss_acc.p, 0, sizeof(double), c->stream));
+        launch_train_pack(c->mlp_theta.p, c->train_packed.p, c->stream);
         for (long long off = 0; off < count; off += kLossChunk) {
             const int b = (int)std::min<long long>(kLossChunk, count - off);
             TrainArgs a = train_args(c, first + off, b, b, 0, 0, 0, 0);
-            launch_train_fwd(a, c->stream);
+            launch_train_grad(a, c->stream);
             launch_loss_sum(c->train_sample_loss.p, b, c->loss_acc.p, c->stream);
         }
         double acc = 0.0;
