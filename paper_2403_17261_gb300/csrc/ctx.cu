@@ -898,18 +898,18 @@ SolvePlan plan_solve(ovl_ctx *c, float dt_override, int iters) {
     return pl;
 }
 
-// The geodesic phase is 2 beta + 4 small launches whose arguments change only
+// The geodesic phase is beta + 4 small launches whose arguments change only
 // when a buffer is reallocated or the entry count changes, so it is captured
 // once as a CUDA graph and replayed while they stay the same.
 void enqueue_geodesics(ovl_ctx *c, cudaStream_t s) {
     CK(cudaMemsetAsync(c->visited.p, 0, sizeof(uint32_t) * ((size_t)((c->vb_bits + 31) / 32) + 1), s));
-    CK(cudaMemsetAsync(c->qctl.p, 0, sizeof(int) * ((size_t)c->beta_max + 4), s));
+    CK(cudaMemsetAsync(c->qctl.p, 0, sizeof(int) * 2 * ((size_t)c->beta_max + 4), s));
     fill_u8(c->D.p, 255, c->D.cap, s);   // the whole buffer: the graph then outlives entry counts
     GeoArgs a{};
     a.n = c->n; a.mask = c->mask.p; a.sob = c->sob.p; a.scene_beta = c->scene_beta.p;
     a.body_base = c->body_base.p; a.vb_base = c->vb_base.p; a.row_ptr = c->row_ptr.p; a.col = c->col.p;
     a.entry_ptr = c->entry_ptr.p; a.visited = c->visited.p; a.queue = c->queue.p; a.qctl = c->qctl.p;
-    a.D = c->D.p;
+    a.done = c->qctl.p + c->beta_max + 4; a.D = c->D.p;
     launch_geo_sources(a, s);
     for (int L = 1; L <= c->beta_max; ++L) launch_geo_level(a, L, s);
 }
@@ -919,7 +919,7 @@ void phase_geodesics(ovl_ctx *c, cudaStream_t s) {
     c->D.ensure(c->ne + 1);
     c->visited.ensure((size_t)((c->vb_bits + 31) / 32) + 1);
     c->queue.ensure((size_t)c->vb_bits + 1);
-    c->qctl.ensure((size_t)c->beta_max + 4);
+    c->qctl.ensure(2 * ((size_t)c->beta_max + 4));
     const std::vector<const void *> key = {
         c->D.p, c->visited.p, c->queue.p, c->qctl.p, c->mask.p, c->row_ptr.p, c->col.p,
         c->entry_ptr.p, c->sob.p, c->scene_beta.p, c->body_base.p, c->vb_base.p,

@@ -272,6 +272,7 @@ struct GeoArgs {
     uint32_t *visited;         // bitmap
     uint32_t *queue;           // (body << 6 | worker)
     int *qctl;                 // [0] = tail, [1 + L] = start of level L
+    int *done;                 // [L] blocks of the launch before level L that finished; all zeroed by the caller
     uint8_t *D;                // per entry
 };
 void launch_geo_sources(const GeoArgs &a, cudaStream_t s);
