@@ -345,7 +345,7 @@ bool solve_masses_fit(ovl_ctx *c, int slots, int ctas_per_sm) {
 // shape gives the same bits (no implicit FMA contraction in the solver),
 // so the plan changes only the time.  Returns false when some worker does
 // not fit even 8 CTAs (the uniform launch then takes it to global memory).
-struct SolveClass { int C, first, count, slots, rows; };
+struct SolveClass { int C, first, count, slots, rows; bool small; };
 
 // The growth leaves this many SMs unclaimed: clusters must fit inside one GPC,
 // so a launch that claims every SM can leave a cluster waiting for a second
@@ -420,22 +420,38 @@ std::vector<int> plan_worker_counts(ovl_ctx *c, int cap, long long budget) {
     return C;
 }
 
+// Where CTAs share SMs, one-CTA workers whose bodies and impulses take at most
+// a kSmallPerSm-th of an SM's shared memory form a class of their own with
+// kSmallThreads threads: the whole class's shared memory is its largest
+// worker's, which left two small workers on an SM that holds five (512 scenes:
+// solve 3.34 -> 2.91 ms; a third with 192 threads 3.40, an eighth with 64 2.91).
+constexpr int kSmallPerSm = 5, kSmallThreads = 128;
+
 // launch classes of a CTA-count plan: workers with equal counts, most CTAs
 // first and longest first inside; the worker order goes to buf
 void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveClass> &classes,
-                       DBuf<uint32_t> &buf) {
+                       DBuf<uint32_t> &buf, bool split) {
     const int P = c->n_parts;
     const std::vector<int> &pb = c->h_pb, &pp = c->h_pp;
     std::vector<int> order(P);
     std::iota(order.begin(), order.end(), 0);
+    std::vector<char> small(P, 0);
+    if (split)
+        for (int p = 0; p < P; ++p)
+            small[p] = C[p] == 1 && solve_smem_bytes(pb[p + 1] - pb[p], true) + 12 * (pp[p + 1] - pp[p]) + 16 <=
+                                        c->smem_per_sm / kSmallPerSm - 3584;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         if (C[x] != C[y]) return C[x] > C[y];
+        if (small[x] != small[y]) return small[x] < small[y];
         return pp[x + 1] - pp[x] > pp[y + 1] - pp[y];
     });
     classes.clear();
+    c->h_class_of.resize(P);
     for (int i = 0; i < P; ++i) {
         const int p = order[i], nb = pb[p + 1] - pb[p];
-        if (classes.empty() || classes.back().C != C[p]) classes.push_back({C[p], i, 0, 1, 0});
+        if (classes.empty() || classes.back().C != C[p] || classes.back().small != (bool)small[p])
+            classes.push_back({C[p], i, 0, 1, 0, (bool)small[p]});
+        c->h_class_of[p] = (int)classes.size() - 1;
         SolveClass &k = classes.back();
         k.count++;
         k.slots = std::max(k.slots, (nb + C[p] - 1) / C[p]);
@@ -452,7 +468,7 @@ bool plan_worker_classes(ovl_ctx *c, int cap, long long budget, std::vector<Solv
                          DBuf<uint32_t> &buf) {
     const std::vector<int> C = plan_worker_counts(c, cap, budget);
     if (C.empty() && c->n_parts > 0) return false;
-    plan_classes_from(c, C, classes, buf);
+    plan_classes_from(c, C, classes, buf, false);
     return true;
 }
 
@@ -490,7 +506,8 @@ bool plan_solve_classes(ovl_ctx *c, const SolveShape &shape, std::vector<SolveCl
     }
     const std::vector<int> C = plan_worker_counts(c, cap, budget);
     if (C.empty() && c->n_parts > 0) return false;
-    plan_classes_from(c, C, classes, c->class_order);
+    // contexts with boxes, and a slot limit, keep one shape
+    plan_classes_from(c, C, classes, c->class_order, shape.per_sm > 1 && !c->has_boxes && c->P.smem_slot_limit <= 0);
     return true;
 }
 
@@ -539,8 +556,8 @@ void launch_solve_classes(ovl_ctx *c, const SolveArgs &a, const SolveShape &shap
         b.order = c->class_order.p + classes[k].first;
         b.smem_slots = classes[k].slots;
         b.smem_rows = classes[k].rows;
-        launch_solve(b, shape.threads, classes[k].C, shape.unroll, solve_masses_fit(c, classes[k].slots, shape.per_sm),
-                     solve_smem_budget(c, shape.per_sm), sk);
+        launch_solve(b, classes[k].small ? kSmallThreads : shape.threads, classes[k].C, shape.unroll,
+                     solve_masses_fit(c, classes[k].slots, shape.per_sm), solve_smem_budget(c, shape.per_sm), sk);
     }, class_launch_order(c, classes));
 }
 
@@ -763,13 +780,11 @@ void apply_solve_order(ovl_ctx *c, const SolvePlan &pl) {
     if (pl.shape >= 0) C = c->h_class_C;
     upload(c->solve_C, C.data(), (size_t)P, c->stream);
     // which workers' launches keep the masses in shared memory (their rows
-    // take the packed form); the classes of a per-worker plan differ in C
+    // take the packed form)
     std::vector<int> M(P, 0);
     if (pl.shape >= 0) {
         const int per_sm = kSolveShapes[pl.shape].per_sm;
-        for (int p = 0; p < P; ++p)
-            for (const SolveClass &k : pl.classes)
-                if (k.C == C[p]) M[p] = solve_masses_fit(c, k.slots, per_sm) ? 1 : 0;
+        for (int p = 0; p < P; ++p) M[p] = solve_masses_fit(c, pl.classes[c->h_class_of[p]].slots, per_sm) ? 1 : 0;
     } else {
         std::fill(M.begin(), M.end(), solve_masses_fit(c, pl.slots, solve_ctas_per_sm(pl.unroll)) ? 1 : 0);
     }

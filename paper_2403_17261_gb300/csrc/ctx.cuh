@@ -105,6 +105,7 @@ struct ovl_ctx {
     std::vector<int> h_pb, h_pp;                 // part_bstart, part_pstart of this step on the host
     HBuf<int> h_starts;                          // both as the kernels write them
     std::vector<int> h_class_C;                  // CTAs per worker of the last per-worker plan
+    std::vector<int> h_class_of;                 // and its launch class
     DBuf<int> solve_C, solve_M, solve_banked, col_off2, pair_of_row2;   // solve: CTAs per worker, masses in shared memory, rows in bank order, rows by owner CTA
     DBuf<uint8_t> row_owner;                     // bucket of every row (scratch of the ordering)
     DBuf<int> row_by_owner;                      // rows by owner CTA (scratch of the ordering)
