@@ -212,10 +212,12 @@ void load_balance_range(const HostScene &sc, Membership &mem, const int2 *ab, in
             const int Bn = ab[i + kAhead].y;
             __builtin_prefetch(mem.mask_ptr() + Bn);
             __builtin_prefetch(row_ptr + Bn);
-            __builtin_prefetch(sc.sob.data() + ab[i + kAhead].x);
         }
         const int A = ab[i].x, B = ab[i].y;
         const uint64_t WA = mem.W(A), WB = mem.W(B);
+        // both in the same single worker, most contacts of a scene: no branch
+        // changes anything (the last would keep that worker in both)
+        if (WA == WB && !(WA & (WA - 1))) continue;
         const int scene = sc.sob[A];
         if ((WA & WB) == 0) {                                   // activation branch
             if (!do_activate) continue;
