@@ -249,12 +249,17 @@ __global__ void k_mlp_pack(const float *th, uint32_t *pk) {
     for (int e = threadIdx.x; e < 16; e += blockDim.x) bias[PK_B3 + e] = e < 3 ? th[OFF_B3 + e] : 0.f;
 }
 
+// float4 per row of the inference's input: the step's records of 16 words, or
+// (mode 0, rows from the caller) the 12 features alone
+template <int MODE>
+__device__ constexpr int infer_stride() { return MODE == 0 ? 3 : 4; }
+
 template <int MODE>
 __device__ __forceinline__ void infer_store(int r, int n, float y0, float y1, float y2,
                                             const float4 *feat, float4 *lam0, float *y3) {
     if (r >= n) return;
     // skip connection: features 4-6 (previous impulses / s), in FP32
-    const float4 f1 = feat[4 * (size_t)r + 1];
+    const float4 f1 = feat[infer_stride<MODE>() * (size_t)r + 1];
     y0 += f1.x; y1 += f1.y; y2 += f1.z;
     if (MODE == 0) {
         y3[3 * (size_t)r] = y0; y3[3 * (size_t)r + 1] = y1; y3[3 * (size_t)r + 2] = y2;
@@ -324,7 +329,7 @@ __global__ void __launch_bounds__(INFER_THREADS) k_mlp_infer(const uint32_t *pk,
 #pragma unroll
         for (int k = 0; k < 12; ++k) x[k] = 0.f;
         if (t < tiles && rr < n) {
-            const float4 *f = feat + 4 * (size_t)rr;
+            const float4 *f = feat + infer_stride<MODE>() * (size_t)rr;
             const float4 a = f[0], b = f[1], c = f[2];
             x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y;
             x[6] = b.z; x[7] = b.w; x[8] = c.x; x[9] = c.y; x[10] = c.z; x[11] = c.w;

@@ -330,7 +330,7 @@ void launch_depth(const uint64_t *mask, const int *row_ptr, const int *col, int 
                   cudaStream_t s);
 void launch_features(const FeatArgs &a, cudaStream_t s);
 void launch_mlp_pack(const float *theta, uint32_t *packed, cudaStream_t s);
-// mode 0: raw outputs to y3 [n][3]; 1: warm start of every contact into lam0;
+// mode 0: raw outputs to y3 [n][3] of feature rows [n][12]; 1: warm start of every contact into lam0;
 // 2: warm start of the contacts without previous impulses into lam0.  On the
 // tensor cores (tcgen05); a wait on them that gives up sets *status to
 // DEV_ERR_TIMEOUT.

@@ -169,10 +169,10 @@ ovl_status ovl_mlp_forward(ovl_ctx *c, int64_t n, const float *feat12, float *y3
         if (n < 0 || n > (int64_t)1 << 30 || (n > 0 && (!feat12 || !y3)))
             return fail(c, OVL_ERR_ARG, "bad size or null array");
         if (n == 0) return OVL_OK;
-        std::vector<float> rows(16 * (size_t)n, 0.f);
-        for (int64_t k = 0; k < n; ++k) std::memcpy(&rows[16 * k], feat12 + 12 * k, 12 * sizeof(float));
-        c->infer_feat.ensure(4 * (size_t)n);
-        CK(cudaMemcpyAsync(c->infer_feat.p, rows.data(), rows.size() * sizeof(float), cudaMemcpyHostToDevice, c->stream));
+        // the rows as the caller holds them: the kernel reads 48 B per row (a
+        // host pass that padded them to 64 B first took half of the call)
+        c->infer_feat.ensure(3 * (size_t)n);
+        CK(cudaMemcpyAsync(c->infer_feat.p, feat12, 12 * sizeof(float) * (size_t)n, cudaMemcpyHostToDevice, c->stream));
         c->infer_y.ensure(3 * (size_t)n);
         launch_mlp_infer(c->mlp_packed.p, c->infer_feat.p, (int)n, 0, nullptr, c->infer_y.p, 0, c->status.p, c->stream);
         download(y3, c->infer_y.p, 3 * (size_t)n, c->stream);
