@@ -55,9 +55,14 @@ struct DBuf {
     // device memory (cudaFree waits for the device)
     void ensure(size_t n) {
         if (n <= cap && p) return;
-        if (p) CK(cudaFree(p));
+        T *old = p;
+        p = nullptr;   // a call that fails leaves the buffer empty
+        cap = 0;
+        if (old) CK(cudaFree(old));
         size_t c = n < 16 ? 16 : 2 * n;
-        CK(cudaMalloc(&p, c * sizeof(T)));
+        T *fresh = nullptr;
+        CK(cudaMalloc(&fresh, c * sizeof(T)));
+        p = fresh;
         cap = c;
     }
     void release() {
@@ -74,9 +79,14 @@ struct HBuf {
     size_t cap = 0;
     void ensure(size_t n) {
         if (n <= cap && p) return;
-        if (p) CK(cudaFreeHost(p));
+        T *old = p;
+        p = nullptr;
+        cap = 0;
+        if (old) CK(cudaFreeHost(old));
         size_t c = n < 16 ? 16 : 2 * n;
-        CK(cudaMallocHost(&p, c * sizeof(T)));
+        T *fresh = nullptr;
+        CK(cudaMallocHost(&fresh, c * sizeof(T)));
+        p = fresh;
         cap = c;
     }
     void release() {
