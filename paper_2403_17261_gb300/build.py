@@ -44,7 +44,7 @@ def sources() -> list[str]:
 
 
 def _headers() -> list[str]:
-    return glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    return [f for d in (CSRC, INCLUDE) for e in ("*.cuh", "*.h") for f in glob.glob(os.path.join(d, e))]
 
 
 def up_to_date() -> bool:

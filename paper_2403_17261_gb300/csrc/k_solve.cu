@@ -1166,14 +1166,9 @@ __global__ void __launch_bounds__(SOLVE_THREADS, U == 1 ? 2 : 1) k_solve(SolveAr
 
 }  // namespace
 
-int solve_slot_bytes(bool masses) { return (int)(masses ? 2 * sizeof(float4) : sizeof(float4) + sizeof(float2)); }
-
-// a CTA's slots and its zero slot
-int solve_smem_bytes(int slots, bool masses) { return (slots + 1) * solve_slot_bytes(masses); }
-
 template <int C, int U, bool P, bool X>
 static void launch_solve_c(const SolveArgs &a, int threads, cudaStream_t s) {
-    int smem = solve_smem_bytes(a.smem_slots, false);
+    const int smem = (int)solve_smem_bytes(a.smem_slots, false);
     CK(cudaFuncSetAttribute(k_solve<C, U, P, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.n_parts * C);
@@ -1207,8 +1202,7 @@ template <int C, bool X>
 static void launch_solve_m(const SolveArgs &a, int threads, int budget, cudaStream_t s) {
     SolveArgs b = a;
     if (X) threads = std::min(threads, SOLVE_THREADS / 2);
-    b.smem_bytes = std::min(budget, solve_smem_bytes(a.smem_slots, true) + 12 * a.smem_rows + 16 +
-                                        (X ? 2 * FULL_ROW_WORDS * 16 * threads : 0));
+    b.smem_bytes = solve_dynamic_bytes(budget, a.smem_slots, a.smem_rows, X ? 2 * FULL_ROW_WORDS * 16 * threads : 0);
     CK(cudaFuncSetAttribute(k_solve_m<C, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.n_parts * C);

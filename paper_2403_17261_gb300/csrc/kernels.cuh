@@ -2,6 +2,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "solve_plan.h"
 
 namespace ovl {
 
@@ -255,8 +256,6 @@ struct SolveArgs {
 // budget: dynamic shared memory a CTA may take
 void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool masses, int budget, cudaStream_t s);
 int solve_ctas_per_sm(int unroll);
-int solve_slot_bytes(bool masses);              // bytes of one shared-memory body slot
-int solve_smem_bytes(int slots, bool masses);   // a CTA's slots plus its zero slot
 
 // ---- geodesics, weights, blend (k_blend.cu) --------------------------------
 struct GeoArgs {
