@@ -18,4 +18,15 @@ inline int solve_dynamic_bytes(int budget, long long slots, long long rows, long
     return (int)std::min<long long>(budget, solve_smem_bytes(slots, true) + 12 * rows + 16 + stage);
 }
 
+// Rows a CTA of a worker's group of C makes room for: its even share, plus a
+// quarter (and a little) for uneven owners.
+inline long long solve_cta_rows(long long np, int C) { return C == 1 ? np : (long long)(1.25 * np / C) + 64; }
+
+// the most of them over P workers, worker p's rows being [start[p], start[p + 1])
+inline long long solve_most_rows(const int *start, int P, int C) {
+    long long most = 0;
+    for (int p = 0; p < P; ++p) most = std::max(most, solve_cta_rows((long long)start[p + 1] - start[p], C));
+    return most;
+}
+
 }  // namespace ovl

@@ -15,6 +15,7 @@ extern "C" {
 int dynamic_bytes(int budget, long long slots, long long rows, long long stage) {
     return ovl::solve_dynamic_bytes(budget, slots, rows, stage);
 }
+long long most_rows(const int *start, int P, int C) { return ovl::solve_most_rows(start, P, C); }
 }
 """
 
@@ -31,6 +32,8 @@ def plan(tmp_path_factory):
     lib = ctypes.CDLL(str(so))
     L = ctypes.c_longlong
     lib.dynamic_bytes.argtypes = [ctypes.c_int, L, L, L]
+    lib.most_rows.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
+    lib.most_rows.restype = L
     return lib
 
 
@@ -43,3 +46,16 @@ def test_rows_beyond_32_bit_bytes_take_the_budget(plan, rows):
 def test_small_launches_take_what_they_need(plan):
     assert plan.dynamic_bytes(220_000, 99, 200, 0) == 100 * 32 + 200 * 12 + 16
     assert plan.dynamic_bytes(220_000, 99, 200, 65536) == 100 * 32 + 200 * 12 + 16 + 65536
+
+
+@pytest.mark.parametrize("rows,C,want", [
+    ([10], 1, 10),
+    ([10, 490, 10], 1, 490),                # the largest worker's rows, not the sum
+    ([10, 490, 10], 4, 153 + 64),
+    ([300] * 600, 1, 300),
+    ([0, 0], 2, 64),
+    ([], 1, 0),
+])
+def test_uniform_launch_makes_room_for_its_largest_worker(plan, rows, C, want):
+    start = (ctypes.c_int * (len(rows) + 1))(*[sum(rows[:i]) for i in range(len(rows) + 1)])
+    assert plan.most_rows(start, len(rows), C) == want
