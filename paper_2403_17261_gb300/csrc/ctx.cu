@@ -345,7 +345,7 @@ bool solve_masses_fit(ovl_ctx *c, int slots, int ctas_per_sm) {
 // shape gives the same bits (no implicit FMA contraction in the solver),
 // so the plan changes only the time.  Returns false when some worker does
 // not fit even 8 CTAs (the uniform launch then takes it to global memory).
-struct SolveClass { int C, first, count, slots, rows; bool small; };
+struct SolveClass { int C, first, count, slots; long long room; bool small; };
 
 // The growth leaves this many SMs unclaimed: clusters must fit inside one GPC,
 // so a launch that claims every SM can leave a cluster waiting for a second
@@ -425,6 +425,9 @@ std::vector<int> plan_worker_counts(ovl_ctx *c, int cap, long long budget) {
 // kSmallThreads threads: the whole class's shared memory is its largest
 // worker's, which left two small workers on an SM that holds five (512 scenes:
 // solve 3.34 -> 2.91 ms; a third with 192 threads 3.40, an eighth with 64 2.91).
+// The class asks for the most that one of its workers wants: its largest body
+// and row counts together belonged to no worker and left four CTAs on an SM
+// (2.95 -> 2.87 ms; 100 scenes of up to 2000 bodies 0.281 -> 0.290).
 constexpr int kSmallPerSm = 5, kSmallThreads = 128;
 
 // launch classes of a CTA-count plan: workers with equal counts, most CTAs
@@ -438,7 +441,7 @@ void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveC
     std::vector<char> small(P, 0);
     if (split)
         for (int p = 0; p < P; ++p)
-            small[p] = C[p] == 1 && solve_smem_bytes(pb[p + 1] - pb[p], true) + 12 * (pp[p + 1] - pp[p]) + 16 <=
+            small[p] = C[p] == 1 && solve_worker_room(pb[p + 1] - pb[p], pp[p + 1] - pp[p], 1) <=
                                         c->smem_per_sm / kSmallPerSm - 3584;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         if (C[x] != C[y]) return C[x] > C[y];
@@ -455,7 +458,7 @@ void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveC
         SolveClass &k = classes.back();
         k.count++;
         k.slots = std::max(k.slots, (nb + C[p] - 1) / C[p]);
-        k.rows = std::max(k.rows, (int)solve_cta_rows(pp[p + 1] - pp[p], C[p]));
+        k.room = std::max(k.room, solve_worker_room(nb, pp[p + 1] - pp[p], C[p]));
     }
     std::vector<uint32_t> o(order.begin(), order.end());
     upload(buf, o.data(), o.size(), c->stream);
@@ -553,7 +556,7 @@ void launch_solve_classes(ovl_ctx *c, const SolveArgs &a, const SolveShape &shap
         b.n_parts = classes[k].count;
         b.order = c->class_order.p + classes[k].first;
         b.smem_slots = classes[k].slots;
-        b.smem_rows = classes[k].rows;
+        b.smem_room = classes[k].room;
         launch_solve(b, classes[k].small ? kSmallThreads : shape.threads, classes[k].C, shape.unroll,
                      solve_masses_fit(c, classes[k].slots, shape.per_sm), solve_smem_budget(c, shape.per_sm), sk);
     }, class_launch_order(c, classes));
@@ -826,7 +829,7 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
     // the largest worker's rows, not all workers': many small workers then
     // share an SM (600 scenes of two workers: solve 0.60 -> 0.27 ms with 64
     // threads per CTA, 0.55 -> 0.32 with 128)
-    a.smem_rows = (int)solve_most_rows(c->h_pp.data(), P, pl.cluster);
+    a.smem_room = solve_most_room(c->h_pb.data(), c->h_pp.data(), P, pl.cluster);
     launch_solve(a, pl.threads, pl.cluster, pl.unroll, masses, solve_smem_budget(c, solve_ctas_per_sm(pl.unroll)), c->stream);
     c->last_ctas = (long long)pl.cluster * P;
     c->last_ctas_masses = masses ? c->last_ctas : 0;

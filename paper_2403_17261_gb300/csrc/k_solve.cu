@@ -1202,7 +1202,7 @@ template <int C, bool X>
 static void launch_solve_m(const SolveArgs &a, int threads, int budget, cudaStream_t s) {
     SolveArgs b = a;
     if (X) threads = std::min(threads, SOLVE_THREADS / 2);
-    b.smem_bytes = solve_dynamic_bytes(budget, a.smem_slots, a.smem_rows, X ? 2 * FULL_ROW_WORDS * 16 * threads : 0);
+    b.smem_bytes = solve_dynamic_bytes(budget, a.smem_room, X ? 2 * FULL_ROW_WORDS * 16 * threads : 0);
     CK(cudaFuncSetAttribute(k_solve_m<C, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.n_parts * C);

@@ -239,7 +239,7 @@ struct SolveArgs {
     float4 *scratch;           // [ne] float4 + [ne] float2: velocities of workers too large for shared memory
     int iters;
     int smem_slots;
-    int smem_rows;             // room asked for: rows per CTA whose impulses are kept in shared memory
+    long long smem_room;       // bytes wanted for a CTA's slots and its rows' impulses (launches with the masses)
     int smem_bytes;            // dynamic shared memory of the launch
     int flags;                 // OVL_FLAG_*
     float res_tol;

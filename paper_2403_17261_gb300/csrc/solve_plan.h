@@ -11,22 +11,30 @@ constexpr int solve_slot_bytes(bool masses) { return masses ? 32 : 24; }
 // a CTA's slots and its zero slot
 constexpr long long solve_smem_bytes(long long slots, bool masses) { return (slots + 1) * solve_slot_bytes(masses); }
 
-// the dynamic shared memory a CTA of the launch with the masses asks for:
-// slots, the impulses of its rows (12 B each, padded to 16) and `stage` bytes,
-// as far as the budget goes.  64-bit: a worker may have more rows than 32-bit bytes.
-inline int solve_dynamic_bytes(int budget, long long slots, long long rows, long long stage) {
-    return (int)std::min<long long>(budget, solve_smem_bytes(slots, true) + 12 * rows + 16 + stage);
-}
-
 // Rows a CTA of a worker's group of C makes room for: its even share, plus a
 // quarter (and a little) for uneven owners.
 inline long long solve_cta_rows(long long np, int C) { return C == 1 ? np : (long long)(1.25 * np / C) + 64; }
 
-// the most of them over P workers, worker p's rows being [start[p], start[p + 1])
-inline long long solve_most_rows(const int *start, int P, int C) {
+// Shared memory a CTA of the launch with the masses wants for a worker of nb
+// bodies and np rows: slots and the impulses of its rows (12 B each, padded to
+// 16).  64-bit: a worker may have more rows than 32-bit bytes.
+inline long long solve_worker_room(int nb, long long np, int C) {
+    return solve_smem_bytes((nb + C - 1) / C, true) + 12 * solve_cta_rows(np, C) + 16;
+}
+
+// The most of it over P workers, bodies and rows of worker p from b[p] and
+// q[p] on.  The worker with the most bodies is seldom the one with the most
+// rows (a chain has one row per body, a pile three), so the maximum is taken
+// over workers, not over bodies and rows apart.
+inline long long solve_most_room(const int *b, const int *q, int P, int C) {
     long long most = 0;
-    for (int p = 0; p < P; ++p) most = std::max(most, solve_cta_rows((long long)start[p + 1] - start[p], C));
+    for (int p = 0; p < P; ++p) most = std::max(most, solve_worker_room(b[p + 1] - b[p], (long long)q[p + 1] - q[p], C));
     return most;
+}
+
+// the dynamic shared memory of that launch: the room and `stage` bytes, as far as the budget goes
+inline int solve_dynamic_bytes(int budget, long long room, long long stage) {
+    return (int)std::min<long long>(budget, room + stage);
 }
 
 }  // namespace ovl

@@ -13,9 +13,9 @@ EXPORTS = r"""
 #include "csrc/solve_plan.h"
 extern "C" {
 int dynamic_bytes(int budget, long long slots, long long rows, long long stage) {
-    return ovl::solve_dynamic_bytes(budget, slots, rows, stage);
+    return ovl::solve_dynamic_bytes(budget, ovl::solve_worker_room((int)slots, rows, 1), stage);
 }
-long long most_rows(const int *start, int P, int C) { return ovl::solve_most_rows(start, P, C); }
+long long most_room(const int *b, const int *q, int P, int C) { return ovl::solve_most_room(b, q, P, C); }
 }
 """
 
@@ -32,8 +32,8 @@ def plan(tmp_path_factory):
     lib = ctypes.CDLL(str(so))
     L = ctypes.c_longlong
     lib.dynamic_bytes.argtypes = [ctypes.c_int, L, L, L]
-    lib.most_rows.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
-    lib.most_rows.restype = L
+    lib.most_room.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
+    lib.most_room.restype = L
     return lib
 
 
@@ -48,14 +48,33 @@ def test_small_launches_take_what_they_need(plan):
     assert plan.dynamic_bytes(220_000, 99, 200, 65536) == 100 * 32 + 200 * 12 + 16 + 65536
 
 
+def _starts(counts):
+    return (ctypes.c_int * (len(counts) + 1))(*[sum(counts[:i]) for i in range(len(counts) + 1)])
+
+
+def _room(plan, bodies, rows, C):
+    return plan.most_room(_starts(bodies), _starts(rows), len(rows), C)
+
+
 @pytest.mark.parametrize("rows,C,want", [
     ([10], 1, 10),
     ([10, 490, 10], 1, 490),                # the largest worker's rows, not the sum
     ([10, 490, 10], 4, 153 + 64),
     ([300] * 600, 1, 300),
     ([0, 0], 2, 64),
-    ([], 1, 0),
 ])
 def test_uniform_launch_makes_room_for_its_largest_worker(plan, rows, C, want):
-    start = (ctypes.c_int * (len(rows) + 1))(*[sum(rows[:i]) for i in range(len(rows) + 1)])
-    assert plan.most_rows(start, len(rows), C) == want
+    assert _room(plan, [0] * len(rows), rows, C) == 32 + 12 * want + 16
+
+
+@pytest.mark.parametrize("bodies,rows,C,want", [
+    ([974, 300], [300, 1900], 1, (974 + 1) * 32 + 12 * 300 + 16),       # not 974 bodies with 1900 rows
+    ([300, 200], [300, 1900], 1, (200 + 1) * 32 + 12 * 1900 + 16),
+    ([301, 10], [100, 20], 2, (151 + 1) * 32 + 12 * (62 + 64) + 16),
+])
+def test_room_is_one_workers(plan, bodies, rows, C, want):
+    assert _room(plan, bodies, rows, C) == want
+
+
+def test_no_workers_want_no_room(plan):
+    assert plan.most_room(_starts([]), _starts([]), 0, 1) == 0
