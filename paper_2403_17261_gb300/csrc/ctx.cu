@@ -316,25 +316,21 @@ void colour_config(ovl_ctx *c, int *cluster, int *slots) {
     *slots = cap;
 }
 
-// Dynamic shared memory a solver CTA may use with 1 or 2 resident CTAs per SM
-// (the solver's static shared memory -- row-bucket offsets, reductions -- takes
-// up to 2.2 KB, the system 1 KB per CTA)
-int solve_smem_budget(ovl_ctx *c, int ctas_per_sm) {
-    return ctas_per_sm == 1 ? c->smem_optin - 2560 : (c->smem_per_sm / 2) - 3584;
+int solve_smem_budget(const ovl_ctx *c, int ctas_per_sm, bool masses) {
+    return ovl::solve_smem_budget(c->smem_optin, c->smem_per_sm, ctas_per_sm, masses);
 }
 
 // Shared-memory body slots per CTA (24 B each, the layout without masses: the
-// CTA counts are planned with it, so adding the masses never adds CTAs), less
-// the CTA's zero slot
-int solve_slot_capacity(ovl_ctx *c, int ctas_per_sm) {
-    int n = std::max(0, solve_smem_budget(c, ctas_per_sm) / solve_slot_bytes(false) - 1);
+// CTA counts are planned with it, so adding the masses never adds CTAs)
+int solve_slot_capacity(const ovl_ctx *c, int ctas_per_sm) {
+    const int n = ovl::solve_slot_capacity(c->smem_optin, c->smem_per_sm, ctas_per_sm, false);
     return c->P.smem_slot_limit > 0 ? std::min(n, c->P.smem_slot_limit) : n;
 }
 
 // a launch keeps the masses in shared memory (32 B per slot) when its slots
 // still fit that way
-bool solve_masses_fit(ovl_ctx *c, int slots, int ctas_per_sm) {
-    return c->P.smem_slot_limit <= 0 && solve_smem_bytes(slots, true) <= solve_smem_budget(c, ctas_per_sm);
+bool solve_masses_fit(const ovl_ctx *c, int slots, int ctas_per_sm) {
+    return c->P.smem_slot_limit <= 0 && solve_smem_bytes(slots, true) <= solve_smem_budget(c, ctas_per_sm, true);
 }
 
 // Per-worker CTA counts for the default launch: every worker starts at the
@@ -501,7 +497,7 @@ bool plan_solve_classes(ovl_ctx *c, const SolveShape &shape, std::vector<SolveCl
     const int cap_plain = solve_slot_capacity(c, shape.per_sm);
     int cap = cap_plain;
     if (c->P.smem_slot_limit <= 0) {
-        const int cap_m = solve_smem_budget(c, shape.per_sm) / solve_slot_bytes(true) - 1;
+        const int cap_m = ovl::solve_slot_capacity(c->smem_optin, c->smem_per_sm, shape.per_sm, true);
         const long long with_m = fewest_ctas(c, cap_m), plain = fewest_ctas(c, cap_plain);
         if (with_m > 0 && (with_m <= slots || plain < 0 || plain > 2 * slots)) cap = cap_m;
     }
@@ -558,7 +554,7 @@ void launch_solve_classes(ovl_ctx *c, const SolveArgs &a, const SolveShape &shap
         b.smem_slots = classes[k].slots;
         b.smem_room = classes[k].room;
         launch_solve(b, classes[k].small ? kSmallThreads : shape.threads, classes[k].C, shape.unroll,
-                     solve_masses_fit(c, classes[k].slots, shape.per_sm), solve_smem_budget(c, shape.per_sm), sk);
+                     solve_masses_fit(c, classes[k].slots, shape.per_sm), solve_smem_budget(c, shape.per_sm, true), sk);
     }, class_launch_order(c, classes));
 }
 
@@ -830,7 +826,7 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
     // share an SM (600 scenes of two workers: solve 0.60 -> 0.27 ms with 64
     // threads per CTA, 0.55 -> 0.32 with 128)
     a.smem_room = solve_most_room(c->h_pb.data(), c->h_pp.data(), P, pl.cluster);
-    launch_solve(a, pl.threads, pl.cluster, pl.unroll, masses, solve_smem_budget(c, solve_ctas_per_sm(pl.unroll)), c->stream);
+    launch_solve(a, pl.threads, pl.cluster, pl.unroll, masses, solve_smem_budget(c, solve_ctas_per_sm(pl.unroll), true), c->stream);
     c->last_ctas = (long long)pl.cluster * P;
     c->last_ctas_masses = masses ? c->last_ctas : 0;
     c->last_cluster = pl.cluster;

@@ -253,7 +253,7 @@ struct SolveArgs {
 };
 // masses: the shared-memory slots hold the inverse masses and inertias (32 B
 // per slot; contact rows read as two records); else 24 B per slot
-// budget: dynamic shared memory a CTA may take
+// budget: dynamic shared memory a CTA may take with the masses
 void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool masses, int budget, cudaStream_t s);
 int solve_ctas_per_sm(int unroll);
 

@@ -11,6 +11,20 @@ constexpr int solve_slot_bytes(bool masses) { return masses ? 32 : 24; }
 // a CTA's slots and its zero slot
 constexpr long long solve_smem_bytes(long long slots, bool masses) { return (slots + 1) * solve_slot_bytes(masses); }
 
+// Dynamic shared memory a CTA may use with one resident CTA per SM (of the
+// `optin` bytes a block may have) or two (of the SM's `per_sm`, less 1 KB that
+// the system takes per block), beside its static memory: 1.8 KB of row-bucket
+// offsets and reductions without the masses, 2.2 KB with them.
+inline int solve_smem_budget(int optin, int per_sm, int ctas_per_sm, bool masses) {
+    const int fixed = masses ? 2560 : 2048;
+    return ctas_per_sm == 1 ? optin - fixed : per_sm / 2 - 1024 - fixed;
+}
+
+// body slots of that memory, less the CTA's zero slot
+inline int solve_slot_capacity(int optin, int per_sm, int ctas_per_sm, bool masses) {
+    return std::max(0, solve_smem_budget(optin, per_sm, ctas_per_sm, masses) / solve_slot_bytes(masses) - 1);
+}
+
 // Rows a CTA of a worker's group of C makes room for: its even share, plus a
 // quarter (and a little) for uneven owners.
 inline long long solve_cta_rows(long long np, int C) { return C == 1 ? np : (long long)(1.25 * np / C) + 64; }

@@ -15,6 +15,7 @@ extern "C" {
 int dynamic_bytes(int budget, long long slots, long long rows, long long stage) {
     return ovl::solve_dynamic_bytes(budget, ovl::solve_worker_room((int)slots, rows, 1), stage);
 }
+int slot_capacity(int optin, int per_sm, int ctas, int masses) { return ovl::solve_slot_capacity(optin, per_sm, ctas, masses); }
 long long most_room(const int *b, const int *q, int P, int C) { return ovl::solve_most_room(b, q, P, C); }
 }
 """
@@ -78,3 +79,16 @@ def test_room_is_one_workers(plan, bodies, rows, C, want):
 
 def test_no_workers_want_no_room(plan):
     assert plan.most_room(_starts([]), _starts([]), 0, 1) == 0
+
+
+@pytest.mark.parametrize("ctas,masses,static", [(1, 0, 1808), (2, 0, 1808), (1, 1, 2192), (2, 1, 2192)])
+def test_slots_fill_the_shared_memory(plan, ctas, masses, static):
+    """static: the kernels' own (ptxas -v).  One more KB of slots would not fit beside it."""
+    optin, per_sm, system = 232448, 233472, 1024
+    slot = 32 if masses else 24
+    used = (plan.slot_capacity(optin, per_sm, ctas, masses) + 1) * slot + static
+    most = optin if ctas == 1 else per_sm // 2 - system
+    assert used <= most
+    assert used + 1024 > most
+    # the layout without the masses gives nothing to the other kernel's tables
+    assert masses or used + 256 > most - 15
