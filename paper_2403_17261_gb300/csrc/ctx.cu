@@ -341,7 +341,7 @@ bool solve_masses_fit(const ovl_ctx *c, int slots, int ctas_per_sm) {
 // shape gives the same bits (no implicit FMA contraction in the solver),
 // so the plan changes only the time.  Returns false when some worker does
 // not fit even 8 CTAs (the uniform launch then takes it to global memory).
-struct SolveClass { int C, first, count, slots; long long room; bool small; };
+struct SolveClass { int C, first, count, slots; long long room; bool small, masses; };
 
 // The growth leaves this many SMs unclaimed: clusters must fit inside one GPC,
 // so a launch that claims every SM can leave a cluster waiting for a second
@@ -449,7 +449,7 @@ void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveC
     for (int i = 0; i < P; ++i) {
         const int p = order[i], nb = pb[p + 1] - pb[p];
         if (classes.empty() || classes.back().C != C[p] || classes.back().small != (bool)small[p])
-            classes.push_back({C[p], i, 0, 1, 0, (bool)small[p]});
+            classes.push_back({C[p], i, 0, 1, 0, (bool)small[p], false});
         c->h_class_of[p] = (int)classes.size() - 1;
         SolveClass &k = classes.back();
         k.count++;
@@ -505,6 +505,10 @@ bool plan_solve_classes(ovl_ctx *c, const SolveShape &shape, std::vector<SolveCl
     if (C.empty() && c->n_parts > 0) return false;
     // contexts with boxes, and a slot limit, keep one shape
     plan_classes_from(c, C, classes, c->class_order, shape.per_sm > 1 && !c->has_boxes && c->P.smem_slot_limit <= 0);
+    const long long ctas = std::accumulate(C.begin(), C.end(), 0ll);
+    for (SolveClass &k : classes)
+        k.masses = solve_masses_fit(c, k.slots, shape.per_sm) &&
+                   (shape.unroll == 2 || c->has_boxes || solve_takes_masses(shape.threads, ctas, c->num_sms, c->smem_per_sm, k.slots));
     return true;
 }
 
@@ -554,7 +558,7 @@ void launch_solve_classes(ovl_ctx *c, const SolveArgs &a, const SolveShape &shap
         b.smem_slots = classes[k].slots;
         b.smem_room = classes[k].room;
         launch_solve(b, classes[k].small ? kSmallThreads : shape.threads, classes[k].C, shape.unroll,
-                     solve_masses_fit(c, classes[k].slots, shape.per_sm), solve_smem_budget(c, shape.per_sm, true), sk);
+                     classes[k].masses, solve_smem_budget(c, shape.per_sm, true), sk);
     }, class_launch_order(c, classes));
 }
 
@@ -768,6 +772,14 @@ struct SolvePlan {
     int cluster = 1, threads = 512, unroll = 1, slots = 0;
 };
 
+// whether a uniform launch keeps the masses in shared memory (the kernels of
+// contexts with boxes have registers for one CTA per SM either way)
+bool uniform_masses(const ovl_ctx *c, const SolvePlan &pl) {
+    return solve_masses_fit(c, pl.slots, solve_ctas_per_sm(pl.unroll)) &&
+           (pl.unroll == 2 || c->has_boxes ||
+            solve_takes_masses(pl.threads, (long long)pl.cluster * c->n_parts, c->num_sms, c->smem_per_sm, pl.slots));
+}
+
 // Every worker's CTA count goes to the device and the rows of every colour
 // are regrouped by the CTA that owns them (it holds the row's first dynamic
 // body); the row build then follows that order.
@@ -780,10 +792,9 @@ void apply_solve_order(ovl_ctx *c, const SolvePlan &pl) {
     // take the packed form)
     std::vector<int> M(P, 0);
     if (pl.shape >= 0) {
-        const int per_sm = kSolveShapes[pl.shape].per_sm;
-        for (int p = 0; p < P; ++p) M[p] = solve_masses_fit(c, pl.classes[c->h_class_of[p]].slots, per_sm) ? 1 : 0;
+        for (int p = 0; p < P; ++p) M[p] = pl.classes[c->h_class_of[p]].masses ? 1 : 0;
     } else {
-        std::fill(M.begin(), M.end(), solve_masses_fit(c, pl.slots, solve_ctas_per_sm(pl.unroll)) ? 1 : 0);
+        std::fill(M.begin(), M.end(), uniform_masses(c, pl) ? 1 : 0);
     }
     upload(c->solve_M, M.data(), (size_t)P, c->stream);
     // the bank order is for k_solve_m's rows
@@ -811,7 +822,7 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
         launch_solve_classes(c, a, kSolveShapes[pl.shape], pl.classes);
         for (const SolveClass &k : pl.classes) {
             c->last_ctas += (long long)k.C * k.count;
-            if (solve_masses_fit(c, k.slots, kSolveShapes[pl.shape].per_sm)) c->last_ctas_masses += (long long)k.C * k.count;
+            if (k.masses) c->last_ctas_masses += (long long)k.C * k.count;
         }
         c->last_cluster = pl.classes.front().C;
         c->last_plan_per_worker = true;
@@ -821,7 +832,7 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
     }
     a.smem_slots = pl.slots;
     a.order = uniform_order(c);
-    const bool masses = solve_masses_fit(c, pl.slots, solve_ctas_per_sm(pl.unroll));
+    const bool masses = uniform_masses(c, pl);
     // the largest worker's rows, not all workers': many small workers then
     // share an SM (600 scenes of two workers: solve 0.60 -> 0.27 ms with 64
     // threads per CTA, 0.55 -> 0.32 with 128)

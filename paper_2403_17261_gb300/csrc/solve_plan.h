@@ -51,4 +51,20 @@ inline int solve_dynamic_bytes(int budget, long long room, long long stage) {
     return (int)std::min<long long>(budget, room + stage);
 }
 
+// Whether a launch of one row per thread whose slots fit with the masses takes
+// the kernel that keeps them and the impulses in shared memory (k_solve_m).
+// Its 91 to 124 registers leave an SM 512 / threads CTAs; the kernel without
+// them has 64 and leaves twice as many, if its slots fit that often and there
+// are CTAs enough.  The launch gives the masses up only where the other kernel
+// runs twice as many CTAs at once: a row costs it about 15 % more.  (Solves,
+// ms, with and without: 1200 small workers with 256 threads 0.54 and 0.30,
+// with 512 threads 0.99 and 0.53, two CTAs each 3.66 and 2.52; 64 workers of
+// eight 512-thread CTAs 2.43 and 1.50, larger ones 4.55 and 3.83; of eight
+// 256-thread CTAs, two or three of which share an SM, 3.55 and 3.87.)
+inline bool solve_takes_masses(int threads, long long ctas, int sms, int per_sm, long long slots) {
+    const long long other = std::min<long long>(std::max(1, 1024 / threads),
+                                                std::max(1ll, per_sm / (solve_smem_bytes(slots, false) + 3072)));
+    return 2 * std::max(1, 512 / threads) > std::min(other, (ctas + sms - 1) / sms);
+}
+
 }  // namespace ovl

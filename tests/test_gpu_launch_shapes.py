@@ -1,0 +1,47 @@
+"""Launches whose CTAs share an SM: the kernel they take and that it computes
+the same bits."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _batch(n_scenes, iters=8):
+    """small piles of uneven sizes, two workers each"""
+    from paper_2403_17261_gb300 import scenes as S
+    rng = S.SplitMix64(3)
+    parts = []
+    for k in range(n_scenes):
+        side = 2 + k % 5
+        pos = S._lattice_pile(side, side, 3, 1.0, 0.5, 0.01, rng)
+        n = pos.shape[0]
+        parts.append(S._single(f"p{k}", pos, np.full(n, 0.5), np.ones(n), [[0, 0, 1, 0]], mu=0.5, dt=1 / 60, flags=1, gamma=1,
+                               beta=4, n_sets=2, set_of_body=(np.arange(n) * 2) // n))
+    sc = S.concat_scenes("batch", parts, iters=iters)
+    sc.state[:, 7:13] = rng.uniform(6 * sc.n_bodies, -0.3, 0.3).reshape(-1, 6).astype(np.float32)
+    return sc
+
+
+def _run(sc, par, steps=2):
+    from paper_2403_17261_gb300 import ovl
+    sim = ovl.Simulation(sc, par)
+    for _ in range(steps):
+        sim.step()
+    out, st = sim.state(), sim.stats()
+    sim.close()
+    return out.view(np.uint32), st
+
+
+@pytest.mark.parametrize("par,masses", [
+    (dict(pgs_cluster=1), False),                     # 512 threads: twice as many CTAs without the masses
+    (dict(pgs_cluster=2), False),
+    (dict(pgs_threads=256), False),
+    (dict(pgs_cluster=1, pgs_threads=32), True),      # registers for all that are there
+])
+def test_shared_sms(par, masses):
+    sc = _batch(350)
+    ref, st = _run(sc, {})
+    assert st["solve_ctas_masses"] == st["solve_ctas"]
+    out, st = _run(sc, par)
+    assert np.array_equal(out, ref)
+    assert st["solve_ctas_masses"] == (st["solve_ctas"] if masses else 0)

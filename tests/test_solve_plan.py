@@ -15,6 +15,9 @@ extern "C" {
 int dynamic_bytes(int budget, long long slots, long long rows, long long stage) {
     return ovl::solve_dynamic_bytes(budget, ovl::solve_worker_room((int)slots, rows, 1), stage);
 }
+int takes_masses(int threads, long long ctas, int sms, int per_sm, long long slots) {
+    return ovl::solve_takes_masses(threads, ctas, sms, per_sm, slots);
+}
 int slot_capacity(int optin, int per_sm, int ctas, int masses) { return ovl::solve_slot_capacity(optin, per_sm, ctas, masses); }
 long long most_room(const int *b, const int *q, int P, int C) { return ovl::solve_most_room(b, q, P, C); }
 }
@@ -33,6 +36,7 @@ def plan(tmp_path_factory):
     lib = ctypes.CDLL(str(so))
     L = ctypes.c_longlong
     lib.dynamic_bytes.argtypes = [ctypes.c_int, L, L, L]
+    lib.takes_masses.argtypes = [ctypes.c_int, L, ctypes.c_int, ctypes.c_int, L]
     lib.most_room.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
     lib.most_room.restype = L
     return lib
@@ -92,3 +96,21 @@ def test_slots_fill_the_shared_memory(plan, ctas, masses, static):
     assert used + 1024 > most
     # the layout without the masses gives nothing to the other kernel's tables
     assert masses or used + 256 > most - 15
+
+
+@pytest.mark.parametrize("threads,ctas,slots,masses", [
+    (512, 152, 200, 1),          # every CTA has an SM of its own
+    (512, 153, 200, 0),          # two per SM: the registers leave one
+    (512, 153, 4600, 0),
+    (512, 153, 8000, 1),         # but the slots leave one too
+    (256, 1200, 200, 0),
+    (256, 512, 3500, 1),         # two per SM, by registers and by slots
+    (256, 512, 2500, 1),         # two and three
+    (256, 512, 2000, 0),         # two and four
+    (128, 152 * 7, 200, 1),
+    (128, 152 * 7 + 1, 200, 0),
+    (32, 152 * 16, 20, 1),
+    (1024, 100, 200, 1),
+])
+def test_ctas_that_share_an_sm_find_registers(plan, threads, ctas, slots, masses):
+    assert plan.takes_masses(threads, ctas, 152, 233472, slots) == masses
