@@ -549,6 +549,12 @@ void run_on_streams(ovl_ctx *c, size_t n, F &&launch, const std::vector<size_t> 
     }
 }
 
+// threads of a class's CTAs
+int class_threads(const ovl_ctx *c, const SolveShape &shape, const SolveClass &k) {
+    if (k.small) return kSmallThreads;
+    return c->has_boxes && k.masses ? solve_box_threads(shape.threads, shape.per_sm) : shape.threads;
+}
+
 void launch_solve_classes(ovl_ctx *c, const SolveArgs &a, const SolveShape &shape,
                           const std::vector<SolveClass> &classes) {
     run_on_streams(c, classes.size(), [&](size_t k, cudaStream_t sk) {
@@ -557,8 +563,8 @@ void launch_solve_classes(ovl_ctx *c, const SolveArgs &a, const SolveShape &shap
         b.order = c->class_order.p + classes[k].first;
         b.smem_slots = classes[k].slots;
         b.smem_room = classes[k].room;
-        launch_solve(b, classes[k].small ? kSmallThreads : shape.threads, classes[k].C, shape.unroll,
-                     classes[k].masses, solve_smem_budget(c, shape.per_sm, true), sk);
+        launch_solve(b, class_threads(c, shape, classes[k]), classes[k].C, shape.unroll, classes[k].masses,
+                     solve_smem_budget(c, shape.per_sm, true), sk);
     }, class_launch_order(c, classes));
 }
 
@@ -780,6 +786,11 @@ bool uniform_masses(const ovl_ctx *c, const SolvePlan &pl) {
             solve_takes_masses(pl.threads, (long long)pl.cluster * c->n_parts, c->num_sms, c->smem_per_sm, pl.slots));
 }
 
+// threads of a uniform launch's CTAs
+int uniform_threads(const ovl_ctx *c, const SolvePlan &pl, bool masses) {
+    return c->has_boxes && masses ? solve_box_threads(pl.threads, solve_ctas_per_sm(pl.unroll)) : pl.threads;
+}
+
 // Every worker's CTA count goes to the device and the rows of every colour
 // are regrouped by the CTA that owns them (it holds the row's first dynamic
 // body); the row build then follows that order.
@@ -837,7 +848,8 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
     // share an SM (600 scenes of two workers: solve 0.60 -> 0.27 ms with 64
     // threads per CTA, 0.55 -> 0.32 with 128)
     a.smem_room = solve_most_room(c->h_pb.data(), c->h_pp.data(), P, pl.cluster);
-    launch_solve(a, pl.threads, pl.cluster, pl.unroll, masses, solve_smem_budget(c, solve_ctas_per_sm(pl.unroll), true), c->stream);
+    launch_solve(a, uniform_threads(c, pl, masses), pl.cluster, pl.unroll, masses,
+                 solve_smem_budget(c, solve_ctas_per_sm(pl.unroll), true), c->stream);
     c->last_ctas = (long long)pl.cluster * P;
     c->last_ctas_masses = masses ? c->last_ctas : 0;
     c->last_cluster = pl.cluster;

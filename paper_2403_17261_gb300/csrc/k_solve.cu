@@ -1056,7 +1056,8 @@ __device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM 
 // and words one after the other, made a colour step 1.4 us (building 2.93 ms,
 // bridge 1.13); with the impulses in shared memory and the words a colour
 // ahead it takes 0.75 us (1.59 and 0.62 ms).  256 threads: the stages take
-// 512 B per thread.
+// 512 B per thread.  (Registers bounded to 128, for two such CTAs per SM,
+// cost clusters 4 to 15 %: 155 to 226 are in use.)
 template <int C, bool X>
 __global__ void __launch_bounds__(X ? SOLVE_THREADS / 2 : SOLVE_THREADS, 1) k_solve_m(SolveArgs a) {
     extern __shared__ float4 sm[];

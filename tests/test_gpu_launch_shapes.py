@@ -45,3 +45,16 @@ def test_shared_sms(par, masses):
     out, st = _run(sc, par)
     assert np.array_equal(out, ref)
     assert st["solve_ctas_masses"] == (st["solve_ctas"] if masses else 0)
+
+
+def test_box_batch():
+    """more workers of boxes than SMs: two CTAs per SM, full rows staged, the bits of one CTA per SM"""
+    from paper_2403_17261_gb300 import scenes as S
+    parts = [S.box_building(seed=7 + k, storeys=1, cells=1 + k % 3, n_sets=2, iters=8) for k in range(90)]
+    sc = S.concat_scenes("boxes", parts, iters=8)
+    sc.half_extents = np.concatenate([p.half_extents for p in parts]).astype(np.float32)
+    ref, st = _run(sc, {}, 3)
+    assert st["solve_ctas_masses"] == st["solve_ctas"] >= 180
+    for par in (dict(smem_slot_limit=5000), dict(pgs_cluster=2), dict(pgs_threads=32), dict(pgs_cluster=1, pgs_threads=512)):
+        out, _ = _run(sc, par, 3)
+        assert np.array_equal(out, ref), par

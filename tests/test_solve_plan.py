@@ -18,6 +18,7 @@ int dynamic_bytes(int budget, long long slots, long long rows, long long stage) 
 int takes_masses(int threads, long long ctas, int sms, int per_sm, long long slots) {
     return ovl::solve_takes_masses(threads, ctas, sms, per_sm, slots);
 }
+int box_threads(int threads, int ctas_per_sm) { return ovl::solve_box_threads(threads, ctas_per_sm); }
 int slot_capacity(int optin, int per_sm, int ctas, int masses) { return ovl::solve_slot_capacity(optin, per_sm, ctas, masses); }
 long long most_room(const int *b, const int *q, int P, int C) { return ovl::solve_most_room(b, q, P, C); }
 }
@@ -114,3 +115,10 @@ def test_slots_fill_the_shared_memory(plan, ctas, masses, static):
 ])
 def test_ctas_that_share_an_sm_find_registers(plan, threads, ctas, slots, masses):
     assert plan.takes_masses(threads, ctas, 152, 233472, slots) == masses
+
+
+@pytest.mark.parametrize("threads,ctas,want", [(512, 1, 256), (256, 1, 256), (96, 1, 96), (256, 2, 128), (512, 2, 128), (64, 2, 64)])
+def test_box_ctas_leave_room_for_their_stages(plan, threads, ctas, want):
+    """two CTAs per SM: 128 threads, whose two stages of 16 records take 64 KB of the half SM's 110"""
+    assert plan.box_threads(threads, ctas) == want
+    assert 2 * 16 * 16 * want < (232448 if ctas == 1 else 233472 // 2 - 3584)
