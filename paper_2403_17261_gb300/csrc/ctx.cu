@@ -227,6 +227,7 @@ MemberArgs member_args(ovl_ctx *c) {
     a.pair_cons = c->pair_cons.p; a.pair_part = c->pair_part.p; a.ps_cons = c->ps_cons.p;
     a.ps_part = c->ps_part.p; a.part_pstart = c->part_pstart.p; a.p_key = c->p_key.p;
     a.p_slot = c->p_slot.p; a.p_lam0 = c->p_lam0.p; a.status = c->status.p;
+    if (c->has_boxes) { a.half = c->half.p; a.full_count = c->full_count.p; }
     return a;
 }
 
@@ -235,8 +236,12 @@ void phase_membership(ovl_ctx *c) {
     const int n = c->n, P = c->n_parts, bits = bits_for(P);
     c->entry_count.ensure((size_t)n + 1);
     c->entry_ptr.ensure((size_t)n + 1);
-    c->h_starts.ensure(2 * (size_t)P + 2);
-    int *const h_bstart = c->h_starts.p, *const h_pstart = h_bstart + P + 1;
+    c->h_starts.ensure(3 * (size_t)P + 2);
+    int *const h_bstart = c->h_starts.p, *const h_pstart = h_bstart + P + 1, *const h_full = h_pstart + P + 1;
+    if (c->has_boxes) {
+        c->full_count.ensure((size_t)P + 1);
+        CK(cudaMemsetAsync(c->full_count.p, 0, sizeof(int) * (size_t)P, s));
+    }
     MemberArgs a = member_args(c);
     launch_entry_count(a, s);
     scan_i32(c->entry_count.p, c->entry_ptr.p, n, c->scan_tmp, s, c->h_counts.p + COUNT_ENTRIES);
@@ -275,8 +280,11 @@ void phase_membership(ovl_ctx *c) {
     w.ws_pstart = c->ws_pstart.p; w.ws_key = c->ws_key.p; w.ws_lam = c->ws_lam.p;
     w.factor = c->P.warmstart;
     launch_pair_setup(a, w, reinterpret_cast<const uint32_t *>(order.p), npr, s);
+    if (c->has_boxes) download(h_full, c->full_count.p, (size_t)P, s);
     // per-worker bodies and constraints on the host, for the launch plans
     CK(cudaStreamSynchronize(s));
+    c->h_full.assign((size_t)P, 0);
+    if (c->has_boxes) c->h_full.assign(h_full, h_full + P);
     c->h_pb.assign(h_bstart, h_bstart + P + 1);
     c->h_pp.assign(h_pstart, h_pstart + P + 1);
     c->nb_max = 0;
@@ -341,7 +349,7 @@ bool solve_masses_fit(const ovl_ctx *c, int slots, int ctas_per_sm) {
 // shape gives the same bits (no implicit FMA contraction in the solver),
 // so the plan changes only the time.  Returns false when some worker does
 // not fit even 8 CTAs (the uniform launch then takes it to global memory).
-struct SolveClass { int C, first, count, slots; long long room; bool small, masses; };
+struct SolveClass { int C, first, count, slots; long long room; bool small, masses; int full; };   // full: FULL_*
 
 // The growth leaves this many SMs unclaimed: clusters must fit inside one GPC,
 // so a launch that claims every SM can leave a cluster waiting for a second
@@ -358,7 +366,7 @@ constexpr int kSolveSmSlack = 8;
 // four; 16 of 40,000 1.29 with four, 1.65 with eight (of which 15 clusters fit
 // at once); boxes: 16 of 4200 1.59 with one and 2.14 with four, 16 of 6100
 // 1.96 and 2.35.
-constexpr double kGrow[2][2] = {{5000, 3000}, {9000, 2500}};   // [boxes][first, next]
+constexpr double kGrow[2][2] = {{5000, 3000}, {9000, 2500}};   // [most rows full][first, next]
 constexpr int kMaxGrow = 4;
 
 // CTA shapes of the per-class launches: threads, rows per thread, CTAs per SM
@@ -370,6 +378,18 @@ constexpr SolveShape kSolveShapes[3] = {{512, 2, 1}, {512, 1, 2}, {256, 2, 2}};
 // CTAs per worker the plans choose from (each a cluster size both the solver
 // and the colouring are built for)
 constexpr int kClusterSizes[] = {1, 2, 3, 4, 6, 8};
+
+// how many of worker p's rows are full
+int full_kind(const ovl_ctx *c, int p) { return solve_full_kind(c->h_full[p], c->h_pp[p + 1] - c->h_pp[p], c->h_pb[p + 1] - c->h_pb[p]); }
+// and, for what all workers share, where the larger part of the full rows lies
+int full_kind(const ovl_ctx *c) {
+    long long all = 0, most = 0;
+    for (int p = 0; p < c->n_parts; ++p) {
+        all += c->h_full[p];
+        if (full_kind(c, p) == FULL_MOST) most += c->h_full[p];
+    }
+    return all == 0 ? FULL_NONE : (2 * most >= all ? FULL_MOST : FULL_FEW);
+}
 
 int default_solve_shape(const ovl_ctx *c) { return c->n_parts <= c->num_sms ? 0 : 2; }
 
@@ -393,7 +413,7 @@ std::vector<int> plan_worker_counts(ovl_ctx *c, int cap, long long budget) {
         C[p] = k;
         total += k;
     }
-    auto load = [&](int p) { return (double)(pp[p + 1] - pp[p]) / C[p]; };
+    auto load = [&](int p) { return solve_grow_rows(c->h_full[p], pp[p + 1] - pp[p], pb[p + 1] - pb[p]) / C[p]; };
     if (total <= budget) {
         std::vector<int> heap(P);
         std::iota(heap.begin(), heap.end(), 0);
@@ -403,7 +423,7 @@ std::vector<int> plan_worker_counts(ovl_ctx *c, int cap, long long budget) {
             std::pop_heap(heap.begin(), heap.end(), less);
             const int p = heap.back();
             const int up = next(C[p]);
-            if (load(p) < kGrow[c->has_boxes][C[p] > 1]) {
+            if (load(p) < kGrow[full_kind(c, p) == FULL_MOST][C[p] > 1]) {
                 heap.pop_back();
                 continue;
             }
@@ -434,13 +454,15 @@ void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveC
     const std::vector<int> &pb = c->h_pb, &pp = c->h_pp;
     std::vector<int> order(P);
     std::iota(order.begin(), order.end(), 0);
-    std::vector<char> small(P, 0);
+    std::vector<char> small(P, 0), full(P);
+    for (int p = 0; p < P; ++p) full[p] = (char)full_kind(c, p);
     if (split)
         for (int p = 0; p < P; ++p)
-            small[p] = C[p] == 1 && solve_worker_room(pb[p + 1] - pb[p], pp[p + 1] - pp[p], 1) <=
+            small[p] = C[p] == 1 && full[p] == FULL_NONE && solve_worker_room(pb[p + 1] - pb[p], pp[p + 1] - pp[p], 1) <=
                                         c->smem_per_sm / kSmallPerSm - 3584;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         if (C[x] != C[y]) return C[x] > C[y];
+        if (full[x] != full[y]) return full[x] > full[y];
         if (small[x] != small[y]) return small[x] < small[y];
         return pp[x + 1] - pp[x] > pp[y + 1] - pp[y];
     });
@@ -448,8 +470,9 @@ void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveC
     c->h_class_of.resize(P);
     for (int i = 0; i < P; ++i) {
         const int p = order[i], nb = pb[p + 1] - pb[p];
-        if (classes.empty() || classes.back().C != C[p] || classes.back().small != (bool)small[p])
-            classes.push_back({C[p], i, 0, 1, 0, (bool)small[p], false});
+        if (classes.empty() || classes.back().C != C[p] || classes.back().full != full[p] ||
+            classes.back().small != (bool)small[p])
+            classes.push_back({C[p], i, 0, 1, 0, (bool)small[p], false, full[p]});
         c->h_class_of[p] = (int)classes.size() - 1;
         SolveClass &k = classes.back();
         k.count++;
@@ -503,12 +526,12 @@ bool plan_solve_classes(ovl_ctx *c, const SolveShape &shape, std::vector<SolveCl
     }
     const std::vector<int> C = plan_worker_counts(c, cap, budget);
     if (C.empty() && c->n_parts > 0) return false;
-    // contexts with boxes, and a slot limit, keep one shape
-    plan_classes_from(c, C, classes, c->class_order, shape.per_sm > 1 && !c->has_boxes && c->P.smem_slot_limit <= 0);
+    // workers of boxes, and a slot limit, keep one shape
+    plan_classes_from(c, C, classes, c->class_order, shape.per_sm > 1 && c->P.smem_slot_limit <= 0);
     const long long ctas = std::accumulate(C.begin(), C.end(), 0ll);
     for (SolveClass &k : classes)
         k.masses = solve_masses_fit(c, k.slots, shape.per_sm) &&
-                   (shape.unroll == 2 || c->has_boxes || solve_takes_masses(shape.threads, ctas, c->num_sms, c->smem_per_sm, k.slots));
+                   (shape.unroll == 2 || k.full != FULL_NONE || solve_takes_masses(shape.threads, ctas, c->num_sms, c->smem_per_sm, k.slots));
     return true;
 }
 
@@ -552,7 +575,7 @@ void run_on_streams(ovl_ctx *c, size_t n, F &&launch, const std::vector<size_t> 
 // threads of a class's CTAs
 int class_threads(const ovl_ctx *c, const SolveShape &shape, const SolveClass &k) {
     if (k.small) return kSmallThreads;
-    return c->has_boxes && k.masses ? solve_box_threads(shape.threads, shape.per_sm) : shape.threads;
+    return k.full == FULL_MOST && k.masses ? solve_box_threads(shape.threads, shape.per_sm) : shape.threads;
 }
 
 void launch_solve_classes(ovl_ctx *c, const SolveArgs &a, const SolveShape &shape,
@@ -563,6 +586,8 @@ void launch_solve_classes(ovl_ctx *c, const SolveArgs &a, const SolveShape &shap
         b.order = c->class_order.p + classes[k].first;
         b.smem_slots = classes[k].slots;
         b.smem_room = classes[k].room;
+        if (classes[k].full == FULL_NONE) b.row_full = nullptr;
+        b.few = classes[k].full == FULL_FEW;
         launch_solve(b, class_threads(c, shape, classes[k]), classes[k].C, shape.unroll, classes[k].masses,
                      solve_smem_budget(c, shape.per_sm, true), sk);
     }, class_launch_order(c, classes));
@@ -678,7 +703,7 @@ void phase_rows(ovl_ctx *c, float dt_override) {
     a.scene_dt = c->scene_dt.p; a.scene_mu = c->scene_mu.p; a.dt_override = dt_override;
     a.erp = c->P.erp; a.slop = c->P.slop;
     a.r0 = c->r0.p; a.r1 = c->r1.p; a.r2 = c->r2.p; a.r3 = c->r3.p; a.rlam = c->rlam.p;
-    a.part_bstart = c->part_bstart.p; a.solve_C = c->solve_C.p; a.solve_M = c->solve_M.p;
+    a.part_bstart = c->part_bstart.p; a.part_pstart = c->part_pstart.p; a.solve_C = c->solve_C.p; a.solve_M = c->solve_M.p;
     a.rpair = c->rpair.p; a.status = c->status.p;
     if (c->has_boxes) {
         c->row_full.ensure(npr + 1);
@@ -744,7 +769,7 @@ SolveArgs solve_args(ovl_ctx *c, float dt_override, int iters) {
     a.iters = iters; a.flags = c->P.flags;
     a.res_tol = c->P.res_tol; a.res_check_every = c->P.res_check_every;
     a.part_iters = c->part_iters.p; a.part_res_sq = c->part_res_sq.p; a.status = c->status.p;
-    if (c->has_boxes) { a.row_full = c->row_full.p; a.rfull = c->rfull.p; a.np = c->npairs; }
+    if (c->has_boxes) { a.row_full = c->row_full.p; a.rfull = c->rfull.p; }
     return a;
 }
 
@@ -778,17 +803,17 @@ struct SolvePlan {
     int cluster = 1, threads = 512, unroll = 1, slots = 0;
 };
 
-// whether a uniform launch keeps the masses in shared memory (the kernels of
-// contexts with boxes have registers for one CTA per SM either way)
+// whether a uniform launch keeps the masses in shared memory (the kernels
+// with full rows have registers for one CTA per SM either way)
 bool uniform_masses(const ovl_ctx *c, const SolvePlan &pl) {
     return solve_masses_fit(c, pl.slots, solve_ctas_per_sm(pl.unroll)) &&
-           (pl.unroll == 2 || c->has_boxes ||
+           (pl.unroll == 2 || full_kind(c) != FULL_NONE ||
             solve_takes_masses(pl.threads, (long long)pl.cluster * c->n_parts, c->num_sms, c->smem_per_sm, pl.slots));
 }
 
 // threads of a uniform launch's CTAs
 int uniform_threads(const ovl_ctx *c, const SolvePlan &pl, bool masses) {
-    return c->has_boxes && masses ? solve_box_threads(pl.threads, solve_ctas_per_sm(pl.unroll)) : pl.threads;
+    return full_kind(c) == FULL_MOST && masses ? solve_box_threads(pl.threads, solve_ctas_per_sm(pl.unroll)) : pl.threads;
 }
 
 // Every worker's CTA count goes to the device and the rows of every colour
@@ -807,10 +832,15 @@ void apply_solve_order(ovl_ctx *c, const SolvePlan &pl) {
     } else {
         std::fill(M.begin(), M.end(), uniform_masses(c, pl) ? 1 : 0);
     }
+    // the bank order is for k_solve_m's plain rows; the layout of the full rows
+    std::vector<int> banked(M);
+    for (int p = 0; p < P; ++p)
+        if ((pl.shape >= 0 ? full_kind(c, p) : full_kind(c)) == FULL_MOST) {
+            banked[p] = 0;
+            M[p] |= 2;
+        }
     upload(c->solve_M, M.data(), (size_t)P, c->stream);
-    // the bank order is for k_solve_m's rows
-    if (c->has_boxes) std::fill(M.begin(), M.end(), 0);
-    upload(c->solve_banked, M.data(), (size_t)P, c->stream);
+    upload(c->solve_banked, banked.data(), (size_t)P, c->stream);
     c->col_off2.ensure((size_t)P * OWNER_NB + 1);
     c->pair_of_row2.ensure((size_t)c->npairs + 1);
     c->row_owner.ensure((size_t)c->npairs + 1);
@@ -848,6 +878,8 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
     // share an SM (600 scenes of two workers: solve 0.60 -> 0.27 ms with 64
     // threads per CTA, 0.55 -> 0.32 with 128)
     a.smem_room = solve_most_room(c->h_pb.data(), c->h_pp.data(), P, pl.cluster);
+    if (full_kind(c) == FULL_NONE) a.row_full = nullptr;
+    a.few = full_kind(c) == FULL_FEW;
     launch_solve(a, uniform_threads(c, pl, masses), pl.cluster, pl.unroll, masses,
                  solve_smem_budget(c, solve_ctas_per_sm(pl.unroll), true), c->stream);
     c->last_ctas = (long long)pl.cluster * P;
@@ -1184,7 +1216,7 @@ void release_all(ovl_ctx *c) {
     c->part_bstart.release(); c->group.release(); c->cons_count.release(); c->cons_start.release();
     c->pair_cons.release(); c->pair_part.release(); c->ps_cons.release(); c->ps_part.release();
     c->part_pstart.release(); c->p_colour.release(); c->part_ncol.release(); c->part_rounds.release();
-    c->col_off.release(); c->pair_of_row.release(); c->p_key.release(); c->p_slot.release();
+    c->full_count.release(); c->col_off.release(); c->pair_of_row.release(); c->p_key.release(); c->p_slot.release();
     c->p_lam0.release(); c->colour_scratch.release(); c->worklist.release(); c->worklist2.release(); c->list_prio.release(); c->list_sorted.release(); c->list_queue.release(); c->wprio.release(); c->wprio2.release(); c->r0.release(); c->r1.release();
     c->r2.release(); c->rlam.release(); c->lam_out.release(); c->r3.release(); c->rpair.release(); c->ws_pstart.release();
     c->ws_key.release(); c->ws_lam.release(); c->copies.release(); c->solve_scratch.release();

@@ -78,6 +78,7 @@ struct ovl_ctx {
     DBuf<float4> r0, r1, r2, r3, rlam, lam_out;
     DBuf<int> rpair;
     DBuf<int> ws_pstart;
+    DBuf<int> full_count;      // constraints with a box end of every worker (contexts with boxes)
     DBuf<uint64_t> ws_key;
     DBuf<float4> ws_lam;
     int64_t ws_n = 0;
@@ -103,7 +104,8 @@ struct ovl_ctx {
     DBuf<uint32_t> worker_order;                 // workers longest first (order of a uniform launch)
     DBuf<uint32_t> class_order, colour_order;    // solve / colouring: workers grouped by CTAs per worker
     std::vector<int> h_pb, h_pp;                 // part_bstart, part_pstart of this step on the host
-    HBuf<int> h_starts;                          // both as the kernels write them
+    HBuf<int> h_starts;                          // both as the kernels write them, and full_count
+    std::vector<int> h_full;                     // full_count of this step on the host (zeros without boxes)
     std::vector<int> h_class_C;                  // CTAs per worker of the last per-worker plan
     std::vector<int> h_class_of;                 // and its launch class
     DBuf<int> solve_C, solve_M, solve_banked, col_off2, pair_of_row2;   // solve: CTAs per worker, masses in shared memory, rows in bank order, rows by owner CTA

@@ -343,6 +343,12 @@ k_row_owner(int P, const int *part_bstart, const int *part_ncol, const int *solv
     }
 }
 
+__device__ __forceinline__ bool body_is_box(const float4 *half, int b) {
+    if (!half || b < 0) return false;
+    const float4 h = half[b];
+    return h.x > 0.f || h.y > 0.f || h.z > 0.f;
+}
+
 // manifold index of contact i (0 without boxes)
 __device__ __forceinline__ int contact_point(const MemberArgs &a, int i) {
     return a.c_p ? __float_as_int(a.c_p[i].w) : 0;
@@ -364,6 +370,12 @@ __global__ void k_pair_setup(MemberArgs a, WarmArgs ws, const uint32_t *order, i
         } else {
             e = a.jab[i - a.nc];
             key = (1ull << 62) | (uint64_t)(i - a.nc);
+        }
+        if (a.half) {
+            // a worker's pairs are neighbours, so a warp adds to one or two counts
+            const bool full = body_is_box(a.half, e.x) || (e.y < a.n && body_is_box(a.half, e.y));
+            const unsigned peers = __match_any_sync(__activemask(), full ? p : -1);
+            if (full && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&a.full_count[p], __popc(peers));
         }
         a.p_key[k] = key;
         a.p_slot[k] = make_int2(body_slot(a, e.x, w), body_slot(a, e.y, w));
@@ -1010,12 +1022,6 @@ __device__ __forceinline__ SlotWords slot_words(const RowArgs &a, int p, int2 sl
     return SlotWords{__uint_as_float(code(sl.x, 24)), __uint_as_float(code(sl.y, 24)), __uint_as_float(p16)};
 }
 
-__device__ __forceinline__ bool body_is_box(const float4 *half, int b) {
-    if (!half || b < 0) return false;
-    const float4 h = half[b];
-    return h.x > 0.f || h.y > 0.f || h.z > 0.f;
-}
-
 // I^-1 v for body b: a box's R diag(1/I) R^T (R from its blended
 // orientation), a sphere's isotropic 1/I
 __device__ float3 inv_inertia_times(const RowArgs &a, int b, float3 v) {
@@ -1029,12 +1035,14 @@ __device__ float3 inv_inertia_times(const RowArgs &a, int b, float3 v) {
     return quat_rotate(q, make_float3(d.x * lb.x, d.y * lb.y, d.z * lb.z));
 }
 
-// one full row (see FULL_ROW_WORDS): lever arms rA, rB (world), ends ea, eb
+// one full row of worker p (see FULL_ROW_WORDS): lever arms rA, rB (world), ends ea, eb
 // (-1: static or not in this worker), directions dir[3], targets tg[3]
-__device__ void write_full_row(const RowArgs &a, int r, int ea, int eb, float3 rA, float3 rB, const float3 *dir,
+__device__ void write_full_row(const RowArgs &a, int r, int p, int ea, int eb, float3 rA, float3 rB, const float3 *dir,
                                const float *tg) {
-    const size_t np = (size_t)a.np;
-    float4 *F = a.rfull + r;
+    const bool most = a.solve_M[p] & 2;
+    const int q0 = a.part_pstart[p];
+    const size_t w = most ? (size_t)(a.part_pstart[p + 1] - q0) : 1;
+    float4 *F = a.rfull + (most ? (size_t)(FULL_ROW_WORDS - 1) * q0 + r : (size_t)FULL_ROW_WORDS * r);
     const float imA = ea >= 0 ? a.st[4 * ea + 2].w : 0.f, imB = eb >= 0 ? a.st[4 * eb + 2].w : 0.f;
     for (int i = 0; i < 3; ++i) {
         const float3 d = dir[i];
@@ -1043,13 +1051,13 @@ __device__ void write_full_row(const RowArgs &a, int r, int ea, int eb, float3 r
         const float3 iA = ea >= 0 ? inv_inertia_times(a, ea, jA) : make_float3(0.f, 0.f, 0.f);
         const float3 iB = eb >= 0 ? inv_inertia_times(a, eb, jB) : make_float3(0.f, 0.f, 0.f);
         const float s = (imA + imB) + ((jA.x * iA.x + jA.y * iA.y + jA.z * iA.z) + (jB.x * iB.x + jB.y * iB.y + jB.z * iB.z));
-        F[i * np] = make_float4(d.x, d.y, d.z, tg[i]);
-        F[(3 + i) * np] = make_float4(jA.x, jA.y, jA.z, s > 0.f ? 1.f / s : 0.f);
-        F[(6 + i) * np] = make_float4(iA.x, iA.y, iA.z, 0.f);
-        F[(9 + i) * np] = make_float4(jB.x, jB.y, jB.z, 0.f);
-        F[(12 + i) * np] = make_float4(iB.x, iB.y, iB.z, 0.f);
+        F[i * w] = make_float4(d.x, d.y, d.z, tg[i]);
+        F[(3 + i) * w] = make_float4(jA.x, jA.y, jA.z, s > 0.f ? 1.f / s : 0.f);
+        F[(6 + i) * w] = make_float4(iA.x, iA.y, iA.z, 0.f);
+        F[(9 + i) * w] = make_float4(jB.x, jB.y, jB.z, 0.f);
+        F[(12 + i) * w] = make_float4(iB.x, iB.y, iB.z, 0.f);
     }
-    F[15 * np] = make_float4(imA, imB, 0.f, 0.f);
+    F[15 * w] = make_float4(imA, imB, 0.f, 0.f);
 }
 
 __global__ void k_rows(RowArgs a) {
@@ -1059,7 +1067,7 @@ __global__ void k_rows(RowArgs a) {
         const int2 sl = a.p_slot[k];
         const int scene = a.part_scene[a.ps_part[k]];
         const float h = a.dt_override > 0.f ? a.dt_override : a.scene_dt[scene];
-        const bool pack = a.solve_M && a.solve_M[a.ps_part[k]];   // a launch with the masses in shared memory
+        const bool pack = a.solve_M[a.ps_part[k]] & 1;   // a launch with the masses in shared memory
         const SlotWords sw = slot_words(a, a.ps_part[k], sl, pack);
         float lam_w = 0.f;   // a plain contact row: k_n (see below)
         if (a.row_full) {
@@ -1121,7 +1129,7 @@ __global__ void k_rows(RowArgs a) {
                     a.r2[r] = make_float4(0.f, 0.f, sw.a, sw.b);
                     a.r3[r] = z;
                 }
-                write_full_row(a, r, ea, eb, rA, rB, dir, tg);
+                write_full_row(a, r, a.ps_part[k], ea, eb, rA, rB, dir, tg);
                 a.rpair[r] = k;
                 a.rlam[r] = a.p_lam0[k];
                 continue;

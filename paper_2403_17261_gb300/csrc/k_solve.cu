@@ -372,7 +372,22 @@ struct FullStaged {
     int stride;
     __device__ __forceinline__ float4 operator()(int j) const { return p[j * stride]; }
 };
-__device__ __forceinline__ FullGlobal full_of(const SolveArgs &a, int r) { return {a.rfull + r, (size_t)a.np}; }
+// Where the full rows of a worker with rows [row0, row1) lie (see
+// FULL_ROW_WORDS).  K: FULL_MOST or FULL_FEW, 0 the launch's argument says which.
+template <int K>
+struct FullRows {
+    const float4 *p;
+    size_t rs, ws;   // from row to row, from word to word
+    __device__ __forceinline__ FullRows(const SolveArgs &a, int row0, int row1) {
+        const bool few = K == 0 ? a.few : K == FULL_FEW;
+        p = few ? a.rfull : a.rfull + (size_t)(FULL_ROW_WORDS - 1) * row0;
+        rs = few ? FULL_ROW_WORDS : 1;
+        ws = few ? 1 : (size_t)(row1 - row0);
+    }
+    __device__ __forceinline__ FullGlobal at(int r) const {
+        return {p + r * (K == 0 ? rs : (K == FULL_FEW ? FULL_ROW_WORDS : 1)), K == FULL_FEW ? 1 : ws};
+    }
+};
 
 // impulse dl along direction i of a full row
 template <class FR>
@@ -418,9 +433,9 @@ __device__ __forceinline__ void full_warm(const FR &F, Body &A, Body &B, float4 
 
 // a row of the sweep: full (box end) or plain
 template <class S, bool X>
-__device__ __forceinline__ void solve_any(const SolveArgs &a, int r, Body &A, Body &B, const Row &w, float mu,
-                                          float4 &lam) {
-    if (is_full<X>(a, r)) full_rows(full_of(a, r), w.joint, A, B, mu, lam);
+__device__ __forceinline__ void solve_any(const SolveArgs &a, const FullRows<0> &fr, int r, Body &A, Body &B, const Row &w,
+                                          float mu, float4 &lam) {
+    if (is_full<X>(a, r)) full_rows(fr.at(r), w.joint, A, B, mu, lam);
     else solve_row<S>(A, B, w, mu, lam);
 }
 
@@ -552,7 +567,7 @@ struct Buckets {
 };
 
 template <class S, bool X>
-__device__ float rows_residual_sq(const SolveArgs &a, const S &st, const Buckets &bk, int ncol, float mu,
+__device__ float rows_residual_sq(const SolveArgs &a, const FullRows<0> &fr, const S &st, const Buckets &bk, int ncol, float mu,
                                   int tid, int T) {
     float sq = 0.f;
     for (int c = 0; c < ncol; ++c)
@@ -566,7 +581,7 @@ __device__ float rows_residual_sq(const SolveArgs &a, const S &st, const Buckets
                 Body A, B;
                 load_pair(st, w, A, B);
                 if (is_full<X>(a, r)) {
-                    sq += full_residual_sq(full_of(a, r), w.joint, A, B, mu, lam);
+                    sq += full_residual_sq(fr.at(r), w.joint, A, B, mu, lam);
                 } else if (w.joint) {
                     sq += joint_residual_sq(A, B, w.x, w.y, w.z);
                 } else {
@@ -606,6 +621,7 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
                              int row0, int row1) {
     __shared__ float red[32];
     __shared__ float part_sum;
+    const FullRows<0> fr(a, row0, row1);
     const int tid = threadIdx.x, T = blockDim.x;
     const int g = rank * T + tid, G = C * T;
     const int b0 = a.part_bstart[p], nb = a.part_bstart[p + 1] - b0;
@@ -651,7 +667,7 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
             Body A, B;
             load_pair(st, w, A, B);
             if (is_full<X>(a, r)) {
-                full_warm(full_of(a, r), A, B, lam);
+                full_warm(fr.at(r), A, B, lam);
             } else if (!w.joint) {
                 const float3 t1 = contact_t1(w);
                 const float3 n = f3(w.x);
@@ -699,8 +715,8 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
                     Body A, B, D, E;
                     load_pair(st, u, A, B);
                     load_pair(st, w, D, E);
-                    solve_any<S, X>(a, r, A, B, u, mu, xl);
-                    solve_any<S, X>(a, q, D, E, w, mu, yl);
+                    solve_any<S, X>(a, fr, r, A, B, u, mu, xl);
+                    solve_any<S, X>(a, fr, q, D, E, w, mu, yl);
                     store_pair(st, row_slots<S>(u), A, B);
                     store_pair(st, row_slots<S>(w), D, E);
                     a.rlam[r] = xl;
@@ -714,7 +730,7 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
                     float4 lam = cur.l0;
                     Body A, B;
                     load_pair(st, w, A, B);
-                    solve_any<S, X>(a, r, A, B, w, mu, lam);
+                    solve_any<S, X>(a, fr, r, A, B, w, mu, lam);
                     store_pair(st, row_slots<S>(w), A, B);
                     a.rlam[r] = lam;
                 }
@@ -730,8 +746,8 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
                         Body A, B, D, E;
                         load_pair(st, u, A, B);
                         load_pair(st, w, D, E);
-                        solve_any<S, X>(a, r, A, B, u, mu, xl);
-                        solve_any<S, X>(a, q, D, E, w, mu, yl);
+                        solve_any<S, X>(a, fr, r, A, B, u, mu, xl);
+                        solve_any<S, X>(a, fr, q, D, E, w, mu, yl);
                         store_pair(st, row_slots<S>(u), A, B);
                         store_pair(st, row_slots<S>(w), D, E);
                         a.rlam[r] = xl;
@@ -744,7 +760,7 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
                     float4 lam = a.rlam[r];
                     Body A, B;
                     load_pair(st, w, A, B);
-                    solve_any<S, X>(a, r, A, B, w, mu, lam);
+                    solve_any<S, X>(a, fr, r, A, B, w, mu, lam);
                     store_pair(st, row_slots<S>(w), A, B);
                     a.rlam[r] = lam;
                 }
@@ -764,14 +780,14 @@ __device__ void solve_worker(const SolveArgs &a, const S &st, int p, int rank, i
         }
         it_done = it + 1;
         if (a.res_tol > 0.f && a.res_check_every > 0 && it_done % a.res_check_every == 0 && it_done < a.iters) {
-            float tot = group_sum<C>(rows_residual_sq<S, X>(a, st, bk, ncol, mu, tid, T), red, &part_sum);
+            float tot = group_sum<C>(rows_residual_sq<S, X>(a, fr, st, bk, ncol, mu, tid, T), red, &part_sum);
             int nrows = 3 * (row1 - row0);
             if (nrows == 0 || sqrtf(tot / nrows) <= a.res_tol) break;   // the same total in every CTA
         }
     }
     // residual of every row at the final iterate
     if (a.flags & OVL_FLAG_RESIDUAL) {
-        float tot = group_sum<C>(rows_residual_sq<S, X>(a, st, bk, ncol, mu, tid, T), red, &part_sum);
+        float tot = group_sum<C>(rows_residual_sq<S, X>(a, fr, st, bk, ncol, mu, tid, T), red, &part_sum);
         if (rank == 0 && tid == 0) a.part_res_sq[p] = (double)tot;
     }
     if (rank == 0 && tid == 0) a.part_iters[p] = it_done;
@@ -829,12 +845,12 @@ __device__ __forceinline__ void fetch_head(const SolveArgs &a, int r, int end, R
 // A full row's words copied to shared memory ahead of use, word j of thread
 // tid at stage[j T + tid]: read by the thread that copied them, so a
 // wait on its own copies is enough.
-__device__ __forceinline__ void stage_full(const SolveArgs &a, int r, float4 *stage) {
-    const float4 *src = a.rfull + r;
+__device__ __forceinline__ void stage_full(const FullRows<FULL_MOST> &fr, int r, float4 *stage) {
+    const float4 *src = fr.p + r;
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage + threadIdx.x);
 #pragma unroll
     for (int j = 0; j < FULL_ROW_WORDS; ++j)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 16u * j * blockDim.x), "l"(src + (size_t)j * a.np) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + 16u * j * blockDim.x), "l"(src + j * fr.ws) : "memory");
 }
 __device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 // all but the newest n groups of this thread's copies have landed
@@ -959,8 +975,8 @@ struct SolveRow {
 // the full rows among a thread's first rows of the colours are copied to
 // shared memory a colour ahead too (two stages of FULL_ROW_WORDS float4 per
 // thread), further ones of a colour come straight from global memory.
-template <int C, bool X, class LM>
-__device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM &lam, const int4 *tab, int ncol, float mu,
+template <int C, int X, class LM>
+__device__ void sweep_rows(const SolveArgs &a, const FullRows<X> &fr, const LocalSlotsM &own, const LM &lam, const int4 *tab, int ncol, float mu,
                            int p, int rank, int nrows, float4 *stage, float *red, float *part_sum) {
     const int tid = threadIdx.x, T = blockDim.x;
     RowHead nx;
@@ -970,10 +986,11 @@ __device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM 
         fetch_head(a, o.x + tid, o.z, nx);
         if (X) {
             fullx = o.x + tid < o.z && __ldg(a.row_full + o.x + tid);
-            if (stage) {
-                if (fullx) stage_full(a, o.x + tid, st);
-                stage_commit();
-            }
+            if constexpr (X == FULL_MOST)
+                if (stage) {
+                    if (fullx) stage_full(fr, o.x + tid, st);
+                    stage_commit();
+                }
         }
     };
     if (ncol > 0) ahead_of(tab[0], stage);
@@ -998,7 +1015,7 @@ __device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM 
                     });
                 } else {
                     visit_row<C>(a, own, (uint32_t)rank, lam, i, r, r >= o.y, true, cur, [&](Body &A, Body &B, const Row &w, float4 &l) {
-                        return f.full(full_of(a, r), A, B, w, l);
+                        return f.full(fr.at(r), A, B, w, l);
                     });
                 }
             } else {
@@ -1019,7 +1036,7 @@ __device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM 
                 fetch_head(a, r, o.z, q);
                 const bool full = X && a.row_full[r];
                 visit_row<C>(a, own, (uint32_t)rank, lam, r - o.x + o.w, r, r >= o.y, full, q, [&](Body &A, Body &B, const Row &w, float4 &l) {
-                    if (full) sq += full_residual_sq(full_of(a, r), w.joint, A, B, mu, l);
+                    if (full) sq += full_residual_sq(fr.at(r), w.joint, A, B, mu, l);
                     else if (w.joint) sq += joint_residual_sq(A, B, w.x, w.y, w.z);
                     else sq += contact_residual_sq(A, B, w.x, w.y, contact_t1(w), l.w, w.x.w, mu, l);
                     return false;
@@ -1052,14 +1069,17 @@ __device__ void sweep_rows(const SolveArgs &a, const LocalSlotsM &own, const LM 
 // rows takes about 900 cycles, of which 95 are the CTA barrier (560 a
 // cluster's), the rest one row's chain; 512 threads (measured on the large
 // pile: 256 1.14 ms, 384 1.00, 512 0.94, 768 0.92 but slower on small piles).
-// X: a context with boxes.  Rows read straight from global memory, flag, head
+// X: how many rows are full.  FULL_FEW: they come straight from global memory;
+// the CTAs are those of the spheres, 512 threads (128 registers) and rows in
+// bank order (a pile of 30,000 with 4 boxes 1.11 -> 0.83 ms, with 400 1.35 -> 0.99).
+// FULL_MOST: rows read straight from global memory, flag, head
 // and words one after the other, made a colour step 1.4 us (building 2.93 ms,
 // bridge 1.13); with the impulses in shared memory and the words a colour
 // ahead it takes 0.75 us (1.59 and 0.62 ms).  256 threads: the stages take
 // 512 B per thread.  (Registers bounded to 128, for two such CTAs per SM,
 // cost clusters 4 to 15 %: 155 to 226 are in use.)
-template <int C, bool X>
-__global__ void __launch_bounds__(X ? SOLVE_THREADS / 2 : SOLVE_THREADS, 1) k_solve_m(SolveArgs a) {
+template <int C, int X>
+__global__ void __launch_bounds__(X == FULL_MOST ? SOLVE_THREADS / 2 : SOLVE_THREADS, 1) k_solve_m(SolveArgs a) {
     extern __shared__ float4 sm[];
     __shared__ int4 tab[OVL_MAX_COLOURS];
     __shared__ float red[32];
@@ -1095,7 +1115,7 @@ __global__ void __launch_bounds__(X ? SOLVE_THREADS / 2 : SOLVE_THREADS, 1) k_so
     float *const L = reinterpret_cast<float *>(sm + 2 * (per + 1));
     const bool fits = 32ll * (per + 1) + 12ll * mine <= a.smem_bytes;
     const long long used = fits ? (32ll * (per + 1) + 12ll * mine + 15) / 16 : 2ll * (per + 1);
-    float4 *const stage = X && 16 * (used + 2ll * FULL_ROW_WORDS * T) <= a.smem_bytes ? sm + used : nullptr;
+    float4 *const stage = X == FULL_MOST && 16 * (used + 2ll * FULL_ROW_WORDS * T) <= a.smem_bytes ? sm + used : nullptr;
     // velocities after the external force (h f), from the blended state; the
     // zero slot (static ends); the impulses
     for (int s = s_lo + tid; s < s_hi; s += T) {
@@ -1111,8 +1131,9 @@ __global__ void __launch_bounds__(X ? SOLVE_THREADS / 2 : SOLVE_THREADS, 1) k_so
             for (int r = tab[c].x + tid; r < tab[c].z; r += T) ls.store(r - tab[c].x + tab[c].w, r, a.rlam[r]);
     group_sync<C>();
     const LocalSlotsM own{V, W};
-    if (fits) sweep_rows<C, X>(a, own, ls, tab, ncol, mu, p, rank, 3 * (row1 - row0), stage, red, &part_sum);
-    else sweep_rows<C, X>(a, own, LamGlobal{a.rlam}, tab, ncol, mu, p, rank, 3 * (row1 - row0), stage, red, &part_sum);
+    const FullRows<X> fr(a, row0, row1);
+    if (fits) sweep_rows<C, X>(a, fr, own, ls, tab, ncol, mu, p, rank, 3 * (row1 - row0), stage, red, &part_sum);
+    else sweep_rows<C, X>(a, fr, own, LamGlobal{a.rlam}, tab, ncol, mu, p, rank, 3 * (row1 - row0), stage, red, &part_sum);
     // impulses back in canonical pair order (next step's warm start)
     for (int c = 0; c < ncol; ++c)
         for (int r = tab[c].x + tid; r < tab[c].z; r += T) {
@@ -1199,11 +1220,11 @@ static void launch_solve_u(const SolveArgs &a, int threads, int cluster, cudaStr
     }
 }
 
-template <int C, bool X>
+template <int C, int X>
 static void launch_solve_m(const SolveArgs &a, int threads, int budget, cudaStream_t s) {
     SolveArgs b = a;
-    if (X) threads = std::min(threads, SOLVE_THREADS / 2);
-    b.smem_bytes = solve_dynamic_bytes(budget, a.smem_room, X ? 2 * FULL_ROW_WORDS * 16 * threads : 0);
+    if (X == FULL_MOST) threads = std::min(threads, SOLVE_THREADS / 2);
+    b.smem_bytes = solve_dynamic_bytes(budget, a.smem_room, X == FULL_MOST ? 2 * FULL_ROW_WORDS * 16 * threads : 0);
     CK(cudaFuncSetAttribute(k_solve_m<C, X>, cudaFuncAttributeMaxDynamicSharedMemorySize, b.smem_bytes));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(a.n_parts * C);
@@ -1221,7 +1242,7 @@ static void launch_solve_m(const SolveArgs &a, int threads, int budget, cudaStre
     note_launch();
 }
 
-template <bool X>
+template <int X>
 static void launch_solve_masses(const SolveArgs &a, int threads, int cluster, int budget, cudaStream_t s) {
     switch (cluster) {
         case 8: launch_solve_m<8, X>(a, threads, budget, s); break;
@@ -1237,8 +1258,9 @@ void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool
     if (!a.n_parts) return;
     if (threads > SOLVE_THREADS) threads = SOLVE_THREADS;
     if (masses) {
-        if (a.row_full) launch_solve_masses<true>(a, threads, cluster, budget, s);
-        else launch_solve_masses<false>(a, threads, cluster, budget, s);
+        if (!a.row_full) launch_solve_masses<FULL_NONE>(a, threads, cluster, budget, s);
+        else if (a.few) launch_solve_masses<FULL_FEW>(a, threads, cluster, budget, s);
+        else launch_solve_masses<FULL_MOST>(a, threads, cluster, budget, s);
     } else if (a.row_full) {
         // a context with boxes: the kernels that hold the full rows (two rows
         // per thread, no rows loaded ahead; one CTA per SM at 512 threads)

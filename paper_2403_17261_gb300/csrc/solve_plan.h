@@ -67,7 +67,32 @@ inline bool solve_takes_masses(int threads, long long ctas, int sms, int per_sm,
     return 2 * std::max(1, 512 / threads) > std::min(other, (ctas + sms - 1) / sms);
 }
 
-// Threads of a CTA that keeps the masses in a context with boxes: at most 256
+// How many of a worker's rows are full rows (a box end), as its launch takes
+// them.  The kernel for workers of boxes (FULL_MOST) copies the full row of a
+// thread's first row of a colour to shared memory ahead of use, which leaves a
+// CTA half the threads: 256 rows of a colour in one pass.  It pays where seven
+// in ten rows are full, or a quarter in a worker of up to 1000 bodies (a colour
+// holds a body once, so about bodies / 2.6 rows).  Other workers with full rows
+// (FULL_FEW) keep the spheres' CTAs.  (Solves of piles with boxes, ms, as
+// FULL_FEW and as FULL_MOST: 8 workers of about 1600 bodies, 2 % of them boxes,
+// 0.71 and 0.96, 20 % 1.25 and 1.54, 75 % 2.46 and 1.89; 8 of 450, 20 %, 1.09
+// and 0.77; 8 of 800, 20 %, 1.06 and 0.95.)
+enum { FULL_NONE, FULL_FEW, FULL_MOST };
+inline int solve_full_kind(long long full, long long rows, int bodies) {
+    if (full == 0) return FULL_NONE;
+    return 10 * full >= 7 * rows || (4 * full >= rows && bodies <= 1000) ? FULL_MOST : FULL_FEW;
+}
+
+// Rows as the growth of a worker's CTAs counts them: where few are full, such a
+// row, read straight from global memory, costs as much as six plain ones; below
+// 2500 rows a worker has too few to share.  (One and four CTAs per worker, a
+// sixth of the rows full: 2200 rows 0.53 and 0.61 ms, 2800 0.66 and 0.61, 4300
+// 0.87 and 0.63; spheres cross at 5000.)
+inline double solve_grow_rows(long long full, long long rows, int bodies) {
+    return solve_full_kind(full, rows, bodies) == FULL_FEW && rows >= 2500 ? rows + 5.0 * full : (double)rows;
+}
+
+// Threads of a CTA that keeps the masses of a worker of boxes: at most 256
 // (its 155 to 226 registers leave no more), and 128 where it is to share its SM
 // with another, which 256 leave neither the registers nor, for the two stages
 // of full rows (512 B per thread), the shared memory.  (Solves of box batches,

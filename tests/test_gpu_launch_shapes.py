@@ -6,18 +6,20 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
+def _pile(side, rng):
+    """side x side x 3 spheres, two workers"""
+    from paper_2403_17261_gb300 import scenes as S
+    pos = S._lattice_pile(side, side, 3, 1.0, 0.5, 0.01, rng)
+    n = pos.shape[0]
+    return S._single("p", pos, np.full(n, 0.5), np.ones(n), [[0, 0, 1, 0]], mu=0.5, dt=1 / 60, flags=1, gamma=1, beta=4, n_sets=2,
+                     set_of_body=(np.arange(n) * 2) // n)
+
+
 def _batch(n_scenes, iters=8):
-    """small piles of uneven sizes, two workers each"""
+    """small piles of uneven sizes"""
     from paper_2403_17261_gb300 import scenes as S
     rng = S.SplitMix64(3)
-    parts = []
-    for k in range(n_scenes):
-        side = 2 + k % 5
-        pos = S._lattice_pile(side, side, 3, 1.0, 0.5, 0.01, rng)
-        n = pos.shape[0]
-        parts.append(S._single(f"p{k}", pos, np.full(n, 0.5), np.ones(n), [[0, 0, 1, 0]], mu=0.5, dt=1 / 60, flags=1, gamma=1,
-                               beta=4, n_sets=2, set_of_body=(np.arange(n) * 2) // n))
-    sc = S.concat_scenes("batch", parts, iters=iters)
+    sc = S.concat_scenes("batch", [_pile(2 + k % 5, rng) for k in range(n_scenes)], iters=iters)
     sc.state[:, 7:13] = rng.uniform(6 * sc.n_bodies, -0.3, 0.3).reshape(-1, 6).astype(np.float32)
     return sc
 
@@ -56,5 +58,33 @@ def test_box_batch():
     ref, st = _run(sc, {}, 3)
     assert st["solve_ctas_masses"] == st["solve_ctas"] >= 180
     for par in (dict(smem_slot_limit=5000), dict(pgs_cluster=2), dict(pgs_threads=32), dict(pgs_cluster=1, pgs_threads=512)):
+        out, _ = _run(sc, par, 3)
+        assert np.array_equal(out, ref), par
+
+
+def _with_boxes(sc, share, seed=5):
+    """turns a share of a pile's spheres into cubes of their width (the radius then bounds the cube)"""
+    from paper_2403_17261_gb300 import scenes as S
+    rng = S.SplitMix64(seed)
+    pick = rng.uniform(sc.n_bodies) < share
+    sc.half_extents = np.where(pick[:, None], 0.9 * sc.radius[:, None], 0.0).repeat(3, 1).astype(np.float32)
+    sc.radius = np.where(pick, 1.6 * sc.radius, sc.radius).astype(np.float32)
+    return sc
+
+
+@pytest.mark.parametrize("n_scenes", [1, 60])
+def test_workers_with_no_few_and_many_boxes(n_scenes):
+    """one context with all kinds of workers, on one CTA per SM and on two, in clusters and without the masses"""
+    from paper_2403_17261_gb300 import scenes as S
+    rng = S.SplitMix64(7)
+    parts = [_with_boxes(_pile(side, rng), share, 5 + j) for share in (0.0, 0.02, 0.3, 1.0) for j in range(n_scenes)
+             for side in ((4, 5) if n_scenes > 1 else (9, 22))]
+    he = np.concatenate([p.half_extents for p in parts])
+    sc = S.concat_scenes("kinds", parts, iters=8)
+    sc.half_extents = he
+    sc.state[:, 7:13] = rng.uniform(6 * sc.n_bodies, -0.3, 0.3).reshape(-1, 6).astype(np.float32)
+    ref, st = _run(sc, {}, 3)
+    assert st["solve_ctas_masses"] == st["solve_ctas"]
+    for par in (dict(smem_slot_limit=5000), dict(pgs_cluster=2), dict(pgs_cluster=1, pgs_threads=64), dict(pgs_cluster=4, smem_slot_limit=10)):
         out, _ = _run(sc, par, 3)
         assert np.array_equal(out, ref), par

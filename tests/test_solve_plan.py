@@ -18,6 +18,8 @@ int dynamic_bytes(int budget, long long slots, long long rows, long long stage) 
 int takes_masses(int threads, long long ctas, int sms, int per_sm, long long slots) {
     return ovl::solve_takes_masses(threads, ctas, sms, per_sm, slots);
 }
+int full_kind(long long full, long long rows, int bodies) { return ovl::solve_full_kind(full, rows, bodies); }
+double grow_rows(long long full, long long rows, int bodies) { return ovl::solve_grow_rows(full, rows, bodies); }
 int box_threads(int threads, int ctas_per_sm) { return ovl::solve_box_threads(threads, ctas_per_sm); }
 int slot_capacity(int optin, int per_sm, int ctas, int masses) { return ovl::solve_slot_capacity(optin, per_sm, ctas, masses); }
 long long most_room(const int *b, const int *q, int P, int C) { return ovl::solve_most_room(b, q, P, C); }
@@ -37,6 +39,8 @@ def plan(tmp_path_factory):
     lib = ctypes.CDLL(str(so))
     L = ctypes.c_longlong
     lib.dynamic_bytes.argtypes = [ctypes.c_int, L, L, L]
+    lib.full_kind.argtypes = lib.grow_rows.argtypes = [L, L, ctypes.c_int]
+    lib.grow_rows.restype = ctypes.c_double
     lib.takes_masses.argtypes = [ctypes.c_int, L, ctypes.c_int, ctypes.c_int, L]
     lib.most_room.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
     lib.most_room.restype = L
@@ -122,3 +126,27 @@ def test_box_ctas_leave_room_for_their_stages(plan, threads, ctas, want):
     """two CTAs per SM: 128 threads, whose two stages of 16 records take 64 KB of the half SM's 110"""
     assert plan.box_threads(threads, ctas) == want
     assert 2 * 16 * 16 * want < (232448 if ctas == 1 else 233472 // 2 - 3584)
+
+
+@pytest.mark.parametrize("full,rows,bodies,kind", [
+    (0, 40_000, 14_000, 0),       # no box end: the spheres' kernel
+    (1, 40_000, 14_000, 1),       # one box does not change its worker's launch
+    (2000, 40_000, 14_000, 1),
+    (28_000, 40_000, 14_000, 2),
+    (250, 1000, 300, 2),
+    (249, 1000, 300, 1),
+    (250, 1000, 1001, 1),
+    (4200, 4200, 170, 2),         # the building
+])
+def test_full_rows_of_a_worker(plan, full, rows, bodies, kind):
+    assert plan.full_kind(full, rows, bodies) == kind
+
+
+@pytest.mark.parametrize("full,rows,bodies,want", [
+    (0, 5000, 1700, 5000.0),
+    (500, 3000, 1100, 5500.0),
+    (500, 2400, 1100, 2400.0),
+    (4200, 4200, 170, 4200.0),
+])
+def test_full_rows_weigh_in_the_growth(plan, full, rows, bodies, want):
+    assert plan.grow_rows(full, rows, bodies) == want
