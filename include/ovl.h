@@ -152,9 +152,9 @@ typedef struct ovl_stats {
                                   workers do not outnumber the SMs, and the phases then add up to
                                   more than the total (index 9) */
     int64_t n_launches;        /* CUDA kernels the library launched during the last step */
-    int32_t solve_cluster;     /* CTAs per worker of the last solve */
-    int32_t solve_threads;     /* threads per CTA of the last solve */
-    int32_t solve_rows_per_thread; /* rows a thread takes at once in a colour (colour block) */
+    int32_t solve_cluster;     /* CTAs per worker of the last solve (the most of its launches) */
+    int32_t solve_threads;     /* threads per CTA of the last solve (of its launch with the most CTAs) */
+    int32_t solve_rows_per_thread; /* rows a thread of that launch takes at once in a colour */
     int32_t colour_rounds_max; /* most colouring rounds any worker needed */
     int64_t lb_candidates;     /* contacts handed to the host load balance in the last step */
     double lb_host_ms;         /* host time of the load balance in the last step (copies included) */

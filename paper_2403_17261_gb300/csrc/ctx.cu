@@ -813,7 +813,8 @@ bool uniform_masses(const ovl_ctx *c, const SolvePlan &pl) {
 
 // threads of a uniform launch's CTAs
 int uniform_threads(const ovl_ctx *c, const SolvePlan &pl, bool masses) {
-    return full_kind(c) == FULL_MOST && masses ? solve_box_threads(pl.threads, solve_ctas_per_sm(pl.unroll)) : pl.threads;
+    const int t = std::min(pl.threads, SOLVE_THREADS);
+    return full_kind(c) == FULL_MOST && masses ? solve_box_threads(t, solve_ctas_per_sm(pl.unroll)) : t;
 }
 
 // Every worker's CTA count goes to the device and the rows of every colour
@@ -861,14 +862,18 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
     c->last_ctas = c->last_ctas_masses = 0;
     if (pl.shape >= 0) {
         launch_solve_classes(c, a, kSolveShapes[pl.shape], pl.classes);
+        long long largest = -1;
         for (const SolveClass &k : pl.classes) {
-            c->last_ctas += (long long)k.C * k.count;
-            if (k.masses) c->last_ctas_masses += (long long)k.C * k.count;
+            const long long ctas = (long long)k.C * k.count;
+            c->last_ctas += ctas;
+            if (k.masses) c->last_ctas_masses += ctas;
+            if (ctas <= largest) continue;
+            largest = ctas;
+            c->last_threads = class_threads(c, kSolveShapes[pl.shape], k);
+            c->last_rows_at_once = solve_rows_at_once(k.masses, k.full, kSolveShapes[pl.shape].unroll);
         }
         c->last_cluster = pl.classes.front().C;
         c->last_plan_per_worker = true;
-        c->last_threads = kSolveShapes[pl.shape].threads;
-        c->last_unroll = kSolveShapes[pl.shape].unroll;
         return;
     }
     a.smem_slots = pl.slots;
@@ -880,14 +885,14 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
     a.smem_room = solve_most_room(c->h_pb.data(), c->h_pp.data(), P, pl.cluster);
     if (full_kind(c) == FULL_NONE) a.row_full = nullptr;
     a.few = full_kind(c) == FULL_FEW;
-    launch_solve(a, uniform_threads(c, pl, masses), pl.cluster, pl.unroll, masses,
+    c->last_threads = uniform_threads(c, pl, masses);
+    c->last_rows_at_once = solve_rows_at_once(masses, full_kind(c), pl.unroll);
+    launch_solve(a, c->last_threads, pl.cluster, pl.unroll, masses,
                  solve_smem_budget(c, solve_ctas_per_sm(pl.unroll), true), c->stream);
     c->last_ctas = (long long)pl.cluster * P;
     c->last_ctas_masses = masses ? c->last_ctas : 0;
     c->last_cluster = pl.cluster;
     c->last_plan_per_worker = false;
-    c->last_threads = pl.threads;
-    c->last_unroll = pl.unroll;
 }
 
 // K13: time every feasible uniform launch (CTAs per worker, threads per CTA,
@@ -1701,7 +1706,7 @@ ovl_status ovl_read_stats(ovl_ctx *c, ovl_stats *out) {
         out->n_launches = c->last_launches;
         out->solve_cluster = c->last_cluster;
         out->solve_threads = c->last_threads;
-        out->solve_rows_per_thread = c->last_unroll;
+        out->solve_rows_per_thread = c->last_rows_at_once;
         out->solve_ctas = c->last_ctas;
         out->solve_ctas_masses = c->last_ctas_masses;
         out->lb_candidates = c->lb_candidates;

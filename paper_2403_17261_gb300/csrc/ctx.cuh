@@ -24,7 +24,7 @@ struct ovl_ctx {
     int num_sms = 0;
     int smem_per_sm = 0;
     int nb_max = 0;          // most bodies in one worker (last membership phase)
-    int last_cluster = 1, last_threads = 512, last_unroll = 1;
+    int last_cluster = 1, last_threads = 512, last_rows_at_once = 1;   // threads and rows: of the launch with the most CTAs
     bool last_plan_per_worker = false;   // the last solve used h_class_C (else last_cluster for all)
     long long last_ctas = 0, last_ctas_masses = 0;   // CTAs of the last solve, those with masses in shared memory
     // a tuned solve launch: uniform (cluster > 0) or per-worker plan (shape = 1 + its index)

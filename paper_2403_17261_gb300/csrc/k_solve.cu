@@ -57,8 +57,6 @@ namespace ovl {
 
 namespace {
 
-constexpr int SOLVE_THREADS = 512;
-
 // The file is built without FMA contraction, and its fused multiply-adds are
 // written out (fmaf): every instantiation (cluster size, rows per thread,
 // slot layout, CTA width) then rounds the same way and gives the same bits.
@@ -1256,7 +1254,6 @@ static void launch_solve_masses(const SolveArgs &a, int threads, int cluster, in
 
 void launch_solve(const SolveArgs &a, int threads, int cluster, int unroll, bool masses, int budget, cudaStream_t s) {
     if (!a.n_parts) return;
-    if (threads > SOLVE_THREADS) threads = SOLVE_THREADS;
     if (masses) {
         if (!a.row_full) launch_solve_masses<FULL_NONE>(a, threads, cluster, budget, s);
         else if (a.few) launch_solve_masses<FULL_FEW>(a, threads, cluster, budget, s);

@@ -5,6 +5,8 @@
 
 namespace ovl {
 
+constexpr int SOLVE_THREADS = 512;   // most threads of a CTA
+
 // bytes of one shared-memory body slot: with the inverse mass and inertia, or without
 constexpr int solve_slot_bytes(bool masses) { return masses ? 32 : 24; }
 
@@ -90,6 +92,12 @@ inline int solve_full_kind(long long full, long long rows, int bodies) {
 // 0.87 and 0.63; spheres cross at 5000.)
 inline double solve_grow_rows(long long full, long long rows, int bodies) {
     return solve_full_kind(full, rows, bodies) == FULL_FEW && rows >= 2500 ? rows + 5.0 * full : (double)rows;
+}
+
+// Rows a thread takes at once in a colour: with the masses one (k_solve_m), the
+// kernels with full rows that read the masses two, else what the shape asks for.
+inline int solve_rows_at_once(bool masses, int full, int rows_per_thread) {
+    return masses ? 1 : (full != FULL_NONE ? 2 : rows_per_thread);
 }
 
 // Threads of a CTA that keeps the masses of a worker of boxes: at most 256

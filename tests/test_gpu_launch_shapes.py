@@ -88,3 +88,18 @@ def test_workers_with_no_few_and_many_boxes(n_scenes):
     for par in (dict(smem_slot_limit=5000), dict(pgs_cluster=2), dict(pgs_cluster=1, pgs_threads=64), dict(pgs_cluster=4, smem_slot_limit=10)):
         out, _ = _run(sc, par, 3)
         assert np.array_equal(out, ref), par
+
+
+def test_stats_name_the_launch():
+    """threads and rows at once as the kernels ran them, not as the plan's shape table has them"""
+    from paper_2403_17261_gb300 import scenes as S
+    seen = lambda sc, par: tuple(_run(sc, par, 1)[1][k] for k in ("solve_threads", "solve_rows_per_thread"))
+    pile, building = S.pile_small(), S.box_building(storeys=2, cells=3, n_sets=3, iters=4)
+    assert seen(pile, {}) == (512, 1)
+    assert seen(pile, dict(pgs_threads=1024)) == (512, 1)
+    assert seen(pile, dict(pgs_threads=96)) == (96, 1)
+    assert seen(pile, dict(smem_slot_limit=5000)) == (512, 2)
+    assert seen(building, {}) == (256, 1)
+    assert seen(building, dict(pgs_cluster=1)) == (128, 1)
+    assert seen(building, dict(smem_slot_limit=5000)) == (512, 2)
+    assert seen(_batch(350), {}) == (128, 1)
