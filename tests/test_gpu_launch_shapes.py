@@ -103,3 +103,23 @@ def test_stats_name_the_launch():
     assert seen(building, dict(pgs_cluster=1)) == (128, 1)
     assert seen(building, dict(smem_slot_limit=5000)) == (512, 2)
     assert seen(_batch(350), {}) == (128, 1)
+
+
+@pytest.mark.parametrize("boxes,most", [(False, 11), (True, 15)])
+def test_autotuner_times_a_launch_once(boxes, most):
+    """four cluster sizes, two thread counts and two row counts come to the same launches where the masses are kept: one row at
+    a time, room enough with one CTA per SM or two; for boxes 128 threads where two share an SM, 256 and 512 the same otherwise.
+    A candidate is three kernels (row order, row build, solve); three plans are timed too."""
+    from paper_2403_17261_gb300 import ovl
+    from paper_2403_17261_gb300 import scenes as S
+    sc = S.box_building(storeys=2, cells=3, n_sets=3, iters=4) if boxes else S.pile_small()
+    sim = ovl.Simulation(sc, dict(flags=ovl.OVL_FLAG_AUTOTUNE))
+    state = sim.state()
+    n = []
+    for _ in range(2):
+        sim.set_state(state)
+        sim.set_step_index(0)
+        sim.step()
+        n.append(sim.stats()["n_launches"])
+    sim.close()
+    assert n[0] - n[1] <= 3 * most + 3
