@@ -169,11 +169,10 @@ ovl_status ovl_load(ovl_ctx *c, const void *buf, size_t len) {
         give(c->ws_lam.p, sizeof(float4) * (size_t)h.ws_n);
         if (h.mlp_ready) {
             c->mlp_theta.ensure(OVL_MLP_N_PARAMS); c->mlp_m.ensure(OVL_MLP_N_PARAMS); c->mlp_v.ensure(OVL_MLP_N_PARAMS);
-            c->mlp_packed.ensure(MLP_PK_WORDS);
             give(c->mlp_theta.p, sizeof(float) * OVL_MLP_N_PARAMS);
             give(c->mlp_m.p, sizeof(float) * OVL_MLP_N_PARAMS);
             give(c->mlp_v.p, sizeof(float) * OVL_MLP_N_PARAMS);
-            launch_mlp_pack(c->mlp_theta.p, c->mlp_packed.p, c->stream);
+            pack_parameters(c);
         }
         CK(cudaStreamSynchronize(c->stream));
         const std::string tune(p, (size_t)h.tune_bytes);

@@ -156,7 +156,7 @@ struct ovl_ctx {
     DBuf<double> loss_acc;
     DBuf<float> train_c12;            // Adam bias corrections per step of a training call
     DBuf<long long> train_step;       // step counter of a training call (graph replay), scratch
-    DBuf<uint32_t> train_packed;      // BF16 operands of a training call
+    DBuf<uint32_t> train_packed;      // the parameters as BF16 operands of training (mlp_packed: of inference)
 };
 
 namespace ovl {
@@ -206,5 +206,7 @@ ovl_status check_device_status(ovl_ctx *c);
 void phase_warmstart(ovl_ctx *c, float dt_override);
 void phase_log(ovl_ctx *c);
 void release_mlp(ovl_ctx *c);
+// the operands of inference and training from new parameters (mlp_theta)
+void pack_parameters(ovl_ctx *c);
 
 }  // namespace ovl

@@ -19,7 +19,6 @@ bool features_needed(const ovl_ctx *c) {
 }
 
 void ensure_train_buffers(ovl_ctx *c, int batch) {
-    c->train_packed.ensure(MLP_TRAIN_PK_WORDS);
     c->train_sample_loss.ensure((size_t)batch);
     c->train_partials.ensure((size_t)train_blocks(batch) * (MLP_N_PARAMS + 1));
     c->mlp_grad.ensure(MLP_N_PARAMS);
@@ -47,6 +46,13 @@ void check_log_range(const ovl_ctx *c, long long first, long long count) {
 }
 
 }  // namespace
+
+void pack_parameters(ovl_ctx *c) {
+    c->mlp_packed.ensure(MLP_PK_WORDS);
+    c->train_packed.ensure(MLP_TRAIN_PK_WORDS);
+    launch_mlp_pack(c->mlp_theta.p, c->mlp_packed.p, c->stream);
+    launch_train_pack(c->mlp_theta.p, c->train_packed.p, c->stream);
+}
 
 void phase_warmstart(ovl_ctx *c, float dt_override) {
     c->feat_valid = false;
@@ -144,8 +150,7 @@ ovl_status ovl_mlp_set_params(ovl_ctx *c, const float *theta, int32_t n) {
         c->mlp_m.ensure(n); c->mlp_v.ensure(n);
         CK(cudaMemsetAsync(c->mlp_m.p, 0, sizeof(float) * n, c->stream));
         CK(cudaMemsetAsync(c->mlp_v.p, 0, sizeof(float) * n, c->stream));
-        c->mlp_packed.ensure(MLP_PK_WORDS);
-        launch_mlp_pack(c->mlp_theta.p, c->mlp_packed.p, c->stream);
+        pack_parameters(c);
         CK(cudaStreamSynchronize(c->stream));
         c->adam_t = 0;
         c->mlp_ready = true;
@@ -262,7 +267,6 @@ ovl_status ovl_mlp_train(ovl_ctx *c, const ovl_train_desc *d, float *loss_per_st
         upload(c->train_c12, c12.data(), c12.size(), c->stream);
         c->train_step.ensure(2);
         CK(cudaMemsetAsync(c->train_step.p, 0, 2 * sizeof(long long), c->stream));
-        launch_train_pack(c->mlp_theta.p, c->train_packed.p, c->stream);
         const int blocks = train_blocks(d->batch);
         TrainArgs a = train_args(c, d->first, d->count, d->batch, d->sampling, d->seed, 0, 1);
         a.step_dev = c->train_step.p;
@@ -299,6 +303,7 @@ ovl_status ovl_mlp_train(ovl_ctx *c, const ovl_train_desc *d, float *loss_per_st
         }
         for (; done < steps; ++done) one_step(c->stream);
         c->adam_t += steps;
+        // every step left its training operands packed
         launch_mlp_pack(c->mlp_theta.p, c->mlp_packed.p, c->stream);
         if (loss_per_step && d->steps > 0) download(loss_per_step, c->train_loss_hist.p, (size_t)d->steps, c->stream);
         CK(cudaStreamSynchronize(c->stream));
@@ -314,7 +319,6 @@ ovl_status ovl_mlp_grad(ovl_ctx *c, int64_t first, int64_t count, float *grad, d
         const int batch = (int)count;
         ensure_train_buffers(c, batch);
         TrainArgs a = train_args(c, first, count, batch, 0, 0, 0, 1);
-        launch_train_pack(c->mlp_theta.p, c->train_packed.p, c->stream);
         launch_train_grad(a, c->stream);
         launch_train_reduce(c->train_partials.p, train_blocks(batch), batch, c->mlp_grad.p,
                             c->mlp_loss.p, 0, nullptr, nullptr, nullptr, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f,
@@ -336,7 +340,6 @@ ovl_status ovl_mlp_loss(ovl_ctx *c, int64_t first, int64_t count, double *loss) 
         ensure_train_buffers(c, kLossChunk);
         c->loss_acc.ensure(1);
         CK(cudaMemsetAsync(c->loss_acc.p, 0, sizeof(double), c->stream));
-        launch_train_pack(c->mlp_theta.p, c->train_packed.p, c->stream);
         for (long long off = 0; off < count; off += kLossChunk) {
             const int b = (int)std::min<long long>(kLossChunk, count - off);
             TrainArgs a = train_args(c, first + off, b, b, 0, 0, 0, 0);
