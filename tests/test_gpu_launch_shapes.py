@@ -123,3 +123,24 @@ def test_autotuner_times_a_launch_once(boxes, most):
         n.append(sim.stats()["n_launches"])
     sim.close()
     assert n[0] - n[1] <= 3 * most + 3
+
+
+@pytest.mark.parametrize("share", [0.0, 0.01])
+def test_impulses_in_global_memory(share):
+    """the masses in shared memory, the impulses not: two CTAs of some 5000 bodies and 10,000 rows each, spheres alone or with a
+    few boxes.  One slot per body and 12 B per row are more than the 229,888 B a CTA may use."""
+    from paper_2403_17261_gb300 import scenes as S
+    rng = S.SplitMix64(11)
+    pos = S._lattice_pile(22, 22, 21, 1.0, 0.5, 0.02, rng)
+    n = pos.shape[0]
+    sc = S._single("pile", pos, rng.uniform(n, 0.45, 0.52), rng.uniform(n, 0.5, 2.0), [[0, 0, 1, 0]], mu=0.5, dt=1 / 60, flags=1,
+                   gamma=1, beta=4, n_sets=1, set_of_body=np.zeros(n, int), iters=12)
+    sc.state[:, 7:13] = rng.uniform(6 * n, -0.3, 0.3).reshape(n, 6).astype(np.float32)
+    if share:
+        sc = _with_boxes(sc, share)
+    out, st = _run(sc, dict(pgs_cluster=2))
+    assert st["solve_ctas_masses"] == st["solve_ctas"] == 2
+    assert 32 * (n // 2 + 1) + 12 * (st["n_pairs"] // 2) > 229888
+    for par in ({}, dict(pgs_cluster=8), dict(pgs_cluster=4, smem_slot_limit=6000)):
+        other, st = _run(sc, par)
+        assert np.array_equal(other, out), par
