@@ -451,7 +451,7 @@ constexpr int kSmallPerSm = 5, kSmallThreads = 128;
 // launch classes of a CTA-count plan: workers with equal counts, most CTAs
 // first and longest first inside; the worker order goes to buf
 void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveClass> &classes,
-                       DBuf<uint32_t> &buf, bool split) {
+                       DBuf<uint32_t> &buf, int room_budget, bool split) {
     const int P = c->n_parts;
     const std::vector<int> &pb = c->h_pb, &pp = c->h_pp;
     std::vector<int> order(P);
@@ -460,7 +460,7 @@ void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveC
     for (int p = 0; p < P; ++p) full[p] = (char)full_kind(c, p);
     if (split)
         for (int p = 0; p < P; ++p)
-            small[p] = C[p] == 1 && full[p] == FULL_NONE && solve_worker_room(pb[p + 1] - pb[p], pp[p + 1] - pp[p], 1) <=
+            small[p] = C[p] == 1 && full[p] == FULL_NONE && solve_worker_room(pb[p + 1] - pb[p], pp[p + 1] - pp[p], 1, 1ll << 62) <=
                                         c->smem_per_sm / kSmallPerSm - 3584;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         if (C[x] != C[y]) return C[x] > C[y];
@@ -479,7 +479,7 @@ void plan_classes_from(ovl_ctx *c, const std::vector<int> &C, std::vector<SolveC
         SolveClass &k = classes.back();
         k.count++;
         k.slots = std::max(k.slots, (nb + C[p] - 1) / C[p]);
-        k.room = std::max(k.room, solve_worker_room(nb, pp[p + 1] - pp[p], C[p]));
+        k.room = std::max(k.room, solve_worker_room(nb, pp[p + 1] - pp[p], C[p], room_budget));
     }
     std::vector<uint32_t> o(order.begin(), order.end());
     upload(buf, o.data(), o.size(), c->stream);
@@ -490,7 +490,7 @@ bool plan_worker_classes(ovl_ctx *c, int cap, long long budget, std::vector<Solv
                          DBuf<uint32_t> &buf) {
     const std::vector<int> C = plan_worker_counts(c, cap, budget);
     if (C.empty() && c->n_parts > 0) return false;
-    plan_classes_from(c, C, classes, buf, false);
+    plan_classes_from(c, C, classes, buf, 0, false);
     return true;
 }
 
@@ -529,7 +529,8 @@ bool plan_solve_classes(ovl_ctx *c, const SolveShape &shape, std::vector<SolveCl
     const std::vector<int> C = plan_worker_counts(c, cap, budget);
     if (C.empty() && c->n_parts > 0) return false;
     // workers of boxes, and a slot limit, keep one shape
-    plan_classes_from(c, C, classes, c->class_order, shape.per_sm > 1 && c->P.smem_slot_limit <= 0);
+    plan_classes_from(c, C, classes, c->class_order, solve_smem_budget(c, shape.per_sm, true),
+                      shape.per_sm > 1 && c->P.smem_slot_limit <= 0);
     const long long ctas = std::accumulate(C.begin(), C.end(), 0ll);
     for (SolveClass &k : classes)
         k.masses = solve_masses_fit(c, k.slots, shape.per_sm) &&
@@ -884,13 +885,13 @@ void launch_solve_plan(ovl_ctx *c, const SolvePlan &pl, float dt_override, int i
     // the largest worker's rows, not all workers': many small workers then
     // share an SM (600 scenes of two workers: solve 0.60 -> 0.27 ms with 64
     // threads per CTA, 0.55 -> 0.32 with 128)
-    a.smem_room = solve_most_room(c->h_pb.data(), c->h_pp.data(), P, pl.cluster);
+    const int budget = solve_smem_budget(c, solve_ctas_per_sm(pl.unroll), true);
+    a.smem_room = solve_most_room(c->h_pb.data(), c->h_pp.data(), P, pl.cluster, budget);
     if (full_kind(c) == FULL_NONE) a.row_full = nullptr;
     a.few = full_kind(c) == FULL_FEW;
     c->last_threads = uniform_threads(c, pl, masses);
     c->last_rows_at_once = solve_rows_at_once(masses, full_kind(c), pl.unroll);
-    launch_solve(a, c->last_threads, pl.cluster, pl.unroll, masses,
-                 solve_smem_budget(c, solve_ctas_per_sm(pl.unroll), true), c->stream);
+    launch_solve(a, c->last_threads, pl.cluster, pl.unroll, masses, budget, c->stream);
     c->last_ctas = (long long)pl.cluster * P;
     c->last_ctas_masses = masses ? c->last_ctas : 0;
     c->last_cluster = pl.cluster;
@@ -928,8 +929,9 @@ void autotune(ovl_ctx *c, float dt_override, int iters, const std::string &key) 
                 const bool masses = uniform_masses(c, pl);
                 pl.threads = uniform_threads(c, pl, masses);
                 const int rows = solve_rows_at_once(masses, full_kind(c), un);
-                const int bytes = masses ? solve_dynamic_bytes(solve_smem_budget(c, solve_ctas_per_sm(un), true),
-                                                               solve_most_room(c->h_pb.data(), c->h_pp.data(), c->n_parts, cl), 0) : 0;
+                const int budget = solve_smem_budget(c, solve_ctas_per_sm(un), true);
+                const int bytes = masses ? solve_dynamic_bytes(
+                    budget, solve_most_room(c->h_pb.data(), c->h_pp.data(), c->n_parts, cl, budget), 0) : 0;
                 if (!timed.insert({cl, pl.threads, rows, bytes}).second) continue;
                 const float ms = time_plan(pl);
                 if (ms < best.ms) best = {cl, pl.threads, un, ms, 0};

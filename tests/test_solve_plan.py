@@ -13,7 +13,7 @@ EXPORTS = r"""
 #include "csrc/solve_plan.h"
 extern "C" {
 int dynamic_bytes(int budget, long long slots, long long rows, long long stage) {
-    return ovl::solve_dynamic_bytes(budget, ovl::solve_worker_room((int)slots, rows, 1), stage);
+    return ovl::solve_dynamic_bytes(budget, ovl::solve_worker_room((int)slots, rows, 1, 1ll << 62), stage);
 }
 int takes_masses(int threads, long long ctas, int sms, int per_sm, long long slots) {
     return ovl::solve_takes_masses(threads, ctas, sms, per_sm, slots);
@@ -22,7 +22,8 @@ int full_kind(long long full, long long rows, int bodies) { return ovl::solve_fu
 double grow_rows(long long full, long long rows, int bodies) { return ovl::solve_grow_rows(full, rows, bodies); }
 int box_threads(int threads, int ctas_per_sm) { return ovl::solve_box_threads(threads, ctas_per_sm); }
 int slot_capacity(int optin, int per_sm, int ctas, int masses) { return ovl::solve_slot_capacity(optin, per_sm, ctas, masses); }
-long long most_room(const int *b, const int *q, int P, int C) { return ovl::solve_most_room(b, q, P, C); }
+long long most_room(const int *b, const int *q, int P, int C) { return ovl::solve_most_room(b, q, P, C, 1ll << 62); }
+long long worker_room(int nb, long long np, int C, long long budget) { return ovl::solve_worker_room(nb, np, C, budget); }
 }
 """
 
@@ -42,6 +43,8 @@ def plan(tmp_path_factory):
     lib.full_kind.argtypes = lib.grow_rows.argtypes = [L, L, ctypes.c_int]
     lib.grow_rows.restype = ctypes.c_double
     lib.takes_masses.argtypes = [ctypes.c_int, L, ctypes.c_int, ctypes.c_int, L]
+    lib.worker_room.argtypes = [ctypes.c_int, L, ctypes.c_int, L]
+    lib.worker_room.restype = L
     lib.most_room.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int]
     lib.most_room.restype = L
     return lib
@@ -150,3 +153,12 @@ def test_full_rows_of_a_worker(plan, full, rows, bodies, kind):
 ])
 def test_full_rows_weigh_in_the_growth(plan, full, rows, bodies, want):
     assert plan.grow_rows(full, rows, bodies) == want
+
+
+@pytest.mark.parametrize("nb,np,C,fits", [(1000, 16000, 1, True), (1000, 17000, 1, False), (7500, 75000, 4, False),
+                                          (7500, 56000, 4, True), (7183, 0, 1, True), (7184, 0, 1, False)])
+def test_no_room_for_impulses_that_do_not_fit(plan, nb, np, C, fits):
+    """an even share beyond the budget leaves the rest of the shared memory to the L1 cache"""
+    slots = ((nb + C - 1) // C + 1) * 32
+    rows = np if C == 1 else int(1.25 * np / C) + 64
+    assert plan.worker_room(nb, np, C, 229888) == slots + (12 * rows + 16 if fits else 0)
