@@ -415,7 +415,7 @@ std::vector<int> plan_worker_counts(ovl_ctx *c, int cap, long long budget) {
         C[p] = k;
         total += k;
     }
-    auto load = [&](int p) { return solve_grow_rows(c->h_full[p], pp[p + 1] - pp[p], pb[p + 1] - pb[p]) / C[p]; };
+    auto load = [&](int p) { return solve_grow_rows(c->h_full[p], pp[p + 1] - pp[p], pb[p + 1] - pb[p], c->nj > c->nc) / C[p]; };
     if (total <= budget) {
         std::vector<int> heap(P);
         std::iota(heap.begin(), heap.end(), 0);

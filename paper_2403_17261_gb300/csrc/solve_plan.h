@@ -91,13 +91,20 @@ inline int solve_full_kind(long long full, long long rows, int bodies) {
     return 10 * full >= 7 * rows || (4 * full >= rows && bodies <= 1000) ? FULL_MOST : FULL_FEW;
 }
 
-// Rows as the growth of a worker's CTAs counts them: where few are full, such a
-// row, read straight from global memory, costs as much as six plain ones; below
-// 2500 rows a worker has too few to share.  (One and four CTAs per worker, a
-// sixth of the rows full: 2200 rows 0.53 and 0.61 ms, 2800 0.66 and 0.61, 4300
-// 0.87 and 0.63; spheres cross at 5000.)
-inline double solve_grow_rows(long long full, long long rows, int bodies) {
-    return solve_full_kind(full, rows, bodies) == FULL_FEW && rows >= 2500 ? rows + 5.0 * full : (double)rows;
+// Rows as the growth of a worker's CTAs counts them, in rows of a pile (three
+// per body, 13 colours).  Where few are full, such a row, read straight from
+// global memory, costs as much as six plain ones; below 2500 rows a worker has
+// too few to share.  (One and four CTAs per worker, a sixth of the rows full:
+// 2200 rows 0.53 and 0.61 ms, 2800 0.66 and 0.61, 4300 0.87 and 0.63; spheres
+// cross at 5000.)  Where joints outnumber contacts the colours are few, about
+// 2.9 per row and body, so a worker has more rows in each (a chain, one CTA and
+// four: 1100 rows 0.13 and 0.15 ms, 2200 0.21 and 0.15, 4400 0.39 and 0.18).
+// Contacts alone do not say so: the fullest body sets the colours.
+inline double solve_grow_rows(long long full, long long rows, int bodies, bool jointed) {
+    const int kind = solve_full_kind(full, rows, bodies);
+    if (kind == FULL_MOST) return (double)rows;
+    const double plain = kind == FULL_FEW && rows >= 2500 ? rows + 5.0 * full : (double)rows;
+    return jointed && rows > 0 ? plain * std::max(1.0, 13.5 / 2.9 * bodies / rows) : plain;
 }
 
 // Rows a thread takes at once in a colour: with the masses one (k_solve_m), the

@@ -19,7 +19,7 @@ int takes_masses(int threads, long long ctas, int sms, int per_sm, long long slo
     return ovl::solve_takes_masses(threads, ctas, sms, per_sm, slots);
 }
 int full_kind(long long full, long long rows, int bodies) { return ovl::solve_full_kind(full, rows, bodies); }
-double grow_rows(long long full, long long rows, int bodies) { return ovl::solve_grow_rows(full, rows, bodies); }
+double grow_rows(long long full, long long rows, int bodies, int jointed) { return ovl::solve_grow_rows(full, rows, bodies, jointed); }
 int box_threads(int threads, int ctas_per_sm) { return ovl::solve_box_threads(threads, ctas_per_sm); }
 int slot_capacity(int optin, int per_sm, int ctas, int masses) { return ovl::solve_slot_capacity(optin, per_sm, ctas, masses); }
 long long most_room(const int *b, const int *q, int P, int C) { return ovl::solve_most_room(b, q, P, C, 1ll << 62); }
@@ -40,7 +40,8 @@ def plan(tmp_path_factory):
     lib = ctypes.CDLL(str(so))
     L = ctypes.c_longlong
     lib.dynamic_bytes.argtypes = [ctypes.c_int, L, L, L]
-    lib.full_kind.argtypes = lib.grow_rows.argtypes = [L, L, ctypes.c_int]
+    lib.full_kind.argtypes = [L, L, ctypes.c_int]
+    lib.grow_rows.argtypes = [L, L, ctypes.c_int, ctypes.c_int]
     lib.grow_rows.restype = ctypes.c_double
     lib.takes_masses.argtypes = [ctypes.c_int, L, ctypes.c_int, ctypes.c_int, L]
     lib.worker_room.argtypes = [ctypes.c_int, L, ctypes.c_int, L]
@@ -145,14 +146,19 @@ def test_full_rows_of_a_worker(plan, full, rows, bodies, kind):
     assert plan.full_kind(full, rows, bodies) == kind
 
 
-@pytest.mark.parametrize("full,rows,bodies,want", [
-    (0, 5000, 1700, 5000.0),
-    (500, 3000, 1100, 5500.0),
-    (500, 2400, 1100, 2400.0),
-    (4200, 4200, 170, 4200.0),
+@pytest.mark.parametrize("full,rows,bodies,jointed,want", [
+    (0, 5000, 1700, 0, 5000.0),
+    (500, 3000, 1100, 0, 5500.0),
+    (500, 2400, 1100, 0, 2400.0),
+    (4200, 4200, 170, 0, 4200.0),
+    (4200, 4200, 170, 1, 4200.0),
+    (0, 2200, 1250, 0, 2200.0),               # few rows per body, but the fullest body sets the colours
+    (0, 2200, 1250, 1, 13.5 / 2.9 * 1250),    # a chain: five colours where a pile has 13
+    (0, 60_000, 10_000, 1, 60_000.0),
+    (0, 0, 0, 1, 0.0),
 ])
-def test_full_rows_weigh_in_the_growth(plan, full, rows, bodies, want):
-    assert plan.grow_rows(full, rows, bodies) == want
+def test_rows_in_the_growth(plan, full, rows, bodies, jointed, want):
+    assert plan.grow_rows(full, rows, bodies, jointed) == pytest.approx(want, rel=1e-12)
 
 
 @pytest.mark.parametrize("nb,np,C,fits", [(1000, 16000, 1, True), (1000, 17000, 1, False), (7500, 75000, 4, False),
