@@ -346,8 +346,9 @@ bool solve_masses_fit(const ovl_ctx *c, int slots, int ctas_per_sm) {
 // Per-worker CTA counts for the default launch: every worker starts at the
 // fewest CTAs (1, 2, 3, 4, 6 or 8) whose shares of its bodies fit one CTA's
 // shared memory; while all CTAs still fit the SMs, the worker with the most
-// rows per CTA moves to the next count while kGrow allows.  Workers with the same count form one launch, and
-// the launches run side by side on the context's streams.  Every launch
+// rows per CTA moves to the next count while kGrow allows.  Workers with the
+// same count (and kind of rows) form one launch, and the launches run side by
+// side on the context's streams.  Every launch
 // shape gives the same bits (no implicit FMA contraction in the solver),
 // so the plan changes only the time.  Returns false when some worker does
 // not fit even 8 CTAs (the uniform launch then takes it to global memory).
@@ -357,9 +358,9 @@ struct SolveClass { int C, first, count, slots; long long room; bool small, mass
 // so a launch that claims every SM can leave a cluster waiting for a second
 // wave.
 constexpr int kSolveSmSlack = 8;
-// A worker grows past one CTA above the first number of constraints, and
-// further, up to four, while its CTAs hold more than the second each (boxes have more colours,
-// so fewer rows in each).  A
+// A worker grows past one CTA above the first number of constraints (as
+// solve_grow_rows counts them), and further, up to four, while its CTAs hold
+// more than the second each (boxes have more colours, so fewer rows in each).  A
 // colour step of one CTA costs about 900 cycles plus 3 per row; a cluster
 // adds its barrier (560 cycles against 95) and the traffic between its CTAs
 // (6 B per cycle), which fewer rows have to pay for.  Measured solves: 2
@@ -375,8 +376,6 @@ constexpr int kMaxGrow = 4;
 struct SolveShape { int threads, unroll, per_sm; };
 constexpr SolveShape kSolveShapes[3] = {{512, 2, 1}, {512, 1, 2}, {256, 2, 2}};
 
-// the shape without tuning: one CTA per SM while the workers do not
-// outnumber the SMs, else two smaller CTAs per SM
 // CTAs per worker the plans choose from (each a cluster size both the solver
 // and the colouring are built for)
 constexpr int kClusterSizes[] = {1, 2, 3, 4, 6, 8};
@@ -393,6 +392,8 @@ int full_kind(const ovl_ctx *c) {
     return all == 0 ? FULL_NONE : (2 * most >= all ? FULL_MOST : FULL_FEW);
 }
 
+// the shape without tuning: one CTA per SM while the workers do not
+// outnumber the SMs, else two smaller CTAs per SM
 int default_solve_shape(const ovl_ctx *c) { return c->n_parts <= c->num_sms ? 0 : 2; }
 
 // CTA count of every worker (shared by the colouring and the solve): the
@@ -793,11 +794,6 @@ int solve_slots_for(ovl_ctx *c, int cluster) {
     return per <= solve_slot_capacity(c, 1) ? per : 0;
 }
 
-// K13: time every feasible uniform launch (CTAs per worker, threads per CTA,
-// rows per thread and colour step) and every per-worker plan shape on this
-// step's rows and keep the fastest for the bucket.
-// Rows of one colour are independent, so every candidate computes the same
-// bits; re-running the row build restores the warm-start impulses.
 // How this step's solve is launched: per-worker classes (shape >= 0) or one
 // uniform launch.
 struct SolvePlan {

@@ -432,8 +432,6 @@ __global__ void k_log_append(const float4 *feat, const float4 *lam, const int *p
 
 // ---- training --------------------------------------------------------------------
 
-constexpr int WGRAD_CHUNK = 128;   // samples of one gradient block (one tensor-core K = 128 product)
-
 __device__ __forceinline__ long long sample_row(const TrainArgs &a, long long step, int j) {
     if (a.sampling == 0) return a.first + (long long)(((unsigned long long)step * a.batch + j) % (unsigned long long)a.count);
     const uint64_t z = mix64(a.seed + 0x9E3779B97F4A7C15ull * (uint64_t)(step * (long long)a.batch + j + 1));

@@ -353,7 +353,7 @@ __device__ __forceinline__ void solve_row(Body &A, Body &B, const Row &w, float 
 __device__ __forceinline__ float clampf(float x, float lo, float hi) { return fminf(fmaxf(x, lo), hi); }
 
 // ---- full rows (a box end: general lever arms and inertia responses) -------
-// Only the kernels of contexts with boxes (X) hold this code: in the sphere
+// Only the kernels for workers with full rows (X) hold this code: in the sphere
 // kernels its registers would add to the rows' loop, which then spills.
 template <bool X>
 __device__ __forceinline__ bool is_full(const SolveArgs &a, int r) { return X && a.row_full[r]; }
@@ -555,8 +555,6 @@ __device__ float group_sum(float v, float *red, float *slot) {
     return tot;
 }
 
-// row buckets of colour c: off[(c OWNER_RANKS + k) 2 + kind], contacts then
-// joints, for the owner ranks k in [k0, k1)
 // Row buckets of this CTA: bucket k of colour c spans rows [tab[c cs + 2k],
 // tab[c cs + 2k + 2]), contacts up to tab[c cs + 2k + 1], for k < nbk.
 struct Buckets {
@@ -969,7 +967,7 @@ struct SolveRow {
 // Warm start, sweeps, residual of one CTA's rows; tab[c] = (first row, first
 // joint, end, rows of earlier colours) of colour c.  A thread's first row of
 // the next colour is loaded before the current colour is solved, its further
-// rows of a colour one ahead.  X (contexts with boxes): with stage != NULL
+// rows of a colour one ahead.  X: FULL_*; with stage != NULL (FULL_MOST)
 // the full rows among a thread's first rows of the colours are copied to
 // shared memory a colour ahead too (two stages of FULL_ROW_WORDS float4 per
 // thread), further ones of a colour come straight from global memory.
@@ -1063,8 +1061,8 @@ __device__ void sweep_rows(const SolveArgs &a, const FullRows<X> &fr, const Loca
 
 // A launch whose slots hold the masses: CTA `rank` of worker p's
 // group holds the slots [rank per, (rank + 1) per), their zero slot and, when
-// they fit, the impulses of its rows and (X) the two stages of full rows.  Latency-bound: a colour step of few
-// rows takes about 900 cycles, of which 95 are the CTA barrier (560 a
+// they fit, the impulses of its rows and (FULL_MOST) the two stages of full
+// rows.  Latency-bound: a colour step of few rows takes about 900 cycles, of which 95 are the CTA barrier (560 a
 // cluster's), the rest one row's chain; 512 threads (measured on the large
 // pile: 256 1.14 ms, 384 1.00, 512 0.94, 768 0.92 but slower on small piles).
 // X: how many rows are full.  FULL_FEW: they come straight from global memory;
@@ -1146,9 +1144,8 @@ __global__ void __launch_bounds__(X == FULL_MOST ? SOLVE_THREADS / 2 : SOLVE_THR
 
 // C CTAs per worker; a worker's slots are spread over their shared memory when
 // they fit (ceil(nb / C) <= smem_slots), else CTA rank 0 solves it alone with
-// its body state in the global scratch area.  M: the shared-memory slots hold
-// the masses (32 B per slot; else 24 B, and rows carry the masses in r3).
-// P: rows loaded ahead (launches of SOLVE_THREADS threads, one CTA per SM).
+// its body state in the global scratch area.  24 B per slot, the rows carry the
+// masses in r3.  U: rows per thread.  P: rows loaded ahead (launches of SOLVE_THREADS threads, one CTA per SM).
 template <int C, int U, bool P, bool X>
 __global__ void __launch_bounds__(SOLVE_THREADS, U == 1 ? 2 : 1) k_solve(SolveArgs a) {
     extern __shared__ float4 sm[];
